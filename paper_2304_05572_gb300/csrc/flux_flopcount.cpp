@@ -66,13 +66,7 @@ using namespace hgks;
 template <int DIM, int STAGE, bool PRFIX>
 static void count(const char* name, int viscous, int tau_zero, bool last)
 {
-    FluxConst fc;
-    fc.gamma = 1.4; fc.gm1 = 0.4;
-    fc.K = DIM == 2 ? 3.0 : 4.0;
-    fc.Kq = fc.K.v + DIM;
-    fc.cslope = 4.0 / fc.Kq.v;
-    fc.mu = 1e-3; fc.c1 = 0.01; fc.c2 = 1.0; fc.viscous = viscous; fc.tau_zero = tau_zero;
-    fc.prfix = PRFIX ? 1.0 / 0.73 - 1.0 : 0.0;
+    const FluxConst fc = flux_const(0.4, 4.0, 1e-3, 0.01, 1.0, PRFIX ? 1.0 / 0.73 - 1.0 : 0.0, viscous, tau_zero);
     // a generic interface: distinct sides, non-zero slopes (the count does not depend on the data
     // as long as both sides and the equilibrium state are physical)
     cnt_double Wl[4] = {1.0, 0.1, 0.2, 2.5}, Wr[4] = {0.8, -0.1, 0.05, 2.0};
@@ -94,13 +88,9 @@ template <int DIM, int STAGE, bool PRFIX>
 static int values(int viscous, int tau_zero, const double* c, const double* w)
 {
     constexpr int NV = DIM + 2;
-    FluxConst fc;
-    fc.gamma = c[0]; fc.gm1 = c[0] - 1.0;
-    fc.K = DIM == 2 ? (5.0 - 3.0 * c[0]) / (c[0] - 1.0) + 1.0 : (3.0 - c[0]) / (c[0] - 1.0);
-    fc.Kq = fc.K.v + DIM;
-    fc.cslope = 4.0 / fc.Kq.v;
-    fc.mu = c[1]; fc.c1 = c[2]; fc.c2 = c[3]; fc.viscous = viscous; fc.tau_zero = tau_zero;
-    fc.prfix = PRFIX ? 1.0 / c[4] - 1.0 : 0.0;
+    // Kt: K + 1 in 2D, K in 1D
+    const double Kt = DIM == 2 ? (5.0 - 3.0 * c[0]) / (c[0] - 1.0) + 2.0 : (3.0 - c[0]) / (c[0] - 1.0);
+    const FluxConst fc = flux_const(c[0] - 1.0, Kt, c[1], c[2], c[3], PRFIX ? 1.0 / c[4] - 1.0 : 0.0, viscous, tau_zero);
     cnt_double in[6][4], o0[4], o1[4];
     for (int q = 0; q < 6; q++)
         for (int k = 0; k < 4; k++) in[q][k] = k < NV ? w[q * 4 + k] : 0.0;

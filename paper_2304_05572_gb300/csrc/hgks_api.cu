@@ -108,10 +108,11 @@ void fill_params(const hgks_config* c, Params& P)
     g.origin = (c->dim == 2 ? (long long)NG * g.pitch : 0) + NG;
     g.dx = (c->x1 - c->x0) / c->nx;
     g.dy = c->dim == 2 ? (c->y1 - c->y0) / c->ny : 1.0;
-    P.gamma = c->gamma; P.K = dof_K(c->dim, c->gamma); P.mu = c->mu; P.c1 = c->c1; P.c2 = c->c2;
+    P.gamma = c->gamma; P.mu = c->mu;
     P.cfl = c->cfl; P.fixed_dt = c->fixed_dt;
-    P.viscous = c->viscous; P.tau_zero = c->tau_zero; P.recon_mode = c->recon_mode;
-    P.prfix = (c->viscous && c->prandtl != 1.0) ? 1.0 / c->prandtl - 1.0 : 0.0;
+    P.viscous = c->viscous; P.recon_mode = c->recon_mode;
+    P.fc = flux_const(c->gamma - 1.0, dof_K(c->dim, c->gamma) + (c->dim - 1), c->mu, c->c1, c->c2,
+                      (c->viscous && c->prandtl != 1.0) ? 1.0 / c->prandtl - 1.0 : 0.0, c->viscous, c->tau_zero);
     for (int k = 0; k < 4; k++) P.bc[k] = c->bc[k];
     P.x0 = c->x0; P.y0 = c->dim == 2 ? c->y0 : 0.0;
     for (int k = 0; k < 4; k++)

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "hgks.h"
+#include "hgks_fluxconst.h"
 
 namespace hgks {
 
@@ -66,9 +67,9 @@ struct Sweep {
 
 struct Params {
     GridGeom g;
-    double gamma, K, mu, c1, c2, cfl, fixed_dt;
-    double prfix;                  // 1/Pr - 1 (viscous runs with Pr != 1), else 0
-    int viscous, tau_zero, recon_mode;
+    double gamma, mu, cfl, fixed_dt;
+    FluxConst fc;
+    int viscous, recon_mode;
     int bc[4];
     double g_ao[4], g3inv, gr[3], eps;
     double x0, y0;                 // domain origin (ghost-cell centres of the prescribed boundaries)

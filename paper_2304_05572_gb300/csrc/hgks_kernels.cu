@@ -813,6 +813,48 @@ __global__ void k_tang_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
 // ---------------------------------------------------------------- flux and update
 constexpr int kFluxMaxBlock = 256;          // largest block of a flux launch (solo 64, batched up to 256)
 
+// State Wv, normal derivative Wn and tangential derivative Wt (2D) of one side (0: left, 1: right) of
+// segment o at Gauss point g.
+template <int DIM>
+__device__ __forceinline__ void side_states(const Params& P, const Sweep& S, int side, int g, long long o,
+                                            double* Wv, double* Wn, double* Wt)
+{
+    constexpr int NV = DIM + 2;
+    if constexpr (DIM == 2) {
+        const long long per = (long long)S.nt * S.nm;
+        // the Gauss-point buffer's quantities: 0 Wl, 1 Wlx, 2 Wly, 3 Wr, 4 Wrx, 5 Wry
+        const double* gp = S.gp + (long long)((g * 6 + 3 * side) * 4) * per + o;
+        // small sweeps: every pass was reconstructed by k_tang / k_tang_ao; large sweeps: the troubled
+        // passes by k_tang_ao, the smooth ones here
+        const unsigned bits = S.tlanes == 4 ? 0xFu : (unsigned)rdc(S.flagT + o, S);
+        const int t = (int)(o / S.nm), m = (int)(o % S.nm);
+        if ((bits >> side) & 1) {
+#pragma unroll
+            for (int k = 0; k < NV; k++) {
+                Wv[k] = ldc(gp + (long long)k * per, S);
+                Wt[k] = ldc(gp + (long long)(8 + k) * per, S);
+            }
+        } else {
+            gp_linear_at(P, S, side, t, m, g, Wv, Wt);
+        }
+        if ((bits >> (2 + side)) & 1) {
+#pragma unroll
+            for (int k = 0; k < NV; k++) Wn[k] = ldc(gp + (long long)(4 + k) * per, S);
+        } else {
+            double unused[NV];
+            gp_linear_at(P, S, 2 + side, t, m, g, Wn, unused);
+        }
+    } else {
+        const long long plane = (long long)S.nlines * S.nm;
+#pragma unroll
+        for (int k = 0; k < NV; k++) {
+            Wv[k] = ldc(S.line + (long long)(side * NV + k) * plane + o, S);
+            Wn[k] = ldc(S.line + (long long)((2 + side) * NV + k) * plane + o, S);
+            Wt[k] = 0.0;
+        }
+    }
+}
+
 template <int DIM, int STAGE, bool PRFIX>
 __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ctrl, long long id)
 {
@@ -831,55 +873,22 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     const bool valid = o < per;
     double o0[NV], o1[NV];
     if (valid) {
-    double Wq[6][NV];
-    if constexpr (DIM == 2) {
-        if (S.tlanes == 4) {
-            // small sweeps: every pass was reconstructed by k_tang / k_tang_ao
-#pragma unroll
-            for (int q = 0; q < 6; q++)
-#pragma unroll
-                for (int k = 0; k < NV; k++) Wq[q][k] = ldc(S.gp + (long long)((g * 6 + q) * 4 + k) * per + o, S);
-        } else {
-            // large sweeps: troubled passes from k_tang_ao, smooth ones reconstructed here
-            const int t = (int)(o / S.nm), m = (int)(o % S.nm);
-            const unsigned bits = rdc(S.flagT + o, S);
-            constexpr int qx[4] = {0, 3, 1, 4};      // Q index: 0 Wl, 1 Wlx, 2 Wly, 3 Wr, 4 Wrx, 5 Wry
-#pragma unroll
-            for (int X = 0; X < 4; X++) {
-                if ((bits >> X) & 1) {
-#pragma unroll
-                    for (int k = 0; k < NV; k++) {
-                        Wq[qx[X]][k] = ldc(S.gp + (long long)((g * 6 + qx[X]) * 4 + k) * per + o, S);
-                        if (X <= 1) Wq[qx[X] + 2][k] = ldc(S.gp + (long long)((g * 6 + qx[X] + 2) * 4 + k) * per + o, S);
-                    }
-                } else {
-                    double v[4], d[4];
-                    gp_linear_at(P, S, X, t, m, g, v, d);
-#pragma unroll
-                    for (int k = 0; k < NV; k++) {
-                        Wq[qx[X]][k] = v[k];
-                        if (X <= 1) Wq[qx[X] + 2][k] = d[k];
-                    }
-                }
-            }
-        }
-    } else {
-        long long plane = (long long)S.nlines * S.nm;
-#pragma unroll
-        for (int k = 0; k < NV; k++) {
-            Wq[0][k] = ldc(S.line + (long long)(0 * NV + k) * plane + o, S);
-            Wq[1][k] = ldc(S.line + (long long)(2 * NV + k) * plane + o, S);
-            Wq[3][k] = ldc(S.line + (long long)(1 * NV + k) * plane + o, S);
-            Wq[4][k] = ldc(S.line + (long long)(3 * NV + k) * plane + o, S);
-            Wq[2][k] = 0.0; Wq[5][k] = 0.0;
-        }
+    // one side after the other: only the side at work holds its states and slopes in registers
+    FluxSums<DIM> sums;
+    double pl, pr;
+    bool ok;
+    {
+        double Wv[NV], Wn[NV], Wt[NV];
+        side_states<DIM>(P, S, 0, g, o, Wv, Wn, Wt);
+        ok = flux_side<DIM, PRFIX, true>(P.fc, Wv, Wn, Wt, sums, pl);
     }
-    FluxConst fc;
-    fc.gamma = P.gamma; fc.gm1 = P.gamma - 1.0; fc.K = P.K;
-    fc.Kq = P.K + (double)DIM; fc.cslope = 4.0 / fc.Kq;
-    fc.mu = P.mu; fc.c1 = P.c1; fc.c2 = P.c2; fc.viscous = P.viscous; fc.tau_zero = P.tau_zero;
-    fc.prfix = P.prfix;
-    if (!gks_flux<DIM, STAGE, PRFIX>(fc, Wq[0], Wq[1], Wq[2], Wq[3], Wq[4], Wq[5], ctrl->dt, o0, o1)) {
+    if (ok) {
+        double Wv[NV], Wn[NV], Wt[NV];
+        side_states<DIM>(P, S, 1, g, o, Wv, Wn, Wt);
+        ok = flux_side<DIM, PRFIX, false>(P.fc, Wv, Wn, Wt, sums, pr);
+    }
+    if (ok) ok = flux_finish<DIM, STAGE, PRFIX>(P.fc, sums, pl, pr, ctrl->dt, o0, o1);
+    if (!ok) {
         // a non-physical state: the status is latched and the flux is a NaN, so that what the
         // failed step leaves behind does not depend on anything but the solve itself
         ctrl->status = HGKS_ENONPHYSICAL;
@@ -1120,7 +1129,7 @@ template <int DIM, int STAGE>
 __global__ void __launch_bounds__(256) kb_flux(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
 {
     HGKS_BATCH_SWEEP_BLOCK();
-    if (d.P.prfix != 0.0) flux_nl<DIM, STAGE, true>(d, dir, id);
+    if (d.P.fc.prfix != 0.0) flux_nl<DIM, STAGE, true>(d, dir, id);
     else flux_nl<DIM, STAGE, false>(d, dir, id);
 }
 
@@ -1307,7 +1316,7 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
     timed(s, KC_FLUX, 1, [&] {
         unsigned int g = pair([](const Sweep& S) { return blocks_for(flux_threads(DIM, (long long)S.nt * S.nm), 64); }, nb);
         const int n0 = (int)nb[0];
-        if (P.prfix != 0.0) {
+        if (P.fc.prfix != 0.0) {
             if (stage == 0) k_flux<DIM, 0, true><<<g, 64, 0, st>>>(D, n0);
             else k_flux<DIM, 1, true><<<g, 64, 0, st>>>(D, n0);
         } else {
