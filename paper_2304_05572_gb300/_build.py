@@ -21,7 +21,7 @@ LIB = os.path.join(OUT_DIR, "libhgks.so")
 LIB_DEBUG = os.path.join(OUT_DIR, "libhgks_debug.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["hgks_kernels.cu", "hgks_api.cu"]
-HEADERS = ["hgks_math.cuh", "hgks_fluxconst.h", "hgks_internal.h", "erfcx_table.inc"]
+HEADERS = ["hgks_math.cuh", "hgks_fluxconst.h", "hgks_fixed.cuh", "hgks_internal.h", "erfcx_table.inc", "exp2_table.inc"]
 
 
 def _nvcc():

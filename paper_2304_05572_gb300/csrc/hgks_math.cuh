@@ -10,17 +10,19 @@
 //    whose fma is explicit.  Any implementation that evaluates the same formulas
 //    in the same order (as written below) takes bit-identical decisions.
 //  * the Gauss-point (tangential) reconstruction and the gas-kinetic flux, which
-//    only feed the update and are written for few FP64 instructions: moments in
-//    the frame of each state's tangential velocity, closed-form micro-slope
-//    solves, one erfc and one exp per side, exp(-dt/(2 tau)) squared for
-//    exp(-dt/tau), and the S2O4 flux combinations formed on scalar coefficients
-//    before the moment vectors are combined.
+//    only feed the update and are written for few FP64 instructions: closed-form
+//    micro-slope solves, one erfc and one exp per side, exp(-dt/(2 tau)) squared
+//    for exp(-dt/tau), and the S2O4 flux combinations formed on scalar
+//    coefficients before the moment vectors are combined.
 #pragma once
 
 #include <cstdint>
 #include <cmath>
 
 #include "hgks_fluxconst.h"
+#if defined(__CUDACC__)
+#include "hgks_fixed.cuh"
+#endif
 
 // flux arithmetic is also compiled for the host (unit checks of the formulas)
 #define HGKS_HD __host__ __device__
@@ -42,40 +44,47 @@ __device__ __forceinline__ ex xfma(ex a, ex b, ex c) { return ex(__fma_rn(a.v, b
 __device__ __forceinline__ ex xabs(ex a) { return ex(fabs(a.v)); }
 __device__ __forceinline__ ex xsqrt(ex a) { return ex(__dsqrt_rn(a.v)); }
 
-// 1/x in free-order arithmetic (the flux, the tangential WENO-AO pass): the hardware's approximate reciprocal refined by two
-// Newton-Raphson steps for 1/x, r <- r + r (1 - x r), each of which squares the relative error;
-// within 1 ulp of the correctly rounded quotient for the normal x the flux meets (checked against
-// IEEE division by hgks_check_reciprocal).  A zero x gives a NaN, which the flux's physical-state
-// tests reject as they rejected the infinity of 1/0.  The host build divides.
+// 1/x and 1/sqrt(x) in free-order arithmetic (the flux, the tangential WENO-AO pass), in fixed
+// point on the device: no FP64 instruction where the hardware's approximation and two
+// Newton-Raphson steps take 4 and 7 of the pipe's 64-cycle slots; within 1 ulp of the correctly
+// rounded quotient and within 2 ulps of IEEE division by the IEEE square root (hgks_check_reciprocal).
+// The host build divides.
 HGKS_HD __forceinline__ double rcp_nr(double x)
 {
 #ifdef __CUDA_ARCH__
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
+    return fixed::rcp(x);
 #else
     return 1.0 / x;
 #endif
 }
 
-// 1/sqrt(x), x > 0, likewise: the hardware's approximation refined by two Newton-Raphson steps
-// for 1/sqrt(x), y <- y + y (1 - x y^2) / 2 (each roughly squares the relative error).  The host
-// build divides by the square root.
 HGKS_HD __forceinline__ double rsqrt_nr(double x)
 {
 #ifdef __CUDA_ARCH__
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double hx = 0.5 * x;
-    double t = fma(-hx * y, y, 0.5);
-    y = fma(y, t, y);
-    t = fma(-hx * y, y, 0.5);
-    return fma(y, t, y);
+    return fixed::rsqrt(x);
 #else
     return 1.0 / sqrt(x);
+#endif
+}
+
+// x 2^K; exp(-y), y >= 0
+template <int K>
+HGKS_HD __forceinline__ double scale2(double x)
+{
+#ifdef __CUDA_ARCH__
+    return fixed::scale2<K>(x);
+#else
+    return x * (K > 0 ? (double)(1 << (K > 0 ? K : 0)) : 1.0 / (double)(1 << (K < 0 ? -K : 0)));
+#endif
+}
+
+HGKS_HD __forceinline__ double exp_neg(double y)
+{
+#ifdef __CUDA_ARCH__
+    if (y < 708.0) return fixed::exp_value(fixed::exp_neg(y));
+    return y >= 708.0 ? 0.0 : y;            // below the normal range; NaN
+#else
+    return exp(-y);
 #endif
 }
 
@@ -545,8 +554,8 @@ struct MState {
     double u2, H;                          // U^2 + h; H = (E + p)/rho, E without the tangential kinetic energy
 };
 
-// Slope constants of one side: ri/h and ri/(2 h^2) carry the 1/rho of <a> = dW/rho (Eq. (8)).
-struct SlopeC { double rih, qh; };
+// Slope constants of one side: ri/h and ri/(2 h^2) carry the 1/rho of <a> = dW/rho (Eq. (8)); 2 U.
+struct SlopeC { double rih, qh, U2; };
 
 // W_k-direction d in the frame of s, with what the closed forms share: R = d1 - U d0 (rho dU),
 // S = d1 + R, dp (pressure), d2, d3 in the frame.
@@ -567,11 +576,11 @@ HGKS_HD __forceinline__ bool make_state(const double* W, const FluxConst& fc, MS
     s.rho = W[0];
     s.ri = rcp_nr(s.rho);
     s.U = W[1] * s.ri;
-    s.hU = 0.5 * s.U;
+    s.hU = scale2<-1>(s.U);
     double E = W[DIM + 1];
     if constexpr (DIM == 2) {
         s.V = W[2] * s.ri;
-        s.hV = 0.5 * s.V;
+        s.hV = scale2<-1>(s.V);
         E = fma(-s.hV, W[2], E);
     } else {
         s.V = s.hV = 0.0;
@@ -641,7 +650,7 @@ template <int DIM>
 HGKS_HD __forceinline__ void slope_solve(const Dir& d, const MState<DIM>& s, const SlopeC& k, Slope& a)
 {
     a.ha3 = k.qh * fma(-s.h, d.d0, d.dp);
-    a.a1 = fma(-2.0 * s.U, a.ha3, k.rih * d.R);
+    a.a1 = fma(-k.U2, a.ha3, k.rih * d.R);
     a.c0 = fma(-s.u2, a.ha3, fma(-s.U, a.a1, d.d0 * s.ri));
     a.a2h = DIM == 2 ? s.ri * d.d2 : 0.0;
 }
@@ -702,34 +711,23 @@ HGKS_HD __forceinline__ void add_psi_lab(const MState<DIM>& s, const Mom& m, int
     acc[1] = FIRST ? m.u[n + 1] : acc[1] + m.u[n + 1];
 }
 
-#include "erfcx_table.inc"
-
-// erfcx(y) = exp(y^2) erfc(y) on [0, 8): per interval [k/4, (k+1)/4) a degree-11 polynomial in
-// y - (k + 1/2)/4 (Chebyshev interpolant, relative error 2.1e-16; gen_erfcx_table.py).
-// Read by device code only.
-__device__ const double c_erfcx[HGKS_ERFCX_INTERVALS * (HGKS_ERFCX_DEGREE + 1)] = HGKS_ERFCX_TABLE;
-
-// erfc(y) for y >= 0, given ey = exp(-y^2): ey erfcx(y) from the table below y = 8 (17 FP64
-// operations instead of a full erfc, which recomputes the exponential), the library erfc above.
-HGKS_HD __forceinline__ double erfc_nonneg(double y, double ey)
-{
-#ifdef __CUDA_ARCH__
-    if (y < 8.0) {
-        // k = round(4y - 1/2) in 0..31 (the interval whose centre is nearest): adding 1.5 2^52
-        // leaves the rounded integer in the low mantissa bits
-        constexpr double kRound = 6755399441055744.0;
-        const double z = fma(y, 4.0, -0.5) + kRound;
-        const int k = __double2loint(z);
-        const double t = y - fma(z - kRound, 0.25, 0.125);
-        const double* a = c_erfcx + k * (HGKS_ERFCX_DEGREE + 1);
-        double p = __ldg(a + HGKS_ERFCX_DEGREE);
-#pragma unroll
-        for (int j = HGKS_ERFCX_DEGREE - 1; j >= 0; j--) p = fma(p, t, __ldg(a + j));
-        return ey * p;
-    }
+#if defined(__CUDACC__)
+__device__ __noinline__ double erfc_far(double y) { return erfc(y); }
 #endif
-    (void)ey;
-    return erfc(y);
+
+// exp(-x^2) and erfc(|x|): below |x| = 8 from the fixed-point exponential and erfcx(|x|) =
+// exp(x^2) erfc(|x|), the library erfc beyond.
+HGKS_HD __forceinline__ void exp_erfc(double x, double& ex2, double& E)
+{
+    const double x2 = x * x;
+#ifdef __CUDA_ARCH__
+    if (x2 < 64.0) { fixed::exp_erfc(fabs(x), x2, ex2, E); return; }
+    ex2 = exp_neg(x2);
+    E = erfc_far(fabs(x));
+#else
+    ex2 = exp(-x2);
+    E = erfc(fabs(x));
+#endif
 }
 
 // Half-line moments of the left state over u > 0 (sign = +1) or of the right state over
@@ -742,17 +740,18 @@ template <int DIM>
 HGKS_HD __forceinline__ void half_moments(const MState<DIM>& s, double sl, int sign, const FluxConst& fc, Mom& m)
 {
     const double x = sl * s.U;
-    const double ex2 = exp(-x * x);
+    double ex2, E;
+    exp_erfc(x, ex2, E);
     const double e = ex2 * (0.56418958354775628695 * s.p * sl);   // rho h sqrt(lam)/sqrt(pi), rho h = p
-    const double E = erfc_nonneg(fabs(x), ex2);
     const bool into = sign > 0 ? x >= 0.0 : x < 0.0;
-    const double hr = 0.5 * s.rho;
+    const double hr = scale2<-1>(s.rho);
     m.u[0] = into ? fma(-hr, E, s.rho) : hr * E;
     m.u[1] = fma(s.U, m.u[0], sign > 0 ? e : -e);
+    const double h2 = scale2<1>(s.h), hn[5] = {s.h, h2, s.h + h2, scale2<1>(h2), 5.0 * s.h};
 #pragma unroll
-    for (int n = 0; n < 5; n++) m.u[n + 2] = fma(s.U, m.u[n + 1], ((double)(n + 1) * s.h) * m.u[n]);
+    for (int n = 0; n < 5; n++) m.u[n + 2] = fma(s.U, m.u[n + 1], hn[n] * m.u[n]);
     m.kk = fc.hKt * s.h;
-    m.kh2 = 2.0 * m.kk * s.h;
+    m.kh2 = scale2<1>(m.kk) * s.h;
 }
 
 // Sums over the two sides (left over u > 0, right over u < 0), lab frame: the equilibrium state
@@ -772,12 +771,13 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
     MState<DIM> s;
     if (!make_state<DIM>(W, fc, s)) return false;
     p = s.p;
-    const double sl = rsqrt_nr(2.0 * s.h);      // sqrt(lambda)
+    const double sl = rsqrt_nr(scale2<1>(s.h));      // sqrt(lambda)
     SlopeC k;
     {
         const double lam = sl * sl;
-        k.rih = 2.0 * lam * s.ri;
+        k.rih = scale2<1>(lam) * s.ri;
         k.qh = lam * k.rih;
+        k.U2 = scale2<1>(s.U);
     }
     Mom m;
     half_moments<DIM>(s, sl, FIRST ? +1 : -1, fc, m);
@@ -810,12 +810,12 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
         if (noneq) {
             // v = V + c: the c part has <u c psi (b.psi)> = b2 h u_1, b2 h u_2, h (T_b(1) + h b3 u_1)
             // and b2 h (u_3 + (Kt + 2) h u_1)/2
-            const double y = 2.0 * s.h * b.ha3, kc = fc.ktp2 * s.h;
+            const double y = scale2<1>(s.h) * b.ha3, kc = fc.ktp2 * s.h, hb = scale2<-1>(b.a2h);
             if constexpr (PRFIX) {
                 L[0] = fma(s.V, g[0], fma(b.a2h, m.u[0], L[0]));
                 L[1] = fma(s.V, g[1], fma(b.a2h, m.u[1], L[1]));
                 L[2] = fma(s.V, g[2], fma(s.h, fma(y, m.u[0], tb0), L[2]));
-                L[3] = fma(s.V, g[3], fma(0.5 * b.a2h, fma(kc, m.u[0], m.u[2]), L[3]));
+                L[3] = fma(s.V, g[3], fma(hb, fma(kc, m.u[0], m.u[2]), L[3]));
                 add_lab<DIM, FIRST>(s, L, q.D5);
             }
             const double tb3 = mom_t(b, m, 3);
@@ -823,7 +823,7 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
             L5[0] = fma(s.V, g[0], L5[0] + g[2]);
             L5[1] = fma(s.V, g[1], fma(b.a2h, m.u[2], L5[1]));
             L5[2] = fma(s.V, g[2], fma(s.h, fma(y, m.u[1], tb1), L5[2]));
-            L5[3] = fma(s.V, g[3], fma(0.5 * b.a2h, fma(kc, m.u[1], m.u[3]), L5[3]));
+            L5[3] = fma(s.V, g[3], fma(hb, fma(kc, m.u[1], m.u[3]), L5[3]));
         }
     } else if constexpr (PRFIX) {
         if (noneq) add_lab<DIM, FIRST>(s, L, q.D5);
@@ -882,7 +882,7 @@ HGKS_HD __forceinline__ void m2_term(const MState<DIM>& s, const FluxConst& fc, 
 template <int STAGE>
 HGKS_HD __forceinline__ void time_coefs(double dt, double tau, double* A0, double* A1)
 {
-    const double e = exp(-0.5 * dt * rcp_nr(tau));
+    const double e = exp_neg(0.5 * dt * rcp_nr(tau));
     const double o = 1.0 - e, P = tau * o, dte = dt * e;
     if constexpr (STAGE == 0) {
         const double hd = 0.5 * dt, td = tau * dt;

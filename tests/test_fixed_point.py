@@ -1,0 +1,95 @@
+"""The fixed-point reciprocal, reciprocal square root, exponential and erfc of the flux kernel
+(csrc/hgks_fixed.cuh), compiled for the host, against long-double references.
+
+Bounds in units of the result's last place: one rounding (1/2), the approximations' own remainders
+(2^-9 for the two reciprocals; for the exponential 2^-5 for the argument's 57 fraction bits and
+2^-4 for series and truncations, bounded here by 1/4), and for erfc the table's 2.1e-16 (up to 1.9
+units) beside the exponential's."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2304_05572_gb300", "csrc")
+
+SRC = r"""
+#include "hgks_fixed.cuh"
+#include <cfloat>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <limits>
+#include <random>
+using namespace hgks::fixed;
+static double ulps(double a, long double r)
+{
+    int e; std::frexp((double)r, &e);
+    return (double)(std::fabs((long double)a - r) / std::ldexp(1.0L, e - 53));
+}
+int main(int argc, char** argv)
+{
+    const char* what = argv[1];
+    std::mt19937_64 g(20230415);
+    std::uniform_real_distribution<double> U(0.0, 1.0);
+    double worst = 0.0;
+    if (!strcmp(what, "special")) {
+        const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
+        bool ok = true;
+        for (double v : {0.0, -0.0, 1e-310, -1e-310, inf, -inf, nan}) ok = ok && std::isnan(rcp(v));
+        ok = ok && rcp(std::ldexp(1.3, 1022)) == 0.0 && rcp(std::ldexp(-1.0, 1023)) == 0.0;
+        for (double v : {0.0, -0.0, 1e-310, -1.0, -inf, inf, nan}) ok = ok && std::isnan(rsqrt(v));
+        for (double v : {0.0, -0.0, 3.0, -1e200, inf, -inf, 1e-300}) ok = ok && scale2<1>(v) == 2 * v && scale2<-1>(v) == 0.5 * v;
+        ok = ok && std::isnan(scale2<1>(nan)) && rcp(1.0) == 1.0 && rcp(-2.0) == -0.5 && rsqrt(4.0) == 0.5 && rsqrt(1.0) == 1.0;
+        ok = ok && exp_value(exp_neg(0.0)) == 1.0 && rcp(std::ldexp(1.0, 1021)) == std::ldexp(1.0, -1021) && rcp(std::ldexp(1.0, -1022)) == std::ldexp(1.0, 1022);
+        printf("%d\n", ok ? 1 : 0);
+        return 0;
+    }
+    for (long i = 0; i < 400000; i++) {
+        // edges of the ranges, neighbours of powers of two, log-uniform and uniform arguments
+        double x = std::exp((U(g) - 0.5) * 1300.0), y = i & 1 ? U(g) : std::exp(-U(g) * 40.0);
+        if (i < 4000) { x = std::ldexp(1.0 + (i / 4) * DBL_EPSILON, (i & 3) - 1); if (i & 2) x = std::nextafter(x, 0.0); }
+        if (!strcmp(what, "rcp")) worst = std::fmax(worst, std::fmax(ulps(rcp(x), 1.0L / x), ulps(-rcp(-x), 1.0L / x)));
+        if (!strcmp(what, "rsqrt")) worst = std::fmax(worst, ulps(rsqrt(x), 1.0L / std::sqrt((long double)x)));
+        if (!strcmp(what, "exp")) {
+            double a = i % 3 ? y * 64.0 : 64.0 + U(g) * (708.0 - 64.0);
+            if (i == 0) a = 64.0;
+            if (i == 1) a = std::nextafter(64.0, 0.0);
+            if (i == 2) a = std::nextafter(708.0, 0.0);
+            worst = std::fmax(worst, ulps(exp_value(exp_neg(a)), std::exp(-(long double)a)));
+        }
+        if (!strcmp(what, "erfc")) {
+            double a = y * 8.0, a2, ex, er;
+            if (i < 96) { a = (i / 3) / 4.0 + (i % 3 == 1 ? 0.125 : 0.0); if (i % 3 == 2) a = std::nextafter(a, 8.0); }
+            if (i == 96) a = std::nextafter(8.0, 0.0);
+            a2 = a * a;
+            if (!(a2 < 64.0)) continue;
+            exp_erfc(a, a2, ex, er);
+            // the exponential is taken of the rounded square
+            const long double ref = std::erfc((long double)a) * std::exp((long double)a * a - (long double)a2);
+            worst = std::fmax(worst, ulps(er, ref));
+        }
+    }
+    printf("%.6f\n", worst);
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def exe(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fixed")
+    (d / "t.cpp").write_text(SRC)
+    subprocess.run(["g++", "-O1", "-std=gnu++17", "-ffp-contract=off", "-I", CSRC, "-o", str(d / "t"), str(d / "t.cpp")],
+                   check=True)
+    return str(d / "t")
+
+
+@pytest.mark.parametrize("what,bound", [("rcp", 0.51), ("rsqrt", 0.51), ("exp", 0.75), ("erfc", 2.7)])
+def test_within_bounds(exe, what, bound):
+    worst = float(subprocess.run([exe, what], check=True, capture_output=True, text=True).stdout)
+    assert worst <= bound, worst
+
+
+def test_special_arguments(exe):
+    assert subprocess.run([exe, "special"], check=True, capture_output=True, text=True).stdout.strip() == "1"
