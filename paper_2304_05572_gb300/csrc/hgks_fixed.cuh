@@ -2,7 +2,7 @@
 // fixed point.
 //
 // The FP64 pipe of this part takes one warp instruction per 64 cycles and scheduler (measured
-// 65-76), while the integer pipe issues a 32 x 32 + 64 bit multiply-add in 2 and everything else in
+// 65-76, comparisons and conversions from and to doubles included), while the integer pipe issues a 32 x 32 + 64 bit multiply-add in 2 and everything else in
 // 1 (a 64 x 64 -> 64 bit high product: 10-22).  A function whose arguments and results have a known
 // range is therefore cheaper in integers, at more bits than a double carries: each routine below
 // works with 61-63 fraction bits, rounds once, and is within one unit in the last place of the exact
@@ -38,7 +38,6 @@ HGKS_FX u32 float_bits(float x) { return __float_as_uint(x); }
 HGKS_FX float float_of(u32 b) { return __uint_as_float(b); }
 HGKS_FX float approx_rcp(float x) { float r; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 HGKS_FX float approx_rsqrt(float x) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
-HGKS_FX i64 to_int(double x) { return __double2ll_rn(x); }
 HGKS_FX int clz32(u32 x) { return __clz((int)x); }
 #else
 HGKS_FX u64 bits_of(double x) { u64 b; memcpy(&b, &x, 8); return b; }
@@ -47,7 +46,6 @@ HGKS_FX u32 float_bits(float x) { u32 b; memcpy(&b, &x, 4); return b; }
 HGKS_FX float float_of(u32 b) { float x; memcpy(&x, &b, 4); return x; }
 HGKS_FX float approx_rcp(float x) { return 1.0f / x; }
 HGKS_FX float approx_rsqrt(float x) { return 1.0f / std::sqrt(x); }
-HGKS_FX i64 to_int(double x) { return std::llrint(x); }
 HGKS_FX int clz32(u32 x) { return __builtin_clz(x); }
 #endif
 
@@ -78,6 +76,32 @@ HGKS_FX i64 smulhi(Half a, Half b)
 {
     const i64 cross = (i64)a.hi * b.lo + (i64)a.lo * b.hi;
     return (i64)a.hi * b.hi + (cross >> 31);
+}
+
+// x > 0 (false for a NaN), x = 0, x finite, |x| <= y for y >= 0 (false for a NaN): on the bit patterns
+HGKS_FX bool is_pos(double x) { return bits_of(x) - 1u < 0x7FF0000000000000ull; }
+HGKS_FX bool is_zero(double x) { return bits_of(x) << 1 == 0u; }
+HGKS_FX bool is_finite(double x) { return ((u32)(bits_of(x) >> 32) & 0x7FF00000u) != 0x7FF00000u; }
+HGKS_FX bool abs_le(double x, double y) { return (bits_of(x) & 0x7FFFFFFFFFFFFFFFull) <= bits_of(y); }
+
+// x rounded towards zero to a float; below 2^-126 to zero, from 2^128 on (and a NaN) to an infinity
+HGKS_FX float to_float(double x)
+{
+    const u64 b = bits_of(x);
+    const u32 hi = (u32)(b >> 32), e = hi & 0x7FF00000u;
+    u32 f = (u32)(b >> 29) - 0xC0000000u;
+    f = e < 0x38100000u ? 0u : e > 0x47E00000u ? 0x7F800000u : f;
+    return float_of((f & 0x7FFFFFFFu) | (hi & 0x80000000u));
+}
+
+// y 2^Q rounded down, for 0 <= y < 2^(64-Q)
+HGKS_FX u64 to_fixed(double y, int q)
+{
+    const u64 b = bits_of(y);
+    const u32 e = (u32)(b >> 52);
+    const u32 s = 1086u - (u32)q - e;                                      // >= 0 in range
+    const u64 m = (b << 11) | 0x8000000000000000ull;
+    return s < 64u ? m >> s : 0u;
 }
 
 // x 2^k for a finite x (zeros and subnormals stay as they are, infinities and NaNs too): an integer
@@ -154,9 +178,8 @@ HGKS_FX u64 load_exp2(u32 j)
 
 HGKS_FX Exp exp_neg(double y)
 {
-    const u64 b = bits_of(y);
-    const int q = (u32)(b >> 32) < 0x40500000u ? 57 : 53;                   // y < 64
-    const u64 yf = (u64)to_int(of_bits(b + ((u64)q << 52)));               // y in 2^-q
+    const int q = (u32)(bits_of(y) >> 32) < 0x40500000u ? 57 : 53;                   // y < 64
+    const u64 yf = to_fixed(y, q);                                         // y in 2^-q
     const u64 t = umulhi_exact(yf, 0xB8AA3B295C17F0BCull), tl = yf * 0xB8AA3B295C17F0BCull;   // y log2(e), 2^-(q+63)
     Exp r;
     r.n = (int)(t >> (q - 1));
@@ -211,7 +234,7 @@ HGKS_FX_DATA constexpr ErfcxQ c_erfcx_q = make_erfcx_q();
 // erfcx(y) in 2^-62 for 0 <= y < 8
 HGKS_FX u64 erfcx_q(double y)
 {
-    const u64 yf = (u64)to_int(of_bits(bits_of(y) + (58ull << 52)));       // 2^-58
+    const u64 yf = to_fixed(y, 58);                                        // 2^-58
     u32 k = (u32)(yf >> 56);
     k = k < HGKS_ERFCX_INTERVALS ? k : HGKS_ERFCX_INTERVALS - 1;
     const i64 t = (i64)(yf - ((u64)k << 56)) - (1ll << 55);                // y - centre, 2^-58

@@ -191,7 +191,7 @@ __device__ __forceinline__ void b_dt(const Params& P, const double* __restrict__
             if (dv.v < d.v) d = dv;
         }
         unsigned long long bits = (unsigned long long)__double_as_longlong(d.v);
-        if (!(d.v > 0.0)) bits = 0x7FF8000000000000ull;   // non-physical cells are caught by the update
+        if (!fixed::is_pos(d.v)) bits = 0x7FF8000000000000ull;   // non-physical cells are caught by the update
         best = bits < best ? bits : best;
     }
     for (int o = 16; o > 0; o >>= 1) {
@@ -281,10 +281,11 @@ __device__ __forceinline__ void b_raw_nflags(const Params& P, const Sweep& S, co
 #pragma unroll
         for (int k = 0; k < NV; k++) {
             double q[5];
+            float f[5];
             const double* b = base + (long long)S.perm[k] * P.g.plane;
 #pragma unroll
-            for (int s = 0; s < 5; s++) q[s] = ldc(b + (long long)s * S.sN, S);
-            tr |= indicator_raw(q, S.Z1n);
+            for (int s = 0; s < 5; s++) { q[s] = ldc(b + (long long)s * S.sN, S); f[s] = fixed::to_float(q[s]); }
+            tr |= indicator_raw(q, f, S.Z1n);
         }
     }
     stc(S.rawN + id, tr, S);
@@ -513,9 +514,10 @@ __device__ __forceinline__ void b_raw_tflags_x4(const Params& P, const Sweep& S,
 #pragma unroll
         for (int X = 0; X < 4; X++) {
             double qv[5];
+            float f[5];
 #pragma unroll
-            for (int s = 0; s < 5; s++) qv[s] = lineval(S, X, q, t - 2 + s, m);
-            bits |= (unsigned)indicator_raw(qv, S.Z1t) << X;
+            for (int s = 0; s < 5; s++) { qv[s] = lineval(S, X, q, t - 2 + s, m); f[s] = fixed::to_float(qv[s]); }
+            bits |= (unsigned)indicator_raw(qv, f, S.Z1t) << X;
         }
         bits |= __shfl_xor_sync(gmask, bits, 1);
         bits |= __shfl_xor_sync(gmask, bits, 2);
@@ -523,29 +525,46 @@ __device__ __forceinline__ void b_raw_tflags_x4(const Params& P, const Sweep& S,
     if (q == 0) stc(S.rawT + seg, bits, S);
 }
 
+// Large sweeps: each thread takes kTRows consecutive lines of one interface, so that a line value is
+// loaded and truncated once for up to 5 windows (8 rows instead of 20 for 4 segments).
+constexpr int kTRows = 4;
+
 __device__ __forceinline__ void b_raw_tflags_x1(const Params& P, const Sweep& S, const Ctrl* __restrict__ ctrl, long long id)
 {
     if (ctrl->done) return;
-    long long total = (long long)(S.nt + 2) * S.nm;
-    if (id >= total) return;
-    int m = (int)(id % S.nm);
-    int t = (int)(id / S.nm) - 1;
-    uint8_t bits = 0;
+    const int m = (int)(id % S.nm);
+    const int r0 = (int)(id / S.nm) * kTRows;              // row of rawT: line r0 - 1
+    const int rows = S.nt + 2 - r0 < kTRows ? S.nt + 2 - r0 : kTRows;
+    if (rows <= 0) return;
+    unsigned bits[kTRows] = {};
     if (P.recon_mode == HGKS_RECON_HYBRID) {
-#pragma unroll
+#pragma unroll 1
         for (int X = 0; X < 4; X++) {
-            int tr = 0;
-#pragma unroll
+#pragma unroll 1
             for (int k = 0; k < 4; k++) {
-                double q[5];
+                double q[kTRows + 4];
+                float f[kTRows + 4];
 #pragma unroll
-                for (int s = 0; s < 5; s++) q[s] = lineval(S, X, k, t - 2 + s, m);
-                tr |= indicator_raw(q, S.Z1t);
+                for (int s = 0; s < kTRows + 4; s++) {
+                    // (lines past the last window repeat the last one: loaded, not used)
+                    q[s] = lineval(S, X, k, r0 - 3 + (s < rows + 4 ? s : rows + 3), m);
+                    f[s] = fixed::to_float(q[s]);
+                }
+#pragma unroll
+                for (int r = 0; r < kTRows; r++)
+                    if (r < rows) bits[r] |= (unsigned)indicator_raw(q + r, f + r, S.Z1t) << X;
             }
-            bits |= (uint8_t)(tr << X);
         }
     }
-    stc(S.rawT + id, bits, S);
+#pragma unroll
+    for (int r = 0; r < kTRows; r++)
+        if (r < rows) stc(S.rawT + (long long)(r0 + r) * S.nm + m, bits[r], S);
+}
+
+// Threads of the raw tangential flag kernel on sweep S.
+inline long long raw_t_threads(const Sweep& S)
+{
+    return S.tlanes == 4 ? (long long)(S.nt + 2) * S.nm * 4 : (long long)((S.nt + 2 + kTRows - 1) / kTRows) * S.nm;
 }
 
 // Small sweeps (fewer segments than a few warps per scheduler) spread a segment over 4 lanes,
@@ -1002,7 +1021,7 @@ __device__ __forceinline__ void b_update(const Params& P, const Sweep& Sx, const
     // rho > 0 and p > 0, the latter as rho E - |m|^2/2 > 0 (no division)
     double ke = DIM == 2 ? 0.5 * fma(out[1], out[1], out[2] * out[2]) : 0.5 * out[1] * out[1];
     double pr = fma(out[NV - 1], out[0], -ke);
-    if (!(out[0] > 0.0) || !(pr > 0.0) || !isfinite(out[0]) || !isfinite(pr)) ctrl->status = HGKS_ENONPHYSICAL;
+    if (!fixed::is_pos(out[0]) || !fixed::is_pos(pr) || !fixed::is_finite(out[0]) || !fixed::is_finite(pr)) ctrl->status = HGKS_ENONPHYSICAL;
 }
 
 template <int DIM, int STAGE>
@@ -1293,7 +1312,7 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
     });
     if constexpr (DIM == 2) {
         timed(s, KC_RAWT, 1, [&] {
-            unsigned int g = pair([](const Sweep& S) { return blocks_for((long long)(S.nt + 2) * S.nm * S.tlanes, TPB); }, nb);
+            unsigned int g = pair([](const Sweep& S) { return blocks_for(raw_t_threads(S), TPB); }, nb);
             k_raw_tflags<<<g, TPB, 0, st>>>(D, (int)nb[0]);
         });
         timed(s, KC_TANG, 1, [&] {
@@ -1411,7 +1430,7 @@ static long long batch_unit_blocks(const SolveDesc& d, int dim, int c, int dir, 
         case BK_RAWN: b = blocks_for((long long)S.nlines * (S.nn + 4), t); break;
         case BK_NORMAL: b = blocks_for((long long)S.nlines * S.nm, t); break;
         case BK_NAO: b = blocks_for((long long)S.nlines * S.nm * 2 * 4, t * 8); break;
-        case BK_RAWT: if (dim != 2) return 0; b = blocks_for((long long)(S.nt + 2) * S.nm * S.tlanes, t); break;
+        case BK_RAWT: if (dim != 2) return 0; b = blocks_for(raw_t_threads(S), t); break;
         case BK_TANG: if (dim != 2) return 0; b = blocks_for((long long)S.nt * S.nm * S.tlanes, t); break;
         case BK_TAO: if (dim != 2) return 0; b = blocks_for((long long)S.nt * S.nm * 4 * 4, t * 8); break;
         case BK_FLUX: b = blocks_for(flux_threads(dim, (long long)S.nt * S.nm), t); break;

@@ -67,6 +67,25 @@ HGKS_HD __forceinline__ double rsqrt_nr(double x)
 #endif
 }
 
+// x > 0, x = 0: integer tests on the device, where a comparison occupies the FP64 pipe too
+HGKS_HD __forceinline__ bool positive(double x)
+{
+#ifdef __CUDA_ARCH__
+    return fixed::is_pos(x);
+#else
+    return x > 0.0;
+#endif
+}
+
+HGKS_HD __forceinline__ bool is_zero(double x)
+{
+#ifdef __CUDA_ARCH__
+    return fixed::is_zero(x);
+#else
+    return x == 0.0;
+#endif
+}
+
 // x 2^K; exp(-y), y >= 0
 template <int K>
 HGKS_HD __forceinline__ double scale2(double x)
@@ -81,8 +100,9 @@ HGKS_HD __forceinline__ double scale2(double x)
 HGKS_HD __forceinline__ double exp_neg(double y)
 {
 #ifdef __CUDA_ARCH__
-    if (y < 708.0) return fixed::exp_value(fixed::exp_neg(y));
-    return y >= 708.0 ? 0.0 : y;            // below the normal range; NaN
+    const unsigned hi = (unsigned)__double2hiint(y);
+    if (hi < 0x40862000u) return fixed::exp_value(fixed::exp_neg(y));       // y < 708
+    return hi <= 0x7FF00000u ? 0.0 : y;     // below the normal range; NaN
 #else
     return exp(-y);
 #endif
@@ -113,7 +133,7 @@ template <> struct exact_order<ex> { static constexpr bool value = true; };
 // and Z1 = 17 zeta1 dx^2 (Eq. (24): abar2 = D/34).  Step 2: xbar = -abar1/(2 abar2) with
 // abar1 = -N/10, N = (2Q_{i-2}+Q_{i-1}) - (2Q_{i+2}+Q_{i+1}); inside iff |xbar| <= 5/2.
 // Step 3: xhat from the conservative 3-cell quadratic; non-troubled iff |xbar - xhat| <= 1/4.
-__device__ __forceinline__ int indicator_raw(const double* q, double Z1)
+__device__ __forceinline__ int indicator_exact(const double* q, double Z1)
 {
     ex q0(q[0]), q1(q[1]), q2(q[2]), q3(q[3]), q4(q[4]);
     ex D = xfma(ex(-10.0), q2, xfma(ex(4.0), q0, q1) + xfma(ex(4.0), q4, q3));
@@ -130,6 +150,47 @@ __device__ __forceinline__ int indicator_raw(const double* q, double Z1)
     if (fabs((xbar - xhat).v) <= 0.25) return 0;
     return 1;
 }
+
+#if defined(__CUDACC__)
+// The same decision with few or no FP64 instructions (a comparison and a conversion occupy the FP64
+// pipe as long as an addition), f[j] = q[j] truncated to FP32 (fixed::to_float).  Each test is first taken in
+// FP32 with a margin above its rounding errors; only a test that falls inside its margin is decided by
+// the exact chain.
+//   Step 1: |D| against Z1 from the truncated window: truncation (2^-23) and four roundings (2^-24) of terms
+//     |c| m with coefficients summing to 20, m = max |q|: error below 20 m (2^-23 + 4 2^-24) = 7.2e-6 m.
+//   Steps 2, 3 on D, N, d = q3 - q1, s = (q1 + q3) - 2 q2, rounded as the exact chain rounds them (10 FP64
+//     operations): xbar = 1.7 N/D and xhat = -d/(2 s) (s = 2 ah2, the halves are exact), their FP32 ratios
+//     within 2^-20 relative; margins 1e-5.  Quantities outside 1e-30..1e30 go to the exact chain, and
+//     s = 0 does unless d = 0, where xhat = 0.
+// The exact chain takes 5 FP64 slots of the pipe on smooth data and, behind Step 1, four IEEE
+// divisions more, where one troubled lane holds up its warp.  Raw flags per step at 1024^2: normal
+// 253 -> 160 us, tangential 702 -> 251 us (with the shared row loads of b_raw_tflags_x1).
+__device__ __forceinline__ int indicator_raw(const double* q, const float* f, double Z1)
+{
+    const float m = fmaxf(fmaxf(fmaxf(fabsf(f[0]), fabsf(f[1])), fmaxf(fabsf(f[3]), fabsf(f[4]))), fabsf(f[2]));
+    const float Df = fmaf(-10.0f, f[2], fmaf(4.0f, f[0], f[1]) + fmaf(4.0f, f[4], f[3]));
+    // (an infinity among the f makes the sum infinite or a NaN: the comparison fails)
+    if (fmaf(8.0e-6f, m, fabsf(Df)) < 0.999999f * fixed::to_float(Z1)) return 0;
+    const ex q0(q[0]), q1(q[1]), q2(q[2]), q3(q[3]), q4(q[4]);
+    const ex D = xfma(ex(-10.0), q2, xfma(ex(4.0), q0, q1) + xfma(ex(4.0), q4, q3));
+    if (fixed::abs_le(D.v, Z1)) return 0;
+    const ex N = xfma(ex(2.0), q0, q1) - xfma(ex(2.0), q4, q3);
+    const float Dt = fixed::to_float(D.v), Nt = 1.7f * fixed::to_float(N.v);
+    const bool range = fabsf(Dt) > 1e-30f && fabsf(Dt) < 1e30f;
+    if (range && fabsf(Nt) > 2.50003f * fabsf(Dt)) return 0;
+    const ex d = q3 - q1, s = xfma(ex(-2.0), q2, q1 + q3);
+    const float sf = fixed::to_float(s.v), df = fixed::to_float(d.v);
+    const bool flat = fixed::is_zero(s.v) && fixed::is_zero(d.v);
+    if (range && fabsf(Nt) < 2.49997f * fabsf(Dt) && (flat || (fabsf(sf) > 1e-30f && fabsf(sf) < 1e30f && fabsf(df) < 1e30f))) {
+        const float xb = __fdividef(Nt, Dt);
+        const float xh = flat ? 0.0f : __fdividef(-0.5f * df, sf);
+        const float gap = fabsf(xb - xh), tol = 1e-5f * (1.0f + fabsf(xh));
+        if (gap < 0.25f - tol) return 0;
+        if (gap > 0.25f + tol) return 1;
+    }
+    return indicator_exact(q, Z1);
+}
+#endif
 
 // Step 5, Eqs. (26)-(27): value and derivative at x_{i+1/2} from cell i's window.
 __device__ __forceinline__ void linear_left(const double* q, double inv12h, double& val, double& der)
@@ -412,7 +473,7 @@ __device__ __forceinline__ bool nonphysical(double gam, const double* Q)
     if constexpr (NV == 4) ke = ex(0.5) * (ex(Q[1]) * ex(Q[1]) + ex(Q[2]) * ex(Q[2]));
     else ke = ex(0.5) * (ex(Q[1]) * ex(Q[1]));
     ex pr = ex(Q[NV - 1]) * ex(Q[0]) - ke;
-    return !(Q[0] > 0.0) || !(pr.v > 0.0);
+    return !(positive(Q[0]) && positive(pr.v));
 }
 
 // ---------------------------------------------------------------- Gauss-point reconstruction
@@ -589,7 +650,7 @@ HGKS_HD __forceinline__ bool make_state(const double* W, const FluxConst& fc, MS
     s.h = s.p * s.ri;
     s.u2 = fma(s.U, s.U, s.h);
     s.H = fma(s.hU, s.U, fc.gq * s.h);
-    return s.rho > 0.0 && s.p > 0.0;
+    return positive(s.rho) && positive(s.p);
 }
 
 // A direction d of the conserved variables (lab frame) in the frame of s.
@@ -721,7 +782,7 @@ HGKS_HD __forceinline__ void exp_erfc(double x, double& ex2, double& E)
 {
     const double x2 = x * x;
 #ifdef __CUDA_ARCH__
-    if (x2 < 64.0) { fixed::exp_erfc(fabs(x), x2, ex2, E); return; }
+    if ((unsigned)__double2hiint(x2) < 0x40500000u) { fixed::exp_erfc(fabs(x), x2, ex2, E); return; }
     ex2 = exp_neg(x2);
     E = erfc_far(fabs(x));
 #else
@@ -743,7 +804,12 @@ HGKS_HD __forceinline__ void half_moments(const MState<DIM>& s, double sl, int s
     double ex2, E;
     exp_erfc(x, ex2, E);
     const double e = ex2 * (0.56418958354775628695 * s.p * sl);   // rho h sqrt(lam)/sqrt(pi), rho h = p
-    const bool into = sign > 0 ? x >= 0.0 : x < 0.0;
+#ifdef __CUDA_ARCH__
+    const bool neg = __double2hiint(x) < 0;         // (at x = 0 both forms below give half the mass)
+#else
+    const bool neg = x < 0.0;
+#endif
+    const bool into = (sign > 0) != neg;
     const double hr = scale2<-1>(s.rho);
     m.u[0] = into ? fma(-hr, E, s.rho) : hr * E;
     m.u[1] = fma(s.U, m.u[0], sign > 0 ? e : -e);
@@ -936,7 +1002,8 @@ HGKS_HD __forceinline__ bool flux_finish(const FluxConst& fc, const FluxSums<DIM
     else tau = fma(fc.c2, jump, fc.c1) * dt;
 
     double A0[6], A1[6];
-    if (tau == 0.0) {
+    const bool eq_only = is_zero(tau);
+    if (eq_only) {
         // F(d) = d M1 + d^2/2 M3
         A0[0] = STAGE == 0 ? 0.5 * dt : 0.0;
         A0[2] = STAGE == 0 ? 0.125 * dt * dt : (1.0 / 3.0) * dt * dt;
@@ -953,7 +1020,7 @@ HGKS_HD __forceinline__ bool flux_finish(const FluxConst& fc, const FluxSums<DIM
         if constexpr (STAGE == 0) c1[k] = DIM == 2 && k == 2 ? m1 : fma(A1[0], M1[k], m1);
     }
     double M2[NV];
-    if (tau != 0.0) {
+    if (!eq_only) {
         m2_term<DIM>(sc, fc, dx, dy, M2);
 #pragma unroll
         for (int k = 0; k < NV; k++) {
@@ -963,7 +1030,7 @@ HGKS_HD __forceinline__ bool flux_finish(const FluxConst& fc, const FluxSums<DIM
     }
     add_lab<DIM, true>(sc, c0, o0);
     if constexpr (STAGE == 0) add_lab<DIM, true>(sc, c1, o1);
-    if (tau == 0.0) return true;
+    if (eq_only) return true;
 #pragma unroll
     for (int k = 0; k < NV; k++) {
         o0[k] = fma(A0[3], q.S4[k], fma(A0[4], q.S5[k], fma(-A0[5], q.S6n[k], o0[k])));
