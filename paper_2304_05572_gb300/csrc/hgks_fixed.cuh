@@ -266,5 +266,109 @@ HGKS_FX void exp_erfc(double y, double y2, double& ex, double& er)
     er = pack(umulhi(e.r << 1, erfcx_q(y) << 1), e.n);
 }
 
+// ---------------------------------------------------------------- linear forms of a 5-value window
+// Five values in one unit, v[j] = q[j] 2^(1083-E) truncated, E the largest biased exponent among them
+// (|v| < 2^61: 60 fraction bits of the window's largest value, where a double sum rounds to 53 of it).
+// False where the exponents leave the range in which every result below is a normal double (or a
+// value is infinite or a NaN); a window of zeros gives zeros.
+HGKS_FX bool window(const double* q, i64* v, int& E)
+{
+    u32 top = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int j = 0; j < 5; j++) {
+        const u32 h = (u32)(bits_of(q[j]) >> 32) & 0x7FFFFFFFu;
+        top = h > top ? h : top;
+    }
+    const u32 e = top >> 20;
+    E = e == 0 ? 100 : (int)e;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int j = 0; j < 5; j++) {
+        const u64 b = bits_of(q[j]);
+        const u32 hi = (u32)(b >> 32);
+        const u32 s = 3u + (u32)E - ((hi >> 20) & 0x7FFu);
+        const u64 m = (b << 11) | 0x8000000000000000ull;
+        const u64 a = s < 64u ? m >> s : 0u;
+        v[j] = (int)hi < 0 ? (i64)(0u - a) : (i64)a;
+    }
+    return e == 0 || e - 200u < 1700u;
+}
+
+// r 2^(E-1023-F) as a double
+HGKS_FX double from_fixed(i64 r, int E, int F)
+{
+    const u64 a = r < 0 ? 0u - (u64)r : (u64)r;
+    const u32 h = (u32)(a >> 32);
+    const int lz = h ? clz32(h) : 32 + clz32((u32)a | 1u);
+    const u64 m = a << lz;
+    const u64 d = ((u64)(u32)(E + 62 - F - lz) << 52) + (m >> 11) + ((m >> 10) & 1u);
+    return of_bits(a == 0 ? 0u : d | ((u64)r & 0x8000000000000000ull));
+}
+
+// Multiplier in [1, 2) as 2^-62 halves, and its exponent
+struct Scale { Half m; int e; };
+HGKS_FX Scale scale_of(double x)
+{
+    const u64 b = bits_of(x);
+    return Scale{halves((i64)((b << 10 & 0x3FFFFFFFFFFFFC00ull) | 0x4000000000000000ull)), (int)(b >> 52) - 1023};
+}
+
+// The quartic through the averages of cells i-2..i+2 at its two Gauss points xi = -+1/(2 sqrt 3): v[0], v[1],
+// and (DER) its derivatives there times `inv` (1/h), d[0], d[1].  The values at +-xi are the sum and the
+// difference of an even and an odd form, on q2, q1 + q3, q0 + q4 and q3 - q1, q4 - q0, so that both points take 5
+// products together (5 more for the derivatives).  Coefficients in 2^-62 (719/720, 1/1080, -1/4320;
+// 25 sqrt3/216, -7 sqrt3/432; 2/3, -1/12; -4 sqrt3/9, 13 sqrt3/54, -sqrt3/54), with the last places of one
+// of each set chosen so that constants and linear data come out exactly.  Products keep 58 fraction
+// bits of the window's largest value: values within 2^-54 of it, derivatives within 2^-53 of it times
+// inv, beside their rounding (the FP64 chain: up to 2^-52 and 2^-50).
+// A product of halves drops the two low halves' term, and the partial sums stay below 2^63:
+// |hi| <= 2^30 for a sum of two values, 3.8 2^61 for the largest set.
+HGKS_FX void dot2(Half a, Half ca, Half b, Half cb, i64& hi, i64& cross)
+{
+    cross += (i64)a.hi * ca.lo + (i64)a.lo * ca.hi;
+    hi += (i64)a.hi * ca.hi;
+    cross += (i64)b.hi * cb.lo + (i64)b.lo * cb.hi;
+    hi += (i64)b.hi * cb.hi;
+}
+
+HGKS_FX i64 form2(Half a, i64 ca, Half b, i64 cb)
+{
+    i64 hi = 0, cross = 0;
+    dot2(a, halves(ca), b, halves(cb), hi, cross);
+    return hi + (cross >> 31);
+}
+
+HGKS_FX i64 form3(Half c, i64 cc, Half a, i64 ca, Half b, i64 cb)
+{
+    const Half k = halves(cc);
+    i64 hi = (i64)c.hi * k.hi, cross = (i64)c.hi * k.lo + (i64)c.lo * k.hi;
+    dot2(a, halves(ca), b, halves(cb), hi, cross);
+    return hi + (cross >> 31);
+}
+
+template <bool DER>
+HGKS_FX bool quartic_pair(const double* q, Scale inv, double* v, double* d)
+{
+    i64 w[5];
+    int E;
+    if (!window(q, w, E) || (DER && (u32)(E + inv.e - 100) > 1900u)) return false;
+    const Half c = halves(w[2]), s1 = halves(w[1] + w[3]), s2 = halves(w[0] + w[4]);
+    const Half d1 = halves(w[3] - w[1]), d2 = halves(w[4] - w[0]);
+    const i64 even = form3(c, 4605280898957349864ll, s1, 4270079646692026ll, s2, -1067519911673006ll);
+    const i64 odd = form2(d1, 924499362554543698ll, d2, -129429910757636118ll);
+    v[0] = from_fixed(even - odd, E, 58);
+    v[1] = from_fixed(even + odd, E, 58);
+    if (DER) {
+        const i64 n = form2(d1, 3074457345618258602ll, d2, -384307168202282325ll);
+        const i64 s = form3(c, -3550077552209447800ll, s1, 1922958674113450892ll, s2, -147919898008726992ll);
+        d[0] = from_fixed(smulhi(halves(n - s), inv.m), E + inv.e, 56);
+        d[1] = from_fixed(smulhi(halves(n + s), inv.m), E + inv.e, 56);
+    }
+    return true;
+}
+
 }  // namespace fixed
 }  // namespace hgks

@@ -627,6 +627,7 @@ __device__ __forceinline__ void b_tang_x4(const Params& P, const Sweep& S, Ctrl*
     warp_count(&ctrl->examined[stage][S.dir][1], lead ? 4u : 0u);
     const long long plane = (long long)S.nt * S.nm;
     const long long o = (long long)t * S.nm + m;
+    const fixed::Scale inv = fixed::scale_of(S.inv_ht);
 #pragma unroll
     for (int X = 0; X < 4; X++) {
         bool f = active && ((bits >> X) & 1);
@@ -635,7 +636,8 @@ __device__ __forceinline__ void b_tang_x4(const Params& P, const Sweep& S, Ctrl*
         double qv[5], v[2], d[2];
 #pragma unroll
         for (int s = 0; s < 5; s++) qv[s] = lineval(S, X, q, t - 2 + s, m);
-        gauss_linear(qv, v, d);
+        if (X <= 1) gauss_linear<true>(qv, inv, S.inv_ht, v, d);
+        else gauss_linear<false>(qv, inv, S.inv_ht, v, d);
         if (X <= 1) {
             // Reading: a reconstructed state with rho <= 0 or p <= 0 falls back to first order
 #pragma unroll
@@ -651,14 +653,14 @@ __device__ __forceinline__ void b_tang_x4(const Params& P, const Sweep& S, Ctrl*
 #pragma unroll
         for (int g = 0; g < 2; g++) {
             stc(S.gp + (long long)((g * 6 + qx[X]) * 4 + q) * plane + o, v[g], S);
-            if (X <= 1) stc(S.gp + (long long)((g * 6 + qx[X] + 2) * 4 + q) * plane + o, d[g] * S.inv_ht, S);
+            if (X <= 1) stc(S.gp + (long long)((g * 6 + qx[X] + 2) * 4 + q) * plane + o, d[g], S);
         }
     }
 }
 
 // Large sweeps: the Step-4 spread flags of a segment (stored, counted, troubled passes appended
 // to the WENO-AO work list); the smooth passes are reconstructed inside the flux kernel
-// (b_flux, gp_linear_at), so their Gauss-point states never go to memory.
+// (b_flux, side_pair), so their Gauss-point states never go to memory.
 __device__ __forceinline__ void b_tflags_x1(const Params& P, const Sweep& S, Ctrl* ctrl, int stage, long long id)
 {
     if (ctrl->done) return;
@@ -681,36 +683,6 @@ __device__ __forceinline__ void b_tflags_x1(const Params& P, const Sweep& S, Ctr
         bool f = active && ((bits >> X) & 1);
         warp_push(&ctrl->cnt[S.dir][1], S.itemsT, f, (uint32_t)((((long long)t * S.nm + m) << 2) | X), S);
     }
-}
-
-// Gauss-point state of the smooth pass X of segment (t, m) at Gauss point g (0: -xi_g, 1: +xi_g):
-// the quartic of each component (the FMA chain of gauss_linear, so the same bits), the
-// first-order fallback of the Q^l, Q^r passes, the tangential derivative in 1/h_t units.
-__device__ __forceinline__ void gp_linear_at(const Params& P, const Sweep& S, int X, int t, int m, int g,
-                                             double* v, double* d)
-{
-    const double* cv = g == 0 ? c_gauss.VM[3] : c_gauss.VP[3];
-    const double* cd = g == 0 ? c_gauss.DM[3] : c_gauss.DP[3];
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        double q[5];
-#pragma unroll
-        for (int j = 0; j < 5; j++) q[j] = lineval(S, X, k, t - 2 + j, m);
-        double a = cv[2] * q[2], e = cd[2] * q[2];
-#pragma unroll
-        for (int j = 0; j < 5; j++) {
-            if (j == 2) continue;
-            a = fma(cv[j], q[j], a);
-            e = fma(cd[j], q[j], e);
-        }
-        v[k] = a; d[k] = e;
-    }
-    if (X <= 1 && nonphysical<4>(P.gamma, v)) {
-#pragma unroll
-        for (int k = 0; k < 4; k++) { v[k] = lineval(S, X, k, t, m); d[k] = 0.0; }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; k++) d[k] = d[k] * S.inv_ht;
 }
 
 __device__ __forceinline__ void b_tang(const Params& P, const Sweep& S, Ctrl* ctrl, int stage, long long id)
@@ -830,38 +802,104 @@ __global__ void k_tang_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
 
 
 // ---------------------------------------------------------------- flux and update
-constexpr int kFluxMaxBlock = 256;          // largest block of a flux launch (solo 64, batched up to 256)
 
-// State Wv, normal derivative Wn and tangential derivative Wt (2D) of one side (0: left, 1: right) of
-// segment o at Gauss point g.
+// Shared memory of a 2D flux block of `threads`: the reconstructed side states (24 doubles a
+// thread, see b_flux), then the segment fluxes of the Gauss point 1 warps (8 doubles a pair of threads).
+constexpr int kFluxSideDoubles = 24;
+inline size_t flux_smem(int dim, int threads)
+{
+    return dim == 2 ? (size_t)threads * (kFluxSideDoubles + 4) * sizeof(double) : 0;
+}
+
+// State, tangential and normal derivative of one side (0: left, 1: right) of segment (t, m) at both Gauss
+// points (2D, large sweeps): the troubled passes from k_tang_ao, the smooth ones reconstructed
+// here.  x[(12 g + j) stride]: j = 0..3 state, 4..7 normal, 8..11 tangential derivative at Gauss point g.
+__device__ __forceinline__ void side_pair(const Params& P, const Sweep& S, int side, long long o, double* __restrict__ x, int stride)
+{
+    const long long per = (long long)S.nt * S.nm;
+    const unsigned bits = rdc(S.flagT + o, S);
+    const int t = (int)((unsigned)o / (unsigned)S.nm), m = (int)((unsigned)o - (unsigned)t * (unsigned)S.nm);   // o < 2^31
+    // the Gauss-point buffer's quantities: 0 Wl, 1 Wlx, 2 Wly, 3 Wr, 4 Wrx, 5 Wry
+    const double* gp = S.gp + (long long)(3 * side * 4) * per + o;
+    const fixed::Scale inv = fixed::scale_of(S.inv_ht);
+    if ((bits >> side) & 1) {
+#pragma unroll 1
+        for (int g = 0; g < 2; g++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                x[(12 * g + k) * stride] = ldc(gp + (long long)(24 * g + k) * per, S);
+                x[(12 * g + 8 + k) * stride] = ldc(gp + (long long)(24 * g + 8 + k) * per, S);
+            }
+    } else {
+        double v[4][2], d[2];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            double q[5];
+#pragma unroll
+            for (int j = 0; j < 5; j++) q[j] = lineval(S, side, k, t - 2 + j, m);
+            gauss_linear<true>(q, inv, S.inv_ht, v[k], d);
+            x[(8 + k) * stride] = d[0];
+            x[(20 + k) * stride] = d[1];
+        }
+#pragma unroll
+        for (int g = 0; g < 2; g++) {
+            const double Q[4] = {v[0][g], v[1][g], v[2][g], v[3][g]};
+            if (nonphysical<4>(P.gamma, Q)) {
+                // Reading: a reconstructed state with rho <= 0 or p <= 0 falls back to first order
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    x[(12 * g + k) * stride] = lineval(S, side, k, t, m);
+                    x[(12 * g + 8 + k) * stride] = 0.0;
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; k++) x[(12 * g + k) * stride] = Q[k];
+            }
+        }
+    }
+    if ((bits >> (2 + side)) & 1) {
+#pragma unroll
+        for (int g = 0; g < 2; g++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) x[(12 * g + 4 + k) * stride] = ldc(gp + (long long)(24 * g + 4 + k) * per, S);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            double q[5], v[2];
+#pragma unroll
+            for (int j = 0; j < 5; j++) q[j] = lineval(S, 2 + side, k, t - 2 + j, m);
+            gauss_linear<false>(q, inv, S.inv_ht, v, nullptr);
+            x[(4 + k) * stride] = v[0];
+            x[(16 + k) * stride] = v[1];
+        }
+    }
+}
+
+// State Wv, normal derivative Wn and tangential derivative Wt (2D) of one side of segment o at Gauss point
+// g: in 1D from the line buffer, in 2D from the Gauss-point buffer (small sweeps, where k_tang and
+// k_tang_ao reconstructed every pass) or from shared memory (large sweeps, side_pair).
 template <int DIM>
-__device__ __forceinline__ void side_states(const Params& P, const Sweep& S, int side, int g, long long o,
+__device__ __forceinline__ void side_states(const Params& P, const Sweep& S, int side, int g, long long o, const double* x, int stride,
                                             double* Wv, double* Wn, double* Wt)
 {
     constexpr int NV = DIM + 2;
     if constexpr (DIM == 2) {
         const long long per = (long long)S.nt * S.nm;
-        // the Gauss-point buffer's quantities: 0 Wl, 1 Wlx, 2 Wly, 3 Wr, 4 Wrx, 5 Wry
         const double* gp = S.gp + (long long)((g * 6 + 3 * side) * 4) * per + o;
-        // small sweeps: every pass was reconstructed by k_tang / k_tang_ao; large sweeps: the troubled
-        // passes by k_tang_ao, the smooth ones here
-        const unsigned bits = S.tlanes == 4 ? 0xFu : (unsigned)rdc(S.flagT + o, S);
-        const int t = (int)(o / S.nm), m = (int)(o % S.nm);
-        if ((bits >> side) & 1) {
+        if (S.tlanes == 4) {
 #pragma unroll
             for (int k = 0; k < NV; k++) {
                 Wv[k] = ldc(gp + (long long)k * per, S);
+                Wn[k] = ldc(gp + (long long)(4 + k) * per, S);
                 Wt[k] = ldc(gp + (long long)(8 + k) * per, S);
             }
         } else {
-            gp_linear_at(P, S, side, t, m, g, Wv, Wt);
-        }
-        if ((bits >> (2 + side)) & 1) {
 #pragma unroll
-            for (int k = 0; k < NV; k++) Wn[k] = ldc(gp + (long long)(4 + k) * per, S);
-        } else {
-            double unused[NV];
-            gp_linear_at(P, S, 2 + side, t, m, g, Wn, unused);
+            for (int k = 0; k < NV; k++) {
+                Wv[k] = x[(12 * g + k) * stride];
+                Wn[k] = x[(12 * g + 4 + k) * stride];
+                Wt[k] = x[(12 * g + 8 + k) * stride];
+            }
         }
     } else {
         const long long plane = (long long)S.nlines * S.nm;
@@ -891,6 +929,19 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     }
     const bool valid = o < per;
     double o0[NV], o1[NV];
+    extern __shared__ double flux_sh[];
+    const int stride = blockDim.x;
+    const int pair0 = threadIdx.x & ~32;         // this thread's lane in the pair's first warp
+    if constexpr (DIM == 2) {
+        // large sweeps: warp 0 of the pair reconstructs the left side at both Gauss points, warp 1 the right
+        // side, and they exchange through shared memory: every line value is loaded and converted once, and
+        // the two points share their products (with the products in FP64 and each warp reconstructing both
+        // sides at its own point the launch took 5.04 ms at 1024^2, so 4.18 ms)
+        if (S.tlanes != 4) {
+            if (valid) side_pair(P, S, g, o, flux_sh + threadIdx.x, stride);
+            __syncthreads();
+        }
+    }
     if (valid) {
     // one side after the other: only the side at work holds its states and slopes in registers
     FluxSums<DIM> sums;
@@ -898,12 +949,12 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     bool ok;
     {
         double Wv[NV], Wn[NV], Wt[NV];
-        side_states<DIM>(P, S, 0, g, o, Wv, Wn, Wt);
+        side_states<DIM>(P, S, 0, g, o, flux_sh + pair0, stride, Wv, Wn, Wt);
         ok = flux_side<DIM, PRFIX, true>(P.fc, Wv, Wn, Wt, sums, pl);
     }
     if (ok) {
         double Wv[NV], Wn[NV], Wt[NV];
-        side_states<DIM>(P, S, 1, g, o, Wv, Wn, Wt);
+        side_states<DIM>(P, S, 1, g, o, flux_sh + pair0 + 32, stride, Wv, Wn, Wt);
         ok = flux_side<DIM, PRFIX, false>(P.fc, Wv, Wn, Wt, sums, pr);
     }
     if (ok) ok = flux_finish<DIM, STAGE, PRFIX>(P.fc, sums, pl, pr, ctrl->dt, o0, o1);
@@ -920,21 +971,22 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     // through shared memory; stored per segment as [output][component][segment]
     constexpr int NO = STAGE == 0 ? 2 : 1;
     if constexpr (DIM == 2) {
-        __shared__ double pair[kFluxMaxBlock / 2][2 * 4];
-        const int slot = ((threadIdx.x >> 6) << 5) + (threadIdx.x & 31);
+        // [output component][lane pair]
+        double* pair = flux_sh + kFluxSideDoubles * stride + ((threadIdx.x >> 6) << 5) + (threadIdx.x & 31);
+        const int ps = stride >> 1;
         if (g == 1 && valid) {
 #pragma unroll
             for (int k = 0; k < NV; k++) {
-                pair[slot][k] = o0[k];
-                if (STAGE == 0) pair[slot][NV + k] = o1[k];
+                pair[k * ps] = o0[k];
+                if (STAGE == 0) pair[(NV + k) * ps] = o1[k];
             }
         }
         __syncthreads();
         if (g == 1 || !valid) return;
 #pragma unroll
         for (int k = 0; k < NV; k++) {
-            o0[k] = fma(0.5, o0[k], 0.5 * pair[slot][k]);
-            if (STAGE == 0) o1[k] = fma(0.5, o1[k], 0.5 * pair[slot][NV + k]);
+            o0[k] = fma(0.5, o0[k], 0.5 * pair[k * ps]);
+            if (STAGE == 0) o1[k] = fma(0.5, o1[k], 0.5 * pair[(NV + k) * ps]);
         }
     } else {
         if (!valid) return;
@@ -1145,7 +1197,7 @@ __global__ void kb_tang_ao(const SolveDesc* __restrict__ D, const int* __restric
 }
 
 template <int DIM, int STAGE>
-__global__ void __launch_bounds__(256) kb_flux(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
+__global__ void __launch_bounds__(128) kb_flux(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
 {
     HGKS_BATCH_SWEEP_BLOCK();
     if (d.P.fc.prfix != 0.0) flux_nl<DIM, STAGE, true>(d, dir, id);
@@ -1336,11 +1388,11 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
         unsigned int g = pair([](const Sweep& S) { return blocks_for(flux_threads(DIM, (long long)S.nt * S.nm), 64); }, nb);
         const int n0 = (int)nb[0];
         if (P.fc.prfix != 0.0) {
-            if (stage == 0) k_flux<DIM, 0, true><<<g, 64, 0, st>>>(D, n0);
-            else k_flux<DIM, 1, true><<<g, 64, 0, st>>>(D, n0);
+            if (stage == 0) k_flux<DIM, 0, true><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
+            else k_flux<DIM, 1, true><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
         } else {
-            if (stage == 0) k_flux<DIM, 0, false><<<g, 64, 0, st>>>(D, n0);
-            else k_flux<DIM, 1, false><<<g, 64, 0, st>>>(D, n0);
+            if (stage == 0) k_flux<DIM, 0, false><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
+            else k_flux<DIM, 1, false><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
         }
     });
 }
@@ -1514,8 +1566,8 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
         mark(BK_FLUX, 0);
         const int tf = tp(BK_FLUX);
         if (dim == 2) {
-            if (stage == 0) kb_flux<2, 0><<<grid(BK_FLUX), tf, 0, st>>>(dd, bo(BK_FLUX), n);
-            else kb_flux<2, 1><<<grid(BK_FLUX), tf, 0, st>>>(dd, bo(BK_FLUX), n);
+            if (stage == 0) kb_flux<2, 0><<<grid(BK_FLUX), tf, flux_smem(2, tf), st>>>(dd, bo(BK_FLUX), n);
+            else kb_flux<2, 1><<<grid(BK_FLUX), tf, flux_smem(2, tf), st>>>(dd, bo(BK_FLUX), n);
         } else {
             if (stage == 0) kb_flux<1, 0><<<grid(BK_FLUX), tf, 0, st>>>(dd, bo(BK_FLUX), n);
             else kb_flux<1, 1><<<grid(BK_FLUX), tf, 0, st>>>(dd, bo(BK_FLUX), n);

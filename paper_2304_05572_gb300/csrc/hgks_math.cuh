@@ -499,9 +499,14 @@ __device__ __constant__ GaussCoef c_gauss = {
      {1.15408348288312548e-01, -1.08364186108139648e+00, 7.69800358919501049e-01, 2.49691472251936941e-01, -5.12583183783541230e-02}},
 };
 
-// quartic at the two Gauss points: v[0] at -g, v[1] at +g (and cell-unit derivatives)
-__device__ __forceinline__ void gauss_linear(const double* q, double* v, double* d)
+#if defined(__CUDACC__)
+// Quartic of the window q at the two Gauss points: v[0] at -g, v[1] at +g, and (DER) its derivatives
+// there times inv_ht (`inv` the same as a fixed-point factor).  In fixed point (fixed::quartic_pair); FP64
+// for exponents outside its range, infinities and NaNs.
+template <bool DER>
+__device__ __forceinline__ void gauss_linear(const double* q, fixed::Scale inv, double inv_ht, double* v, double* d)
 {
+    if (fixed::quartic_pair<DER>(q, inv, v, d)) return;
     const double* vm = c_gauss.VM[3]; const double* vp = c_gauss.VP[3];
     const double* dm = c_gauss.DM[3]; const double* dp = c_gauss.DP[3];
     double a = vm[2] * q[2], b = vp[2] * q[2], e = dm[2] * q[2], f = dp[2] * q[2];
@@ -511,8 +516,10 @@ __device__ __forceinline__ void gauss_linear(const double* q, double* v, double*
         a = fma(vm[j], q[j], a); b = fma(vp[j], q[j], b);
         e = fma(dm[j], q[j], e); f = fma(dp[j], q[j], f);
     }
-    v[0] = a; v[1] = b; d[0] = e; d[1] = f;
+    v[0] = a; v[1] = b;
+    if (DER) { d[0] = e * inv_ht; d[1] = f * inv_ht; }
 }
+#endif
 
 __device__ __forceinline__ void gauss_ao(const fx* q, const AOConst& k, double* v, double* d)
 {

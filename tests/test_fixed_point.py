@@ -4,7 +4,10 @@
 Bounds in units of the result's last place: one rounding (1/2), the approximations' own remainders
 (2^-9 for the two reciprocals; for the exponential 2^-5 for the argument's 57 fraction bits and
 2^-4 for series and truncations, bounded here by 1/4), and for erfc the table's 2.1e-16 (up to 1.9
-units) beside the exponential's."""
+units) beside the exponential's.  The Gauss-point quartic (quartic_pair) loses, beside its rounding,
+at most 1.5 2^-60 by the window's truncation and 1.5 2^-58 per product and set (values: 5 products, 2
+sets; derivatives the same and 3 2^-56 for the factor 1/h) of the window's largest value: within
+2^-54 and 2^-53."""
 import os
 import subprocess
 
@@ -33,6 +36,44 @@ int main(int argc, char** argv)
     std::mt19937_64 g(20230415);
     std::uniform_real_distribution<double> U(0.0, 1.0);
     double worst = 0.0;
+    if (!strcmp(what, "quartic")) {
+        // error beyond one rounding, relative to the window's largest value (and 1/h): values, derivatives
+        const long double r3 = std::sqrt(3.0L);
+        double wv = 0.0, wd = 0.0;
+        bool ok = true;
+        for (long i = 0; i < 200000; i++) {
+            double q[5], v[2], d[2], mx = 0.0;
+            const double base = i & 1 ? 6.0 * U(g) - 3.0 : 0.0, amp = i & 1 ? std::exp(-U(g) * 40.0) : 1.0;
+            const double sc = std::ldexp(1.0, (int)(U(g) * 600.0) - 300), inv = std::exp(40.0 * U(g) - 20.0);
+            for (double& x : q) x = sc * (base + amp * (2.0 * U(g) - 1.0) * (i & 4 ? std::exp(-U(g) * 20.0) : 1.0));
+            if (i % 50 == 0) for (int j = 1; j < 5; j++) q[j] = q[0];
+            if (i % 50 == 1) { q[0] = q[1] = 0.0; q[3] = -q[3]; }
+            for (double x : q) mx = std::fmax(mx, std::fabs(x));
+            ok = ok && quartic_pair<true>(q, scale_of(inv), v, d);
+            double u[2];
+            ok = ok && quartic_pair<false>(q, scale_of(inv), u, nullptr) && u[0] == v[0] && u[1] == v[1];
+            if (i % 50 == 0) ok = ok && v[0] == q[0] && v[1] == q[0];
+            for (int k = 0; k < 2; k++) {
+                const long double s = k ? r3 : -r3;
+                const long double c[5] = {-1 / 4320.0L + 7 * s / 432, 1 / 1080.0L - 25 * s / 216, 719 / 720.0L,
+                                          1 / 1080.0L + 25 * s / 216, -1 / 4320.0L - 7 * s / 432};
+                const long double e[5] = {1 / 12.0L - s / 54, -2 / 3.0L + 13 * s / 54, -4 * s / 9, 2 / 3.0L + 13 * s / 54, -1 / 12.0L - s / 54};
+                long double a = 0, b = 0;
+                for (int j = 0; j < 5; j++) { a += c[j] * q[j]; b += e[j] * q[j]; }
+                b *= inv;
+                wv = std::fmax(wv, (double)((std::fabs(v[k] - a) - std::fabs(a) * 0x1p-53L) / mx));
+                wd = std::fmax(wd, (double)((std::fabs(d[k] - b) - std::fabs(b) * 0x1p-53L) / (mx * (long double)inv)));
+            }
+        }
+        double z[5] = {0.0, -0.0, 0.0, 0.0, 0.0}, v[2], d[2];
+        ok = ok && quartic_pair<true>(z, scale_of(3.0), v, d) && v[0] == 0 && v[1] == 0 && d[0] == 0 && d[1] == 0;
+        for (double bad : {std::numeric_limits<double>::infinity(), std::numeric_limits<double>::quiet_NaN(), 1e-280, 1e280}) {
+            z[1] = bad;
+            ok = ok && !quartic_pair<true>(z, scale_of(3.0), v, d);
+        }
+        printf("%d %.6f %.6f\n", ok ? 1 : 0, std::ldexp(wv, 54), std::ldexp(wd, 53));
+        return 0;
+    }
     if (!strcmp(what, "special")) {
         const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
         bool ok = true;
@@ -93,3 +134,8 @@ def test_within_bounds(exe, what, bound):
 
 def test_special_arguments(exe):
     assert subprocess.run([exe, "special"], check=True, capture_output=True, text=True).stdout.strip() == "1"
+
+
+def test_gauss_point_quartic(exe):
+    ok, wv, wd = subprocess.run([exe, "quartic"], check=True, capture_output=True, text=True).stdout.split()
+    assert ok == "1" and float(wv) <= 1.0 and float(wd) <= 1.0, (ok, wv, wd)
