@@ -115,14 +115,10 @@ HGKS_FX double scale2(double x)
     return of_bits(((u64)h << 32) | (u32)b);
 }
 
-// 1/x: the 23-bit reciprocal of the leading bits and one third-order Newton step in fixed point,
-// 1/m = y (1 + e + e^2), e = 1 - m y.  Out of range: |x| >= 2^1022 gives 0; zero, subnormal, infinite and NaN
-// arguments give a NaN (which the flux's physical-state tests reject).
-HGKS_FX double rcp(double x)
+// 1/m for m in [1, 2) given in units of 2^-63, as r 2^-63, r in (2^62, 2^63], within 2 units: the 23-bit
+// reciprocal of the leading bits and one third-order Newton step, 1/m = y (1 + e + e^2), e = 1 - m y.
+HGKS_FX u64 rcp_mantissa(u64 m)
 {
-    const u64 b = bits_of(x);
-    const u32 hi = (u32)(b >> 32), e0 = (hi >> 20) & 0x7FF;
-    const u64 m = (b << 11) | 0x8000000000000000ull;                       // [1, 2) in 2^-63
     float y0 = approx_rcp(float_of(0x3F800000u | (u32)(m << 1 >> 41)));
     y0 = y0 < 0.99999994f ? y0 : 0.99999994f;                              // (1/2, 1)
     const u32 y = (float_bits(y0) << 8) | 0x80000000u;                     // 2^-32
@@ -130,22 +126,13 @@ HGKS_FX double rcp(double x)
     const i64 e = (i64)(0x8000000000000000ull - p);                        // |e| < 2^42
     const i64 eh = (int)(e >> 12);
     const i64 s = e + ((eh * eh) >> 39);
-    const u64 r = ((u64)y << 31) + (u64)((i64)((int)(s >> 32)) * (i64)y) + (((u64)(u32)s * y) >> 32);   // 2^-63, (1/2, 1]
-    const u64 mant = ((u64)(2044u - e0) << 52) + ((r + 512u) >> 10);
-    const bool in = e0 - 1u < 2044u;
-    const u32 h = in ? (u32)(mant >> 32) : e0 - 2045u < 2u ? 0u : 0x7FF80000u;
-    return of_bits((((u64)(h | (hi & 0x80000000u))) << 32) | (in ? (u32)mant : 0u));
+    return ((u64)y << 31) + (u64)((i64)((int)(s >> 32)) * (i64)y) + (((u64)(u32)s * y) >> 32);
 }
 
-// 1/sqrt(x): the same with 1/sqrt(m) = y (1 + e/2 + 3 e^2/8), e = 1 - m y^2.  A NaN unless x is positive,
-// normal and finite.
-HGKS_FX double rsqrt(double x)
+// 1/sqrt(m) for m in [1, 4) in units of 2^-62 (frac: 23 fraction bits of m or m/2, odd: m < 2), as r 2^-63:
+// the same with 1/sqrt(m) = y (1 + e/2 + 3 e^2/8), e = 1 - m y^2.
+HGKS_FX u64 rsqrt_mantissa(u64 m, u32 frac, u32 odd)
 {
-    const u64 b = bits_of(x);
-    const u32 hi = (u32)(b >> 32), e0 = hi >> 20;                          // with the sign bit
-    const u32 odd = e0 & 1u;                                               // odd biased exponent: m in [1, 2)
-    const u64 m = ((b << 11) | 0x8000000000000000ull) >> odd;              // [1, 4) in 2^-62
-    const u32 frac = (hi << 3 & 0x007FFFF8u) | ((u32)b >> 29);
     float y0 = approx_rsqrt(float_of((odd ? 0x3F800000u : 0x40000000u) | frac));
     y0 = y0 < 0.99999994f ? y0 : 0.99999994f;
     const u32 y = (float_bits(y0) << 8) | 0x80000000u;                     // 2^-32, [1/2, 1)
@@ -153,10 +140,73 @@ HGKS_FX double rsqrt(double x)
     const i64 e = (i64)(0x4000000000000000ull - p);                        // e in 2^-62 = e/2 in 2^-63
     const i64 eh = (int)(e >> 11);                                         // 2^-51
     const i64 s = e + ((eh * eh) >> 42) * 3;
-    const u64 r = ((u64)y << 31) + (u64)((i64)((int)(s >> 32)) * (i64)y) + (((u64)(u32)s * y) >> 32);
+    return ((u64)y << 31) + (u64)((i64)((int)(s >> 32)) * (i64)y) + (((u64)(u32)s * y) >> 32);
+}
+
+// 1/x.  Out of range: |x| >= 2^1022 gives 0; zero, subnormal, infinite and NaN arguments give a NaN
+// (which the flux's physical-state tests reject).
+HGKS_FX double rcp(double x)
+{
+    const u64 b = bits_of(x);
+    const u32 hi = (u32)(b >> 32), e0 = (hi >> 20) & 0x7FF;
+    const u64 r = rcp_mantissa((b << 11) | 0x8000000000000000ull);
+    const u64 mant = ((u64)(2044u - e0) << 52) + ((r + 512u) >> 10);
+    const bool in = e0 - 1u < 2044u;
+    const u32 h = in ? (u32)(mant >> 32) : e0 - 2045u < 2u ? 0u : 0x7FF80000u;
+    return of_bits((((u64)(h | (hi & 0x80000000u))) << 32) | (in ? (u32)mant : 0u));
+}
+
+// 1/sqrt(x); a NaN unless x is positive, normal and finite.
+HGKS_FX double rsqrt(double x)
+{
+    const u64 b = bits_of(x);
+    const u32 hi = (u32)(b >> 32), e0 = hi >> 20;                          // with the sign bit
+    const u32 odd = e0 & 1u;                                               // odd biased exponent: m in [1, 2)
+    const u64 r = rsqrt_mantissa(((b << 11) | 0x8000000000000000ull) >> odd, (hi << 3 & 0x007FFFF8u) | ((u32)b >> 29), odd);
     const u64 mant = ((u64)(1021u - (u32)(((int)e0 - 1023) >> 1)) << 52) + ((r + 512u) >> 10);
     const u32 h = e0 - 1u < 2046u ? (u32)(mant >> 32) : 0x7FF80000u;
     return of_bits(((u64)h << 32) | (u32)mant);
+}
+
+// IEEE a / b (round to nearest) where a is zero or normal, b normal and the quotient normal and
+// below 2^1023; false elsewhere.  The quotient of the mantissas to 61 bits, rounded to 53 and corrected by the sign of the
+// exact remainder against half a unit (a quotient of two doubles is never half way between two).
+HGKS_FX bool div_rn(double a, double b, double& q)
+{
+    const u64 ab = bits_of(a), bb = bits_of(b);
+    const u32 ah = (u32)(ab >> 32), bh = (u32)(bb >> 32);
+    const u32 ea = (ah >> 20) & 0x7FFu, eb = (bh >> 20) & 0x7FFu;
+    const u64 ma = (ab & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull, mb = (bb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+    const u64 t = umulhi(ma << 11, rcp_mantissa(mb << 11));                // ma/mb in 2^-62, (1/2, 2)
+    const u32 small = t < 0x4000000000000000ull ? 1u : 0u;                 // quotient below 1
+    const u32 sh = 10u - small;
+    u64 c = (t + (256ull << (1u - small))) >> sh;                          // 53 bits, unit 2^-52 or 2^-53
+    const i64 r2 = (i64)((ma << (52u + small)) - c * mb) * 2;              // twice the remainder (its low 64 bits are all of it)
+    c += r2 > (i64)mb ? 1u : 0u;
+    c -= r2 < -(i64)mb ? 1u : 0u;
+    const u32 e = ea + 1022u - eb - small;                                 // exponent field less 1 (c carries the hidden bit)
+    const u64 z = ((u64)e << 52) + c;
+    const bool zero = ab << 1 == 0u;
+    q = of_bits((zero ? 0u : z) | ((ab ^ bb) & 0x8000000000000000ull));
+    return eb - 1u < 2046u && (zero || (ea - 1u < 2046u && e < 2045u));
+}
+
+// IEEE sqrt(x) (round to nearest) for positive normal x; false elsewhere.  Rounded from x/sqrt(x) in 2^-61
+// and corrected by the remainder x - c^2, which must lie in (-c, c].
+HGKS_FX bool sqrt_rn(double x, double& q)
+{
+    const u64 b = bits_of(x);
+    const u32 hi = (u32)(b >> 32), e0 = hi >> 20;
+    const u32 odd = e0 & 1u;
+    const u64 m = ((b << 11) | 0x8000000000000000ull) >> odd;              // [1, 4) in 2^-62
+    const u64 t = umulhi(m, rsqrt_mantissa(m, (hi << 3 & 0x007FFFF8u) | ((u32)b >> 29), odd));   // 2^-61, [1, 2)
+    u64 c = (t + 256u) >> 9;
+    const u64 m53 = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+    const i64 r = (i64)((m53 << (53u - odd)) - c * c);                     // low 64 bits of m 2^104 - c^2
+    c += r > (i64)c ? 1u : 0u;
+    c -= r <= -(i64)c ? 1u : 0u;
+    q = of_bits((((u64)(u32)(((int)e0 - 1023) >> 1) + 1022u) << 52) + c);
+    return e0 - 1u < 2046u;
 }
 
 #include "exp2_table.inc"

@@ -38,11 +38,31 @@ struct ex {
 __device__ __forceinline__ ex operator+(ex a, ex b) { return ex(__dadd_rn(a.v, b.v)); }
 __device__ __forceinline__ ex operator-(ex a, ex b) { return ex(__dsub_rn(a.v, b.v)); }
 __device__ __forceinline__ ex operator*(ex a, ex b) { return ex(__dmul_rn(a.v, b.v)); }
+#if defined(__CUDACC__)
+// IEEE quotients and roots in integers: the same bits, where the compiler's sequences take 10 to 15
+// FP64 instructions; those remain for zeros, subnormals, infinities, NaNs and the ends of the range.
+// WENO-AO everywhere on 500^2: normal passes 4.65 -> 3.85 ms per step; dt at 1024^2 97 -> 46 us.
+__device__ __noinline__ double div_far(double a, double b) { return __ddiv_rn(a, b); }
+__device__ __noinline__ double sqrt_far(double a) { return __dsqrt_rn(a); }
+__device__ __forceinline__ ex operator/(ex a, ex b)
+{
+    double q;
+    if (!fixed::div_rn(a.v, b.v, q)) q = div_far(a.v, b.v);
+    return ex(q);
+}
+__device__ __forceinline__ ex xsqrt(ex a)
+{
+    double q;
+    if (!fixed::sqrt_rn(a.v, q)) q = sqrt_far(a.v);
+    return ex(q);
+}
+#else
 __device__ __forceinline__ ex operator/(ex a, ex b) { return ex(__ddiv_rn(a.v, b.v)); }
+__device__ __forceinline__ ex xsqrt(ex a) { return ex(__dsqrt_rn(a.v)); }
+#endif
 __device__ __forceinline__ ex operator-(ex a) { return ex(-a.v); }
 __device__ __forceinline__ ex xfma(ex a, ex b, ex c) { return ex(__fma_rn(a.v, b.v, c.v)); }
 __device__ __forceinline__ ex xabs(ex a) { return ex(fabs(a.v)); }
-__device__ __forceinline__ ex xsqrt(ex a) { return ex(__dsqrt_rn(a.v)); }
 
 // 1/x and 1/sqrt(x) in free-order arithmetic (the flux, the tangential WENO-AO pass), in fixed
 // point on the device: no FP64 instruction where the hardware's approximation and two

@@ -74,6 +74,33 @@ int main(int argc, char** argv)
         printf("%d %.6f %.6f\n", ok ? 1 : 0, std::ldexp(wv, 54), std::ldexp(wd, 53));
         return 0;
     }
+    if (!strcmp(what, "ieee")) {
+        // quotients and roots: the host's bits on random operands, on short mantissas and on operands made
+        // so that the result lies next to the middle between two doubles
+        long wrong = 0, taken = 0, n = 400000;
+        for (long i = 0; i < n; i++) {
+            auto draw = [&](bool wide) {
+                u64 m = g() & 0xFFFFFFFFFFFFFull, e = wide ? 1 + g() % 2046 : 900 + g() % 200;
+                const int sh = (int)(g() % 53);
+                if (i % 4 == 1) m &= ~((1ull << sh) - 1);
+                if (i % 4 == 2) m |= (1ull << sh) - 1;
+                return of_bits((g() & 0x8000000000000000ull) | (e << 52) | m);
+            };
+            double a = draw(i & 1), b = draw(i & 1), q;
+            if (i % 5 == 0) a = of_bits(bits_of(b * draw(false)) + g() % 3 - 1);
+            if (i % 1000 == 0) a = std::copysign(0.0, a);
+            if (div_rn(a, b, q)) { taken++; wrong += bits_of(q) != bits_of(a / b); }
+            double x = std::fabs(draw(i & 1));
+            if (i % 3 == 0) { const double y = draw(false); x = of_bits(bits_of(y * y) + g() % 3 - 1); }
+            if (sqrt_rn(x, q)) wrong += bits_of(q) != bits_of(std::sqrt(x));
+        }
+        const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
+        double q;
+        for (double v : {0.0, -0.0, 1e-310, inf, nan}) wrong += div_rn(1.0, v, q) + sqrt_rn(v, q) + (v == 0.0 ? 0 : div_rn(v, 1.0, q));
+        wrong += sqrt_rn(-1.0, q) + div_rn(1e300, 1e-300, q) + div_rn(1e-300, 1e300, q) + div_rn(1e-200, 1e108, q);
+        printf("%ld %d\n", wrong, taken > n / 2 ? 1 : 0);
+        return 0;
+    }
     if (!strcmp(what, "special")) {
         const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
         bool ok = true;
@@ -139,3 +166,7 @@ def test_special_arguments(exe):
 def test_gauss_point_quartic(exe):
     ok, wv, wd = subprocess.run([exe, "quartic"], check=True, capture_output=True, text=True).stdout.split()
     assert ok == "1" and float(wv) <= 1.0 and float(wd) <= 1.0, (ok, wv, wd)
+
+
+def test_ieee_division_and_root(exe):
+    assert subprocess.run([exe, "ieee"], check=True, capture_output=True, text=True).stdout.split() == ["0", "1"]
