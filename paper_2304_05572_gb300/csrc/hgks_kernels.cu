@@ -702,24 +702,24 @@ __global__ void k_tang(const SolveDesc* __restrict__ D, int nb0, int stage)
 // The troubled tangential pass `it`: its pass X, segment (t, m), the eigenvectors at the face
 // average (tangential direction) and the pass's 5 line values.
 __device__ __forceinline__ void tang_ao_item(const Params& P, const Sweep& S, const double* __restrict__ W, uint32_t it,
-                                             int& X, int& t, int& m, fx (*Lm)[4], fx (*Rm)[4], fx (*x)[4])
+                                             int& X, int& t, int& m, TangEig& e, double (*x)[4])
 {
     X = it & 3;
-    const long long tm = it >> 2;
-    m = (int)(tm % S.nm); t = (int)(tm / S.nm);
-    fx qs[4];
+    const uint32_t tm = it >> 2;
+    t = (int)(tm / (uint32_t)S.nm); m = (int)(tm - (uint32_t)t * (uint32_t)S.nm);
+    double qs[4];
     const double* cl = cellp(P, S, W, t, m - 1);
     const double* cr = cellp(P, S, W, t, m);
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         long long o = (long long)S.perm[k] * P.g.plane;
-        qs[k] = (fx(ldc(cl + o, S)) + fx(ldc(cr + o, S))) * fx(0.5);
+        qs[k] = scale2<-1>(ldc(cl + o, S) + ldc(cr + o, S));
     }
-    eigvec<4>(P.gamma, qs, 0.0, 1.0, Lm, Rm);
+    tang_eig(P.gamma, qs, e);
 #pragma unroll
     for (int s = 0; s < 5; s++)
 #pragma unroll
-        for (int k = 0; k < 4; k++) x[s][k] = fx(lineval(S, X, k, t - 2 + s, m));
+        for (int k = 0; k < 4; k++) x[s][k] = lineval(S, X, k, t - 2 + s, m);
 }
 
 // The troubled tangential passes: one per lane (tang_ao) from kAoOneLaneMin items on, else one
@@ -739,10 +739,10 @@ __device__ __forceinline__ void b_tang_ao(const Params& P, const Sweep& S, const
     if (n >= kAoOneLaneMin) {
         for (unsigned int i = (unsigned int)lane; i < n; i += (unsigned int)lanes) {
             int X, t, m;
-            fx Lm[4][4], Rm[4][4], x[5][4];
-            tang_ao_item(P, S, W, rdc(S.itemsT + i, S), X, t, m, Lm, Rm, x);
-            double v[4][2], d[4][2];
-            tang_ao(Lm, Rm, x, ak, v, d);
+            TangEig e;
+            double x[5][4], v[4][2], d[4][2];
+            tang_ao_item(P, S, W, rdc(S.itemsT + i, S), X, t, m, e, x);
+            tang_ao(e, x, ak, X <= 1, v, d);
             gp_positivity(P, S, t, m, X, v, d);
             const long long o = (long long)t * S.nm + m;
             const int qv = X == 0 ? 0 : (X == 1 ? 3 : (X == 2 ? 1 : 4));
@@ -761,10 +761,10 @@ __device__ __forceinline__ void b_tang_ao(const Params& P, const Sweep& S, const
     const unsigned gmask = 0xFu << lane0;
     for (unsigned int i = (unsigned int)(lane >> 2); i < n; i += (unsigned int)(lanes >> 2)) {
         int X, t, m;
-        fx Lm[4][4], Rm[4][4], x[5][4];
-        tang_ao_item(P, S, W, rdc(S.itemsT + i, S), X, t, m, Lm, Rm, x);
-        double vq[2], dq[2];
-        tang_ao_x4(Lm, Rm, x, ak, gmask, vq, dq);
+        TangEig e;
+        double x[5][4], vq[2], dq[2];
+        tang_ao_item(P, S, W, rdc(S.itemsT + i, S), X, t, m, e, x);
+        tang_ao_x4(e, x, ak, X <= 1, gmask, vq, dq);
         if (X <= 1) {
             // positivity of the reconstructed Q^l, Q^r states (gp_positivity), on the gathered components
 #pragma unroll

@@ -128,26 +128,6 @@ HGKS_HD __forceinline__ double exp_neg(double y)
 #endif
 }
 
-// Free-order FP64 with the same interface: the compiler may contract a*b + c into an FMA, and
-// divisions and square roots go through the Newton-refined reciprocals above.  Used where the
-// outputs only feed the flux (the tangential WENO-AO pass), never a flag decision.
-struct fx {
-    double v;
-    __device__ __forceinline__ fx() {}
-    __device__ __forceinline__ fx(double x) : v(x) {}
-};
-__device__ __forceinline__ fx operator+(fx a, fx b) { return fx(a.v + b.v); }
-__device__ __forceinline__ fx operator-(fx a, fx b) { return fx(a.v - b.v); }
-__device__ __forceinline__ fx operator*(fx a, fx b) { return fx(a.v * b.v); }
-__device__ __forceinline__ fx operator/(fx a, fx b) { return fx(a.v * rcp_nr(b.v)); }
-__device__ __forceinline__ fx operator-(fx a) { return fx(-a.v); }
-__device__ __forceinline__ fx xfma(fx a, fx b, fx c) { return fx(fma(a.v, b.v, c.v)); }
-__device__ __forceinline__ fx xabs(fx a) { return fx(fabs(a.v)); }
-__device__ __forceinline__ fx xsqrt(fx a) { return fx(a.v * rsqrt_nr(a.v)); }
-
-template <typename T> struct exact_order { static constexpr bool value = false; };
-template <> struct exact_order<ex> { static constexpr bool value = true; };
-
 // Troubled-cell indicator, Sec. 2.3.1 Steps 1-3, on the window q[0..4] = Q_{i-2..i+2}
 // (cell units).  Step 1: |D| <= Z1 with D = (4Q_{i-2}+Q_{i-1}) + (4Q_{i+2}+Q_{i+1}) - 10 Q_i
 // and Z1 = 17 zeta1 dx^2 (Eq. (24): abar2 = D/34).  Step 2: xbar = -abar1/(2 abar2) with
@@ -268,29 +248,14 @@ __device__ __forceinline__ void ao_betas(const T* q, T* b)
 }
 
 // Normalised nonlinear weights, Eqs. (37), (38), (40), with the ratio delta/(beta_k + eps) squared.
-// With T = fx the four ratios share one division (1/(e0 e1 e2 e3) times the other three factors)
-// whenever that product is a finite positive number.
 template <typename T>
 __device__ __forceinline__ void ao_weights(const T* q, const AOConst& k, T* wb)
 {
     T b[4], w[4], r[4];
     ao_betas(q, b);
     T d = ((xabs(b[3] - b[0]) + xabs(b[3] - b[1])) + xabs(b[3] - b[2])) * T(1.0 / 3.0);
-    bool done = false;
-    if constexpr (!exact_order<T>::value) {
-        const double e0 = b[0].v + k.eps, e1 = b[1].v + k.eps, e2 = b[2].v + k.eps, e3 = b[3].v + k.eps;
-        const double e01 = e0 * e1, e23 = e2 * e3, prod = e01 * e23;
-        if (prod > 0.0 && prod < 1e300) {
-            const double di = d.v * rcp_nr(prod);
-            r[0] = T(di * (e1 * e23)); r[1] = T(di * (e0 * e23));
-            r[2] = T(di * (e3 * e01)); r[3] = T(di * (e2 * e01));
-            done = true;
-        }
-    }
-    if (!done) {
 #pragma unroll
-        for (int j = 0; j < 4; j++) r[j] = d / (b[j] + T(k.eps));
-    }
+    for (int j = 0; j < 4; j++) r[j] = d / (b[j] + T(k.eps));
 #pragma unroll
     for (int j = 0; j < 4; j++) w[j] = T(k.g[j]) * (T(1.0) + r[j] * r[j]);
     T inv = T(1.0) / (((w[0] + w[1]) + w[2]) + w[3]);
@@ -497,28 +462,6 @@ __device__ __forceinline__ bool nonphysical(double gam, const double* Q)
 }
 
 // ---------------------------------------------------------------- Gauss-point reconstruction
-// Coefficients (cell units) of the three quadratics and the quartic through the averages of
-// cells i-2..i+2, evaluated at xi = +-1/(2 sqrt 3): values V and derivatives D, at +g (P) and -g (M).
-struct GaussCoef { double VP[4][5], DP[4][5], VM[4][5], DM[4][5]; };
-__device__ __constant__ GaussCoef c_gauss = {
-    {{1.44337567297406433e-01, -5.77350269189625731e-01, 1.43301270189221941e+00, 0.0, 0.0},
-     {0.0, -1.44337567297406433e-01, 1.00000000000000000e+00, 1.44337567297406433e-01, 0.0},
-     {0.0, 0.0, 5.66987298107780702e-01, 5.77350269189625731e-01, -1.44337567297406433e-01},
-     {2.78341566041253249e-02, -1.99542917542694126e-01, 9.98611111111111116e-01, 2.01394769394545980e-01, -2.82971195670882886e-02}},
-    {{7.88675134594812866e-01, -2.57735026918962573e+00, 1.78867513459481287e+00, 0.0, 0.0},
-     {0.0, -2.11324865405187107e-01, -5.77350269189625731e-01, 7.88675134594812866e-01, 0.0},
-     {0.0, 0.0, -1.21132486540518713e+00, 1.42264973081037427e+00, -2.11324865405187107e-01},
-     {5.12583183783541230e-02, -2.49691472251936941e-01, -7.69800358919501049e-01, 1.08364186108139648e+00, -1.15408348288312548e-01}},
-    {{-1.44337567297406433e-01, 5.77350269189625731e-01, 5.66987298107780702e-01, 0.0, 0.0},
-     {0.0, 1.44337567297406433e-01, 1.00000000000000000e+00, -1.44337567297406433e-01, 0.0},
-     {0.0, 0.0, 1.43301270189221941e+00, -5.77350269189625731e-01, 1.44337567297406433e-01},
-     {-2.82971195670882886e-02, 2.01394769394545980e-01, 9.98611111111111116e-01, -1.99542917542694126e-01, 2.78341566041253249e-02}},
-    {{2.11324865405187107e-01, -1.42264973081037427e+00, 1.21132486540518713e+00, 0.0, 0.0},
-     {0.0, -7.88675134594812866e-01, 5.77350269189625731e-01, 2.11324865405187107e-01, 0.0},
-     {0.0, 0.0, -1.78867513459481287e+00, 2.57735026918962573e+00, -7.88675134594812866e-01},
-     {1.15408348288312548e-01, -1.08364186108139648e+00, 7.69800358919501049e-01, 2.49691472251936941e-01, -5.12583183783541230e-02}},
-};
-
 #if defined(__CUDACC__)
 // Quartic of the window q at the two Gauss points: v[0] at -g, v[1] at +g, and (DER) its derivatives
 // there times inv_ht (`inv` the same as a fixed-point factor).  In fixed point (fixed::quartic_pair); FP64
@@ -527,98 +470,168 @@ template <bool DER>
 __device__ __forceinline__ void gauss_linear(const double* q, fixed::Scale inv, double inv_ht, double* v, double* d)
 {
     if (fixed::quartic_pair<DER>(q, inv, v, d)) return;
-    const double* vm = c_gauss.VM[3]; const double* vp = c_gauss.VP[3];
-    const double* dm = c_gauss.DM[3]; const double* dp = c_gauss.DP[3];
-    double a = vm[2] * q[2], b = vp[2] * q[2], e = dm[2] * q[2], f = dp[2] * q[2];
-#pragma unroll
-    for (int j = 0; j < 5; j++) {
-        if (j == 2) continue;
-        a = fma(vm[j], q[j], a); b = fma(vp[j], q[j], b);
-        e = fma(dm[j], q[j], e); f = fma(dp[j], q[j], f);
+    const double s1 = q[1] + q[3], s2 = q[0] + q[4], d1 = q[3] - q[1], d2 = q[4] - q[0];
+    const double even = fma(719.0 / 720.0, q[2], fma(1.0 / 1080.0, s1, (-1.0 / 4320.0) * s2));
+    const double odd = fma(0.20046884346862004, d1, -0.028065638085606807 * d2);      // 25 sqrt3/216, 7 sqrt3/432
+    v[0] = even - odd; v[1] = even + odd;
+    if (DER) {
+        const double n = fma(2.0 / 3.0, d1, (-1.0 / 12.0) * d2);
+        // 4 sqrt3/9, 13 sqrt3/54, sqrt3/54
+        const double t = fma(-0.76980035891950105, q[2], fma(0.4169751944147297, s1, -0.032075014954979206 * s2));
+        d[0] = (n - t) * inv_ht; d[1] = (n + t) * inv_ht;
     }
-    v[0] = a; v[1] = b;
-    if (DER) { d[0] = e * inv_ht; d[1] = f * inv_ht; }
 }
 #endif
 
-__device__ __forceinline__ void gauss_ao(const fx* q, const AOConst& k, double* v, double* d)
+// The tangential WENO-AO pass (free-order arithmetic: the outputs only feed the flux).
+//
+// AO reconstruction of one characteristic field at the two Gauss points xi = -+g, g^2 = 1/12: v[0], v[1], and
+// (der) its derivatives d[0], d[1] in cell units.  With t_k/2 the slope at the cell's centre and s_k the
+// curvature of sub-stencil k (the terms its smoothness indicator is made of) and c1..c4 the quartic's
+// coefficients, the polynomials' values there are
+//     p_k = q2 +- g t_k/2,           p_k' = t_k/2 +- g s_k          (xi^2 - 1/12 vanishes),
+//     p_3 = q2 - c4/180 +- g (c1 + c3/12),   p_3' = c1 + c3/4 +- 2 g (c2 + c4/6),
+// so the combination of Eq. (41) takes two sums over the sub-stencils and the indicators' own terms: 27
+// FP64 operations in place of 72 on the tabulated point values of each polynomial.  With the shared rows of
+// the projections (tang_project, tang_back) WENO-AO everywhere on 500^2 went from 7.35 to 3.45 ms per
+// step of tangential passes, the 1024^2 four-quadrant step's from 0.25 to 0.14 ms.
+__device__ __forceinline__ void gauss_ao(const double* q, const AOConst& k, bool der, double* v, double* d)
 {
-    fx wb[4];
-    ao_weights(q, k, wb);
-    double w3 = wb[3].v * k.g3inv;
-    // weight of each polynomial in the AO combination (Eq. (41)):
-    //   quartic: wb3/g3;   quadratic s: wb_s - wb3 g_s/g3
-    double ws[4] = {wb[0].v - wb[3].v * k.gr[0], wb[1].v - wb[3].v * k.gr[1], wb[2].v - wb[3].v * k.gr[2], w3};
-    double a = 0.0, b = 0.0, e = 0.0, f = 0.0;
-#pragma unroll
-    for (int s = 0; s < 4; s++) {
-        double pa = 0.0, pb = 0.0, pe = 0.0, pf = 0.0;
-#pragma unroll
-        for (int j = 0; j < 5; j++) {
-            if (c_gauss.VM[s][j] == 0.0 && c_gauss.DM[s][j] == 0.0) continue;
-            pa = fma(c_gauss.VM[s][j], q[j].v, pa); pb = fma(c_gauss.VP[s][j], q[j].v, pb);
-            pe = fma(c_gauss.DM[s][j], q[j].v, pe); pf = fma(c_gauss.DP[s][j], q[j].v, pf);
-        }
-        a = fma(ws[s], pa, a); b = fma(ws[s], pb, b); e = fma(ws[s], pe, e); f = fma(ws[s], pf, f);
+    const double q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3], q4 = q[4];
+    // smoothness indicators, Eq. (39), as ao_betas
+    const double s0 = fma(-2.0, q1, q0) + q2, s1 = fma(-2.0, q2, q1) + q3, s2 = fma(-2.0, q3, q2) + q4;
+    const double d13 = q3 - q1, d04 = q4 - q0, a13 = q1 + q3, a04 = q0 + q4;
+    const double t0 = fma(3.0, q2, fma(-4.0, q1, q0)), t1 = d13, t2 = fma(-3.0, q2, fma(4.0, q3, -q4));
+    const double c1 = fma(17.0 / 24.0, d13, (-5.0 / 48.0) * d04);
+    const double c2 = fma(-1.375, q2, fma(0.75, a13, -0.0625 * a04));
+    const double c3 = fma(-1.0 / 6.0, d13, (1.0 / 12.0) * d04);
+    const double c4 = fma(0.25, q2, fma(-1.0 / 6.0, a13, (1.0 / 24.0) * a04));
+    constexpr double b1312 = 13.0 / 12.0;
+    const double b0 = fma(b1312 * s0, s0, (0.25 * t0) * t0);
+    const double b1 = fma(b1312 * s1, s1, (0.25 * t1) * t1);
+    const double b2 = fma(b1312 * s2, s2, (0.25 * t2) * t2);
+    const double b3 = fma(c1, fma(0.5, c3, c1), fma(c2, fma(13.0 / 3.0, c2, 4.2 * c4),
+                      fma((3129.0 / 80.0) * c3, c3, ((87617.0 / 140.0) * c4) * c4)));
+    // nonlinear weights, Eqs. (37), (38), not yet normalised (the reciprocals take no FP64 operation)
+    const double dl = ((fabs(b3 - b0) + fabs(b3 - b1)) + fabs(b3 - b2)) * (1.0 / 3.0);
+    const double r0 = dl * rcp_nr(b0 + k.eps), r1 = dl * rcp_nr(b1 + k.eps), r2 = dl * rcp_nr(b2 + k.eps), r3 = dl * rcp_nr(b3 + k.eps);
+    const double w0 = fma(k.g[0] * r0, r0, k.g[0]), w1 = fma(k.g[1] * r1, r1, k.g[1]);
+    const double w2 = fma(k.g[2] * r2, r2, k.g[2]), w3 = fma(k.g[3] * r3, r3, k.g[3]);
+    const double inv = rcp_nr((w0 + w1) + (w2 + w3));
+    // weights of the polynomials in the combination: sub-stencil k: w_k - w3 g_k/g3; quartic: w3/g3
+    const double m0 = fma(-w3, k.gr[0], w0), m1 = fma(-w3, k.gr[1], w1), m2 = fma(-w3, k.gr[2], w2);
+    const double m3 = w3 * k.g3inv, m32 = scale2<1>(m3);
+    const double B = fma(m0, t0, fma(m1, t1, m2 * t2));
+    const double ev = (m3 * (-1.0 / 180.0)) * c4;
+    const double od = 0.14433756729740644 * fma(m32, fma(1.0 / 12.0, c3, c1), B);          // g/2
+    v[0] = fma(inv, ev - od, q2);
+    v[1] = fma(inv, ev + od, q2);
+    if (der) {
+        const double C = fma(m0, s0, fma(m1, s1, m2 * s2));
+        const double De = fma(m32, fma(0.25, c3, c1), B), Do = fma(m32, fma(1.0 / 6.0, c4, c2), C);
+        const double ih = scale2<-1>(inv);
+        d[0] = ih * fma(-0.57735026918962576, Do, De);                                     // 2g
+        d[1] = ih * fma(0.57735026918962576, Do, De);
+    } else {
+        d[0] = d[1] = 0.0;
     }
-    v[0] = a; v[1] = b; d[0] = e; d[1] = f;
 }
 
-// Tangential WENO-AO of one pass (4 components, one lane) at the two Gauss points: projection of
-// the 5 line values x[s][] onto the characteristic fields (rows of Lm), gauss_ao per field, and
-// the projection back with Rm.  Free-order arithmetic (the outputs only feed the flux).
-__device__ __forceinline__ void tang_ao(const fx (*Lm)[4], const fx (*Rm)[4], const fx (*x)[4], const AOConst& ak,
+// Eigenvectors of the flux Jacobian in the tangential direction at the face average Qs: the projections onto
+// and from the fields in the few terms their rows share (L and R have zeros and repeated entries).
+struct TangEig { double U, V, c, H, hq2, b1h, ci2; };
+
+__device__ __forceinline__ void tang_eig(double gam, const double* Qs, TangEig& e)
+{
+    const double gm1 = gam - 1.0, ri = rcp_nr(Qs[0]);
+    e.U = Qs[1] * ri;
+    e.V = Qs[2] * ri;
+    e.hq2 = scale2<-1>(fma(e.U, e.U, e.V * e.V));
+    const double p = gm1 * fma(-Qs[0], e.hq2, Qs[3]);
+    const double c2 = (gam * p) * ri, ci = rsqrt_nr(c2);
+    e.c = c2 * ci;
+    e.H = (Qs[3] + p) * ri;
+    e.ci2 = scale2<-1>(ci);
+    e.b1h = (scale2<-1>(gm1) * ci) * ci;
+}
+
+// Fields of one state x
+__device__ __forceinline__ void tang_project(const TangEig& e, const double* x, double* f)
+{
+    const double w = e.b1h * fma(e.hq2, x[0], fma(-e.U, x[1], fma(-e.V, x[2], x[3])));
+    const double z = e.ci2 * fma(e.V, x[0], -x[2]);
+    f[0] = w + z;
+    f[1] = fma(-2.0, w, x[0]);
+    f[2] = fma(e.U, x[0], -x[1]);
+    f[3] = w - z;
+}
+
+__device__ __forceinline__ void tang_back(const TangEig& e, const double* f, double* x)
+{
+    const double s = f[0] + f[3], cd = e.c * (f[3] - f[0]);
+    x[0] = s + f[1];
+    x[1] = fma(e.U, x[0], -f[2]);
+    x[2] = fma(e.V, x[0], cd);
+    x[3] = fma(e.H, s, fma(e.hq2, f[1], fma(-e.U, f[2], e.V * cd)));
+}
+
+// One pass (4 components, one lane) at the two Gauss points: projection of the 5 line values x[s][],
+// gauss_ao per field, projection back.
+__device__ __forceinline__ void tang_ao(const TangEig& e, const double (*x)[4], const AOConst& ak, bool der,
                                         double (*v)[2], double (*d)[2])
 {
-    // all 20 projections first: the line values are dead before the four fields' weights are
-    // formed (134 registers against 170 with the projection inside the field loop)
-    fx uc[4][5];
+    // all projections first: the line values are dead before the four fields' weights are formed
+    double uc[5][4];
 #pragma unroll
-    for (int s = 0; s < 5; s++)
+    for (int s = 0; s < 5; s++) tang_project(e, x[s], uc[s]);
+    double cv[2][4], cd[2][4];
 #pragma unroll
-        for (int c = 0; c < 4; c++)
-            uc[c][s] = xfma(Lm[c][3], x[s][3], xfma(Lm[c][2], x[s][2], xfma(Lm[c][1], x[s][1], Lm[c][0] * x[s][0])));
-    double cv[4][2], cd[4][2];
+    for (int c = 0; c < 4; c++) {
+        const double u[5] = {uc[0][c], uc[1][c], uc[2][c], uc[3][c], uc[4][c]};
+        double vv[2], dd[2];
+        gauss_ao(u, ak, der, vv, dd);
 #pragma unroll
-    for (int c = 0; c < 4; c++) gauss_ao(uc[c], ak, cv[c], cd[c]);
+        for (int g = 0; g < 2; g++) { cv[g][c] = vv[g]; cd[g][c] = dd[g]; }
+    }
 #pragma unroll
-    for (int g = 0; g < 2; g++)
+    for (int g = 0; g < 2; g++) {
+        double xv[4], xd[4] = {0.0, 0.0, 0.0, 0.0};
+        tang_back(e, cv[g], xv);
+        if (der) tang_back(e, cd[g], xd);
 #pragma unroll
-        for (int r = 0; r < 4; r++) {
-            double a = 0.0, b = 0.0;
-#pragma unroll
-            for (int c = 0; c < 4; c++) { a = fma(Rm[r][c].v, cv[c][g], a); b = fma(Rm[r][c].v, cd[c][g], b); }
-            v[r][g] = a; d[r][g] = b;
-        }
+        for (int r = 0; r < 4; r++) { v[r][g] = xv[r]; d[r][g] = xd[r]; }
+    }
 }
 
 #if defined(__CUDACC__)
-// The same pass spread over the 4 lanes of an aligned lane group like weno_ao_face_x4: lane q
-// projects the 5 line values onto field q (row q of Lm), runs gauss_ao for it, the fields'
-// Gauss-point values and derivatives are exchanged with shuffles, and lane q projects back its
-// own component (row q of Rm): vq[g], dq[g] at the two Gauss points.
-__device__ __forceinline__ void tang_ao_x4(const fx (*Lm)[4], const fx (*Rm)[4], const fx (*x)[4], const AOConst& ak,
+// The same pass spread over the 4 lanes of an aligned lane group: lane q projects the 5 line values onto
+// field q with its row of L, runs gauss_ao for it, the fields' Gauss-point values and derivatives are
+// exchanged with shuffles, and lane q forms its own component with its row of R: vq[g], dq[g].
+__device__ __forceinline__ void tang_ao_x4(const TangEig& e, const double (*x)[4], const AOConst& ak, bool der,
                                            unsigned gmask, double* vq, double* dq)
 {
     const int q = threadIdx.x & 3;
     const int lane0 = threadIdx.x & 28;
-    fx Lq[4], Rq[4];
-    select_row<4>(Lm, q, Lq);
-    select_row<4>(Rm, q, Rq);
-    fx u[5];
+    const double bU = e.b1h * e.U, bV = e.b1h * e.V, b2h = e.b1h * e.hq2, Vci = e.V * e.ci2, Vc = e.V * e.c;
+    auto pick = [&](double a, double b, double c, double d) { return q == 0 ? a : q == 1 ? b : q == 2 ? c : d; };
+    const double l0 = pick(b2h + Vci, fma(-2.0, b2h, 1.0), e.U, b2h - Vci), l1 = pick(-bU, scale2<1>(bU), -1.0, -bU);
+    const double l2 = pick(-(bV + e.ci2), scale2<1>(bV), 0.0, e.ci2 - bV), l3 = pick(e.b1h, -scale2<1>(e.b1h), 0.0, e.b1h);
+    double u[5];
 #pragma unroll
-    for (int s = 0; s < 5; s++) u[s] = xfma(Lq[3], x[s][3], xfma(Lq[2], x[s][2], xfma(Lq[1], x[s][1], Lq[0] * x[s][0])));
-    double cvq[2], cdq[2];
-    gauss_ao(u, ak, cvq, cdq);
+    for (int s = 0; s < 5; s++) u[s] = fma(l3, x[s][3], fma(l2, x[s][2], fma(l1, x[s][1], l0 * x[s][0])));
+    double cv[2], cd[2];
+    gauss_ao(u, ak, der, cv, cd);
+    const double r0 = pick(1.0, e.U, e.V - e.c, e.H - Vc), r1 = pick(1.0, e.U, e.V, e.hq2);
+    const double r2 = pick(0.0, -1.0, 0.0, -e.U), r3 = pick(1.0, e.U, e.V + e.c, e.H + Vc);
 #pragma unroll
     for (int g = 0; g < 2; g++) {
-        double a = 0.0, b = 0.0;
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-            a = fma(Rq[c].v, __shfl_sync(gmask, cvq[g], lane0 + c), a);
-            b = fma(Rq[c].v, __shfl_sync(gmask, cdq[g], lane0 + c), b);
-        }
-        vq[g] = a; dq[g] = b;
+        auto back = [&](double f) {
+            const double f0 = __shfl_sync(gmask, f, lane0), f1 = __shfl_sync(gmask, f, lane0 + 1);
+            const double f2 = __shfl_sync(gmask, f, lane0 + 2), f3 = __shfl_sync(gmask, f, lane0 + 3);
+            return fma(r3, f3, fma(r2, f2, fma(r1, f1, r0 * f0)));
+        };
+        vq[g] = back(cv[g]);
+        dq[g] = der ? back(cd[g]) : 0.0;          // `der` is the same for the 4 lanes
     }
 }
 #endif
