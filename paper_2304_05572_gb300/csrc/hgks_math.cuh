@@ -128,6 +128,23 @@ HGKS_HD __forceinline__ double exp_neg(double y)
 #endif
 }
 
+// x 2^K with the bits of the FP64 multiplication.  INT: an integer add to the exponent (the multiplication
+// itself where the result could leave the normal range): for kernels bound by the FP64 pipe.  A lane
+// group's short dependent chain is no faster with it (128 against 125 us on the 512^2 step's normal
+// passes) and multiplies.
+template <int K, bool INT>
+__device__ __forceinline__ ex xscale(ex x)
+{
+    constexpr double f = K > 0 ? (double)(1 << (K > 0 ? K : 0)) : 1.0 / (double)(1 << (K < 0 ? -K : 0));
+#if defined(__CUDACC__)
+    if constexpr (INT) {
+        const unsigned e = (unsigned)(__double2hiint(x.v) >> 20) & 0x7FFu;
+        return e - 8u < 2032u || fixed::is_zero(x.v) ? ex(fixed::scale2<K>(x.v)) : x * ex(f);
+    }
+#endif
+    return x * ex(f);
+}
+
 // Troubled-cell indicator, Sec. 2.3.1 Steps 1-3, on the window q[0..4] = Q_{i-2..i+2}
 // (cell units).  Step 1: |D| <= Z1 with D = (4Q_{i-2}+Q_{i-1}) + (4Q_{i+2}+Q_{i+1}) - 10 Q_i
 // and Z1 = 17 zeta1 dx^2 (Eq. (24): abar2 = D/34).  Step 2: xbar = -abar1/(2 abar2) with
@@ -228,37 +245,39 @@ struct AOConst {
     double eps;
 };
 
-// Smoothness indicators of Eq. (39) in cell units (with T = ex: the evaluation order the
-// decisions need).
-template <typename T>
-__device__ __forceinline__ void ao_betas(const T* q, T* b)
+// Smoothness indicators of Eq. (39) in cell units, in the evaluation order the decisions need
+// (factors 2, 4, 1/2, 1/4, 1/16 are exact).
+template <bool INT>
+__device__ __forceinline__ void ao_betas(const ex* q, ex* b)
 {
-    T s0 = (q[0] - T(2.0) * q[1]) + q[2], t0 = (q[0] - T(4.0) * q[1]) + T(3.0) * q[2];
-    T s1 = (q[1] - T(2.0) * q[2]) + q[3], t1 = q[1] - q[3];
-    T s2 = (q[2] - T(2.0) * q[3]) + q[4], t2 = (T(3.0) * q[2] - T(4.0) * q[3]) + q[4];
-    b[0] = T(13.0 / 12.0) * (s0 * s0) + T(0.25) * (t0 * t0);
-    b[1] = T(13.0 / 12.0) * (s1 * s1) + T(0.25) * (t1 * t1);
-    b[2] = T(13.0 / 12.0) * (s2 * s2) + T(0.25) * (t2 * t2);
-    T c1 = T(17.0 / 24.0) * (q[3] - q[1]) - T(5.0 / 48.0) * (q[4] - q[0]);
-    T c2 = ((T(0.75) * (q[1] + q[3]) - T(0.0625) * (q[0] + q[4])) - T(1.375) * q[2]);
-    T c3 = T(1.0 / 6.0) * (q[1] - q[3]) - T(1.0 / 12.0) * (q[0] - q[4]);
-    T c4 = ((T(1.0 / 24.0) * (q[0] + q[4]) - T(1.0 / 6.0) * (q[1] + q[3])) + T(0.25) * q[2]);
-    b[3] = ((((c1 * c1 + T(0.5) * (c1 * c3)) + T(13.0 / 3.0) * (c2 * c2)) + T(21.0 / 5.0) * (c2 * c4))
-            + T(3129.0 / 80.0) * (c3 * c3)) + T(87617.0 / 140.0) * (c4 * c4);
+    const ex q1_2 = xscale<1, INT>(q[1]), q2_2 = xscale<1, INT>(q[2]), q3_2 = xscale<1, INT>(q[3]);
+    const ex s0 = (q[0] - q1_2) + q[2], t0 = (q[0] - xscale<1, INT>(q1_2)) + ex(3.0) * q[2];
+    const ex s1 = (q[1] - q2_2) + q[3], t1 = q[1] - q[3];
+    const ex s2 = (q[2] - q3_2) + q[4], t2 = (ex(3.0) * q[2] - xscale<1, INT>(q3_2)) + q[4];
+    b[0] = ex(13.0 / 12.0) * (s0 * s0) + xscale<-2, INT>(t0 * t0);
+    b[1] = ex(13.0 / 12.0) * (s1 * s1) + xscale<-2, INT>(t1 * t1);
+    b[2] = ex(13.0 / 12.0) * (s2 * s2) + xscale<-2, INT>(t2 * t2);
+    const ex a13 = q[1] + q[3], a04 = q[0] + q[4];
+    const ex c1 = ex(17.0 / 24.0) * (q[3] - q[1]) - ex(5.0 / 48.0) * (q[4] - q[0]);
+    const ex c2 = ((ex(0.75) * a13 - xscale<-4, INT>(a04)) - ex(1.375) * q[2]);
+    const ex c3 = ex(1.0 / 6.0) * t1 - ex(1.0 / 12.0) * (q[0] - q[4]);
+    const ex c4 = ((ex(1.0 / 24.0) * a04 - ex(1.0 / 6.0) * a13) + xscale<-2, INT>(q[2]));
+    b[3] = ((((c1 * c1 + xscale<-1, INT>(c1 * c3)) + ex(13.0 / 3.0) * (c2 * c2)) + ex(21.0 / 5.0) * (c2 * c4))
+            + ex(3129.0 / 80.0) * (c3 * c3)) + ex(87617.0 / 140.0) * (c4 * c4);
 }
 
 // Normalised nonlinear weights, Eqs. (37), (38), (40), with the ratio delta/(beta_k + eps) squared.
-template <typename T>
-__device__ __forceinline__ void ao_weights(const T* q, const AOConst& k, T* wb)
+template <bool INT>
+__device__ __forceinline__ void ao_weights(const ex* q, const AOConst& k, ex* wb)
 {
-    T b[4], w[4], r[4];
-    ao_betas(q, b);
-    T d = ((xabs(b[3] - b[0]) + xabs(b[3] - b[1])) + xabs(b[3] - b[2])) * T(1.0 / 3.0);
+    ex b[4], w[4], r[4];
+    ao_betas<INT>(q, b);
+    const ex d = ((xabs(b[3] - b[0]) + xabs(b[3] - b[1])) + xabs(b[3] - b[2])) * ex(1.0 / 3.0);
 #pragma unroll
-    for (int j = 0; j < 4; j++) r[j] = d / (b[j] + T(k.eps));
+    for (int j = 0; j < 4; j++) r[j] = d / (b[j] + ex(k.eps));
 #pragma unroll
-    for (int j = 0; j < 4; j++) w[j] = T(k.g[j]) * (T(1.0) + r[j] * r[j]);
-    T inv = T(1.0) / (((w[0] + w[1]) + w[2]) + w[3]);
+    for (int j = 0; j < 4; j++) w[j] = ex(k.g[j]) * (ex(1.0) + r[j] * r[j]);
+    const ex inv = ex(1.0) / (((w[0] + w[1]) + w[2]) + w[3]);
 #pragma unroll
     for (int j = 0; j < 4; j++) wb[j] = w[j] * inv;
 }
@@ -272,79 +291,85 @@ __device__ __forceinline__ ex ao_combine(const ex* wb, const AOConst& k, const e
 
 // Face values / cell-unit derivatives of the three quadratics (Eqs. (32), (43), with the
 // p_2(x_{i+1/2}) coefficient corrected to -1/6) and of the quartic (Eqs. (36), (44)).
+template <bool INT>
 __device__ __forceinline__ void face_polys(const ex* q, int side, ex* pv, ex* pd)
 {
     if (side > 0) {
-        pv[0] = ((ex(2.0) * q[0] - ex(7.0) * q[1]) + ex(11.0) * q[2]) * ex(1.0 / 6.0);
-        pv[1] = ((-q[1] + ex(5.0) * q[2]) + ex(2.0) * q[3]) * ex(1.0 / 6.0);
-        pv[2] = ((ex(2.0) * q[2] + ex(5.0) * q[3]) - q[4]) * ex(1.0 / 6.0);
-        pv[3] = ((((ex(2.0) * q[0] - ex(13.0) * q[1]) + ex(47.0) * q[2]) + ex(27.0) * q[3]) - ex(3.0) * q[4]) * ex(1.0 / 60.0);
-        pd[0] = (q[0] - ex(3.0) * q[1]) + ex(2.0) * q[2];
+        pv[0] = ((xscale<1, INT>(q[0]) - ex(7.0) * q[1]) + ex(11.0) * q[2]) * ex(1.0 / 6.0);
+        pv[1] = ((-q[1] + ex(5.0) * q[2]) + xscale<1, INT>(q[3])) * ex(1.0 / 6.0);
+        pv[2] = ((xscale<1, INT>(q[2]) + ex(5.0) * q[3]) - q[4]) * ex(1.0 / 6.0);
+        pv[3] = ((((xscale<1, INT>(q[0]) - ex(13.0) * q[1]) + ex(47.0) * q[2]) + ex(27.0) * q[3]) - ex(3.0) * q[4]) * ex(1.0 / 60.0);
+        pd[0] = (q[0] - ex(3.0) * q[1]) + xscale<1, INT>(q[2]);
         pd[1] = q[3] - q[2];
         pd[2] = q[3] - q[2];
         pd[3] = (((q[1] - ex(15.0) * q[2]) + ex(15.0) * q[3]) - q[4]) * ex(1.0 / 12.0);
     } else {
-        pv[0] = ((-q[0] + ex(5.0) * q[1]) + ex(2.0) * q[2]) * ex(1.0 / 6.0);
-        pv[1] = ((ex(2.0) * q[1] + ex(5.0) * q[2]) - q[3]) * ex(1.0 / 6.0);
-        pv[2] = ((ex(11.0) * q[2] - ex(7.0) * q[3]) + ex(2.0) * q[4]) * ex(1.0 / 6.0);
-        pv[3] = ((((-ex(3.0) * q[0] + ex(27.0) * q[1]) + ex(47.0) * q[2]) - ex(13.0) * q[3]) + ex(2.0) * q[4]) * ex(1.0 / 60.0);
+        pv[0] = ((-q[0] + ex(5.0) * q[1]) + xscale<1, INT>(q[2])) * ex(1.0 / 6.0);
+        pv[1] = ((xscale<1, INT>(q[1]) + ex(5.0) * q[2]) - q[3]) * ex(1.0 / 6.0);
+        pv[2] = ((ex(11.0) * q[2] - ex(7.0) * q[3]) + xscale<1, INT>(q[4])) * ex(1.0 / 6.0);
+        pv[3] = ((((-ex(3.0) * q[0] + ex(27.0) * q[1]) + ex(47.0) * q[2]) - ex(13.0) * q[3]) + xscale<1, INT>(q[4])) * ex(1.0 / 60.0);
         pd[0] = q[2] - q[1];
         pd[1] = q[2] - q[1];
-        pd[2] = (-ex(2.0) * q[2] + ex(3.0) * q[3]) - q[4];
+        pd[2] = (-xscale<1, INT>(q[2]) + ex(3.0) * q[3]) - q[4];
         pd[3] = (((q[0] - ex(15.0) * q[1]) + ex(15.0) * q[2]) - q[3]) * ex(1.0 / 12.0);
     }
 }
 
-// Left (L = R^{-1}, rows) and right (R, columns) eigenvectors of nx dF/dQ + ny dG/dQ at Q.
-template <int NV, typename T>
-__device__ __forceinline__ void eigvec(double gam, const T* Q, double nxd, double nyd, T (*L)[NV], T (*R)[NV])
+// Left (L = R^{-1}, rows) and right (R, columns) eigenvectors of dF/dQ (local normal direction) at Q, the
+// entries that are not 0 or 1 by construction (2D: L[2] = (-V, 0, 1, 0), R's third column (0, 0, 1, V)):
+// a factor 1 and a term 0 leave the other operands' bits as they are.
+template <int NV, bool INT>
+__device__ __forceinline__ void eigvec(double gam, const ex* Q, ex (*L)[NV], ex (*R)[NV])
 {
-    T gm1 = T(gam) - T(1.0);
-    T rho = Q[0], ri = T(1.0) / rho;
-    T U = Q[1] * ri;
+    const ex gm1 = ex(gam) - ex(1.0);
+    const ex rho = Q[0], ri = ex(1.0) / rho;
+    const ex U = Q[1] * ri;
+    ex V(0.0), q2 = U * U;
+    if constexpr (NV == 4) { V = Q[2] * ri; q2 = q2 + V * V; }
+    const ex p = gm1 * (Q[NV - 1] - xscale<-1, INT>(rho) * q2);
+    const ex c2 = (ex(gam) * p) * ri, c = xsqrt(c2), ci = ex(1.0) / c;
+    const ex H = (Q[NV - 1] + p) * ri;
+    const ex b1 = gm1 / c2, b1h = xscale<-1, INT>(b1), b2 = b1h * q2, bU = b1 * U, uci = U * ci, uc = U * c;
+    constexpr int E = NV - 1;
+    R[0][0] = ex(1.0);   R[0][1] = ex(1.0);        R[0][E] = ex(1.0);
+    R[1][0] = U - c;      R[1][1] = U;              R[1][E] = U + c;
+    R[E][0] = H - uc;     R[E][1] = xscale<-1, INT>(q2); R[E][E] = H + uc;
+    L[0][0] = xscale<-1, INT>(b2 + uci); L[0][1] = -xscale<-1, INT>(bU + ci); L[0][E] = b1h;
+    L[1][0] = ex(1.0) - b2;         L[1][1] = bU;                    L[1][E] = -b1;
+    L[E][0] = xscale<-1, INT>(b2 - uci); L[E][1] = -xscale<-1, INT>(bU - ci); L[E][E] = b1h;
     if constexpr (NV == 4) {
-        T nx(nxd), ny(nyd);
-        T V = Q[2] * ri;
-        T q2 = U * U + V * V;
-        T p = gm1 * (Q[3] - (T(0.5) * rho) * q2);
-        T c2 = (T(gam) * p) * ri, c = xsqrt(c2), ci = T(1.0) / c;
-        T H = (Q[3] + p) * ri;
-        T un = U * nx + V * ny, ut = V * nx - U * ny;
-        T b1 = gm1 / c2, b2 = (T(0.5) * b1) * q2;
-        R[0][0] = T(1.0);    R[0][1] = T(1.0);       R[0][2] = T(0.0); R[0][3] = T(1.0);
-        R[1][0] = U - c * nx; R[1][1] = U;             R[1][2] = -ny;     R[1][3] = U + c * nx;
-        R[2][0] = V - c * ny; R[2][1] = V;             R[2][2] = nx;      R[2][3] = V + c * ny;
-        R[3][0] = H - un * c; R[3][1] = T(0.5) * q2;  R[3][2] = ut;      R[3][3] = H + un * c;
-        L[0][0] = T(0.5) * (b2 + un * ci); L[0][1] = -(T(0.5) * (b1 * U + nx * ci)); L[0][2] = -(T(0.5) * (b1 * V + ny * ci)); L[0][3] = T(0.5) * b1;
-        L[1][0] = T(1.0) - b2;             L[1][1] = b1 * U;                          L[1][2] = b1 * V;                          L[1][3] = -b1;
-        L[2][0] = -ut;                      L[2][1] = -ny;                             L[2][2] = nx;                              L[2][3] = T(0.0);
-        L[3][0] = T(0.5) * (b2 - un * ci); L[3][1] = -(T(0.5) * (b1 * U - nx * ci)); L[3][2] = -(T(0.5) * (b1 * V - ny * ci)); L[3][3] = T(0.5) * b1;
-    } else {
-        T q2 = U * U;
-        T p = gm1 * (Q[2] - (T(0.5) * rho) * q2);
-        T c2 = (T(gam) * p) * ri, c = xsqrt(c2), ci = T(1.0) / c;
-        T H = (Q[2] + p) * ri;
-        T b1 = gm1 / c2, b2 = (T(0.5) * b1) * q2;
-        R[0][0] = T(1.0);    R[0][1] = T(1.0);      R[0][2] = T(1.0);
-        R[1][0] = U - c;      R[1][1] = U;            R[1][2] = U + c;
-        R[2][0] = H - U * c;  R[2][1] = T(0.5) * q2; R[2][2] = H + U * c;
-        L[0][0] = T(0.5) * (b2 + U * ci); L[0][1] = -(T(0.5) * (b1 * U + ci)); L[0][2] = T(0.5) * b1;
-        L[1][0] = T(1.0) - b2;            L[1][1] = b1 * U;                     L[1][2] = -b1;
-        L[2][0] = T(0.5) * (b2 - U * ci); L[2][1] = -(T(0.5) * (b1 * U - ci)); L[2][2] = T(0.5) * b1;
+        const ex bV = b1 * V;
+        R[0][2] = ex(0.0); R[1][2] = ex(0.0); R[2][0] = V; R[2][1] = V; R[2][2] = ex(1.0); R[2][3] = V; R[3][2] = V;
+        L[0][2] = -xscale<-1, INT>(bV); L[1][2] = bV; L[3][2] = L[0][2];
+        L[2][0] = -V; L[2][1] = ex(0.0); L[2][2] = ex(1.0); L[2][3] = ex(0.0);
     }
 }
 
-// y = M x with the summation order ((m0 x0 + m1 x1) + m2 x2) + m3 x3.
-template <int NV, typename T>
-__device__ __forceinline__ void matvec(const T (*M)[NV], const T* x, T* y)
+// y = L x and y = R x with the summation order ((m0 x0 + m1 x1) + m2 x2) + m3 x3.
+template <int NV>
+__device__ __forceinline__ void project(const ex (*L)[NV], const ex* x, ex* y)
 {
 #pragma unroll
     for (int r = 0; r < NV; r++) {
-        T s = M[r][0] * x[0] + M[r][1] * x[1];
+        if (NV == 4 && r == 2) { y[2] = L[2][0] * x[0] + x[2]; continue; }
+        ex s = L[r][0] * x[0] + L[r][1] * x[1];
 #pragma unroll
-        for (int c = 2; c < NV; c++) s = s + M[r][c] * x[c];
+        for (int c = 2; c < NV; c++) s = s + L[r][c] * x[c];
         y[r] = s;
     }
+}
+
+template <int NV>
+__device__ __forceinline__ void project_back(const ex (*R)[NV], const ex* x, ex* y)
+{
+    y[0] = (x[0] + x[1]) + x[NV - 1];
+    y[1] = (R[1][0] * x[0] + R[1][1] * x[1]) + R[1][NV - 1] * x[NV - 1];
+    ex s = R[NV - 1][0] * x[0] + R[NV - 1][1] * x[1];
+    if constexpr (NV == 4) {
+        y[2] = ((R[2][0] * x[0] + R[2][1] * x[1]) + x[2]) + R[2][3] * x[3];
+        s = s + R[3][2] * x[2];
+    }
+    y[NV - 1] = s + R[NV - 1][NV - 1] * x[NV - 1];
 }
 
 // Characteristic WENO-AO at the face of side (+1: x_{i+1/2}, -1: x_{i-1/2}) of the cell whose
@@ -357,27 +382,27 @@ __device__ __forceinline__ void weno_ao_face(double gam, const AOConst& k, const
     ex L[NV][NV], R[NV][NV], Uc[5][NV], uv[NV], ud[NV], qs[NV];
 #pragma unroll
     for (int c = 0; c < NV; c++) qs[c] = ex(Qs[c]);
-    eigvec<NV>(gam, qs, 1.0, 0.0, L, R);
+    eigvec<NV, true>(gam, qs, L, R);
 #pragma unroll
     for (int j = 0; j < 5; j++) {
         ex x[NV];
 #pragma unroll
         for (int c = 0; c < NV; c++) x[c] = ex(Qw[j][c]);
-        matvec<NV>(L, x, Uc[j]);
+        project<NV>(L, x, Uc[j]);
     }
 #pragma unroll
     for (int c = 0; c < NV; c++) {
         ex q[5], wb[4], pv[4], pd[4];
 #pragma unroll
         for (int j = 0; j < 5; j++) q[j] = Uc[j][c];
-        ao_weights(q, k, wb);
-        face_polys(q, side, pv, pd);
+        ao_weights<true>(q, k, wb);
+        face_polys<true>(q, side, pv, pd);
         uv[c] = ao_combine(wb, k, pv);
         ud[c] = ao_combine(wb, k, pd);
     }
     ex v[NV], d[NV];
-    matvec<NV>(R, uv, v);
-    matvec<NV>(R, ud, d);
+    project_back<NV>(R, uv, v);
+    project_back<NV>(R, ud, d);
 #pragma unroll
     for (int c = 0; c < NV; c++) { val[c] = v[c].v; der[c] = d[c].v; }
 }
@@ -416,7 +441,7 @@ __device__ __forceinline__ void weno_ao_face_x4(double gam, const AOConst& k, co
     ex L[NV][NV], R[NV][NV], qs[NV];
 #pragma unroll
     for (int c = 0; c < NV; c++) qs[c] = ex(Qs[c]);
-    eigvec<NV>(gam, qs, 1.0, 0.0, L, R);
+    eigvec<NV, false>(gam, qs, L, R);
     ex Lq[NV], Rq[NV];
     select_row<NV>(L, qc, Lq);
     select_row<NV>(R, qc, Rq);
@@ -428,8 +453,8 @@ __device__ __forceinline__ void weno_ao_face_x4(double gam, const AOConst& k, co
         for (int c = 2; c < NV; c++) s = s + Lq[c] * ex(Qw[j][c]);
         u[j] = s;
     }
-    ao_weights(u, k, wb);
-    face_polys(u, side, pv, pd);
+    ao_weights<false>(u, k, wb);
+    face_polys<false>(u, side, pv, pd);
     const double uvq = ao_combine(wb, k, pv).v, udq = ao_combine(wb, k, pd).v;
     ex uv[NV], ud[NV];
 #pragma unroll
@@ -437,7 +462,7 @@ __device__ __forceinline__ void weno_ao_face_x4(double gam, const AOConst& k, co
         uv[c] = ex(__shfl_sync(gmask, uvq, lane0 + c));
         ud[c] = ex(__shfl_sync(gmask, udq, lane0 + c));
     }
-    // row qc of R times uv and ud, in the summation order of matvec
+    // row qc of R times uv and ud, in the summation order of project_back
     ex v = Rq[0] * uv[0] + Rq[1] * uv[1], d = Rq[0] * ud[0] + Rq[1] * ud[1];
 #pragma unroll
     for (int c = 2; c < NV; c++) { v = v + Rq[c] * uv[c]; d = d + Rq[c] * ud[c]; }
