@@ -141,9 +141,9 @@ void fill_sweeps(const hgks_config* c, const Params& P, Sweep* sw)
         S.nt = c->dim == 2 ? (d == 0 ? g.ny : g.nx) : 1;
         S.nm = S.nn + 1;
         S.nlines = c->dim == 2 ? S.nt + 6 : 1;
-        // below ~4 warps per scheduler of segments, spread a segment over 4 lanes (shorter FP64
-        // chains per thread); the results do not depend on the choice
-        S.tlanes = (long long)S.nt * S.nm < 65536 ? 4 : 1;
+        // small sweeps spread an item over lanes (shorter FP64 chains per thread) and take one launch per
+        // reconstruction direction; the line is placed by measurement (see k_normal_small)
+        S.small = (long long)S.nt * S.nm < 65536 ? 1 : 0;
         S.tlo = c->dim == 2 ? -3 : 0;
         S.sN = d == 0 ? 1 : g.pitch;
         S.sT = d == 0 ? g.pitch : 1;
@@ -671,8 +671,8 @@ extern "C" int hgks_batch_step(hgks_batch* b, const double* t_end, int nsteps, i
         for (int k = 0; k < 3 && left > 0; k++) {
             int tpb[BK_COUNT];
             for (int c = 0; c < BK_COUNT; c++) {
-                bool heavy_regs = c == BK_FLUX || c == BK_NAO || c == BK_TAO;
-                tpb[c] = c == BK_CTRL ? 32 : (heavy_regs ? cand_small[k] : cand_big[k]);
+                bool heavy_regs = c == BK_FLUX || c == BK_NAO || c == BK_TAO || c == BK_NSMALL || c == BK_TSMALL;
+                tpb[c] = heavy_regs ? cand_small[k] : cand_big[k];
                 // a flux block keeps 224 bytes of shared memory a thread: 128 threads stay below 48 KB
                 if (c == BK_FLUX && tpb[c] > 128) tpb[c] = 128;
             }
@@ -683,8 +683,8 @@ extern "C" int hgks_batch_step(hgks_batch* b, const double* t_end, int nsteps, i
             b->steps_enqueued++;
             left--;
             for (int c = 0; c < BK_COUNT; c++) {
-                // classes without launches in this dimension (and the control kernels) carry no events
-                if (c == BK_CTRL || b->plan.nblk[c] == 0) continue;
+                // classes without launches carry no events
+                if (b->plan.nblk[c] == 0) continue;
                 float ms = 0.0f;
                 cudaError_t qe = cudaEventElapsedTime(&ms, b->ev[2 * c], b->ev[2 * c + 1]);
                 if (qe != cudaSuccess) { (void)cudaGetLastError(); continue; }

@@ -26,6 +26,7 @@ struct Ctrl {
     int status;                      // 0 or HGKS_ENONPHYSICAL
     long long steps;
     unsigned int cnt[2][2];          // AO work-list lengths [sweep][0 normal, 1 tangential]
+    unsigned int dt_blocks;          // blocks of the time-step reduction that have finished
     unsigned long long troubled[2][2][2];
     unsigned long long examined[2][2][2];
 };
@@ -47,7 +48,7 @@ struct Sweep {
     int nn, nt;                // cells normal / tangential
     int nm;                    // interfaces per line (nn + 1)
     int nlines;                // lines with normal reconstruction (nt + 6 in 2D, 1 in 1D)
-    int tlanes;                // lanes per segment of the tangential kernels: 4 for small sweeps, else 1
+    int small;                 // below 65536 interface segments: one launch per reconstruction direction (lane groups)
     int tlo;                   // first line index (-3 in 2D, 0 in 1D)
     long long sN, sT;          // state strides for +1 in n / t
     int perm[4];               // local component -> global component
@@ -94,8 +95,8 @@ struct SolveDesc {
 // Kernel classes of a batched step, one launch each per stage.  The sweep classes (BK_RAWN to
 // BK_FLUX) cover both sweeps of every solver: their units are (solver s, sweep d), unit 2 s + d.
 enum BatchClass {
-    BK_CTRL = 0, BK_DT, BK_GHX, BK_GHY,
-    BK_RAWN, BK_NORMAL, BK_NAO, BK_RAWT, BK_TANG, BK_TAO, BK_FLUX,
+    BK_DT = 0, BK_GHOST,
+    BK_RAWN, BK_NORMAL, BK_NAO, BK_NSMALL, BK_RAWT, BK_TANG, BK_TAO, BK_TSMALL, BK_FLUX,
     BK_UPD, BK_COUNT
 };
 
@@ -139,7 +140,7 @@ struct hgks_solver {
 namespace hgks {
 
 // kernel classes for timing
-enum KClass { KC_GHOST = 0, KC_DT, KC_RAWN, KC_NORMAL, KC_NORMAL_AO, KC_RAWT, KC_TANG, KC_TANG_AO, KC_FLUX, KC_UPDATE, KC_MISC, KC_COUNT };
+enum KClass { KC_GHOST = 0, KC_DT, KC_RAWN, KC_NORMAL, KC_NORMAL_AO, KC_RAWT, KC_TANG, KC_TANG_AO, KC_FLUX, KC_UPDATE, KC_COUNT };
 extern const char* kclass_names[KC_COUNT];
 
 // host-side launchers (hgks_kernels.cu); all enqueue on s->stream

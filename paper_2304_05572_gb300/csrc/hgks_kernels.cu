@@ -19,7 +19,7 @@ namespace hgks {
 
 const char* kclass_names[KC_COUNT] = {"ghost", "dt", "raw_normal_flags", "normal_recon", "normal_weno_ao",
                                       "raw_tangential_flags", "tangential_recon", "tangential_weno_ao",
-                                      "gks_flux", "stage_update", "misc"};
+                                      "gks_flux", "stage_update"};
 
 namespace {
 
@@ -76,26 +76,18 @@ __device__ __forceinline__ double cell_centre(double origin, int i, double h)
     return (ex(origin) + (ex((double)i) + ex(0.5)) * ex(h)).v;
 }
 
-// The first thread of a stage's x-ghost launch also empties the stage's work lists (no kernel
-// of the stage reads them before the ghost fills are complete).
-__device__ __forceinline__ void b_ghost_x(const Params& P, double* __restrict__ W, Ctrl* __restrict__ ctrl, long long id)
+// Component k of cell (i, j) of an interior row j, i anywhere in the padded width: the interior cell, or
+// the x ghost cell's value by its boundary.
+__device__ __forceinline__ double x_value(const Params& P, const double* W, int k, int i, int j)
 {
-    if (ctrl->done) return;
-    if (id == 0) ctrl->cnt[0][0] = ctrl->cnt[0][1] = ctrl->cnt[1][0] = ctrl->cnt[1][1] = 0;
     const GridGeom& g = P.g;
-    int rowsI = g.dim == 2 ? g.ny : 1;
-    long long total = (long long)g.nv * rowsI * NG * 2;
-    if (id >= total) return;
-    int side = (int)(id % 2); id /= 2;
-    int l = (int)(id % NG) + 1; id /= NG;
-    int j = (int)(id % rowsI);
-    int k = (int)(id / rowsI);
-    int bc = P.bc[side];
-    int dst = side == 0 ? -l : g.nx - 1 + l;
-    double* base = W + g.origin + (long long)k * g.plane + (long long)j * g.pitch;
-    if (bc == HGKS_BC_INFLOW) { stc(base + dst, P.bc_state[side][k], g); return; }
+    const double* base = W + g.origin + (long long)k * g.plane + (long long)j * g.pitch;
+    if (i >= 0 && i < g.nx) return rdc(base + i, g);
+    const int side = i < 0 ? 0 : 1, l = i < 0 ? -i : i - g.nx + 1;
+    const int bc = P.bc[side];
+    if (bc == HGKS_BC_INFLOW) return P.bc_state[side][k];
+    const bool mirror = bc == HGKS_BC_REFLECT || bc == HGKS_BC_SYMMETRY || bc == HGKS_BC_NOSLIP;
     int src;
-    bool mirror = bc == HGKS_BC_REFLECT || bc == HGKS_BC_SYMMETRY || bc == HGKS_BC_NOSLIP;
     if (bc == HGKS_BC_PERIODIC) src = side == 0 ? g.nx - l : l - 1;
     else if (bc == HGKS_BC_EXTRAP) src = side == 0 ? 0 : g.nx - 1;
     else src = side == 0 ? l - 1 : g.nx - l;
@@ -104,68 +96,78 @@ __device__ __forceinline__ void b_ghost_x(const Params& P, double* __restrict__ 
         if (k == 1) v = -v;
         if (bc == HGKS_BC_NOSLIP && g.dim == 2 && k == 2) v = -v;
     }
-    stc(base + dst, v, g);
+    return v;
 }
 
-__global__ void k_ghost_x(Params P, double* __restrict__ W, Ctrl* __restrict__ ctrl)
+// The ghost cells of a stage, one value per thread: the x sides on interior rows, then the y sides over the
+// padded width.  A corner takes its y boundary's image of the x ghost cell beside it, formed from the
+// interior cell behind both (x_value), so no ghost cell is read and one launch fills them all.
+// The first thread also empties the stage's work lists (no kernel of the stage reads them before this launch
+// is complete).
+inline long long ghost_threads(const GridGeom& g)
 {
-    b_ghost_x(P, W, ctrl, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+    const long long x = (long long)g.nv * (g.dim == 2 ? g.ny : 1) * NG * 2;
+    return g.dim == 2 ? x + (long long)g.nv * (g.nx + 2 * NG) * NG * 2 : x;
 }
 
-
-__device__ __forceinline__ void b_ghost_y(const Params& P, double* __restrict__ W, const Ctrl* __restrict__ ctrl, int stage, long long id)
+__device__ __forceinline__ void b_ghost(const Params& P, double* W, Ctrl* __restrict__ ctrl, int stage, long long id)
 {
-    if (ctrl->done) return;
+    if (id == 0) ctrl->cnt[0][0] = ctrl->cnt[0][1] = ctrl->cnt[1][0] = ctrl->cnt[1][1] = 0;
     const GridGeom& g = P.g;
-    int width = g.nx + 2 * NG;
-    long long total = (long long)g.nv * width * NG * 2;
-    if (id >= total) return;
-    int i = (int)(id % width) - NG; id /= width;
-    int side = (int)(id % 2); id /= 2;
-    int l = (int)(id % NG) + 1;
-    int k = (int)(id / NG);
-    int bc = P.bc[2 + side];
-    int dst = side == 0 ? -l : g.ny - 1 + l;
-    double* base = W + g.origin + (long long)k * g.plane + i;
-    if (bc == HGKS_BC_INFLOW) { stc(base + (long long)dst * g.pitch, P.bc_state[2 + side][k], g); return; }
+    const int rowsI = g.dim == 2 ? g.ny : 1;
+    const long long nxg = (long long)g.nv * rowsI * NG * 2;
+    if (id < nxg) {
+        const int side = (int)(id % 2); id /= 2;
+        const int l = (int)(id % NG) + 1; id /= NG;
+        const int j = (int)(id % rowsI);
+        const int k = (int)(id / rowsI);
+        const int dst = side == 0 ? -l : g.nx - 1 + l;
+        stc(W + g.origin + (long long)k * g.plane + (long long)j * g.pitch + dst, x_value(P, W, k, dst, j), g);
+        return;
+    }
+    id -= nxg;
+    const int width = g.nx + 2 * NG;
+    if (g.dim != 2 || id >= (long long)g.nv * width * NG * 2) return;
+    const int i = (int)(id % width) - NG; id /= width;
+    const int side = (int)(id % 2); id /= 2;
+    const int l = (int)(id % NG) + 1;
+    const int k = (int)(id / NG);
+    const int bc = P.bc[2 + side];
+    const int dst = side == 0 ? -l : g.ny - 1 + l;
+    double* to = W + g.origin + (long long)k * g.plane + (long long)dst * g.pitch + i;
+    if (bc == HGKS_BC_INFLOW) { stc(to, P.bc_state[2 + side][k], g); return; }
     if (bc == HGKS_BC_SHOCK_TRACK) {
         const double xc = cell_centre(P.x0, i, g.dx), yc = cell_centre(P.y0, dst, g.dy);
         const double t = stage_time(ctrl, stage);
         const double xs = (ex(P.shock_x0) + ex(P.shock_cot) * (ex(yc) + ex(P.shock_speed) * ex(t))).v;
-        stc(base + (long long)dst * g.pitch, xc < xs ? P.bc_state[2 + side][k] : P.shock_pre[k], g);
+        stc(to, xc < xs ? P.bc_state[2 + side][k] : P.shock_pre[k], g);
         return;
     }
     if (bc == HGKS_BC_SHOCK_WALL && cell_centre(P.x0, i, g.dx) < P.shock_x0) {
-        stc(base + (long long)dst * g.pitch, P.bc_state[2 + side][k], g);
+        stc(to, P.bc_state[2 + side][k], g);
         return;
     }
+    const bool mirror = bc == HGKS_BC_REFLECT || bc == HGKS_BC_SYMMETRY || bc == HGKS_BC_NOSLIP || bc == HGKS_BC_SHOCK_WALL;
     int src;
-    bool mirror = bc == HGKS_BC_REFLECT || bc == HGKS_BC_SYMMETRY || bc == HGKS_BC_NOSLIP || bc == HGKS_BC_SHOCK_WALL;
     if (bc == HGKS_BC_PERIODIC) src = side == 0 ? g.ny - l : l - 1;
     else if (bc == HGKS_BC_EXTRAP) src = side == 0 ? 0 : g.ny - 1;
     else src = side == 0 ? l - 1 : g.ny - l;
-    double v = rdc(base + (long long)src * g.pitch, g);
+    double v = x_value(P, W, k, i, src);
     if (mirror) {
         if (k == 2) v = -v;
         if (bc == HGKS_BC_NOSLIP && k == 1) v = -v;
     }
-    stc(base + (long long)dst * g.pitch, v, g);
+    stc(to, v, g);
 }
 
-__global__ void k_ghost_y(Params P, double* __restrict__ W, const Ctrl* __restrict__ ctrl, int stage)
+// Second stage (W*)
+__global__ void k_ghost(Params P, double* W, Ctrl* __restrict__ ctrl)
 {
-    b_ghost_y(P, W, ctrl, stage, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+    if (ctrl->done) return;
+    b_ghost(P, W, ctrl, 1, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
-
 
 // ---------------------------------------------------------------- time step
-__global__ void k_begin_step(Ctrl* ctrl)
-{
-    ctrl->dtmin_bits = 0x7FF0000000000000ull;   // +inf
-    ctrl->cnt[0][0] = ctrl->cnt[0][1] = ctrl->cnt[1][0] = ctrl->cnt[1][1] = 0;
-}
-
-
 // Sec. 3 preamble: dt = CFL min(h/(|U|+a), h^2/(4 nu)), h = min(dx, dy), nu = mu/rho;
 // same evaluation order as the CPU reference so that dt is reproduced exactly.
 __device__ __forceinline__ void b_dt(const Params& P, const double* __restrict__ W, Ctrl* ctrl, double h, long long start, long long stride)
@@ -201,15 +203,20 @@ __device__ __forceinline__ void b_dt(const Params& P, const double* __restrict__
     if ((threadIdx.x & 31) == 0) atomicMin(&ctrl->dtmin_bits, best);
 }
 
-__global__ void k_dt(Params P, const double* __restrict__ W, Ctrl* ctrl, double h)
+// Called by every thread of each of the `blocks` blocks that reduced a solver's dt: the last block to
+// arrive applies the CFL number (or takes the fixed step), clips to t_end, decides whether the step
+// runs, and leaves the reduction ready for the next step.
+__device__ __forceinline__ void dt_finish(const Params& P, Ctrl* ctrl, double t_end, unsigned int blocks)
 {
-    b_dt(P, W, ctrl, h, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
-}
-
-
-__global__ void k_dt_final(Ctrl* ctrl, double cfl, double fixed_dt, double t_end, double tol)
-{
-    double dt = fixed_dt > 0.0 ? fixed_dt : cfl * __longlong_as_double((long long)ctrl->dtmin_bits);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(&ctrl->dt_blocks, 1u) != blocks - 1u) return;
+    __threadfence();
+    ctrl->dt_blocks = 0;
+    const unsigned long long bits = atomicExch(&ctrl->dtmin_bits, 0x7FF0000000000000ull);
+    const double tol = 1e-12 * (fabs(t_end) > 1.0 ? fabs(t_end) : 1.0);
+    double dt = P.fixed_dt > 0.0 ? P.fixed_dt : P.cfl * __longlong_as_double((long long)bits);
     int done = ctrl->status != 0 || !(t_end - ctrl->t > tol);
     if (!done && ctrl->t + dt > t_end) dt = t_end - ctrl->t;
     if (!done && !(dt > 0.0 && dt < 1e300)) { ctrl->status = HGKS_ENONPHYSICAL; done = 1; }
@@ -217,17 +224,25 @@ __global__ void k_dt_final(Ctrl* ctrl, double cfl, double fixed_dt, double t_end
     ctrl->done = done;
 }
 
-__global__ void k_end_step(Ctrl* ctrl)
+// The first launch of a step: blocks [0, nb) reduce dt, the others fill the ghost cells of W^n (both only
+// read interior cells; a step that turns out to be done has its ghost cells filled for nothing).  One launch
+// for what took five (work-list reset, dt, its decision, two ghost fills).
+__global__ void k_dt_ghost(Params P, double* W, Ctrl* ctrl, double h, double t_end, int nb)
 {
-    if (ctrl->done) return;
-    ctrl->t += ctrl->dt;
-    ctrl->last_dt = ctrl->dt;
-    ctrl->steps += 1;
+    const int b = (int)blockIdx.x;
+    if (b >= nb) {
+        b_ghost(P, W, ctrl, 0, (long long)(b - nb) * blockDim.x + threadIdx.x);
+        return;
+    }
+    if (!(P.fixed_dt > 0.0)) b_dt(P, W, ctrl, h, (long long)b * blockDim.x + threadIdx.x, (long long)nb * blockDim.x);
+    dt_finish(P, ctrl, t_end, (unsigned)nb);
 }
 
 __global__ void k_set_time(Ctrl* ctrl, double t0)
 {
     ctrl->t = t0;
+    ctrl->dtmin_bits = 0x7FF0000000000000ull;   // +inf
+    ctrl->dt_blocks = 0;
     ctrl->dt = 0.0;
     ctrl->last_dt = 0.0;
     ctrl->steps = 0;
@@ -285,7 +300,7 @@ __device__ __forceinline__ void b_raw_nflags(const Params& P, const Sweep& S, co
             const double* b = base + (long long)S.perm[k] * P.g.plane;
 #pragma unroll
             for (int s = 0; s < 5; s++) { q[s] = ldc(b + (long long)s * S.sN, S); f[s] = fixed::to_float(q[s]); }
-            tr |= indicator_raw(q, f, S.Z1n);
+            tr |= indicator_raw<false>(q, f, S.Z1n);
         }
     }
     stc(S.rawN + id, tr, S);
@@ -489,6 +504,102 @@ __global__ void k_normal_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
 }
 
 
+// Small sweeps: flags, linear reconstruction and WENO-AO of the normal pass in one launch, one (line,
+// interface, side) per aligned group of 4 lanes, lane q carrying component q.  The group runs the raw
+// indicator on the three cells the Step-4 spread looks at (7 values a lane, so nothing is read back), ORs it
+// over the components with shuffles, and takes the linear formulas or weno_ao_face_x4.  The arithmetic is
+// b_normal's and b_normal_ao's, so every result is.  Such a sweep's time is made of launches (3 us each)
+// and of each thread's chain of FP64 instructions (31 ns each): with one launch per direction in place of
+// three (flags, linear pass, compacted WENO-AO) and the step's five control and ghost launches in two, a
+// step of 200 cells in 1D went from 133 to 90 us, of 48 x 48 from 210 to 136, of the 200 x 100 viscous tube
+// from 508 to 466.  Compaction and shared flags pay from about 65536 segments on.
+template <int NV>
+__device__ __forceinline__ void b_normal_small(const Params& P, const Sweep& S, const double* __restrict__ W, Ctrl* ctrl, int stage, long long id)
+{
+    if (ctrl->done) return;
+    const long long total = (long long)S.nlines * S.nm * 2;
+    const long long item = id >> 2;
+    const int q = (int)(id & 3), qc = q < NV ? q : NV - 1;
+    const int lane0 = threadIdx.x & 28;
+    const unsigned gmask = 0xFu << lane0;
+    const bool active = item < total;               // the same for the 4 lanes of a group
+    const int side = (int)(item & 1);
+    int L = 0, m = 0, flag = 0;
+    double v[7];
+    if (active) {
+        const unsigned lm = (unsigned)(item >> 1);
+        L = (int)(lm / (unsigned)S.nm); m = (int)(lm - (unsigned)L * (unsigned)S.nm);
+        const double* b = cellp(P, S, W, L + S.tlo, m - 1 + side - 3) + (long long)S.perm[qc] * P.g.plane;
+#pragma unroll
+        for (int s = 0; s < 7; s++) v[s] = ldc(b + (long long)s * S.sN, S);
+        if (P.recon_mode == HGKS_RECON_WENOAO) flag = 1;
+        else if (P.recon_mode == HGKS_RECON_HYBRID) {
+            float f[7];
+#pragma unroll
+            for (int s = 0; s < 7; s++) f[s] = fixed::to_float(v[s]);
+#pragma unroll
+            for (int s = 0; s < 3; s++) flag |= indicator_raw<true>(v + s, f + s, S.Z1n);
+            flag |= __shfl_xor_sync(gmask, flag, 1);
+            flag |= __shfl_xor_sync(gmask, flag, 2);
+        }
+        if (q == 0) {
+            uint8_t* fo = S.flagN + (long long)L * (S.nn + 2);
+            if (side == 1) stc(fo + m + 1, flag, S);
+            else if (m == 0) stc(fo, flag, S);
+        }
+    }
+    const int t = L + S.tlo;
+    const bool counted = active && q == 0 && side == 1 && t >= 0 && t < S.nt && m < S.nn;
+    warp_count(&ctrl->troubled[stage][S.dir][0], counted && flag ? 1u : 0u);
+    warp_count(&ctrl->examined[stage][S.dir][0], counted ? 1u : 0u);
+    if (!active) return;
+    double val, der;
+    if (!flag) {
+        if (side == 0) linear_left(v + 1, S.inv12hn, val, der);
+        else linear_right(v + 1, S.inv12hn, val, der);
+        double Q[NV];
+#pragma unroll
+        for (int k = 0; k < NV; k++) Q[k] = __shfl_sync(gmask, val, lane0 + k);
+        if (nonphysical<NV>(P.gamma, Q)) { val = v[3]; der = 0.0; }
+    } else {
+        AOConst ak;
+        for (int j = 0; j < 4; j++) ak.g[j] = P.g_ao[j];
+        ak.g3inv = P.g3inv; ak.gr[0] = P.gr[0]; ak.gr[1] = P.gr[1]; ak.gr[2] = P.gr[2]; ak.eps = P.eps;
+        double Qw[5][NV], Qs[NV], vs[NV];
+        const double avg = ((ex(side == 0 ? v[3] : v[2]) + ex(side == 0 ? v[4] : v[3])) * ex(0.5)).v;
+#pragma unroll
+        for (int k = 0; k < NV; k++) {
+            Qs[k] = __shfl_sync(gmask, avg, lane0 + k);
+#pragma unroll
+            for (int s = 0; s < 5; s++) Qw[s][k] = __shfl_sync(gmask, v[s + 1], lane0 + k);
+        }
+        weno_ao_face_x4<NV>(P.gamma, ak, Qw, Qs, side == 0 ? +1 : -1, gmask, vs, der);
+        val = 0.0;
+        if (nonphysical<NV>(P.gamma, vs)) {
+            val = v[3];
+            der = 0.0;
+        } else {
+#pragma unroll
+            for (int k = 0; k < NV; k++)
+                if (k == q) val = vs[k];
+            der = (ex(der) * ex(S.inv_hn)).v;
+        }
+    }
+    if (q < NV) {
+        const long long plane = (long long)S.nlines * S.nm, o = (long long)L * S.nm + m;
+        stc(S.line + (long long)(side * NV + q) * plane + o, val, S);
+        stc(S.line + (long long)((2 + side) * NV + q) * plane + o, der, S);
+    }
+}
+
+template <int NV>
+__global__ void k_normal_small(const SolveDesc* __restrict__ D, int nb0, int stage)
+{
+    const SweepBlock b = sweep_block(nb0);
+    const SolveDesc& d = *D;
+    b_normal_small<NV>(d.P, d.sw[b.dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, b.id);
+}
+
 // ---------------------------------------------------------------- tangential passes (2D)
 __device__ __forceinline__ double lineval(const Sweep& S, int X, int k, int t, int m)
 {
@@ -496,40 +607,11 @@ __device__ __forceinline__ double lineval(const Sweep& S, int X, int k, int t, i
     return ldc(S.line + (long long)(X * 4 + k) * plane + (long long)(t - S.tlo) * S.nm + m, S);
 }
 
-// Raw tangential flags, one segment per aligned group of 4 lanes: lane q runs the indicator of
-// every pass X on component q, the 4 components' bits are OR-ed with shuffles (a cell is smooth
-// only if every component is), and lane 0 stores them.  `id` counts lanes.
-__device__ __forceinline__ void b_raw_tflags_x4(const Params& P, const Sweep& S, const Ctrl* __restrict__ ctrl, long long id)
-{
-    if (ctrl->done) return;
-    long long total = (long long)(S.nt + 2) * S.nm;
-    const long long seg = id >> 2;
-    if (seg >= total) return;                       // the same for the 4 lanes of a group
-    const int q = (int)(id & 3);
-    const unsigned gmask = 0xFu << (threadIdx.x & 28);
-    int m = (int)(seg % S.nm);
-    int t = (int)(seg / S.nm) - 1;
-    unsigned int bits = 0;
-    if (P.recon_mode == HGKS_RECON_HYBRID) {
-#pragma unroll
-        for (int X = 0; X < 4; X++) {
-            double qv[5];
-            float f[5];
-#pragma unroll
-            for (int s = 0; s < 5; s++) { qv[s] = lineval(S, X, q, t - 2 + s, m); f[s] = fixed::to_float(qv[s]); }
-            bits |= (unsigned)indicator_raw(qv, f, S.Z1t) << X;
-        }
-        bits |= __shfl_xor_sync(gmask, bits, 1);
-        bits |= __shfl_xor_sync(gmask, bits, 2);
-    }
-    if (q == 0) stc(S.rawT + seg, bits, S);
-}
-
 // Large sweeps: each thread takes kTRows consecutive lines of one interface, so that a line value is
 // loaded and truncated once for up to 5 windows (8 rows instead of 20 for 4 segments).
 constexpr int kTRows = 4;
 
-__device__ __forceinline__ void b_raw_tflags_x1(const Params& P, const Sweep& S, const Ctrl* __restrict__ ctrl, long long id)
+__device__ __forceinline__ void b_raw_tflags(const Params& P, const Sweep& S, const Ctrl* __restrict__ ctrl, long long id)
 {
     if (ctrl->done) return;
     const int m = (int)(id % S.nm);
@@ -552,7 +634,7 @@ __device__ __forceinline__ void b_raw_tflags_x1(const Params& P, const Sweep& S,
                 }
 #pragma unroll
                 for (int r = 0; r < kTRows; r++)
-                    if (r < rows) bits[r] |= (unsigned)indicator_raw(q + r, f + r, S.Z1t) << X;
+                    if (r < rows) bits[r] |= (unsigned)indicator_raw<false>(q + r, f + r, S.Z1t) << X;
             }
         }
     }
@@ -562,19 +644,7 @@ __device__ __forceinline__ void b_raw_tflags_x1(const Params& P, const Sweep& S,
 }
 
 // Threads of the raw tangential flag kernel on sweep S.
-inline long long raw_t_threads(const Sweep& S)
-{
-    return S.tlanes == 4 ? (long long)(S.nt + 2) * S.nm * 4 : (long long)((S.nt + 2 + kTRows - 1) / kTRows) * S.nm;
-}
-
-// Small sweeps (fewer segments than a few warps per scheduler) spread a segment over 4 lanes,
-// which shortens the chain of FP64 instructions per thread; large sweeps keep one segment per
-// thread.  The arithmetic, and so every result, is the same either way.
-__device__ __forceinline__ void b_raw_tflags(const Params& P, const Sweep& S, const Ctrl* __restrict__ ctrl, long long id)
-{
-    if (S.tlanes == 4) b_raw_tflags_x4(P, S, ctrl, id);
-    else b_raw_tflags_x1(P, S, ctrl, id);
-}
+inline long long raw_t_threads(const Sweep& S) { return (long long)((S.nt + 2 + kTRows - 1) / kTRows) * S.nm; }
 
 __global__ void k_raw_tflags(const SolveDesc* __restrict__ D, int nb0)
 {
@@ -597,71 +667,10 @@ __device__ __forceinline__ void gp_positivity(const Params& P, const Sweep& S, i
     }
 }
 
-// Gauss-point reconstruction of the smooth passes, one segment per aligned group of 4 lanes, lane q
-// carrying component q: the Step-4 spread flags of the segment (the same in every lane; lane 0
-// stores them, counts them and appends the troubled passes to the WENO-AO work list), then for
-// every smooth pass the quartic of component q at both Gauss points; the positivity test of the
-// Q^l, Q^r passes gathers the 4 components with shuffles.  `id` counts lanes.  Every lane of the
-// warp reaches the warp-wide counts and appends.
-__device__ __forceinline__ void b_tang_x4(const Params& P, const Sweep& S, Ctrl* ctrl, int stage, long long id)
-{
-    if (ctrl->done) return;
-    long long total = (long long)S.nt * S.nm;
-    const long long seg = id >> 2;
-    const int q = (int)(id & 3);
-    const int lane0 = threadIdx.x & 28;
-    const unsigned gmask = 0xFu << lane0;
-    bool active = seg < total;                      // the same for the 4 lanes of a group
-    int m = 0, t = 0;
-    unsigned int bits = 0;
-    if (active) {
-        m = (int)(seg % S.nm); t = (int)(seg / S.nm);
-        if (P.recon_mode == HGKS_RECON_LINEAR) bits = 0;
-        else if (P.recon_mode == HGKS_RECON_WENOAO) bits = 0xF;
-        else bits = rdc(S.rawT + (long long)t * S.nm + m, S) | rdc(S.rawT + (long long)(t + 1) * S.nm + m, S)
-                    | rdc(S.rawT + (long long)(t + 2) * S.nm + m, S);
-        if (q == 0) stc(S.flagT + seg, bits, S);
-    }
-    const bool lead = active && q == 0;
-    warp_count(&ctrl->troubled[stage][S.dir][1], lead ? (unsigned)__popc(bits) : 0u);
-    warp_count(&ctrl->examined[stage][S.dir][1], lead ? 4u : 0u);
-    const long long plane = (long long)S.nt * S.nm;
-    const long long o = (long long)t * S.nm + m;
-    const fixed::Scale inv = fixed::scale_of(S.inv_ht);
-#pragma unroll
-    for (int X = 0; X < 4; X++) {
-        bool f = active && ((bits >> X) & 1);
-        warp_push(&ctrl->cnt[S.dir][1], S.itemsT, f && q == 0, (uint32_t)((seg << 2) | X), S);
-        if (!active || f) continue;                 // the same for the 4 lanes of a group
-        double qv[5], v[2], d[2];
-#pragma unroll
-        for (int s = 0; s < 5; s++) qv[s] = lineval(S, X, q, t - 2 + s, m);
-        if (X <= 1) gauss_linear<true>(qv, inv, S.inv_ht, v, d);
-        else gauss_linear<false>(qv, inv, S.inv_ht, v, d);
-        if (X <= 1) {
-            // Reading: a reconstructed state with rho <= 0 or p <= 0 falls back to first order
-#pragma unroll
-            for (int g = 0; g < 2; g++) {
-                double Q[4];
-#pragma unroll
-                for (int c = 0; c < 4; c++) Q[c] = __shfl_sync(gmask, v[g], lane0 + c);
-                if (nonphysical<4>(P.gamma, Q)) { v[g] = lineval(S, X, q, t, m); d[g] = 0.0; }
-            }
-        }
-        // Q index: 0 Wl, 1 Wlx, 2 Wly, 3 Wr, 4 Wrx, 5 Wry
-        constexpr int qx[4] = {0, 3, 1, 4};
-#pragma unroll
-        for (int g = 0; g < 2; g++) {
-            stc(S.gp + (long long)((g * 6 + qx[X]) * 4 + q) * plane + o, v[g], S);
-            if (X <= 1) stc(S.gp + (long long)((g * 6 + qx[X] + 2) * 4 + q) * plane + o, d[g], S);
-        }
-    }
-}
-
 // Large sweeps: the Step-4 spread flags of a segment (stored, counted, troubled passes appended
 // to the WENO-AO work list); the smooth passes are reconstructed inside the flux kernel
 // (b_flux, side_pair), so their Gauss-point states never go to memory.
-__device__ __forceinline__ void b_tflags_x1(const Params& P, const Sweep& S, Ctrl* ctrl, int stage, long long id)
+__device__ __forceinline__ void b_tang(const Params& P, const Sweep& S, Ctrl* ctrl, int stage, long long id)
 {
     if (ctrl->done) return;
     long long total = (long long)S.nt * S.nm;
@@ -683,12 +692,6 @@ __device__ __forceinline__ void b_tflags_x1(const Params& P, const Sweep& S, Ctr
         bool f = active && ((bits >> X) & 1);
         warp_push(&ctrl->cnt[S.dir][1], S.itemsT, f, (uint32_t)((((long long)t * S.nm + m) << 2) | X), S);
     }
-}
-
-__device__ __forceinline__ void b_tang(const Params& P, const Sweep& S, Ctrl* ctrl, int stage, long long id)
-{
-    if (S.tlanes == 4) b_tang_x4(P, S, ctrl, stage, id);
-    else b_tflags_x1(P, S, ctrl, stage, id);
 }
 
 __global__ void k_tang(const SolveDesc* __restrict__ D, int nb0, int stage)
@@ -801,6 +804,100 @@ __global__ void k_tang_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
 }
 
 
+// Small sweeps: flags, quartics and WENO-AO of the four tangential passes in one launch, 16 lanes per
+// segment: lanes 4 X + q carry component q of pass X.  As in b_normal_small the raw indicator runs on the three
+// lines the Step-4 spread looks at; every pass ends in the Gauss-point buffer.  Free-order arithmetic:
+// compiled once (tang_small_nl) like tang_ao_nl.
+__device__ __forceinline__ void b_tang_small(const Params& P, const Sweep& S, const double* __restrict__ W, Ctrl* ctrl, int stage, long long id)
+{
+    if (ctrl->done) return;
+    const long long total = (long long)S.nt * S.nm;
+    const long long seg = id >> 4;
+    const int X = (int)(id >> 2) & 3, q = (int)(id & 3);
+    const int lane0 = threadIdx.x & 28;
+    const unsigned gmask = 0xFu << lane0, hmask = 0xFFFFu << (threadIdx.x & 16);
+    const bool active = seg < total;                // the same for the 16 lanes of a segment
+    int t = 0, m = 0;
+    unsigned flag = 0, bits = 0;
+    double v[7];
+    if (active) {
+        t = (int)((unsigned)seg / (unsigned)S.nm); m = (int)((unsigned)seg - (unsigned)t * (unsigned)S.nm);
+#pragma unroll
+        for (int s = 0; s < 7; s++) v[s] = lineval(S, X, q, t - 3 + s, m);
+        if (P.recon_mode == HGKS_RECON_WENOAO) flag = 1;
+        else if (P.recon_mode == HGKS_RECON_HYBRID) {
+            float f[7];
+#pragma unroll
+            for (int s = 0; s < 7; s++) f[s] = fixed::to_float(v[s]);
+#pragma unroll
+            for (int s = 0; s < 3; s++) flag |= (unsigned)indicator_raw<true>(v + s, f + s, S.Z1t);
+            flag |= __shfl_xor_sync(gmask, flag, 1);
+            flag |= __shfl_xor_sync(gmask, flag, 2);
+        }
+        bits = flag << X;
+        bits |= __shfl_xor_sync(hmask, bits, 4);
+        bits |= __shfl_xor_sync(hmask, bits, 8);
+        if ((id & 15) == 0) stc(S.flagT + seg, bits, S);
+    }
+    const bool lead = active && (id & 15) == 0;
+    warp_count(&ctrl->troubled[stage][S.dir][1], lead ? (unsigned)__popc(bits) : 0u);
+    warp_count(&ctrl->examined[stage][S.dir][1], lead ? 4u : 0u);
+    if (!active) return;
+    double vq[2], dq[2] = {0.0, 0.0};
+    if (!flag) {
+        const fixed::Scale inv = fixed::scale_of(S.inv_ht);
+        if (X <= 1) gauss_linear<true>(v + 1, inv, S.inv_ht, vq, dq);
+        else gauss_linear<false>(v + 1, inv, S.inv_ht, vq, dq);
+    } else {
+        AOConst ak;
+        for (int j = 0; j < 4; j++) ak.g[j] = P.g_ao[j];
+        ak.g3inv = P.g3inv; ak.gr[0] = P.gr[0]; ak.gr[1] = P.gr[1]; ak.gr[2] = P.gr[2]; ak.eps = P.eps;
+        // the face average of the segment, one component a lane
+        const long long oc = (long long)S.perm[q] * P.g.plane;
+        const double avg = scale2<-1>(ldc(cellp(P, S, W, t, m - 1) + oc, S) + ldc(cellp(P, S, W, t, m) + oc, S));
+        double qs[4], x[5][4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            qs[k] = __shfl_sync(gmask, avg, lane0 + k);
+#pragma unroll
+            for (int s = 0; s < 5; s++) x[s][k] = __shfl_sync(gmask, v[s + 1], lane0 + k);
+        }
+        TangEig e;
+        tang_eig(P.gamma, qs, e);
+        tang_ao_x4(e, x, ak, X <= 1, gmask, vq, dq);
+        dq[0] *= S.inv_ht;
+        dq[1] *= S.inv_ht;
+    }
+    if (X <= 1) {
+        // Reading: a reconstructed state with rho <= 0 or p <= 0 falls back to first order
+#pragma unroll
+        for (int g = 0; g < 2; g++) {
+            double Q[4];
+#pragma unroll
+            for (int c = 0; c < 4; c++) Q[c] = __shfl_sync(gmask, vq[g], lane0 + c);
+            if (nonphysical<4>(P.gamma, Q)) { vq[g] = v[3]; dq[g] = 0.0; }
+        }
+    }
+    // Q index: 0 Wl, 1 Wlx, 2 Wly, 3 Wr, 4 Wrx, 5 Wry
+    const int qv = X == 0 ? 0 : (X == 1 ? 3 : (X == 2 ? 1 : 4));
+#pragma unroll
+    for (int g = 0; g < 2; g++) {
+        stc(S.gp + (long long)((g * 6 + qv) * 4 + q) * total + seg, vq[g], S);
+        if (X <= 1) stc(S.gp + (long long)((g * 6 + qv + 2) * 4 + q) * total + seg, dq[g], S);
+    }
+}
+
+__device__ __noinline__ void tang_small_nl(const SolveDesc& d, int dir, int stage, long long id)
+{
+    b_tang_small(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, id);
+}
+
+__global__ void k_tang_small(const SolveDesc* __restrict__ D, int nb0, int stage)
+{
+    const SweepBlock b = sweep_block(nb0);
+    tang_small_nl(*D, b.dir, stage, b.id);
+}
+
 // ---------------------------------------------------------------- flux and update
 
 // Shared memory of a 2D flux block of `threads`: the reconstructed side states (24 doubles a
@@ -886,7 +983,7 @@ __device__ __forceinline__ void side_states(const Params& P, const Sweep& S, int
     if constexpr (DIM == 2) {
         const long long per = (long long)S.nt * S.nm;
         const double* gp = S.gp + (long long)((g * 6 + 3 * side) * 4) * per + o;
-        if (S.tlanes == 4) {
+        if (S.small) {
 #pragma unroll
             for (int k = 0; k < NV; k++) {
                 Wv[k] = ldc(gp + (long long)k * per, S);
@@ -937,7 +1034,7 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
         // side, and they exchange through shared memory: every line value is loaded and converted once, and
         // the two points share their products (with the products in FP64 and each warp reconstructing both
         // sides at its own point the launch took 5.04 ms at 1024^2, so 4.18 ms)
-        if (S.tlanes != 4) {
+        if (!S.small) {
             if (valid) side_pair(P, S, g, o, flux_sh + threadIdx.x, stride);
             __syncthreads();
         }
@@ -1026,6 +1123,11 @@ template <int DIM, int STAGE>
 __device__ __forceinline__ void b_update(const Params& P, const Sweep& Sx, const Sweep& Sy, const double* __restrict__ Win, double* __restrict__ Wout, double* __restrict__ Acc, Ctrl* ctrl, long long id)
 {
     if (ctrl->done) return;
+    if (STAGE == 1 && id == 0) {              // the end of the step (no thread of this launch reads these)
+        ctrl->t += ctrl->dt;
+        ctrl->last_dt = ctrl->dt;
+        ctrl->steps += 1;
+    }
     constexpr int NV = DIM + 2;
     const GridGeom& g = P.g;
     int rowsI = DIM == 2 ? g.ny : 1;
@@ -1116,45 +1218,18 @@ __device__ __forceinline__ int find_solve(const int* __restrict__ boff, int n, i
     const long long id = lblk_ * blockDim.x + threadIdx.x;                               \
     (void)nblk_; (void)id;
 
-__global__ void kb_ctrl(const SolveDesc* __restrict__ D, int n, int what, const double* __restrict__ tend)
-{
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    Ctrl* ctrl = D[s].ctrl;
-    if (what == 0) {                       // begin step
-        ctrl->dtmin_bits = 0x7FF0000000000000ull;
-        ctrl->cnt[0][0] = ctrl->cnt[0][1] = ctrl->cnt[1][0] = ctrl->cnt[1][1] = 0;
-    } else if (what == 1) {                // dt final (as k_dt_final, t_end per solver)
-        const Params& P = D[s].P;
-        double t_end = tend[s];
-        double tol = 1e-12 * (fabs(t_end) > 1.0 ? fabs(t_end) : 1.0);
-        double dt = P.fixed_dt > 0.0 ? P.fixed_dt : P.cfl * __longlong_as_double((long long)ctrl->dtmin_bits);
-        int done = ctrl->status != 0 || !(t_end - ctrl->t > tol);
-        if (!done && ctrl->t + dt > t_end) dt = t_end - ctrl->t;
-        if (!done && !(dt > 0.0 && dt < 1e300)) { ctrl->status = HGKS_ENONPHYSICAL; done = 1; }
-        ctrl->dt = dt;
-        ctrl->done = done;
-    } else {                               // end step
-        if (ctrl->done) return;
-        ctrl->t += ctrl->dt;
-        ctrl->last_dt = ctrl->dt;
-        ctrl->steps += 1;
-    }
-}
-
-__global__ void kb_dt(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
+__global__ void kb_dt(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, const double* __restrict__ tend)
 {
     HGKS_BATCH_BLOCK();
-    if (d.P.fixed_dt > 0.0) return;
-    b_dt(d.P, d.W, d.ctrl, d.h, id, nblk_ * blockDim.x);
+    if (!(d.P.fixed_dt > 0.0)) b_dt(d.P, d.W, d.ctrl, d.h, id, nblk_ * blockDim.x);
+    dt_finish(d.P, d.ctrl, tend[s_], (unsigned)nblk_);
 }
 
-__global__ void kb_ghost(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage, int axis)
+__global__ void kb_ghost(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
 {
     HGKS_BATCH_BLOCK();
-    double* W = stage == 0 ? d.W : d.Ws;
-    if (axis == 0) b_ghost_x(d.P, W, d.ctrl, id);
-    else b_ghost_y(d.P, W, d.ctrl, stage, id);
+    if (d.ctrl->done) return;
+    b_ghost(d.P, stage == 0 ? d.W : d.Ws, d.ctrl, stage, id);
 }
 
 template <int NV>
@@ -1176,6 +1251,19 @@ __global__ void kb_normal_ao(const SolveDesc* __restrict__ D, const int* __restr
 {
     HGKS_BATCH_SWEEP_BLOCK();
     b_normal_ao<NV>(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, id, nblk_ * blockDim.x);
+}
+
+template <int NV>
+__global__ void kb_normal_small(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+{
+    HGKS_BATCH_SWEEP_BLOCK();
+    b_normal_small<NV>(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, id);
+}
+
+__global__ void kb_tang_small(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+{
+    HGKS_BATCH_SWEEP_BLOCK();
+    tang_small_nl(d, dir, stage, id);
 }
 
 __global__ void kb_raw_tflags(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
@@ -1211,6 +1299,10 @@ __global__ void kb_update(const SolveDesc* __restrict__ D, const int* __restrict
     if (STAGE == 0) b_update<DIM, 0>(d.P, d.sw[0], d.sw[1], d.W, d.Ws, d.Acc, d.ctrl, id);
     else b_update<DIM, 1>(d.P, d.sw[0], d.sw[1], d.Ws, d.W, d.Acc, d.ctrl, id);
 }
+
+// Threads of the small-sweep reconstruction launches.
+inline long long normal_small_threads(const Sweep& S) { return (long long)S.nlines * S.nm * 2 * 4; }
+inline long long tang_small_threads(const Sweep& S) { return (long long)S.nt * S.nm * 16; }
 
 inline unsigned int blocks_for(long long n, int tpb) { return (unsigned int)((n + tpb - 1) / tpb); }
 
@@ -1339,9 +1431,11 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
     const SolveDesc* D = s->d_self;
     constexpr int NV = DIM + 2;
     const int sms = device_sm_count();
-    auto pair = [&](auto blocks, unsigned int* nb) {
-        nb[0] = blocks(s->sw[0]);
-        nb[1] = DIM == 2 ? blocks(s->sw[1]) : 0u;
+    // nb: the blocks of each sweep, none for a sweep of the other size class; returns their sum
+    enum { LARGE = 0, SMALL = 1, ALL = 2 };
+    unsigned int nb[2];
+    auto pair = [&](int which, auto blocks) {
+        for (int d = 0; d < 2; d++) nb[d] = d < DIM && (which == ALL || s->sw[d].small == which) ? blocks(s->sw[d]) : 0u;
         return nb[0] + nb[1];
     };
     // the compacted WENO-AO passes: a grid for 4 lanes per possible item, capped at 8 blocks per SM
@@ -1349,32 +1443,24 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
         unsigned int b = blocks_for(maxn, 128);
         return b > (unsigned)(sms * 8) ? (unsigned)(sms * 8) : b;
     };
-    unsigned int nb[2];
-    timed(s, KC_RAWN, 1, [&] {
-        unsigned int g = pair([](const Sweep& S) { return blocks_for((long long)S.nlines * (S.nn + 4), TPB); }, nb);
-        k_raw_nflags<NV><<<g, TPB, 0, st>>>(D, (int)nb[0], stage);
-    });
-    timed(s, KC_NORMAL, 1, [&] {
-        unsigned int g = pair([](const Sweep& S) { return blocks_for((long long)S.nlines * S.nm, TPB); }, nb);
-        k_normal<NV><<<g, TPB, 0, st>>>(D, (int)nb[0], stage);
-    });
-    timed(s, KC_NORMAL_AO, 1, [&] {
-        unsigned int g = pair([&](const Sweep& S) { return ao_blocks((long long)S.nlines * S.nm * 2 * 4); }, nb);
-        k_normal_ao<NV><<<g, 128, 0, st>>>(D, (int)nb[0], stage);
-    });
+    unsigned int g;
+    if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for((long long)S.nlines * (S.nn + 4), TPB); })))
+        timed(s, KC_RAWN, 1, [&] { k_raw_nflags<NV><<<g, TPB, 0, st>>>(D, (int)nb[0], stage); });
+    if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for((long long)S.nlines * S.nm, TPB); })))
+        timed(s, KC_NORMAL, 1, [&] { k_normal<NV><<<g, TPB, 0, st>>>(D, (int)nb[0], stage); });
+    if ((g = pair(LARGE, [&](const Sweep& S) { return ao_blocks((long long)S.nlines * S.nm * 2 * 4); })))
+        timed(s, KC_NORMAL_AO, 1, [&] { k_normal_ao<NV><<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
+    if ((g = pair(SMALL, [](const Sweep& S) { return blocks_for(normal_small_threads(S), 128); })))
+        timed(s, KC_NORMAL, 1, [&] { k_normal_small<NV><<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
     if constexpr (DIM == 2) {
-        timed(s, KC_RAWT, 1, [&] {
-            unsigned int g = pair([](const Sweep& S) { return blocks_for(raw_t_threads(S), TPB); }, nb);
-            k_raw_tflags<<<g, TPB, 0, st>>>(D, (int)nb[0]);
-        });
-        timed(s, KC_TANG, 1, [&] {
-            unsigned int g = pair([](const Sweep& S) { return blocks_for((long long)S.nt * S.nm * S.tlanes, TPB); }, nb);
-            k_tang<<<g, TPB, 0, st>>>(D, (int)nb[0], stage);
-        });
-        timed(s, KC_TANG_AO, 1, [&] {
-            unsigned int g = pair([&](const Sweep& S) { return ao_blocks((long long)S.nt * S.nm * 4 * 4); }, nb);
-            k_tang_ao<<<g, 128, 0, st>>>(D, (int)nb[0], stage);
-        });
+        if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for(raw_t_threads(S), TPB); })))
+            timed(s, KC_RAWT, 1, [&] { k_raw_tflags<<<g, TPB, 0, st>>>(D, (int)nb[0]); });
+        if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for((long long)S.nt * S.nm, TPB); })))
+            timed(s, KC_TANG, 1, [&] { k_tang<<<g, TPB, 0, st>>>(D, (int)nb[0], stage); });
+        if ((g = pair(LARGE, [&](const Sweep& S) { return ao_blocks((long long)S.nt * S.nm * 4 * 4); })))
+            timed(s, KC_TANG_AO, 1, [&] { k_tang_ao<<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
+        if ((g = pair(SMALL, [](const Sweep& S) { return blocks_for(tang_small_threads(S), 128); })))
+            timed(s, KC_TANG, 1, [&] { k_tang_small<<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
     }
     if (s->capture) {
         for (int d = 0; d < DIM; d++) {
@@ -1385,7 +1471,7 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
         }
     }
     timed(s, KC_FLUX, 1, [&] {
-        unsigned int g = pair([](const Sweep& S) { return blocks_for(flux_threads(DIM, (long long)S.nt * S.nm), 64); }, nb);
+        g = pair(ALL, [](const Sweep& S) { return blocks_for(flux_threads(DIM, (long long)S.nt * S.nm), 64); });
         const int n0 = (int)nb[0];
         if (P.fc.prfix != 0.0) {
             if (stage == 0) k_flux<DIM, 0, true><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
@@ -1403,12 +1489,8 @@ static void enqueue_stage(hgks_solver* s, int stage)
     NvtxRange range(stage == 0 ? "S2O4 stage 1" : "S2O4 stage 2");
     const Params& P = s->P;
     cudaStream_t st = s->stream;
-    double* Win = stage == 0 ? s->W : s->Ws;
-    timed(s, KC_GHOST, DIM == 2 ? 2 : 1, [&] {
-        int rowsI = DIM == 2 ? P.g.ny : 1;
-        k_ghost_x<<<blocks_for((long long)P.g.nv * rowsI * NG * 2, TPB), TPB, 0, st>>>(P, Win, s->ctrl);
-        if (DIM == 2) k_ghost_y<<<blocks_for((long long)P.g.nv * (P.g.nx + 2 * NG) * NG * 2, TPB), TPB, 0, st>>>(P, Win, s->ctrl, stage);
-    });
+    if (stage == 1)
+        timed(s, KC_GHOST, 1, [&] { k_ghost<<<blocks_for(ghost_threads(P.g), TPB), TPB, 0, st>>>(P, s->Ws, s->ctrl); });
     enqueue_sweeps<DIM>(s, stage);
     timed(s, KC_UPDATE, 1, [&] {
         long long n = (long long)(DIM == 2 ? P.g.ny : 1) * P.g.nx;
@@ -1422,34 +1504,32 @@ cudaError_t launch_step(hgks_solver* s, double t_end)
     NvtxRange range("hgks_step");
     const Params& P = s->P;
     cudaStream_t st = s->stream;
-    double tol = 1e-12 * (fabs(t_end) > 1.0 ? fabs(t_end) : 1.0);
-    double h = P.g.dim == 2 ? (P.g.dx < P.g.dy ? P.g.dx : P.g.dy) : P.g.dx;
-    timed(s, KC_DT, P.fixed_dt > 0.0 ? 2 : 3, [&] {
-        k_begin_step<<<1, 1, 0, st>>>(s->ctrl);
+    const double h = P.g.dim == 2 ? (P.g.dx < P.g.dy ? P.g.dx : P.g.dy) : P.g.dx;
+    timed(s, KC_DT, 1, [&] {
+        unsigned int nb = 1;
         if (!(P.fixed_dt > 0.0)) {
-            long long n = (long long)(P.g.dim == 2 ? P.g.ny : 1) * P.g.nx;
-            unsigned int b = blocks_for(n, TPB);
-            unsigned int cap = (unsigned)device_sm_count() * 4;
-            if (b > cap) b = cap;
-            k_dt<<<b, TPB, 0, st>>>(P, s->W, s->ctrl, h);
+            nb = blocks_for((long long)(P.g.dim == 2 ? P.g.ny : 1) * P.g.nx, TPB);
+            const unsigned int cap = (unsigned)device_sm_count() * 4;
+            if (nb > cap) nb = cap;
         }
-        k_dt_final<<<1, 1, 0, st>>>(s->ctrl, P.cfl, P.fixed_dt, t_end, tol);
+        k_dt_ghost<<<nb + blocks_for(ghost_threads(P.g), TPB), TPB, 0, st>>>(P, s->W, s->ctrl, h, t_end, (int)nb);
     });
     if (P.g.dim == 2) { enqueue_stage<2>(s, 0); enqueue_stage<2>(s, 1); }
     else { enqueue_stage<1>(s, 0); enqueue_stage<1>(s, 1); }
-    timed(s, KC_MISC, 1, [&] { k_end_step<<<1, 1, 0, st>>>(s->ctrl); });
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- host: batched step
 const int kBatchTpbDefault[BK_COUNT] = {
-    32, 256, 256, 256,        // ctrl, dt, ghost x, ghost y
+    256, 256,                 // dt, ghost cells
     256,                      // raw normal flags
     256,                      // normal reconstruction
     128,                      // normal WENO-AO
+    128,                      // normal reconstruction of small sweeps
     256,                      // raw tangential flags
-    256,                      // tangential reconstruction
+    256,                      // tangential flags
     128,                      // tangential WENO-AO
+    128,                      // tangential reconstruction of small sweeps
     128,                      // flux
     256                       // update
 };
@@ -1473,18 +1553,21 @@ static long long batch_unit_blocks(const SolveDesc& d, int dim, int c, int dir, 
     const Sweep& S = d.sw[dir];
     const long long cells = (long long)(dim == 2 ? g.ny : 1) * g.nx;
     if (batch_sweep_class(c) && dir >= dim) return 0;          // 1D: no y sweep
+    if (dim == 1 && c >= BK_RAWT && c <= BK_TSMALL) return 0;
+    if (S.small && (c == BK_RAWN || c == BK_NORMAL || c == BK_NAO || c == BK_RAWT || c == BK_TANG || c == BK_TAO)) return 0;
+    if (!S.small && (c == BK_NSMALL || c == BK_TSMALL)) return 0;
     long long b = 0;
     switch (c) {
-        case BK_CTRL: return 0;
         case BK_DT: b = (cells + (long long)t * 8 - 1) / ((long long)t * 8); break;
-        case BK_GHX: b = blocks_for((long long)g.nv * (dim == 2 ? g.ny : 1) * NG * 2, t); break;
-        case BK_GHY: if (dim != 2) return 0; b = blocks_for((long long)g.nv * (g.nx + 2 * NG) * NG * 2, t); break;
+        case BK_GHOST: b = blocks_for(ghost_threads(g), t); break;
         case BK_RAWN: b = blocks_for((long long)S.nlines * (S.nn + 4), t); break;
         case BK_NORMAL: b = blocks_for((long long)S.nlines * S.nm, t); break;
         case BK_NAO: b = blocks_for((long long)S.nlines * S.nm * 2 * 4, t * 8); break;
-        case BK_RAWT: if (dim != 2) return 0; b = blocks_for(raw_t_threads(S), t); break;
-        case BK_TANG: if (dim != 2) return 0; b = blocks_for((long long)S.nt * S.nm * S.tlanes, t); break;
-        case BK_TAO: if (dim != 2) return 0; b = blocks_for((long long)S.nt * S.nm * 4 * 4, t * 8); break;
+        case BK_NSMALL: b = blocks_for(normal_small_threads(S), t); break;
+        case BK_RAWT: b = blocks_for(raw_t_threads(S), t); break;
+        case BK_TANG: b = blocks_for((long long)S.nt * S.nm, t); break;
+        case BK_TAO: b = blocks_for((long long)S.nt * S.nm * 4 * 4, t * 8); break;
+        case BK_TSMALL: b = blocks_for(tang_small_threads(S), t); break;
         case BK_FLUX: b = blocks_for(flux_threads(dim, (long long)S.nt * S.nm), t); break;
         case BK_UPD: b = blocks_for(cells, t); break;
     }
@@ -1510,7 +1593,7 @@ void batch_plan(const std::vector<const SolveDesc*>& descs, int dim, const int* 
                       : batch_unit_blocks(*descs[u], dim, c, 0, tpb[c]);
         }
         bo[units] = (int)acc;
-        plan.nblk[c] = c == BK_CTRL ? (int)blocks_for(n, tpb[c]) : (int)acc;
+        plan.nblk[c] = (int)acc;
     }
 }
 
@@ -1524,45 +1607,32 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
     auto mark = [&](int c, int which) { if (ev) cudaEventRecord(ev[2 * c + which], st); };
     auto grid = [&](int c) { return (unsigned int)plan.nblk[c]; };
     auto tp = [&](int c) { return plan.tpb[c]; };
-    const int tc = plan.tpb[BK_CTRL];
-    kb_ctrl<<<grid(BK_CTRL), tc, 0, st>>>(dd, n, 0, dtend);
     mark(BK_DT, 0);
-    if (grid(BK_DT)) kb_dt<<<grid(BK_DT), tp(BK_DT), 0, st>>>(dd, bo(BK_DT), n);
+    kb_dt<<<grid(BK_DT), tp(BK_DT), 0, st>>>(dd, bo(BK_DT), n, dtend);
     mark(BK_DT, 1);
-    kb_ctrl<<<grid(BK_CTRL), tc, 0, st>>>(dd, n, 1, dtend);
     for (int stage = 0; stage < 2; stage++) {
-        mark(BK_GHX, 0);
-        kb_ghost<<<grid(BK_GHX), tp(BK_GHX), 0, st>>>(dd, bo(BK_GHX), n, stage, 0);
-        mark(BK_GHX, 1);
-        if (dim == 2) {
-            mark(BK_GHY, 0);
-            kb_ghost<<<grid(BK_GHY), tp(BK_GHY), 0, st>>>(dd, bo(BK_GHY), n, stage, 1);
-            mark(BK_GHY, 1);
-        }
-        // every sweep class: one launch over both sweeps of every solver
-        mark(BK_RAWN, 0);
-        if (dim == 2) kb_raw_nflags<4><<<grid(BK_RAWN), tp(BK_RAWN), 0, st>>>(dd, bo(BK_RAWN), n, stage);
-        else kb_raw_nflags<3><<<grid(BK_RAWN), tp(BK_RAWN), 0, st>>>(dd, bo(BK_RAWN), n, stage);
-        mark(BK_RAWN, 1);
-        mark(BK_NORMAL, 0);
-        if (dim == 2) kb_normal<4><<<grid(BK_NORMAL), tp(BK_NORMAL), 0, st>>>(dd, bo(BK_NORMAL), n, stage);
-        else kb_normal<3><<<grid(BK_NORMAL), tp(BK_NORMAL), 0, st>>>(dd, bo(BK_NORMAL), n, stage);
-        mark(BK_NORMAL, 1);
-        mark(BK_NAO, 0);
-        if (dim == 2) kb_normal_ao<4><<<grid(BK_NAO), tp(BK_NAO), 0, st>>>(dd, bo(BK_NAO), n, stage);
-        else kb_normal_ao<3><<<grid(BK_NAO), tp(BK_NAO), 0, st>>>(dd, bo(BK_NAO), n, stage);
-        mark(BK_NAO, 1);
-        if (dim == 2) {
-            mark(BK_RAWT, 0);
-            kb_raw_tflags<<<grid(BK_RAWT), tp(BK_RAWT), 0, st>>>(dd, bo(BK_RAWT), n);
-            mark(BK_RAWT, 1);
-            mark(BK_TANG, 0);
-            kb_tang<<<grid(BK_TANG), tp(BK_TANG), 0, st>>>(dd, bo(BK_TANG), n, stage);
-            mark(BK_TANG, 1);
-            mark(BK_TAO, 0);
-            kb_tang_ao<<<grid(BK_TAO), tp(BK_TAO), 0, st>>>(dd, bo(BK_TAO), n, stage);
-            mark(BK_TAO, 1);
-        }
+        mark(BK_GHOST, 0);
+        kb_ghost<<<grid(BK_GHOST), tp(BK_GHOST), 0, st>>>(dd, bo(BK_GHOST), n, stage);
+        mark(BK_GHOST, 1);
+        // every sweep class: one launch over both sweeps of every solver it applies to
+        auto sweep = [&](int c, auto launch) {
+            if (!grid(c)) return;
+            mark(c, 0);
+            launch();
+            mark(c, 1);
+        };
+#define HGKS_BY_DIM(kernel, c) sweep(c, [&] {                                                          \
+            if (dim == 2) kernel<4><<<grid(c), tp(c), 0, st>>>(dd, bo(c), n, stage);                      \
+            else kernel<3><<<grid(c), tp(c), 0, st>>>(dd, bo(c), n, stage); })
+        HGKS_BY_DIM(kb_raw_nflags, BK_RAWN);
+        HGKS_BY_DIM(kb_normal, BK_NORMAL);
+        HGKS_BY_DIM(kb_normal_ao, BK_NAO);
+        HGKS_BY_DIM(kb_normal_small, BK_NSMALL);
+#undef HGKS_BY_DIM
+        sweep(BK_RAWT, [&] { kb_raw_tflags<<<grid(BK_RAWT), tp(BK_RAWT), 0, st>>>(dd, bo(BK_RAWT), n); });
+        sweep(BK_TANG, [&] { kb_tang<<<grid(BK_TANG), tp(BK_TANG), 0, st>>>(dd, bo(BK_TANG), n, stage); });
+        sweep(BK_TAO, [&] { kb_tang_ao<<<grid(BK_TAO), tp(BK_TAO), 0, st>>>(dd, bo(BK_TAO), n, stage); });
+        sweep(BK_TSMALL, [&] { kb_tang_small<<<grid(BK_TSMALL), tp(BK_TSMALL), 0, st>>>(dd, bo(BK_TSMALL), n, stage); });
         mark(BK_FLUX, 0);
         const int tf = tp(BK_FLUX);
         if (dim == 2) {
@@ -1584,7 +1654,6 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
         }
         mark(BK_UPD, 1);
     }
-    kb_ctrl<<<grid(BK_CTRL), tc, 0, st>>>(dd, n, 3, dtend);
     return cudaGetLastError();
 }
 

@@ -150,9 +150,8 @@ __device__ __forceinline__ ex xscale(ex x)
 // and Z1 = 17 zeta1 dx^2 (Eq. (24): abar2 = D/34).  Step 2: xbar = -abar1/(2 abar2) with
 // abar1 = -N/10, N = (2Q_{i-2}+Q_{i-1}) - (2Q_{i+2}+Q_{i+1}); inside iff |xbar| <= 5/2.
 // Step 3: xhat from the conservative 3-cell quadratic; non-troubled iff |xbar - xhat| <= 1/4.
-__device__ __forceinline__ int indicator_exact(const double* q, double Z1)
+__device__ __forceinline__ int indicator_exact(ex q0, ex q1, ex q2, ex q3, ex q4, double Z1)
 {
-    ex q0(q[0]), q1(q[1]), q2(q[2]), q3(q[3]), q4(q[4]);
     ex D = xfma(ex(-10.0), q2, xfma(ex(4.0), q0, q1) + xfma(ex(4.0), q4, q3));
     if (fabs(D.v) <= Z1) return 0;
     ex N = xfma(ex(2.0), q0, q1) - xfma(ex(2.0), q4, q3);
@@ -169,6 +168,11 @@ __device__ __forceinline__ int indicator_exact(const double* q, double Z1)
 }
 
 #if defined(__CUDACC__)
+__device__ __noinline__ int indicator_exact_nl(ex q0, ex q1, ex q2, ex q3, ex q4, double Z1)
+{
+    return indicator_exact(q0, q1, q2, q3, q4, Z1);
+}
+
 // The same decision with few or no FP64 instructions (a comparison and a conversion occupy the FP64
 // pipe as long as an addition), f[j] = q[j] truncated to FP32 (fixed::to_float).  Each test is first taken in
 // FP32 with a margin above its rounding errors; only a test that falls inside its margin is decided by
@@ -182,6 +186,9 @@ __device__ __forceinline__ int indicator_exact(const double* q, double Z1)
 // The exact chain takes 5 FP64 slots of the pipe on smooth data and, behind Step 1, four IEEE
 // divisions more, where one troubled lane holds up its warp.  Raw flags per step at 1024^2: normal
 // 253 -> 160 us, tangential 702 -> 251 us (with the shared row loads of b_raw_tflags_x1).
+// CALL: the exact chain behind a call, where three windows a thread would otherwise unroll it three times
+// (a call costs the large sweeps' tangential flags 20 %, 254 -> 300 us at 1024^2).
+template <bool CALL>
 __device__ __forceinline__ int indicator_raw(const double* q, const float* f, double Z1)
 {
     const float m = fmaxf(fmaxf(fmaxf(fabsf(f[0]), fabsf(f[1])), fmaxf(fabsf(f[3]), fabsf(f[4]))), fabsf(f[2]));
@@ -205,7 +212,7 @@ __device__ __forceinline__ int indicator_raw(const double* q, const float* f, do
         if (gap < 0.25f - tol) return 0;
         if (gap > 0.25f + tol) return 1;
     }
-    return indicator_exact(q, Z1);
+    return CALL ? indicator_exact_nl(q0, q1, q2, q3, q4, Z1) : indicator_exact(q0, q1, q2, q3, q4, Z1);
 }
 #endif
 
