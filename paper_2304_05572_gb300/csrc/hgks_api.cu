@@ -671,10 +671,10 @@ extern "C" int hgks_batch_step(hgks_batch* b, const double* t_end, int nsteps, i
         for (int k = 0; k < 3 && left > 0; k++) {
             int tpb[BK_COUNT];
             for (int c = 0; c < BK_COUNT; c++) {
-                bool heavy_regs = c == BK_FLUX || c == BK_NAO || c == BK_TAO || c == BK_NSMALL || c == BK_TSMALL;
+                // the flux kernels' warps share segments: fixed block sizes
+                if (c >= BK_FLUX && c <= BK_FSMALL_PR) { tpb[c] = kBatchTpbDefault[c]; continue; }
+                bool heavy_regs = c == BK_NAO || c == BK_TAO || c == BK_NSMALL || c == BK_TSMALL;
                 tpb[c] = heavy_regs ? cand_small[k] : cand_big[k];
-                // a flux block keeps 224 bytes of shared memory a thread: 128 threads stay below 48 KB
-                if (c == BK_FLUX && tpb[c] > 128) tpb[c] = 128;
             }
             int st = batch_upload_plan(b, tpb);
             if (st != HGKS_OK) return st;

@@ -93,14 +93,15 @@ struct SolveDesc {
 };
 
 // Kernel classes of a batched step, one launch each per stage.  The sweep classes (BK_RAWN to
-// BK_FLUX) cover both sweeps of every solver: their units are (solver s, sweep d), unit 2 s + d.
+// BK_FSMALL_PR) cover both sweeps of every solver: their units are (solver s, sweep d), unit 2 s + d.
 enum BatchClass {
     BK_DT = 0, BK_GHOST,
-    BK_RAWN, BK_NORMAL, BK_NAO, BK_NSMALL, BK_RAWT, BK_TANG, BK_TAO, BK_TSMALL, BK_FLUX,
+    BK_RAWN, BK_NORMAL, BK_NAO, BK_NSMALL, BK_RAWT, BK_TANG, BK_TAO, BK_TSMALL,
+    BK_FLUX, BK_FLUX_PR, BK_FSMALL, BK_FSMALL_PR,
     BK_UPD, BK_COUNT
 };
 
-inline bool batch_sweep_class(int c) { return c >= BK_RAWN && c <= BK_FLUX; }
+inline bool batch_sweep_class(int c) { return c >= BK_RAWN && c <= BK_FSMALL_PR; }
 
 struct BatchPlan {
     int n = 0, dim = 0;

@@ -11,6 +11,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <cstdio>
+#include <type_traits>
 
 #include "hgks_internal.h"
 #include "hgks_math.cuh"
@@ -973,17 +974,17 @@ __device__ __forceinline__ void side_pair(const Params& P, const Sweep& S, int s
 }
 
 // State Wv, normal derivative Wn and tangential derivative Wt (2D) of one side of segment o at Gauss point
-// g: in 1D from the line buffer, in 2D from the Gauss-point buffer (small sweeps, where k_tang and
-// k_tang_ao reconstructed every pass) or from shared memory (large sweeps, side_pair).
+// g: 1D from the line buffer; 2D from shared memory (large sweeps, side_pair) or, x = nullptr, from the
+// Gauss-point buffer (small sweeps, where every pass was reconstructed before).
 template <int DIM>
-__device__ __forceinline__ void side_states(const Params& P, const Sweep& S, int side, int g, long long o, const double* x, int stride,
+__device__ __forceinline__ void side_states(const Sweep& S, int side, int g, long long o, const double* x, int stride,
                                             double* Wv, double* Wn, double* Wt)
 {
     constexpr int NV = DIM + 2;
     if constexpr (DIM == 2) {
         const long long per = (long long)S.nt * S.nm;
-        const double* gp = S.gp + (long long)((g * 6 + 3 * side) * 4) * per + o;
-        if (S.small) {
+        if (!x) {
+            const double* gp = S.gp + (long long)((g * 6 + 3 * side) * 4) * per + o;
 #pragma unroll
             for (int k = 0; k < NV; k++) {
                 Wv[k] = ldc(gp + (long long)k * per, S);
@@ -1009,6 +1010,19 @@ __device__ __forceinline__ void side_states(const Params& P, const Sweep& S, int
     }
 }
 
+// The segment's fluxes [output][component][segment].
+template <int DIM, int STAGE>
+__device__ __forceinline__ void store_flux(const Sweep& S, long long o, const double* o0, const double* o1)
+{
+    const long long per = (long long)S.nt * S.nm;
+#pragma unroll
+    for (int k = 0; k < DIM + 2; k++) {
+        const int gk = S.perm[k];
+        stc(S.flux + (long long)gk * per + o, o0[k], S);
+        if (STAGE == 0) stc(S.flux + (long long)(DIM + 2 + gk) * per + o, o1[k], S);
+    }
+}
+
 template <int DIM, int STAGE, bool PRFIX>
 __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ctrl, long long id)
 {
@@ -1030,14 +1044,12 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     const int stride = blockDim.x;
     const int pair0 = threadIdx.x & ~32;         // this thread's lane in the pair's first warp
     if constexpr (DIM == 2) {
-        // large sweeps: warp 0 of the pair reconstructs the left side at both Gauss points, warp 1 the right
-        // side, and they exchange through shared memory: every line value is loaded and converted once, and
-        // the two points share their products (with the products in FP64 and each warp reconstructing both
-        // sides at its own point the launch took 5.04 ms at 1024^2, so 4.18 ms)
-        if (!S.small) {
-            if (valid) side_pair(P, S, g, o, flux_sh + threadIdx.x, stride);
-            __syncthreads();
-        }
+        // warp 0 of the pair reconstructs the left side at both Gauss points, warp 1 the right side, and they
+        // exchange through shared memory: every line value is loaded and converted once, and the two points
+        // share their products (with the products in FP64 and each warp reconstructing both sides at its own
+        // point the launch took 5.04 ms at 1024^2, so 4.18 ms)
+        if (valid) side_pair(P, S, g, o, flux_sh + threadIdx.x, stride);
+        __syncthreads();
     }
     if (valid) {
     // one side after the other: only the side at work holds its states and slopes in registers
@@ -1046,13 +1058,13 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     bool ok;
     {
         double Wv[NV], Wn[NV], Wt[NV];
-        side_states<DIM>(P, S, 0, g, o, flux_sh + pair0, stride, Wv, Wn, Wt);
-        ok = flux_side<DIM, PRFIX, true>(P.fc, Wv, Wn, Wt, sums, pl);
+        side_states<DIM>(S, 0, g, o, flux_sh + pair0, stride, Wv, Wn, Wt);
+        ok = flux_side<DIM, PRFIX, true>(P.fc, Wv, Wn, Wt, true, sums, pl);
     }
     if (ok) {
         double Wv[NV], Wn[NV], Wt[NV];
-        side_states<DIM>(P, S, 1, g, o, flux_sh + pair0 + 32, stride, Wv, Wn, Wt);
-        ok = flux_side<DIM, PRFIX, false>(P.fc, Wv, Wn, Wt, sums, pr);
+        side_states<DIM>(S, 1, g, o, flux_sh + pair0 + 32, stride, Wv, Wn, Wt);
+        ok = flux_side<DIM, PRFIX, false>(P.fc, Wv, Wn, Wt, false, sums, pr);
     }
     if (ok) ok = flux_finish<DIM, STAGE, PRFIX>(P.fc, sums, pl, pr, ctrl->dt, o0, o1);
     if (!ok) {
@@ -1065,8 +1077,7 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     }
     }
     // the segment flux (Gauss weights 1/2): the Gauss point 1 warp hands its fluxes to its partner
-    // through shared memory; stored per segment as [output][component][segment]
-    constexpr int NO = STAGE == 0 ? 2 : 1;
+    // through shared memory
     if constexpr (DIM == 2) {
         // [output component][lane pair]
         double* pair = flux_sh + kFluxSideDoubles * stride + ((threadIdx.x >> 6) << 5) + (threadIdx.x & 31);
@@ -1088,13 +1099,96 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     } else {
         if (!valid) return;
     }
-#pragma unroll
-    for (int k = 0; k < NV; k++) {
-        const int gk = S.perm[k];
-        stc(S.flux + (long long)(0 * NV + gk) * per + o, o0[k], S);
-        if (NO == 2) stc(S.flux + (long long)(1 * NV + gk) * per + o, o1[k], S);
-    }
+    store_flux<DIM, STAGE>(S, o, o0, o1);
 }
+
+// Small sweeps: the two sides of a Gauss point on two warps, so that a thread's chain is one side (about 190
+// FP64 instructions) and, on the left side's warp, the sums' completion (about 150) instead of two sides and
+// the completion.  2D: 4 warps on the same 32 segments (side = warp & 1, Gauss point = warp >> 1 of the 4);
+// 1D: 2 warps.  The right side's sums and the second point's fluxes go through shared memory, one column
+// per left thread.  Per launch: 200 cells in 1D 18 -> 15 us, 48 x 48 29 -> 21, 200 x 100 (Prandtl fix) 124 -> 111.
+template <int DIM, bool PRFIX>
+__host__ __device__ constexpr int flux_sums() { return (PRFIX ? 8 : 6) * (DIM + 2) + 1; }
+
+inline size_t flux_small_smem(int dim, bool prfix, int threads)
+{
+    const int n = dim == 2 ? (prfix ? flux_sums<2, true>() : flux_sums<2, false>())
+                           : (prfix ? flux_sums<1, true>() : flux_sums<1, false>());
+    return (size_t)threads / 2 * n * sizeof(double);
+}
+
+template <int DIM, int STAGE, bool PRFIX>
+__device__ __forceinline__ void b_flux_small(const Params& P, const Sweep& S, Ctrl* ctrl, long long id)
+{
+    if (ctrl->done) return;                   // the same for every thread of a block
+    constexpr int NV = DIM + 2, NS = flux_sums<DIM, PRFIX>(), NVEC = PRFIX ? 8 : 6;
+    const long long warp = id >> 5;
+    const int side = (int)(warp & 1), g = DIM == 2 ? (int)(warp >> 1) & 1 : 0;
+    const long long o = ((warp >> DIM) << 5) + (id & 31);
+    const bool valid = o < (long long)S.nt * S.nm;
+    const int cols = blockDim.x >> 1;
+    extern __shared__ double flux_sh[];
+    double* col = flux_sh + ((threadIdx.x >> 6) << 5) + (threadIdx.x & 31);
+    FluxSums<DIM> q;
+    double* vec[8] = {q.Wc, q.Wx, q.Wy, q.S4, q.S5, q.S6n, q.D5, q.D6n};
+    const double nan = __longlong_as_double(0x7FF8000000000000LL);
+    double p = 0.0;
+    bool ok = false;
+    if (valid) {
+        double Wv[NV], Wn[NV], Wt[NV];
+        side_states<DIM>(S, side, g, o, nullptr, 0, Wv, Wn, Wt);
+        ok = flux_side<DIM, PRFIX, true>(P.fc, Wv, Wn, Wt, side == 0, q, p);
+        if (side == 1) {
+            if (!ok) q.Wc[0] = nan;             // the completion finds the state non-physical
+#pragma unroll
+            for (int j = 0; j < NVEC; j++) {
+                if ((DIM == 1 && j == 2) || (j >= 3 && P.fc.tau_zero)) continue;
+#pragma unroll
+                for (int k = 0; k < NV; k++) col[(j * NV + k) * cols] = vec[j][k];
+            }
+            col[(NS - 1) * cols] = p;
+        }
+    }
+    __syncthreads();
+    double o0[NV], o1[NV];
+    if (valid && side == 0) {
+        const double pr = col[(NS - 1) * cols];
+#pragma unroll
+        for (int j = 0; j < NVEC; j++) {
+            if ((DIM == 1 && j == 2) || (j >= 3 && P.fc.tau_zero)) continue;
+#pragma unroll
+            for (int k = 0; k < NV; k++) vec[j][k] += col[(j * NV + k) * cols];
+        }
+        if (ok) ok = flux_finish<DIM, STAGE, PRFIX>(P.fc, q, p, pr, ctrl->dt, o0, o1);
+        if (!ok) {
+            // the status is latched and the flux is a NaN (see b_flux)
+            ctrl->status = HGKS_ENONPHYSICAL;
+#pragma unroll
+            for (int k = 0; k < NV; k++) { o0[k] = nan; o1[k] = nan; }
+        }
+        if (DIM == 2 && g == 1) {
+#pragma unroll
+            for (int k = 0; k < NV; k++) {
+                col[k * cols] = o0[k];
+                if (STAGE == 0) col[(NV + k) * cols] = o1[k];
+            }
+        }
+    }
+    if constexpr (DIM == 2) {
+        __syncthreads();
+        if (g == 0 && side == 0 && valid) {
+            const double* c1 = col + 32;          // Gauss point 1 of the same segment
+#pragma unroll
+            for (int k = 0; k < NV; k++) {
+                o0[k] = fma(0.5, o0[k], 0.5 * c1[k * cols]);
+                if (STAGE == 0) o1[k] = fma(0.5, o1[k], 0.5 * c1[(NV + k) * cols]);
+            }
+        }
+    }
+    if (g == 0 && side == 0 && valid) store_flux<DIM, STAGE>(S, o, o0, o1);
+}
+
+inline long long flux_small_threads(int dim, long long per) { return (dim == 2 ? 4 : 2) * ((per + 31) / 32) * 32; }
 
 // Threads of a 2D flux launch for a sweep of `per` segments: two Gauss points per segment, the
 // segments padded to whole warps (see b_flux).
@@ -1115,6 +1209,21 @@ __global__ void __launch_bounds__(64, 4) k_flux(const SolveDesc* __restrict__ D,
 {
     const SweepBlock b = sweep_block(nb0);
     flux_nl<DIM, STAGE, PRFIX>(*D, b.dir, b.id);
+}
+
+template <int DIM, int STAGE, bool PRFIX>
+__device__ __noinline__ void flux_small_nl(const SolveDesc& d, int dir, long long id)
+{
+    b_flux_small<DIM, STAGE, PRFIX>(d.P, d.sw[dir], d.ctrl, id);
+}
+
+constexpr int kFluxSmallBlock = 128;
+
+template <int DIM, int STAGE, bool PRFIX>
+__global__ void __launch_bounds__(kFluxSmallBlock) k_flux_small(const SolveDesc* __restrict__ D, int nb0)
+{
+    const SweepBlock b = sweep_block(nb0);
+    flux_small_nl<DIM, STAGE, PRFIX>(*D, b.dir, b.id);
 }
 
 // Stage 0: W* = W^n - dF(dt/2)/dx - dG(dt/2)/dy (Eq. (19)), Acc = W^n - d(dt F^n + dt^2/6 dF^n)/dx - ...
@@ -1284,12 +1393,18 @@ __global__ void kb_tang_ao(const SolveDesc* __restrict__ D, const int* __restric
     tang_ao_nl(d, dir, stage, id, nblk_ * blockDim.x);
 }
 
-template <int DIM, int STAGE>
-__global__ void __launch_bounds__(128) kb_flux(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
+template <int DIM, int STAGE, bool PRFIX>
+__global__ void __launch_bounds__(64, 4) kb_flux(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
 {
     HGKS_BATCH_SWEEP_BLOCK();
-    if (d.P.fc.prfix != 0.0) flux_nl<DIM, STAGE, true>(d, dir, id);
-    else flux_nl<DIM, STAGE, false>(d, dir, id);
+    flux_nl<DIM, STAGE, PRFIX>(d, dir, id);
+}
+
+template <int DIM, int STAGE, bool PRFIX>
+__global__ void __launch_bounds__(kFluxSmallBlock) kb_flux_small(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
+{
+    HGKS_BATCH_SWEEP_BLOCK();
+    flux_small_nl<DIM, STAGE, PRFIX>(d, dir, id);
 }
 
 template <int DIM, int STAGE>
@@ -1470,17 +1585,22 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
             if (DIM == 2) cudaMemcpyAsync(s->cap[stage][d][1], S.flagT, (size_t)S.nt * S.nm, cudaMemcpyDeviceToDevice, st);
         }
     }
-    timed(s, KC_FLUX, 1, [&] {
-        g = pair(ALL, [](const Sweep& S) { return blocks_for(flux_threads(DIM, (long long)S.nt * S.nm), 64); });
-        const int n0 = (int)nb[0];
-        if (P.fc.prfix != 0.0) {
-            if (stage == 0) k_flux<DIM, 0, true><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
-            else k_flux<DIM, 1, true><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
-        } else {
-            if (stage == 0) k_flux<DIM, 0, false><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
-            else k_flux<DIM, 1, false><<<g, 64, flux_smem(DIM, 64), st>>>(D, n0);
-        }
-    });
+    auto flux = [&](auto prfix) {
+        constexpr bool PR = decltype(prfix)::value;
+        if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for(flux_threads(DIM, (long long)S.nt * S.nm), 64); })))
+            timed(s, KC_FLUX, 1, [&] {
+                if (stage == 0) k_flux<DIM, 0, PR><<<g, 64, flux_smem(DIM, 64), st>>>(D, (int)nb[0]);
+                else k_flux<DIM, 1, PR><<<g, 64, flux_smem(DIM, 64), st>>>(D, (int)nb[0]);
+            });
+        constexpr int T = kFluxSmallBlock;
+        if ((g = pair(SMALL, [](const Sweep& S) { return blocks_for(flux_small_threads(DIM, (long long)S.nt * S.nm), T); })))
+            timed(s, KC_FLUX, 1, [&] {
+                if (stage == 0) k_flux_small<DIM, 0, PR><<<g, T, flux_small_smem(DIM, PR, T), st>>>(D, (int)nb[0]);
+                else k_flux_small<DIM, 1, PR><<<g, T, flux_small_smem(DIM, PR, T), st>>>(D, (int)nb[0]);
+            });
+    };
+    if (P.fc.prfix != 0.0) flux(std::true_type{});
+    else flux(std::false_type{});
 }
 
 template <int DIM>
@@ -1530,7 +1650,8 @@ const int kBatchTpbDefault[BK_COUNT] = {
     256,                      // tangential flags
     128,                      // tangential WENO-AO
     128,                      // tangential reconstruction of small sweeps
-    128,                      // flux
+    64, 64,                   // flux of large sweeps (Pr = 1, Prandtl fix)
+    kFluxSmallBlock, kFluxSmallBlock,   // flux of small sweeps
     256                       // update
 };
 
@@ -1554,8 +1675,11 @@ static long long batch_unit_blocks(const SolveDesc& d, int dim, int c, int dir, 
     const long long cells = (long long)(dim == 2 ? g.ny : 1) * g.nx;
     if (batch_sweep_class(c) && dir >= dim) return 0;          // 1D: no y sweep
     if (dim == 1 && c >= BK_RAWT && c <= BK_TSMALL) return 0;
-    if (S.small && (c == BK_RAWN || c == BK_NORMAL || c == BK_NAO || c == BK_RAWT || c == BK_TANG || c == BK_TAO)) return 0;
-    if (!S.small && (c == BK_NSMALL || c == BK_TSMALL)) return 0;
+    // the sweep classes of the other size, and the flux classes of the other Prandtl variant
+    const bool small_class = c == BK_NSMALL || c == BK_TSMALL || c == BK_FSMALL || c == BK_FSMALL_PR;
+    if (batch_sweep_class(c) && small_class != (S.small != 0)) return 0;
+    const bool pr = d.P.fc.prfix != 0.0;
+    if (((c == BK_FLUX || c == BK_FSMALL) && pr) || ((c == BK_FLUX_PR || c == BK_FSMALL_PR) && !pr)) return 0;
     long long b = 0;
     switch (c) {
         case BK_DT: b = (cells + (long long)t * 8 - 1) / ((long long)t * 8); break;
@@ -1568,7 +1692,8 @@ static long long batch_unit_blocks(const SolveDesc& d, int dim, int c, int dir, 
         case BK_TANG: b = blocks_for((long long)S.nt * S.nm, t); break;
         case BK_TAO: b = blocks_for((long long)S.nt * S.nm * 4 * 4, t * 8); break;
         case BK_TSMALL: b = blocks_for(tang_small_threads(S), t); break;
-        case BK_FLUX: b = blocks_for(flux_threads(dim, (long long)S.nt * S.nm), t); break;
+        case BK_FLUX: case BK_FLUX_PR: b = blocks_for(flux_threads(dim, (long long)S.nt * S.nm), t); break;
+        case BK_FSMALL: case BK_FSMALL_PR: b = blocks_for(flux_small_threads(dim, (long long)S.nt * S.nm), t); break;
         case BK_UPD: b = blocks_for(cells, t); break;
     }
     return b < 1 ? 1 : b;
@@ -1633,16 +1758,22 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
         sweep(BK_TANG, [&] { kb_tang<<<grid(BK_TANG), tp(BK_TANG), 0, st>>>(dd, bo(BK_TANG), n, stage); });
         sweep(BK_TAO, [&] { kb_tang_ao<<<grid(BK_TAO), tp(BK_TAO), 0, st>>>(dd, bo(BK_TAO), n, stage); });
         sweep(BK_TSMALL, [&] { kb_tang_small<<<grid(BK_TSMALL), tp(BK_TSMALL), 0, st>>>(dd, bo(BK_TSMALL), n, stage); });
-        mark(BK_FLUX, 0);
-        const int tf = tp(BK_FLUX);
-        if (dim == 2) {
-            if (stage == 0) kb_flux<2, 0><<<grid(BK_FLUX), tf, flux_smem(2, tf), st>>>(dd, bo(BK_FLUX), n);
-            else kb_flux<2, 1><<<grid(BK_FLUX), tf, flux_smem(2, tf), st>>>(dd, bo(BK_FLUX), n);
-        } else {
-            if (stage == 0) kb_flux<1, 0><<<grid(BK_FLUX), tf, 0, st>>>(dd, bo(BK_FLUX), n);
-            else kb_flux<1, 1><<<grid(BK_FLUX), tf, 0, st>>>(dd, bo(BK_FLUX), n);
-        }
-        mark(BK_FLUX, 1);
+        auto flux = [&](auto dimc, auto prfix) {
+            constexpr int DIM = decltype(dimc)::value;
+            constexpr bool PR = decltype(prfix)::value;
+            const int cl = PR ? BK_FLUX_PR : BK_FLUX, cs = PR ? BK_FSMALL_PR : BK_FSMALL;
+            sweep(cl, [&] {
+                if (stage == 0) kb_flux<DIM, 0, PR><<<grid(cl), tp(cl), flux_smem(DIM, tp(cl)), st>>>(dd, bo(cl), n);
+                else kb_flux<DIM, 1, PR><<<grid(cl), tp(cl), flux_smem(DIM, tp(cl)), st>>>(dd, bo(cl), n);
+            });
+            sweep(cs, [&] {
+                if (stage == 0) kb_flux_small<DIM, 0, PR><<<grid(cs), tp(cs), flux_small_smem(DIM, PR, tp(cs)), st>>>(dd, bo(cs), n);
+                else kb_flux_small<DIM, 1, PR><<<grid(cs), tp(cs), flux_small_smem(DIM, PR, tp(cs)), st>>>(dd, bo(cs), n);
+            });
+        };
+        auto flux_dim = [&](auto dimc) { flux(dimc, std::false_type{}); flux(dimc, std::true_type{}); };
+        if (dim == 2) flux_dim(std::integral_constant<int, 2>{});
+        else flux_dim(std::integral_constant<int, 1>{});
         mark(BK_UPD, 0);
         const int tu = tp(BK_UPD);
         if (dim == 2) {

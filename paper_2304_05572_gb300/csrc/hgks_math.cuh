@@ -899,10 +899,11 @@ HGKS_HD __forceinline__ void half_moments(const MState<DIM>& s, double sl, int s
 template <int DIM>
 struct FluxSums { double Wc[DIM + 2], Wx[DIM + 2], Wy[DIM + 2], S4[DIM + 2], S5[DIM + 2], S6n[DIM + 2], D5[DIM + 2], D6n[DIM + 2]; };
 
-// One side's share of the sums, from its state and its normal (x) and tangential (y) derivatives.
+// One side's share of the sums (left: over u > 0, else over u < 0), from its state and its normal (x) and
+// tangential (y) derivatives; FIRST: stored, else added.
 // Returns false if the state is non-physical.
 template <int DIM, bool PRFIX, bool FIRST>
-HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, const double* Wx, const double* Wy,
+HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, const double* Wx, const double* Wy, bool left,
                                        FluxSums<DIM>& q, double& p)
 {
     constexpr int NV = DIM + 2;
@@ -918,7 +919,7 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
         k.U2 = scale2<1>(s.U);
     }
     Mom m;
-    half_moments<DIM>(s, sl, FIRST ? +1 : -1, fc, m);
+    half_moments<DIM>(s, sl, left ? +1 : -1, fc, m);
     add_psi_lab<DIM, FIRST>(s, m, 0, q.Wc);
     Dir dx, dy;
     Slope a;
@@ -1153,8 +1154,8 @@ HGKS_HD __forceinline__ bool gks_flux(const FluxConst& fc, const double* Wl, con
 {
     FluxSums<DIM> q;
     double pl, pr;
-    const bool okl = flux_side<DIM, PRFIX, true>(fc, Wl, Wlx, Wly, q, pl);
-    const bool okr = okl && flux_side<DIM, PRFIX, false>(fc, Wr, Wrx, Wry, q, pr);
+    const bool okl = flux_side<DIM, PRFIX, true>(fc, Wl, Wlx, Wly, true, q, pl);
+    const bool okr = okl && flux_side<DIM, PRFIX, false>(fc, Wr, Wrx, Wry, false, q, pr);
     if (!okr) return false;
     return flux_finish<DIM, STAGE, PRFIX>(fc, q, pl, pr, dt, o0, o1);
 }
