@@ -671,9 +671,9 @@ extern "C" int hgks_batch_step(hgks_batch* b, const double* t_end, int nsteps, i
         for (int k = 0; k < 3 && left > 0; k++) {
             int tpb[BK_COUNT];
             for (int c = 0; c < BK_COUNT; c++) {
-                // the flux kernels' warps share segments: fixed block sizes
-                if (c >= BK_FLUX && c <= BK_FSMALL_PR) { tpb[c] = kBatchTpbDefault[c]; continue; }
-                bool heavy_regs = c == BK_NAO || c == BK_TAO || c == BK_NSMALL || c == BK_TSMALL;
+                // kernels whose warps share segments have fixed block sizes
+                if ((c >= BK_FLUX && c <= BK_FSMALL_PR) || c == BK_TSMALL) { tpb[c] = kBatchTpbDefault[c]; continue; }
+                bool heavy_regs = c == BK_NAO || c == BK_TAO || c == BK_NSMALL;
                 tpb[c] = heavy_regs ? cand_small[k] : cand_big[k];
             }
             int st = batch_upload_plan(b, tpb);

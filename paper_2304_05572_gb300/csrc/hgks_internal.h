@@ -105,6 +105,7 @@ inline bool batch_sweep_class(int c) { return c >= BK_RAWN && c <= BK_FSMALL_PR;
 
 struct BatchPlan {
     int n = 0, dim = 0;
+    int tang_rows = 1;             // lines a block of BK_TSMALL
     int tpb[BK_COUNT];
     int nblk[BK_COUNT];            // total blocks of each class
     std::vector<int> boff;         // [BK_COUNT][2 n + 1] block offsets per unit (a solver, or a

@@ -390,7 +390,7 @@ __device__ __forceinline__ void b_normal(const Params& P, const Sweep& S, const 
             if (side == 0) linear_left(q, S.inv12hn, val[k], der[k]);
             else linear_right(q, S.inv12hn, val[k], der[k]);
         }
-        if (nonphysical<NV>(P.gamma, val)) {
+        if (nonphysical<NV>(val)) {
             const double* cc = cellp(P, S, W, t, c);
 #pragma unroll
             for (int k = 0; k < NV; k++) { val[k] = ldc(cc + (long long)S.perm[k] * P.g.plane, S); der[k] = 0.0; }
@@ -461,7 +461,7 @@ __device__ __forceinline__ void b_normal_ao(const Params& P, const Sweep& S, con
             int side, L, m;
             normal_ao_item<NV>(P, S, W, rdc(S.itemsN + i, S), Qw, Qs, side, L, m);
             weno_ao_face<NV>(P.gamma, ak, Qw, Qs, side == 0 ? +1 : -1, val, d);
-            const bool bad = nonphysical<NV>(P.gamma, val);
+            const bool bad = nonphysical<NV>(val);
             const long long o = (long long)L * S.nm + m;
 #pragma unroll
             for (int k = 0; k < NV; k++) {
@@ -479,7 +479,7 @@ __device__ __forceinline__ void b_normal_ao(const Params& P, const Sweep& S, con
         normal_ao_item<NV>(P, S, W, rdc(S.itemsN + i, S), Qw, Qs, side, L, m);
         weno_ao_face_x4<NV>(P.gamma, ak, Qw, Qs, side == 0 ? +1 : -1, gmask, val, dq);
         double vq = 0.0;
-        if (nonphysical<NV>(P.gamma, val)) {
+        if (nonphysical<NV>(val)) {
             vq = Qw[2][q < NV ? q : 0];
             dq = 0.0;
         } else {
@@ -505,79 +505,77 @@ __global__ void k_normal_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
 }
 
 
-// Small sweeps: flags, linear reconstruction and WENO-AO of the normal pass in one launch, one (line,
-// interface, side) per aligned group of 4 lanes, lane q carrying component q.  The group runs the raw
-// indicator on the three cells the Step-4 spread looks at (7 values a lane, so nothing is read back), ORs it
-// over the components with shuffles, and takes the linear formulas or weno_ao_face_x4.  The arithmetic is
-// b_normal's and b_normal_ao's, so every result is.  Such a sweep's time is made of launches (3 us each)
-// and of each thread's chain of FP64 instructions (31 ns each): with one launch per direction in place of
-// three (flags, linear pass, compacted WENO-AO) and the step's five control and ghost launches in two, a
-// step of 200 cells in 1D went from 133 to 90 us, of 48 x 48 from 210 to 136, of the 200 x 100 viscous tube
-// from 508 to 466.  Compaction and shared flags pay from about 65536 segments on.
+// Small sweeps: flags, linear reconstruction and WENO-AO of the normal pass in one launch.  A warp takes 8
+// consecutive cells of a line, 4 lanes each (lane q carries component q), and one side: every group runs the
+// raw indicator of its cell, the groups exchange the decisions for the Step-4 spread (OR over the components,
+// then over the neighbouring groups), and the inner 6 reconstruct their face with the linear formulas or
+// weno_ao_face_x4.  The arithmetic is b_normal's and b_normal_ao's, so every result is.  The warps of a
+// block stand on neighbouring lines, which share the memory sectors of a y sweep.
+// Such a sweep's time is made of launches (3 us each) and of each thread's chain of FP64 instructions (31 ns
+// each): with one launch per direction in place of three (flags, linear pass, compacted WENO-AO) and the
+// step's five control and ghost launches in two, a step of 200 cells in 1D went from 133 to 90 us, of
+// 48 x 48 from 210 to 136.  Compaction and shared flags pay from about 65536 segments on.
+constexpr int kSmallCells = 6;
+
 template <int NV>
 __device__ __forceinline__ void b_normal_small(const Params& P, const Sweep& S, const double* __restrict__ W, Ctrl* ctrl, int stage, long long id)
 {
     if (ctrl->done) return;
-    const long long total = (long long)S.nlines * S.nm * 2;
-    const long long item = id >> 2;
-    const int q = (int)(id & 3), qc = q < NV ? q : NV - 1;
-    const int lane0 = threadIdx.x & 28;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, gi = lane >> 2, q = lane & 3, qc = q < NV ? q : NV - 1;
+    const int lane0 = lane & 28;
     const unsigned gmask = 0xFu << lane0;
-    const bool active = item < total;               // the same for the 4 lanes of a group
-    const int side = (int)(item & 1);
-    int L = 0, m = 0, flag = 0;
-    double v[7];
-    if (active) {
-        const unsigned lm = (unsigned)(item >> 1);
-        L = (int)(lm / (unsigned)S.nm); m = (int)(lm - (unsigned)L * (unsigned)S.nm);
-        const double* b = cellp(P, S, W, L + S.tlo, m - 1 + side - 3) + (long long)S.perm[qc] * P.g.plane;
-#pragma unroll
-        for (int s = 0; s < 7; s++) v[s] = ldc(b + (long long)s * S.sN, S);
-        if (P.recon_mode == HGKS_RECON_WENOAO) flag = 1;
-        else if (P.recon_mode == HGKS_RECON_HYBRID) {
-            float f[7];
-#pragma unroll
-            for (int s = 0; s < 7; s++) f[s] = fixed::to_float(v[s]);
-#pragma unroll
-            for (int s = 0; s < 3; s++) flag |= indicator_raw<true>(v + s, f + s, S.Z1n);
-            flag |= __shfl_xor_sync(gmask, flag, 1);
-            flag |= __shfl_xor_sync(gmask, flag, 2);
-        }
-        if (q == 0) {
-            uint8_t* fo = S.flagN + (long long)L * (S.nn + 2);
-            if (side == 1) stc(fo + m + 1, flag, S);
-            else if (m == 0) stc(fo, flag, S);
-        }
-    }
+    const unsigned w = (unsigned)(id >> 5), nl = (unsigned)S.nlines;
+    const unsigned rest = w / nl;
+    const int L = (int)(w - rest * nl), side = (int)(rest & 1), c = (int)(rest >> 1) * kSmallCells + gi - 2;
+    if ((int)(rest >> 1) * kSmallCells >= S.nn + 2) return;        // the same for the warp
+    const int cc = c <= S.nn + 1 ? c : S.nn + 1;                   // (groups past the last halo cell repeat it)
     const int t = L + S.tlo;
-    const bool counted = active && q == 0 && side == 1 && t >= 0 && t < S.nt && m < S.nn;
+    const double* b = cellp(P, S, W, t, cc - 2) + (long long)S.perm[qc] * P.g.plane;
+    double v[5];
+#pragma unroll
+    for (int s = 0; s < 5; s++) v[s] = ldc(b + (long long)s * S.sN, S);
+    int flag = 0;
+    if (P.recon_mode == HGKS_RECON_WENOAO) flag = 1;
+    else if (P.recon_mode == HGKS_RECON_HYBRID) {
+        float f[5];
+#pragma unroll
+        for (int s = 0; s < 5; s++) f[s] = fixed::to_float(v[s]);
+        flag = indicator_raw<true>(v, f, S.Z1n);
+        flag |= __shfl_xor_sync(full, flag, 1);
+        flag |= __shfl_xor_sync(full, flag, 2);
+        flag |= __shfl_sync(full, flag, lane - 4) | __shfl_sync(full, flag, lane + 4);   // (used by the inner groups)
+    }
+    const bool out = gi >= 1 && gi <= kSmallCells && c <= S.nn;
+    const bool first = out && side == 0 && q == 0;                 // one lane per cell -1..nn
+    if (first) stc(S.flagN + (long long)L * (S.nn + 2) + c + 1, flag, S);
+    const bool counted = first && t >= 0 && t < S.nt && c >= 0 && c < S.nn;
     warp_count(&ctrl->troubled[stage][S.dir][0], counted && flag ? 1u : 0u);
     warp_count(&ctrl->examined[stage][S.dir][0], counted ? 1u : 0u);
-    if (!active) return;
+    // side 0: the left state of interface c + 1; side 1: the right state of interface c
+    const int m = side == 0 ? c + 1 : c;
+    if (!out || m < 0 || m >= S.nm) return;                        // the same for a group
     double val, der;
     if (!flag) {
-        if (side == 0) linear_left(v + 1, S.inv12hn, val, der);
-        else linear_right(v + 1, S.inv12hn, val, der);
-        double Q[NV];
-#pragma unroll
-        for (int k = 0; k < NV; k++) Q[k] = __shfl_sync(gmask, val, lane0 + k);
-        if (nonphysical<NV>(P.gamma, Q)) { val = v[3]; der = 0.0; }
+        if (side == 0) linear_left(v, S.inv12hn, val, der);
+        else linear_right(v, S.inv12hn, val, der);
+        if (nonphysical_x4<NV>(val, lane0, gmask)) { val = v[2]; der = 0.0; }
     } else {
         AOConst ak;
         for (int j = 0; j < 4; j++) ak.g[j] = P.g_ao[j];
         ak.g3inv = P.g3inv; ak.gr[0] = P.gr[0]; ak.gr[1] = P.gr[1]; ak.gr[2] = P.gr[2]; ak.eps = P.eps;
         double Qw[5][NV], Qs[NV], vs[NV];
-        const double avg = ((ex(side == 0 ? v[3] : v[2]) + ex(side == 0 ? v[4] : v[3])) * ex(0.5)).v;
+        const double avg = ((ex(side == 0 ? v[2] : v[1]) + ex(side == 0 ? v[3] : v[2])) * ex(0.5)).v;
 #pragma unroll
         for (int k = 0; k < NV; k++) {
             Qs[k] = __shfl_sync(gmask, avg, lane0 + k);
 #pragma unroll
-            for (int s = 0; s < 5; s++) Qw[s][k] = __shfl_sync(gmask, v[s + 1], lane0 + k);
+            for (int s = 0; s < 5; s++) Qw[s][k] = __shfl_sync(gmask, v[s], lane0 + k);
         }
         weno_ao_face_x4<NV>(P.gamma, ak, Qw, Qs, side == 0 ? +1 : -1, gmask, vs, der);
         val = 0.0;
-        if (nonphysical<NV>(P.gamma, vs)) {
-            val = v[3];
+        if (nonphysical<NV>(vs)) {
+            val = v[2];
             der = 0.0;
         } else {
 #pragma unroll
@@ -661,7 +659,7 @@ __device__ __forceinline__ void gp_positivity(const Params& P, const Sweep& S, i
 #pragma unroll
     for (int g = 0; g < 2; g++) {
         double Q[4] = {v[0][g], v[1][g], v[2][g], v[3][g]};
-        if (nonphysical<4>(P.gamma, Q)) {
+        if (nonphysical<4>(Q)) {
 #pragma unroll
             for (int k = 0; k < 4; k++) { v[k][g] = lineval(S, X, k, t, m); d[k][g] = 0.0; }
         }
@@ -772,12 +770,8 @@ __device__ __forceinline__ void b_tang_ao(const Params& P, const Sweep& S, const
         if (X <= 1) {
             // positivity of the reconstructed Q^l, Q^r states (gp_positivity), on the gathered components
 #pragma unroll
-            for (int g = 0; g < 2; g++) {
-                double Q[4];
-#pragma unroll
-                for (int k = 0; k < 4; k++) Q[k] = __shfl_sync(gmask, vq[g], lane0 + k);
-                if (nonphysical<4>(P.gamma, Q)) { vq[g] = lineval(S, X, q, t, m); dq[g] = 0.0; }
-            }
+            for (int g = 0; g < 2; g++)
+                if (nonphysical_x4<4>(vq[g], lane0, gmask)) { vq[g] = lineval(S, X, q, t, m); dq[g] = 0.0; }
         }
         const long long o = (long long)t * S.nm + m;
         const int qv = X == 0 ? 0 : (X == 1 ? 3 : (X == 2 ? 1 : 4));
@@ -805,98 +799,136 @@ __global__ void k_tang_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
 }
 
 
-// Small sweeps: flags, quartics and WENO-AO of the four tangential passes in one launch, 16 lanes per
-// segment: lanes 4 X + q carry component q of pass X.  As in b_normal_small the raw indicator runs on the three
-// lines the Step-4 spread looks at; every pass ends in the Gauss-point buffer.  Free-order arithmetic:
-// compiled once (tang_small_nl) like tang_ao_nl.
-__device__ __forceinline__ void b_tang_small(const Params& P, const Sweep& S, const double* __restrict__ W, Ctrl* ctrl, int stage, long long id)
+// Small sweeps: flags, quartics and WENO-AO of the four tangential passes in one launch.  A block of 4 warps
+// takes 8 interfaces and `rows` consecutive lines, warp X pass X, 4 lanes an interface (lane q component q).  A
+// warp walks along the lines with the window in registers: one load and one raw indicator per line, the
+// decisions of the line before and the line after kept for the Step-4 spread.  Every pass ends in the
+// Gauss-point buffer.  Free-order arithmetic: compiled once (tang_small_nl) like tang_ao_nl; it does not depend
+// on `rows`, which is chosen for the number of blocks.
+constexpr int kSmallCols = 8, kSmallRowsMax = 8, kSmallTangBlock = 128;
+
+__device__ __forceinline__ void b_tang_small(const Params& P, const Sweep& S, const double* __restrict__ W, Ctrl* ctrl, int stage,
+                                             unsigned block, int rows)
 {
+    __shared__ uint8_t s_flag[4][kSmallRowsMax][kSmallCols];
     if (ctrl->done) return;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, X = threadIdx.x >> 5, gi = lane >> 2, q = lane & 3;
+    const int lane0 = lane & 28;
+    const unsigned gmask = 0xFu << lane0;
+    const unsigned nmb = (unsigned)(S.nm + kSmallCols - 1) / kSmallCols, tb = block / nmb;
+    const int t0 = (int)tb * rows, m0 = (int)(block - tb * nmb) * kSmallCols;
+    const int m = m0 + gi, mc = m < S.nm ? m : S.nm - 1;
+    const bool inside = m < S.nm;
+    const bool hybrid = P.recon_mode == HGKS_RECON_HYBRID;
     const long long total = (long long)S.nt * S.nm;
-    const long long seg = id >> 4;
-    const int X = (int)(id >> 2) & 3, q = (int)(id & 3);
-    const int lane0 = threadIdx.x & 28;
-    const unsigned gmask = 0xFu << lane0, hmask = 0xFFFFu << (threadIdx.x & 16);
-    const bool active = seg < total;                // the same for the 16 lanes of a segment
-    int t = 0, m = 0;
-    unsigned flag = 0, bits = 0;
-    double v[7];
-    if (active) {
-        t = (int)((unsigned)seg / (unsigned)S.nm); m = (int)((unsigned)seg - (unsigned)t * (unsigned)S.nm);
+    const fixed::Scale inv = fixed::scale_of(S.inv_ht);
+    AOConst ak;
+    for (int j = 0; j < 4; j++) ak.g[j] = P.g_ao[j];
+    ak.g3inv = P.g3inv; ak.gr[0] = P.gr[0]; ak.gr[1] = P.gr[1]; ak.gr[2] = P.gr[2]; ak.eps = P.eps;
+
+    double v[6];                                 // lines t-2..t+3 (before the first line: t0-3..t0+2)
+    float f[6];
+    auto raw = [&](const double* vw, const float* fw) {
+        unsigned r = (unsigned)indicator_raw<true>(vw, fw, S.Z1t);
+        r |= __shfl_xor_sync(full, r, 1);
+        return r | __shfl_xor_sync(full, r, 2);
+    };
 #pragma unroll
-        for (int s = 0; s < 7; s++) v[s] = lineval(S, X, q, t - 3 + s, m);
-        if (P.recon_mode == HGKS_RECON_WENOAO) flag = 1;
-        else if (P.recon_mode == HGKS_RECON_HYBRID) {
-            float f[7];
+    for (int s = 0; s < 6; s++) { v[s] = lineval(S, X, q, t0 - 3 + s, mc); f[s] = fixed::to_float(v[s]); }
+    unsigned before = 0, here = 0, troubled = 0, examined = 0;
+    if (hybrid) { before = raw(v, f); here = raw(v + 1, f + 1); }
+#pragma unroll 1
+    for (int r = 0; r < rows; r++) {
+        const int t = t0 + r;
+        if (t >= S.nt) break;                    // the same for the block
 #pragma unroll
-            for (int s = 0; s < 7; s++) f[s] = fixed::to_float(v[s]);
-#pragma unroll
-            for (int s = 0; s < 3; s++) flag |= (unsigned)indicator_raw<true>(v + s, f + s, S.Z1t);
-            flag |= __shfl_xor_sync(gmask, flag, 1);
-            flag |= __shfl_xor_sync(gmask, flag, 2);
+        for (int s = 0; s < 5; s++) { v[s] = v[s + 1]; f[s] = f[s + 1]; }
+        unsigned flag = P.recon_mode == HGKS_RECON_WENOAO ? 1u : 0u;
+        if (hybrid) {
+            v[5] = lineval(S, X, q, t + 3, mc);
+            f[5] = fixed::to_float(v[5]);
+            const unsigned after = raw(v + 1, f + 1);
+            flag = before | here | after;
+            before = here;
+            here = after;
+        } else if (r + 1 < rows && t + 1 < S.nt) {
+            v[5] = lineval(S, X, q, t + 3, mc);
         }
-        bits = flag << X;
-        bits |= __shfl_xor_sync(hmask, bits, 4);
-        bits |= __shfl_xor_sync(hmask, bits, 8);
-        if ((id & 15) == 0) stc(S.flagT + seg, bits, S);
-    }
-    const bool lead = active && (id & 15) == 0;
-    warp_count(&ctrl->troubled[stage][S.dir][1], lead ? (unsigned)__popc(bits) : 0u);
-    warp_count(&ctrl->examined[stage][S.dir][1], lead ? 4u : 0u);
-    if (!active) return;
-    double vq[2], dq[2] = {0.0, 0.0};
-    if (!flag) {
-        const fixed::Scale inv = fixed::scale_of(S.inv_ht);
-        if (X <= 1) gauss_linear<true>(v + 1, inv, S.inv_ht, vq, dq);
-        else gauss_linear<false>(v + 1, inv, S.inv_ht, vq, dq);
-    } else {
-        AOConst ak;
-        for (int j = 0; j < 4; j++) ak.g[j] = P.g_ao[j];
-        ak.g3inv = P.g3inv; ak.gr[0] = P.gr[0]; ak.gr[1] = P.gr[1]; ak.gr[2] = P.gr[2]; ak.eps = P.eps;
-        // the face average of the segment, one component a lane
-        const long long oc = (long long)S.perm[q] * P.g.plane;
-        const double avg = scale2<-1>(ldc(cellp(P, S, W, t, m - 1) + oc, S) + ldc(cellp(P, S, W, t, m) + oc, S));
-        double qs[4], x[5][4];
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            qs[k] = __shfl_sync(gmask, avg, lane0 + k);
-#pragma unroll
-            for (int s = 0; s < 5; s++) x[s][k] = __shfl_sync(gmask, v[s + 1], lane0 + k);
+        if (q == 0) {
+            s_flag[X][r][gi] = (uint8_t)flag;
+            troubled += inside ? flag : 0u;
+            examined += inside ? 1u : 0u;
         }
-        TangEig e;
-        tang_eig(P.gamma, qs, e);
-        tang_ao_x4(e, x, ak, X <= 1, gmask, vq, dq);
-        dq[0] *= S.inv_ht;
-        dq[1] *= S.inv_ht;
-    }
-    if (X <= 1) {
-        // Reading: a reconstructed state with rho <= 0 or p <= 0 falls back to first order
+        if (!inside) continue;                   // the same for a group
+        double vq[2], dq[2] = {0.0, 0.0};
+        if (!flag) {
+            if (X <= 1) gauss_linear<true>(v, inv, S.inv_ht, vq, dq);
+            else gauss_linear<false>(v, inv, S.inv_ht, vq, dq);
+        } else {
+            // the face average of the segment, one component a lane
+            const long long oc = (long long)S.perm[q] * P.g.plane;
+            const double avg = scale2<-1>(ldc(cellp(P, S, W, t, m - 1) + oc, S) + ldc(cellp(P, S, W, t, m) + oc, S));
+            double qs[4], x[5][4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                qs[k] = __shfl_sync(gmask, avg, lane0 + k);
+#pragma unroll
+                for (int s = 0; s < 5; s++) x[s][k] = __shfl_sync(gmask, v[s], lane0 + k);
+            }
+            TangEig e;
+            tang_eig(P.gamma, qs, e);
+            tang_ao_x4(e, x, ak, X <= 1, gmask, vq, dq);
+            dq[0] *= S.inv_ht;
+            dq[1] *= S.inv_ht;
+        }
+        if (X <= 1) {
+            // Reading: a reconstructed state with rho <= 0 or p <= 0 falls back to first order
+#pragma unroll
+            for (int g = 0; g < 2; g++)
+                if (nonphysical_x4<4>(vq[g], lane0, gmask)) { vq[g] = v[2]; dq[g] = 0.0; }
+        }
+        // Q index: 0 Wl, 1 Wlx, 2 Wly, 3 Wr, 4 Wrx, 5 Wry
+        const int qv = X == 0 ? 0 : (X == 1 ? 3 : (X == 2 ? 1 : 4));
+        const long long o = (long long)t * S.nm + m;
 #pragma unroll
         for (int g = 0; g < 2; g++) {
-            double Q[4];
-#pragma unroll
-            for (int c = 0; c < 4; c++) Q[c] = __shfl_sync(gmask, vq[g], lane0 + c);
-            if (nonphysical<4>(P.gamma, Q)) { vq[g] = v[3]; dq[g] = 0.0; }
+            stc(S.gp + (long long)((g * 6 + qv) * 4 + q) * total + o, vq[g], S);
+            if (X <= 1) stc(S.gp + (long long)((g * 6 + qv + 2) * 4 + q) * total + o, dq[g], S);
         }
     }
-    // Q index: 0 Wl, 1 Wlx, 2 Wly, 3 Wr, 4 Wrx, 5 Wry
-    const int qv = X == 0 ? 0 : (X == 1 ? 3 : (X == 2 ? 1 : 4));
-#pragma unroll
-    for (int g = 0; g < 2; g++) {
-        stc(S.gp + (long long)((g * 6 + qv) * 4 + q) * total + seg, vq[g], S);
-        if (X <= 1) stc(S.gp + (long long)((g * 6 + qv + 2) * 4 + q) * total + seg, dq[g], S);
+    __syncwarp();
+    warp_count(&ctrl->troubled[stage][S.dir][1], troubled);
+    warp_count(&ctrl->examined[stage][S.dir][1], examined);
+    __syncthreads();
+    const int r = threadIdx.x / kSmallCols, j = threadIdx.x % kSmallCols;
+    if (r < rows && t0 + r < S.nt && m0 + j < S.nm) {
+        const unsigned bits = s_flag[0][r][j] | s_flag[1][r][j] << 1 | s_flag[2][r][j] << 2 | s_flag[3][r][j] << 3;
+        stc(S.flagT + (long long)(t0 + r) * S.nm + m0 + j, bits, S);
     }
 }
 
-__device__ __noinline__ void tang_small_nl(const SolveDesc& d, int dir, int stage, long long id)
+// Blocks of the small tangential launch on sweep S with `rows` lines a block; rows from the number of blocks
+// that leaves: up to 8 while a launch still has 16 blocks for each of 152 SMs.
+inline long long tang_small_blocks(const Sweep& S, int rows)
 {
-    b_tang_small(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, id);
+    return (long long)((S.nm + kSmallCols - 1) / kSmallCols) * ((S.nt + rows - 1) / rows);
+}
+inline int tang_small_rows(long long blocks1)     // blocks1: blocks of the whole launch with one line a block
+{
+    const long long r = blocks1 / (16 * 152);
+    return r < 1 ? 1 : r > kSmallRowsMax ? kSmallRowsMax : (int)r;
 }
 
-__global__ void k_tang_small(const SolveDesc* __restrict__ D, int nb0, int stage)
+__device__ __noinline__ void tang_small_nl(const SolveDesc& d, int dir, int stage, unsigned block, int rows)
 {
-    const SweepBlock b = sweep_block(nb0);
-    tang_small_nl(*D, b.dir, stage, b.id);
+    b_tang_small(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, block, rows);
+}
+
+__global__ void __launch_bounds__(kSmallTangBlock) k_tang_small(const SolveDesc* __restrict__ D, int nb0, int stage, int rows)
+{
+    const int dir = (int)blockIdx.x >= nb0 ? 1 : 0;
+    tang_small_nl(*D, dir, stage, blockIdx.x - (dir ? (unsigned)nb0 : 0u), rows);
 }
 
 // ---------------------------------------------------------------- flux and update
@@ -942,7 +974,7 @@ __device__ __forceinline__ void side_pair(const Params& P, const Sweep& S, int s
 #pragma unroll
         for (int g = 0; g < 2; g++) {
             const double Q[4] = {v[0][g], v[1][g], v[2][g], v[3][g]};
-            if (nonphysical<4>(P.gamma, Q)) {
+            if (nonphysical<4>(Q)) {
                 // Reading: a reconstructed state with rho <= 0 or p <= 0 falls back to first order
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
@@ -1281,7 +1313,10 @@ __device__ __forceinline__ void b_update(const Params& P, const Sweep& Sx, const
         stc(Wout + cell + (long long)k * g.plane, out[k], g);
         if (STAGE == 0) stc(Acc + cell + (long long)k * g.plane, acc[k], g);
     }
-    // rho > 0 and p > 0, the latter as rho E - |m|^2/2 > 0 (no division)
+    // rho > 0 and p > 0, the latter as rho E - |m|^2/2 > 0 (no division; first in FP32, see surely_physical)
+    if (surely_physical(fixed::to_float(out[0]), fixed::to_float(out[1]), DIM == 2 ? fixed::to_float(out[2]) : 0.0f,
+                        fixed::to_float(out[NV - 1])))
+        return;
     double ke = DIM == 2 ? 0.5 * fma(out[1], out[1], out[2] * out[2]) : 0.5 * out[1] * out[1];
     double pr = fma(out[NV - 1], out[0], -ke);
     if (!fixed::is_pos(out[0]) || !fixed::is_pos(pr) || !fixed::is_finite(out[0]) || !fixed::is_finite(pr)) ctrl->status = HGKS_ENONPHYSICAL;
@@ -1369,10 +1404,10 @@ __global__ void kb_normal_small(const SolveDesc* __restrict__ D, const int* __re
     b_normal_small<NV>(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, id);
 }
 
-__global__ void kb_tang_small(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+__global__ void __launch_bounds__(kSmallTangBlock) kb_tang_small(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage, int rows)
 {
     HGKS_BATCH_SWEEP_BLOCK();
-    tang_small_nl(d, dir, stage, id);
+    tang_small_nl(d, dir, stage, (unsigned)lblk_, rows);
 }
 
 __global__ void kb_raw_tflags(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
@@ -1415,9 +1450,11 @@ __global__ void kb_update(const SolveDesc* __restrict__ D, const int* __restrict
     else b_update<DIM, 1>(d.P, d.sw[0], d.sw[1], d.Ws, d.W, d.Acc, d.ctrl, id);
 }
 
-// Threads of the small-sweep reconstruction launches.
-inline long long normal_small_threads(const Sweep& S) { return (long long)S.nlines * S.nm * 2 * 4; }
-inline long long tang_small_threads(const Sweep& S) { return (long long)S.nt * S.nm * 16; }
+// Threads of the small-sweep normal launch: a warp per 6 cells of -1..nn, side and line.
+inline long long normal_small_threads(const Sweep& S)
+{
+    return (long long)((S.nn + 2 + kSmallCells - 1) / kSmallCells) * 2 * S.nlines * 32;
+}
 
 inline unsigned int blocks_for(long long n, int tpb) { return (unsigned int)((n + tpb - 1) / tpb); }
 
@@ -1574,8 +1611,9 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
             timed(s, KC_TANG, 1, [&] { k_tang<<<g, TPB, 0, st>>>(D, (int)nb[0], stage); });
         if ((g = pair(LARGE, [&](const Sweep& S) { return ao_blocks((long long)S.nt * S.nm * 4 * 4); })))
             timed(s, KC_TANG_AO, 1, [&] { k_tang_ao<<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
-        if ((g = pair(SMALL, [](const Sweep& S) { return blocks_for(tang_small_threads(S), 128); })))
-            timed(s, KC_TANG, 1, [&] { k_tang_small<<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
+        const int rows = tang_small_rows(pair(SMALL, [](const Sweep& S) { return (unsigned)tang_small_blocks(S, 1); }));
+        if ((g = pair(SMALL, [&](const Sweep& S) { return (unsigned)tang_small_blocks(S, rows); })))
+            timed(s, KC_TANG, 1, [&] { k_tang_small<<<g, kSmallTangBlock, 0, st>>>(D, (int)nb[0], stage, rows); });
     }
     if (s->capture) {
         for (int d = 0; d < DIM; d++) {
@@ -1668,7 +1706,7 @@ void batch_fill_desc(const hgks_solver* s, SolveDesc& d)
 }
 
 // Blocks of one unit of class c with t threads per block: solver d (sweep dir for the sweep classes).
-static long long batch_unit_blocks(const SolveDesc& d, int dim, int c, int dir, int t)
+static long long batch_unit_blocks(const SolveDesc& d, int dim, int c, int dir, int t, int rows)
 {
     const GridGeom& g = d.P.g;
     const Sweep& S = d.sw[dir];
@@ -1691,7 +1729,7 @@ static long long batch_unit_blocks(const SolveDesc& d, int dim, int c, int dir, 
         case BK_RAWT: b = blocks_for(raw_t_threads(S), t); break;
         case BK_TANG: b = blocks_for((long long)S.nt * S.nm, t); break;
         case BK_TAO: b = blocks_for((long long)S.nt * S.nm * 4 * 4, t * 8); break;
-        case BK_TSMALL: b = blocks_for(tang_small_threads(S), t); break;
+        case BK_TSMALL: b = tang_small_blocks(S, rows); break;
         case BK_FLUX: case BK_FLUX_PR: b = blocks_for(flux_threads(dim, (long long)S.nt * S.nm), t); break;
         case BK_FSMALL: case BK_FSMALL_PR: b = blocks_for(flux_small_threads(dim, (long long)S.nt * S.nm), t); break;
         case BK_UPD: b = blocks_for(cells, t); break;
@@ -1706,6 +1744,9 @@ void batch_plan(const std::vector<const SolveDesc*>& descs, int dim, const int* 
     plan.n = n;
     plan.dim = dim;
     for (int c = 0; c < BK_COUNT; c++) plan.tpb[c] = tpb[c];
+    long long blocks1 = 0;
+    for (int u = 0; u < 2 * n; u++) blocks1 += batch_unit_blocks(*descs[u >> 1], dim, BK_TSMALL, u & 1, tpb[BK_TSMALL], 1);
+    plan.tang_rows = tang_small_rows(blocks1);
     plan.boff.assign((size_t)BK_COUNT * stride, 0);
     for (int c = 0; c < BK_COUNT; c++) {
         int* bo = plan.boff.data() + (size_t)c * stride;
@@ -1714,8 +1755,8 @@ void batch_plan(const std::vector<const SolveDesc*>& descs, int dim, const int* 
         long long acc = 0;
         for (int u = 0; u < units; u++) {
             bo[u] = (int)acc;
-            acc += sw ? batch_unit_blocks(*descs[u >> 1], dim, c, u & 1, tpb[c])
-                      : batch_unit_blocks(*descs[u], dim, c, 0, tpb[c]);
+            acc += sw ? batch_unit_blocks(*descs[u >> 1], dim, c, u & 1, tpb[c], plan.tang_rows)
+                      : batch_unit_blocks(*descs[u], dim, c, 0, tpb[c], 1);
         }
         bo[units] = (int)acc;
         plan.nblk[c] = (int)acc;
@@ -1757,7 +1798,7 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
         sweep(BK_RAWT, [&] { kb_raw_tflags<<<grid(BK_RAWT), tp(BK_RAWT), 0, st>>>(dd, bo(BK_RAWT), n); });
         sweep(BK_TANG, [&] { kb_tang<<<grid(BK_TANG), tp(BK_TANG), 0, st>>>(dd, bo(BK_TANG), n, stage); });
         sweep(BK_TAO, [&] { kb_tang_ao<<<grid(BK_TAO), tp(BK_TAO), 0, st>>>(dd, bo(BK_TAO), n, stage); });
-        sweep(BK_TSMALL, [&] { kb_tang_small<<<grid(BK_TSMALL), tp(BK_TSMALL), 0, st>>>(dd, bo(BK_TSMALL), n, stage); });
+        sweep(BK_TSMALL, [&] { kb_tang_small<<<grid(BK_TSMALL), kSmallTangBlock, 0, st>>>(dd, bo(BK_TSMALL), n, stage, plan.tang_rows); });
         auto flux = [&](auto dimc, auto prfix) {
             constexpr int DIM = decltype(dimc)::value;
             constexpr bool PR = decltype(prfix)::value;
