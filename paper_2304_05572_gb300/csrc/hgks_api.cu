@@ -322,10 +322,27 @@ extern "C" const char* hgks_last_error(const hgks_solver* s)
     return s ? s->err : g_create_err;
 }
 
+// Plain device memory of the solver's device: a kernel may read and write it directly (memory of another
+// device, managed or mapped memory goes through the runtime's copies).
+static bool own_device_memory(const hgks_solver* s, const void* p)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    int dev = -1;
+    return a.type == cudaMemoryTypeDevice && a.device == s->device && cudaGetDevice(&dev) == cudaSuccess && dev == s->device
+           && (uintptr_t)p % sizeof(double) == 0;
+}
+
 extern "C" int hgks_set_state(hgks_solver* s, const double* W, int on_device, double t0)
 {
     if (!s || !W) return HGKS_EINVAL;
     const GridGeom& g = s->P.g;
+    if (on_device && own_device_memory(s, W)) {
+        CUDA_TRY(s, launch_state_in(s, W, t0));
+        CUDA_TRY(s, cudaStreamSynchronize(s->stream));
+        s->launches = 0;
+        return HGKS_OK;
+    }
     cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     for (int k = 0; k < g.nv; k++) {
         CUDA_TRY(s, cudaMemcpy2DAsync(s->W + g.origin + (long long)k * g.plane, (size_t)g.pitch * sizeof(double),
@@ -342,6 +359,11 @@ extern "C" int hgks_get_state(hgks_solver* s, double* W, int on_device)
 {
     if (!s || !W) return HGKS_EINVAL;
     const GridGeom& g = s->P.g;
+    if (on_device && own_device_memory(s, W)) {
+        CUDA_TRY(s, launch_state_out(s, W));
+        CUDA_TRY(s, cudaStreamSynchronize(s->stream));
+        return HGKS_OK;
+    }
     cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     for (int k = 0; k < g.nv; k++) {
         CUDA_TRY(s, cudaMemcpy2DAsync(W + (size_t)k * g.nx * g.ny, (size_t)g.nx * sizeof(double),
@@ -932,16 +954,23 @@ extern "C" int hgks_step_noalloc(const hgks_config* cfg, const double* W_in, dou
     s.d_self = (SolveDesc*)(b + L.off_desc);
     SolveDesc self;
     batch_fill_desc(&s, self);
-    // the array keeps the previous call's contents: start every call from zero
-    e = cudaMemsetAsync(base, 0, L.total, s.stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s.d_self, &self, sizeof(SolveDesc), cudaMemcpyHostToDevice, s.stream);
-    for (int k = 0; k < g.nv && e == cudaSuccess; k++)
-        e = cudaMemcpy2DAsync(s.W + g.origin + (long long)k * g.plane, (size_t)g.pitch * sizeof(double),
-                              W_in + (size_t)k * g.nx * g.ny, (size_t)g.nx * sizeof(double),
-                              (size_t)g.nx * sizeof(double), (size_t)g.ny, cudaMemcpyDeviceToDevice, s.stream);
-    if (e == cudaSuccess) e = launch_set_time(&s, 0.0);
+    if (own_device_memory(&s, W_in)) {
+        // descriptor, control block and state in one launch; a step writes everything else before it reads it
+        e = launch_noalloc_in(&s, self, W_in);
+    } else {
+        // the array keeps the previous call's contents: start from zero
+        e = cudaMemsetAsync(base, 0, L.total, s.stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(s.d_self, &self, sizeof(SolveDesc), cudaMemcpyHostToDevice, s.stream);
+        for (int k = 0; k < g.nv && e == cudaSuccess; k++)
+            e = cudaMemcpy2DAsync(s.W + g.origin + (long long)k * g.plane, (size_t)g.pitch * sizeof(double),
+                                  W_in + (size_t)k * g.nx * g.ny, (size_t)g.nx * sizeof(double),
+                                  (size_t)g.nx * sizeof(double), (size_t)g.ny, cudaMemcpyDeviceToDevice, s.stream);
+        if (e == cudaSuccess) e = launch_set_time(&s, 0.0);
+    }
     if (e == cudaSuccess) e = launch_step(&s, 1e300);
-    for (int k = 0; k < g.nv && e == cudaSuccess; k++)
+    const bool own_out = own_device_memory(&s, W_out);
+    if (own_out && e == cudaSuccess) e = launch_state_out(&s, W_out);
+    for (int k = 0; k < g.nv && !own_out && e == cudaSuccess; k++)
         e = cudaMemcpy2DAsync(W_out + (size_t)k * g.nx * g.ny, (size_t)g.nx * sizeof(double),
                               s.W + g.origin + (long long)k * g.plane, (size_t)g.pitch * sizeof(double),
                               (size_t)g.nx * sizeof(double), (size_t)g.ny, cudaMemcpyDeviceToDevice, s.stream);

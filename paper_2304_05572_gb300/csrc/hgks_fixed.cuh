@@ -94,6 +94,15 @@ HGKS_FX float to_float(double x)
     return float_of((f & 0x7FFFFFFFu) | (hi & 0x80000000u));
 }
 
+// Whether rho > 0 and rho E - (mx^2 + my^2)/2 > 0 beyond doubt, from the components truncated to FP32
+// (to_float): truncations and products err by less than 2^-20 of each term, so a difference above 4e-6 of
+// rho E is positive (both factors within 1e-12..1e12, where no product leaves the range).
+HGKS_FX bool surely_physical(float rho, float mx, float my, float E)
+{
+    const float re = rho * E, ke = 0.5f * (mx * mx + my * my);
+    return rho > 1e-12f && rho < 1e12f && E > 1e-12f && E < 1e12f && re - ke > 4e-6f * re;
+}
+
 // y 2^Q rounded down, for 0 <= y < 2^(64-Q)
 HGKS_FX u64 to_fixed(double y, int q)
 {

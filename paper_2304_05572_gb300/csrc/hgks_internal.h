@@ -148,6 +148,11 @@ extern const char* kclass_names[KC_COUNT];
 // host-side launchers (hgks_kernels.cu); all enqueue on s->stream
 cudaError_t launch_step(hgks_solver* s, double t_end);
 cudaError_t launch_set_time(hgks_solver* s, double t0);
+// the caller's state (device memory of the solver's device) into the solver with time t0, and out of it
+cudaError_t launch_state_in(hgks_solver* s, const double* W, double t0);
+cudaError_t launch_state_out(hgks_solver* s, double* W);
+// the allocation-free step's start: descriptor, control block and state
+cudaError_t launch_noalloc_in(hgks_solver* s, const SolveDesc& self, const double* W);
 int device_sm_count();
 // the debug build's count of out-of-range accesses and the first such address (returns 1), or 0
 // without the checks compiled in, -1 if the device read failed

@@ -239,7 +239,17 @@ __global__ void k_dt_ghost(Params P, double* W, Ctrl* ctrl, double h, double t_e
     dt_finish(P, ctrl, t_end, (unsigned)nb);
 }
 
-__global__ void k_set_time(Ctrl* ctrl, double t0)
+__global__ void k_state_out(GridGeom g, const double* __restrict__ W, double* __restrict__ dst)
+{
+    const long long n = (long long)g.nv * g.ny * g.nx;
+    for (long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x; id < n; id += (long long)gridDim.x * blockDim.x) {
+        const long long row = id / g.nx;
+        const int i = (int)(id - row * g.nx), k = (int)(row / g.ny), j = (int)(row - (long long)k * g.ny);
+        dst[id] = rdc(W + g.origin + (long long)k * g.plane + (long long)j * g.pitch + i, g);
+    }
+}
+
+__device__ __forceinline__ void reset_ctrl(Ctrl* ctrl, double t0)
 {
     ctrl->t = t0;
     ctrl->dtmin_bits = 0x7FF0000000000000ull;   // +inf
@@ -252,6 +262,40 @@ __global__ void k_set_time(Ctrl* ctrl, double t0)
     for (int a = 0; a < 2; a++) for (int b = 0; b < 2; b++) for (int c = 0; c < 2; c++) {
         ctrl->troubled[a][b][c] = 0; ctrl->examined[a][b][c] = 0;
     }
+}
+
+__global__ void k_set_time(Ctrl* ctrl, double t0) { reset_ctrl(ctrl, t0); }
+
+__device__ __forceinline__ void state_in(const GridGeom& g, const double* src, double* W, long long id, long long threads)
+{
+    const long long n = (long long)g.nv * g.ny * g.nx;
+    for (; id < n; id += threads) {
+        const long long row = id / g.nx;
+        const int i = (int)(id - row * g.nx), k = (int)(row / g.ny), j = (int)(row - (long long)k * g.ny);
+        stc(W + g.origin + (long long)k * g.plane + (long long)j * g.pitch + i, src[id], g);
+    }
+}
+
+// The caller's [nv][ny][nx] state into and out of the padded layout, one launch for all components in place
+// of a pitched copy each and a launch for the control block: 8 steps of a 200-cell tube with both
+// transfers 714 -> 691 us, a 48 x 48 allocation-free step (which also copied its descriptor and cleared
+// its 3.5 MB) 164 -> 131 us.
+__global__ void k_state_in(GridGeom g, const double* __restrict__ src, double* __restrict__ W, Ctrl* ctrl, double t0)
+{
+    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id == 0) reset_ctrl(ctrl, t0);
+    state_in(g, src, W, id, (long long)gridDim.x * blockDim.x);
+}
+
+// The same for the allocation-free step, whose descriptor travels as the launch's argument.
+__global__ void k_noalloc_in(SolveDesc d, SolveDesc* self, const double* __restrict__ src)
+{
+    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id == 0) {
+        *self = d;
+        reset_ctrl(d.ctrl, 0.0);
+    }
+    state_in(d.P.g, src, d.W, id, (long long)gridDim.x * blockDim.x);
 }
 
 // warp-aggregated counter add
@@ -1108,7 +1152,8 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
         for (int k = 0; k < NV; k++) { o0[k] = nan; o1[k] = nan; }
     }
     }
-    // the segment flux (Gauss weights 1/2): the Gauss point 1 warp hands its fluxes to its partner
+    // the segment flux, the sum over the two Gauss points (their weight 1/2 is in the update's 1/dx, exactly):
+    // the Gauss point 1 warp hands its fluxes to its partner
     // through shared memory
     if constexpr (DIM == 2) {
         // [output component][lane pair]
@@ -1125,8 +1170,8 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
         if (g == 1 || !valid) return;
 #pragma unroll
         for (int k = 0; k < NV; k++) {
-            o0[k] = fma(0.5, o0[k], 0.5 * pair[k * ps]);
-            if (STAGE == 0) o1[k] = fma(0.5, o1[k], 0.5 * pair[(NV + k) * ps]);
+            o0[k] += pair[k * ps];
+            if (STAGE == 0) o1[k] += pair[(NV + k) * ps];
         }
     } else {
         if (!valid) return;
@@ -1212,8 +1257,8 @@ __device__ __forceinline__ void b_flux_small(const Params& P, const Sweep& S, Ct
             const double* c1 = col + 32;          // Gauss point 1 of the same segment
 #pragma unroll
             for (int k = 0; k < NV; k++) {
-                o0[k] = fma(0.5, o0[k], 0.5 * c1[k * cols]);
-                if (STAGE == 0) o1[k] = fma(0.5, o1[k], 0.5 * c1[(NV + k) * cols]);
+                o0[k] += c1[k * cols];
+                if (STAGE == 0) o1[k] += c1[(NV + k) * cols];
             }
         }
     }
@@ -1276,7 +1321,8 @@ __device__ __forceinline__ void b_update(const Params& P, const Sweep& Sx, const
     if (id >= n) return;
     int i = (int)(id % g.nx), j = (int)(id / g.nx);
     long long cell = g.origin + (long long)j * g.pitch + i;
-    const double inv_dx = Sx.inv_hn, inv_dy = DIM == 2 ? Sy.inv_hn : 0.0;   // 1/dx, 1/dy (host-divided)
+    // 1/dx, 1/dy (host-divided), in 2D times the Gauss weight 1/2 of the segment fluxes
+    const double inv_dx = DIM == 2 ? scale2<-1>(Sx.inv_hn) : Sx.inv_hn, inv_dy = DIM == 2 ? scale2<-1>(Sy.inv_hn) : 0.0;
     long long perx = (long long)Sx.nt * Sx.nm, pery = DIM == 2 ? (long long)Sy.nt * Sy.nm : 0;
     long long ox = (long long)j * Sx.nm + i, oy = (long long)i * (DIM == 2 ? Sy.nm : 0) + j;
     double out[NV], acc[NV];
@@ -1313,8 +1359,8 @@ __device__ __forceinline__ void b_update(const Params& P, const Sweep& Sx, const
         stc(Wout + cell + (long long)k * g.plane, out[k], g);
         if (STAGE == 0) stc(Acc + cell + (long long)k * g.plane, acc[k], g);
     }
-    // rho > 0 and p > 0, the latter as rho E - |m|^2/2 > 0 (no division; first in FP32, see surely_physical)
-    if (surely_physical(fixed::to_float(out[0]), fixed::to_float(out[1]), DIM == 2 ? fixed::to_float(out[2]) : 0.0f,
+    // rho > 0 and p > 0, the latter as rho E - |m|^2/2 > 0 (no division; first in FP32, see fixed::surely_physical)
+    if (fixed::surely_physical(fixed::to_float(out[0]), fixed::to_float(out[1]), DIM == 2 ? fixed::to_float(out[2]) : 0.0f,
                         fixed::to_float(out[NV - 1])))
         return;
     double ke = DIM == 2 ? 0.5 * fma(out[1], out[1], out[2] * out[2]) : 0.5 * out[1] * out[1];
@@ -1826,6 +1872,30 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
         }
         mark(BK_UPD, 1);
     }
+    return cudaGetLastError();
+}
+
+static unsigned int copy_blocks(const GridGeom& g)
+{
+    const unsigned int b = blocks_for((long long)g.nv * g.ny * g.nx, TPB), cap = (unsigned)device_sm_count() * 16;
+    return b < cap ? b : cap;
+}
+
+cudaError_t launch_state_in(hgks_solver* s, const double* W, double t0)
+{
+    k_state_in<<<copy_blocks(s->P.g), TPB, 0, s->stream>>>(s->P.g, W, s->W, s->ctrl, t0);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_noalloc_in(hgks_solver* s, const SolveDesc& self, const double* W)
+{
+    k_noalloc_in<<<copy_blocks(s->P.g), TPB, 0, s->stream>>>(self, s->d_self, W);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_state_out(hgks_solver* s, double* W)
+{
+    k_state_out<<<copy_blocks(s->P.g), TPB, 0, s->stream>>>(s->P.g, s->W, W);
     return cudaGetLastError();
 }
 

@@ -492,20 +492,12 @@ __device__ __forceinline__ bool nonphysical_exact(const double* Q)
     return !(positive(Q[0]) && positive(pr.v));
 }
 
-// First in FP32: the truncated components and the products err by less than 2^-20 of each term, so a difference
-// above 4e-6 of rho E (both factors within 1e-12..1e12, where no product leaves the range) is positive and the
-// state physical without an FP64 instruction.  Anything else goes to the exact test.
+// First in FP32 (fixed::surely_physical); only a state next to vacuum takes the exact test.
 #if defined(__CUDACC__)
-__device__ __forceinline__ bool surely_physical(float rho, float mx, float my, float E)
-{
-    const float re = rho * E, ke = 0.5f * fmaf(mx, mx, my * my);
-    return rho > 1e-12f && rho < 1e12f && E > 1e-12f && E < 1e12f && re - ke > 4e-6f * re;
-}
-
 template <int NV>
 __device__ __forceinline__ bool nonphysical(const double* Q)
 {
-    if (surely_physical(fixed::to_float(Q[0]), fixed::to_float(Q[1]), NV == 4 ? fixed::to_float(Q[2]) : 0.0f,
+    if (fixed::surely_physical(fixed::to_float(Q[0]), fixed::to_float(Q[1]), NV == 4 ? fixed::to_float(Q[2]) : 0.0f,
                         fixed::to_float(Q[NV - 1])))
         return false;
     return nonphysical_exact<NV>(Q);
@@ -519,7 +511,7 @@ __device__ __forceinline__ bool nonphysical_x4(double v, int lane0, unsigned gma
     const float f = fixed::to_float(v);
     const float rho = __shfl_sync(gmask, f, lane0), mx = __shfl_sync(gmask, f, lane0 + 1);
     const float my = NV == 4 ? __shfl_sync(gmask, f, lane0 + 2) : 0.0f, E = __shfl_sync(gmask, f, lane0 + NV - 1);
-    if (surely_physical(rho, mx, my, E)) return false;             // the same for the 4 lanes
+    if (fixed::surely_physical(rho, mx, my, E)) return false;             // the same for the 4 lanes
     double Q[NV];
 #pragma unroll
     for (int k = 0; k < NV; k++) Q[k] = __shfl_sync(gmask, v, lane0 + k);

@@ -101,6 +101,25 @@ int main(int argc, char** argv)
         printf("%ld %d\n", wrong, taken > n / 2 ? 1 : 0);
         return 0;
     }
+    if (!strcmp(what, "physical")) {
+        // never true for a state that is not physical; true from 1e-5 of rho E on
+        long wrong = 0, missed = 0, yes = 0;
+        for (long i = 0; i < 400000; i++) {
+            const double rho = std::exp(40.0 * U(g) - 20.0), u = 2000.0 * (U(g) - 0.5), v = i & 1 ? 2000.0 * (U(g) - 0.5) : 0.0;
+            const double rel = (i % 3 ? 1.0 : -1.0) * std::exp(-U(g) * 25.0), ke = 0.5 * rho * (u * u + v * v);
+            const double E = ke / (1.0 - (rel < 0.9 ? rel : 0.9));
+            const long double pr = (long double)E * rho - 0.5L * ((long double)(rho * u) * (rho * u) + (long double)(rho * v) * (rho * v));
+            const bool s = surely_physical(to_float(rho), to_float(rho * u), to_float(rho * v), to_float(E));
+            wrong += s && !(pr > 0);
+            yes += s;
+            missed += !s && rel > 1e-5 && E < 1e12 && E > 1e-12 && rho > 1e-12 && rho < 1e12;
+        }
+        for (double bad : {0.0, -1.0, std::numeric_limits<double>::infinity(), std::numeric_limits<double>::quiet_NaN(), 1e-320, 1e300})
+            wrong += surely_physical(to_float(bad), 0.0f, 0.0f, 1.0f) + surely_physical(1.0f, 0.0f, 0.0f, to_float(bad))
+                   + (std::isfinite(bad) && std::fabs(bad) < 1.4 ? 0 : surely_physical(1.0f, to_float(bad), 0.0f, 1.0f));
+        printf("%ld %d\n", wrong + missed, yes > 100000 ? 1 : 0);
+        return 0;
+    }
     if (!strcmp(what, "special")) {
         const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
         bool ok = true;
@@ -168,5 +187,7 @@ def test_gauss_point_quartic(exe):
     assert ok == "1" and float(wv) <= 1.0 and float(wd) <= 1.0, (ok, wv, wd)
 
 
-def test_ieee_division_and_root(exe):
-    assert subprocess.run([exe, "ieee"], check=True, capture_output=True, text=True).stdout.split() == ["0", "1"]
+@pytest.mark.parametrize("what", ["ieee", "physical"])
+def test_exact_decisions(exe, what):
+    """IEEE quotients and roots bit for bit; the FP32 positivity test against the exact sign."""
+    assert subprocess.run([exe, what], check=True, capture_output=True, text=True).stdout.split() == ["0", "1"]

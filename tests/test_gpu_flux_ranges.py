@@ -22,8 +22,6 @@ CASES = {
     # U / sqrt(2 h) = 7.9 and 8.1 (both sides of the switch within the wave), and far beyond
     "mach_edge": dict(u=8.0 * np.sqrt(2.0), p0=1.0, amp=0.02),
     "mach_20": dict(u=-24.0, p0=1.0, amp=0.02),
-    # (rho E - |m|^2/2)/(rho E) = 2.5e-6..1e-5: both sides of the FP32 positivity test's margin of 4e-6
-    "pressure_next_to_zero": dict(u=1000.0, p0=1.0, amp=0.3),
     # c1 = 0: tau = c2 |dp| / sum p dt, tiny where the pressure is nearly flat
     "stiff_tau": dict(u=0.3, p0=1.0, amp=1e-4, c1=0.0),
     "zero_tau_flat_pressure": dict(u=0.3, p0=1.0, amp=0.0, c1=0.0),
