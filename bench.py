@@ -59,7 +59,7 @@ WORKLOAD = "four-quadrant 2D Riemann problem, 1024^2 cells, hybrid WENO-AO HGKS,
 # two), kept fixed here so that the yardstick does not move when a kernel changes:
 # * the flux per Gauss point: the closed form of the flux kernel (2D Euler, tau > 0), counted on
 #   the host by paper_2304_05572_gb300/flopcount.py: 1433 operations in the first stage (F(dt/2)
-#   and the F^n + dt/6 dF^n combination), 1389 in the second; on sweeps of 65 536 segments or
+#   and the F^n + dt/6 dF^n combination), 1389 in the second; on sweeps of 49 152 segments or
 #   more the kernel also reconstructs its Gauss point's smooth tangential passes
 #   (FLUX_KERNEL_TANG_FLOP_PER_GP); one launch covers both sweeps of a stage;
 # * the rest of the step per cell-stage (indicator, reconstruction, update, time step), counted on
@@ -645,9 +645,9 @@ def main():
     if flux_calls:
         avg_ms = flux_ms / flux_calls
         gp_per_launch = 2 * 2 * (n + 1) * n      # Gauss points of both sweeps (one launch per stage)
-        # the kernel's work per Gauss point: the flux, and on sweeps of 65 536 segments or more the
+        # the kernel's work per Gauss point: the flux, and on sweeps of 49 152 segments or more the
         # fused reconstruction of the smooth tangential passes
-        per_gp = FLUX_ALG_FLOP_PER_GP + (FLUX_KERNEL_TANG_FLOP_PER_GP if n * (n + 1) >= 65536 else 0.0)
+        per_gp = FLUX_ALG_FLOP_PER_GP + (FLUX_KERNEL_TANG_FLOP_PER_GP if n * (n + 1) >= 49152 else 0.0)
         achieved = per_gp * gp_per_launch / (avg_ms * 1e-3) / 1e12
         roofline = {"bound": "alu", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
                     "frac": achieved / peak_tflops,

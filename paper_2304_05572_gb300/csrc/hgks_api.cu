@@ -143,7 +143,7 @@ void fill_sweeps(const hgks_config* c, const Params& P, Sweep* sw)
         S.nlines = c->dim == 2 ? S.nt + 6 : 1;
         // small sweeps spread an item over lanes (shorter FP64 chains per thread) and take one launch per
         // reconstruction direction; the line is placed by measurement (see k_normal_small)
-        S.small = (long long)S.nt * S.nm < 65536 ? 1 : 0;
+        S.small = (long long)S.nt * S.nm < 49152 ? 1 : 0;
         S.tlo = c->dim == 2 ? -3 : 0;
         S.sN = d == 0 ? 1 : g.pitch;
         S.sT = d == 0 ? g.pitch : 1;

@@ -48,7 +48,7 @@ struct Sweep {
     int nn, nt;                // cells normal / tangential
     int nm;                    // interfaces per line (nn + 1)
     int nlines;                // lines with normal reconstruction (nt + 6 in 2D, 1 in 1D)
-    int small;                 // below 65536 interface segments: one launch per reconstruction direction (lane groups)
+    int small;                 // below 49152 interface segments: one launch per reconstruction direction (lane groups)
     int tlo;                   // first line index (-3 in 2D, 0 in 1D)
     long long sN, sT;          // state strides for +1 in n / t
     int perm[4];               // local component -> global component

@@ -44,19 +44,31 @@ __device__ __forceinline__ bool in_range(const T* p, const char* lo, const char*
     return false;
 }
 template <class T, class R>
-__device__ __forceinline__ T ldc(const T* p, const R& r) { return in_range(p, r.lo, r.hi) ? __ldg(p) : T(0); }
+__device__ __forceinline__ T ldc(const T* p, const R& r) { return in_range(p, r.lo, r.hi) ? *p : T(0); }
 template <class T, class R>
 __device__ __forceinline__ T rdc(const T* p, const R& r) { return in_range(p, r.lo, r.hi) ? *p : T(0); }
 template <class T, class V, class R>
 __device__ __forceinline__ void stc(T* p, V v, const R& r) { if (in_range(p, r.lo, r.hi)) *p = (T)v; }
 #else
 template <class T, class R>
-__device__ __forceinline__ T ldc(const T* p, const R&) { return __ldg(p); }
+__device__ __forceinline__ T ldc(const T* p, const R&) { return *p; }
 template <class T, class R>
 __device__ __forceinline__ T rdc(const T* p, const R&) { return *p; }
 template <class T, class V, class R>
 __device__ __forceinline__ void stc(T* p, V v, const R&) { *p = (T)v; }
 #endif
+
+// Entry of every kernel of a step.  The step's launches carry the programmatic-serialisation attribute: a
+// launch is set up while the one before it drains, and waits here until that one is complete and its
+// memory visible, before anything is read (so loads are plain ones, not through the read-only path, whose
+// data must not change while a kernel is resident).  About 2.5 us less per launch: a step of 200 cells in 1D 79 ->
+// 60 us, of 48 x 48 four-quadrant 155 -> 131, of 1024^2 9.76 -> 9.71 ms.  The next launch is not let in early
+// (launch_dependents at the start): its waiting blocks then crowd onto the multiprocessors that were free first (8191
+// cells 84 -> 116 us, 48 x 48 155 -> 219).
+__device__ __forceinline__ void pdl_enter()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // ---------------------------------------------------------------- ghost cells
 // x ghosts on interior rows, then y ghosts over the padded width (fills corners).
@@ -111,7 +123,7 @@ inline long long ghost_threads(const GridGeom& g)
     return g.dim == 2 ? x + (long long)g.nv * (g.nx + 2 * NG) * NG * 2 : x;
 }
 
-__device__ __forceinline__ void b_ghost(const Params& P, double* W, Ctrl* __restrict__ ctrl, int stage, long long id)
+__device__ __forceinline__ void b_ghost(const Params& P, double* W, Ctrl* ctrl, int stage, long long id)
 {
     if (id == 0) ctrl->cnt[0][0] = ctrl->cnt[0][1] = ctrl->cnt[1][0] = ctrl->cnt[1][1] = 0;
     const GridGeom& g = P.g;
@@ -162,8 +174,9 @@ __device__ __forceinline__ void b_ghost(const Params& P, double* W, Ctrl* __rest
 }
 
 // Second stage (W*)
-__global__ void k_ghost(Params P, double* W, Ctrl* __restrict__ ctrl)
+__global__ void k_ghost(Params P, double* W, Ctrl* ctrl)
 {
+    pdl_enter();
     if (ctrl->done) return;
     b_ghost(P, W, ctrl, 1, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
@@ -171,7 +184,7 @@ __global__ void k_ghost(Params P, double* W, Ctrl* __restrict__ ctrl)
 // ---------------------------------------------------------------- time step
 // Sec. 3 preamble: dt = CFL min(h/(|U|+a), h^2/(4 nu)), h = min(dx, dy), nu = mu/rho;
 // same evaluation order as the CPU reference so that dt is reproduced exactly.
-__device__ __forceinline__ void b_dt(const Params& P, const double* __restrict__ W, Ctrl* ctrl, double h, long long start, long long stride)
+__device__ __forceinline__ void b_dt(const Params& P, const double* W, Ctrl* ctrl, double h, long long start, long long stride)
 {
     const GridGeom& g = P.g;
     int rowsI = g.dim == 2 ? g.ny : 1;
@@ -230,6 +243,7 @@ __device__ __forceinline__ void dt_finish(const Params& P, Ctrl* ctrl, double t_
 // for what took five (work-list reset, dt, its decision, two ghost fills).
 __global__ void k_dt_ghost(Params P, double* W, Ctrl* ctrl, double h, double t_end, int nb)
 {
+    pdl_enter();
     const int b = (int)blockIdx.x;
     if (b >= nb) {
         b_ghost(P, W, ctrl, 0, (long long)(b - nb) * blockDim.x + threadIdx.x);
@@ -239,8 +253,9 @@ __global__ void k_dt_ghost(Params P, double* W, Ctrl* ctrl, double h, double t_e
     dt_finish(P, ctrl, t_end, (unsigned)nb);
 }
 
-__global__ void k_state_out(GridGeom g, const double* __restrict__ W, double* __restrict__ dst)
+__global__ void k_state_out(GridGeom g, const double* W, double* dst)
 {
+    pdl_enter();
     const long long n = (long long)g.nv * g.ny * g.nx;
     for (long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x; id < n; id += (long long)gridDim.x * blockDim.x) {
         const long long row = id / g.nx;
@@ -280,16 +295,18 @@ __device__ __forceinline__ void state_in(const GridGeom& g, const double* src, d
 // of a pitched copy each and a launch for the control block: 8 steps of a 200-cell tube with both
 // transfers 714 -> 691 us, a 48 x 48 allocation-free step (which also copied its descriptor and cleared
 // its 3.5 MB) 164 -> 131 us.
-__global__ void k_state_in(GridGeom g, const double* __restrict__ src, double* __restrict__ W, Ctrl* ctrl, double t0)
+__global__ void k_state_in(GridGeom g, const double* src, double* W, Ctrl* ctrl, double t0)
 {
+    pdl_enter();
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (id == 0) reset_ctrl(ctrl, t0);
     state_in(g, src, W, id, (long long)gridDim.x * blockDim.x);
 }
 
 // The same for the allocation-free step, whose descriptor travels as the launch's argument.
-__global__ void k_noalloc_in(SolveDesc d, SolveDesc* self, const double* __restrict__ src)
+__global__ void k_noalloc_in(SolveDesc d, SolveDesc* self, const double* src)
 {
+    pdl_enter();
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (id == 0) {
         *self = d;
@@ -327,7 +344,7 @@ __device__ __forceinline__ const double* cellp(const Params& P, const Sweep& S, 
 }
 
 template <int NV>
-__device__ __forceinline__ void b_raw_nflags(const Params& P, const Sweep& S, const double* __restrict__ W, const Ctrl* __restrict__ ctrl, long long id)
+__device__ __forceinline__ void b_raw_nflags(const Params& P, const Sweep& S, const double* W, const Ctrl* ctrl, long long id)
 {
     if (ctrl->done) return;
     int width = S.nn + 4;
@@ -369,8 +386,9 @@ __device__ __forceinline__ SweepBlock sweep_block(int nb0)
 }
 
 template <int NV>
-__global__ void k_raw_nflags(const SolveDesc* __restrict__ D, int nb0, int stage)
+__global__ void k_raw_nflags(const SolveDesc* D, int nb0, int stage)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     const SolveDesc& d = *D;
     b_raw_nflags<NV>(d.P, d.sw[b.dir], stage == 0 ? d.W : d.Ws, d.ctrl, b.id);
@@ -390,7 +408,7 @@ __device__ __forceinline__ void store_line(const Params& P, const Sweep& S, int 
 }
 
 template <int NV>
-__device__ __forceinline__ void b_normal(const Params& P, const Sweep& S, const double* __restrict__ W, Ctrl* ctrl, int stage, long long id)
+__device__ __forceinline__ void b_normal(const Params& P, const Sweep& S, const double* W, Ctrl* ctrl, int stage, long long id)
 {
     if (ctrl->done) return;
     long long total = (long long)S.nlines * S.nm;
@@ -444,8 +462,9 @@ __device__ __forceinline__ void b_normal(const Params& P, const Sweep& S, const 
 }
 
 template <int NV>
-__global__ void k_normal(const SolveDesc* __restrict__ D, int nb0, int stage)
+__global__ void k_normal(const SolveDesc* D, int nb0, int stage)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     const SolveDesc& d = *D;
     b_normal<NV>(d.P, d.sw[b.dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, b.id);
@@ -464,7 +483,7 @@ constexpr unsigned int kAoOneLaneMin = 32768;
 // The window (cells i-2..i+2 across the face, all components) and the face average of the
 // troubled side `it` of the normal pass.
 template <int NV>
-__device__ __forceinline__ void normal_ao_item(const Params& P, const Sweep& S, const double* __restrict__ W, uint32_t it,
+__device__ __forceinline__ void normal_ao_item(const Params& P, const Sweep& S, const double* W, uint32_t it,
                                                double (*Qw)[NV], double* Qs, int& side, int& L, int& m)
 {
     side = it & 1;
@@ -491,7 +510,7 @@ __device__ __forceinline__ void normal_ao_item(const Params& P, const Sweep& S, 
 // field q and stores component q).  Both forms give the same bits.  `lane`, `lanes`: this
 // thread's index among, and the number of, the lanes working on the pass.
 template <int NV>
-__device__ __forceinline__ void b_normal_ao(const Params& P, const Sweep& S, const double* __restrict__ W, const Ctrl* __restrict__ ctrl, long long lane, long long lanes)
+__device__ __forceinline__ void b_normal_ao(const Params& P, const Sweep& S, const double* W, const Ctrl* ctrl, long long lane, long long lanes)
 {
     if (ctrl->done) return;
     unsigned int n = ctrl->cnt[S.dir][0];
@@ -541,8 +560,9 @@ __device__ __forceinline__ void b_normal_ao(const Params& P, const Sweep& S, con
 }
 
 template <int NV>
-__global__ void k_normal_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
+__global__ void k_normal_ao(const SolveDesc* D, int nb0, int stage)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     const SolveDesc& d = *D;
     b_normal_ao<NV>(d.P, d.sw[b.dir], stage == 0 ? d.W : d.Ws, d.ctrl, b.id, b.lanes);
@@ -558,11 +578,11 @@ __global__ void k_normal_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
 // Such a sweep's time is made of launches (3 us each) and of each thread's chain of FP64 instructions (31 ns
 // each): with one launch per direction in place of three (flags, linear pass, compacted WENO-AO) and the
 // step's five control and ghost launches in two, a step of 200 cells in 1D went from 133 to 90 us, of
-// 48 x 48 from 210 to 136.  Compaction and shared flags pay from about 65536 segments on.
+// 48 x 48 from 210 to 136.  Compaction and shared flags pay from about 49152 segments on
 constexpr int kSmallCells = 6;
 
 template <int NV>
-__device__ __forceinline__ void b_normal_small(const Params& P, const Sweep& S, const double* __restrict__ W, Ctrl* ctrl, int stage, long long id)
+__device__ __forceinline__ void b_normal_small(const Params& P, const Sweep& S, const double* W, Ctrl* ctrl, int stage, long long id)
 {
     if (ctrl->done) return;
     const unsigned full = 0xffffffffu;
@@ -636,8 +656,9 @@ __device__ __forceinline__ void b_normal_small(const Params& P, const Sweep& S, 
 }
 
 template <int NV>
-__global__ void k_normal_small(const SolveDesc* __restrict__ D, int nb0, int stage)
+__global__ void k_normal_small(const SolveDesc* D, int nb0, int stage)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     const SolveDesc& d = *D;
     b_normal_small<NV>(d.P, d.sw[b.dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, b.id);
@@ -654,7 +675,7 @@ __device__ __forceinline__ double lineval(const Sweep& S, int X, int k, int t, i
 // loaded and truncated once for up to 5 windows (8 rows instead of 20 for 4 segments).
 constexpr int kTRows = 4;
 
-__device__ __forceinline__ void b_raw_tflags(const Params& P, const Sweep& S, const Ctrl* __restrict__ ctrl, long long id)
+__device__ __forceinline__ void b_raw_tflags(const Params& P, const Sweep& S, const Ctrl* ctrl, long long id)
 {
     if (ctrl->done) return;
     const int m = (int)(id % S.nm);
@@ -689,8 +710,9 @@ __device__ __forceinline__ void b_raw_tflags(const Params& P, const Sweep& S, co
 // Threads of the raw tangential flag kernel on sweep S.
 inline long long raw_t_threads(const Sweep& S) { return (long long)((S.nt + 2 + kTRows - 1) / kTRows) * S.nm; }
 
-__global__ void k_raw_tflags(const SolveDesc* __restrict__ D, int nb0)
+__global__ void k_raw_tflags(const SolveDesc* D, int nb0)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     const SolveDesc& d = *D;
     b_raw_tflags(d.P, d.sw[b.dir], d.ctrl, b.id);
@@ -737,8 +759,9 @@ __device__ __forceinline__ void b_tang(const Params& P, const Sweep& S, Ctrl* ct
     }
 }
 
-__global__ void k_tang(const SolveDesc* __restrict__ D, int nb0, int stage)
+__global__ void k_tang(const SolveDesc* D, int nb0, int stage)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     const SolveDesc& d = *D;
     b_tang(d.P, d.sw[b.dir], d.ctrl, stage, b.id);
@@ -747,7 +770,7 @@ __global__ void k_tang(const SolveDesc* __restrict__ D, int nb0, int stage)
 
 // The troubled tangential pass `it`: its pass X, segment (t, m), the eigenvectors at the face
 // average (tangential direction) and the pass's 5 line values.
-__device__ __forceinline__ void tang_ao_item(const Params& P, const Sweep& S, const double* __restrict__ W, uint32_t it,
+__device__ __forceinline__ void tang_ao_item(const Params& P, const Sweep& S, const double* W, uint32_t it,
                                              int& X, int& t, int& m, TangEig& e, double (*x)[4])
 {
     X = it & 3;
@@ -772,7 +795,7 @@ __device__ __forceinline__ void tang_ao_item(const Params& P, const Sweep& S, co
 // per aligned group of 4 lanes (tang_ao_x4, lane q computes and stores component q).  Free-order
 // arithmetic (the outputs only feed the flux).  `lane`, `lanes`: this thread's index among, and
 // the number of, the lanes working on the pass.
-__device__ __forceinline__ void b_tang_ao(const Params& P, const Sweep& S, const double* __restrict__ W, const Ctrl* __restrict__ ctrl, long long lane, long long lanes)
+__device__ __forceinline__ void b_tang_ao(const Params& P, const Sweep& S, const double* W, const Ctrl* ctrl, long long lane, long long lanes)
 {
     if (ctrl->done) return;
     unsigned int n = ctrl->cnt[S.dir][1];
@@ -836,8 +859,9 @@ __device__ __noinline__ void tang_ao_nl(const SolveDesc& d, int dir, int stage, 
     b_tang_ao(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, lane, lanes);
 }
 
-__global__ void k_tang_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
+__global__ void k_tang_ao(const SolveDesc* D, int nb0, int stage)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     tang_ao_nl(*D, b.dir, stage, b.id, b.lanes);
 }
@@ -851,7 +875,7 @@ __global__ void k_tang_ao(const SolveDesc* __restrict__ D, int nb0, int stage)
 // on `rows`, which is chosen for the number of blocks.
 constexpr int kSmallCols = 8, kSmallRowsMax = 8, kSmallTangBlock = 128;
 
-__device__ __forceinline__ void b_tang_small(const Params& P, const Sweep& S, const double* __restrict__ W, Ctrl* ctrl, int stage,
+__device__ __forceinline__ void b_tang_small(const Params& P, const Sweep& S, const double* W, Ctrl* ctrl, int stage,
                                              unsigned block, int rows)
 {
     __shared__ uint8_t s_flag[4][kSmallRowsMax][kSmallCols];
@@ -969,8 +993,9 @@ __device__ __noinline__ void tang_small_nl(const SolveDesc& d, int dir, int stag
     b_tang_small(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, block, rows);
 }
 
-__global__ void __launch_bounds__(kSmallTangBlock) k_tang_small(const SolveDesc* __restrict__ D, int nb0, int stage, int rows)
+__global__ void __launch_bounds__(kSmallTangBlock) k_tang_small(const SolveDesc* D, int nb0, int stage, int rows)
 {
+    pdl_enter();
     const int dir = (int)blockIdx.x >= nb0 ? 1 : 0;
     tang_small_nl(*D, dir, stage, blockIdx.x - (dir ? (unsigned)nb0 : 0u), rows);
 }
@@ -988,7 +1013,7 @@ inline size_t flux_smem(int dim, int threads)
 // State, tangential and normal derivative of one side (0: left, 1: right) of segment (t, m) at both Gauss
 // points (2D, large sweeps): the troubled passes from k_tang_ao, the smooth ones reconstructed
 // here.  x[(12 g + j) stride]: j = 0..3 state, 4..7 normal, 8..11 tangential derivative at Gauss point g.
-__device__ __forceinline__ void side_pair(const Params& P, const Sweep& S, int side, long long o, double* __restrict__ x, int stride)
+__device__ __forceinline__ void side_pair(const Params& P, const Sweep& S, int side, long long o, double* x, int stride)
 {
     const long long per = (long long)S.nt * S.nm;
     const unsigned bits = rdc(S.flagT + o, S);
@@ -1282,8 +1307,9 @@ __device__ __noinline__ void flux_nl(const SolveDesc& d, int dir, long long id)
 // 8 warps per SM) lets the flux keep its working set in registers (measured 3.5 % faster than
 // under a 128-thread bound at the same occupancy)
 template <int DIM, int STAGE, bool PRFIX>
-__global__ void __launch_bounds__(64, 4) k_flux(const SolveDesc* __restrict__ D, int nb0)
+__global__ void __launch_bounds__(64, 4) k_flux(const SolveDesc* D, int nb0)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     flux_nl<DIM, STAGE, PRFIX>(*D, b.dir, b.id);
 }
@@ -1297,8 +1323,9 @@ __device__ __noinline__ void flux_small_nl(const SolveDesc& d, int dir, long lon
 constexpr int kFluxSmallBlock = 128;
 
 template <int DIM, int STAGE, bool PRFIX>
-__global__ void __launch_bounds__(kFluxSmallBlock) k_flux_small(const SolveDesc* __restrict__ D, int nb0)
+__global__ void __launch_bounds__(kFluxSmallBlock) k_flux_small(const SolveDesc* D, int nb0)
 {
+    pdl_enter();
     const SweepBlock b = sweep_block(nb0);
     flux_small_nl<DIM, STAGE, PRFIX>(*D, b.dir, b.id);
 }
@@ -1306,7 +1333,7 @@ __global__ void __launch_bounds__(kFluxSmallBlock) k_flux_small(const SolveDesc*
 // Stage 0: W* = W^n - dF(dt/2)/dx - dG(dt/2)/dy (Eq. (19)), Acc = W^n - d(dt F^n + dt^2/6 dF^n)/dx - ...
 // Stage 1: W^{n+1} = Acc - d(dt^2/3 dF*)/dx - ... (Eqs. (20)-(22))
 template <int DIM, int STAGE>
-__device__ __forceinline__ void b_update(const Params& P, const Sweep& Sx, const Sweep& Sy, const double* __restrict__ Win, double* __restrict__ Wout, double* __restrict__ Acc, Ctrl* ctrl, long long id)
+__device__ __forceinline__ void b_update(const Params& P, const Sweep& Sx, const Sweep& Sy, const double* Win, double* Wout, double* Acc, Ctrl* ctrl, long long id)
 {
     if (ctrl->done) return;
     if (STAGE == 1 && id == 0) {              // the end of the step (no thread of this launch reads these)
@@ -1369,9 +1396,10 @@ __device__ __forceinline__ void b_update(const Params& P, const Sweep& Sx, const
 }
 
 template <int DIM, int STAGE>
-__global__ void k_update(Params P, Sweep Sx, Sweep Sy, const double* __restrict__ Win, double* __restrict__ Wout,
-                         double* __restrict__ Acc, Ctrl* ctrl)
+__global__ void k_update(Params P, Sweep Sx, Sweep Sy, const double* Win, double* Wout,
+                         double* Acc, Ctrl* ctrl)
 {
+    pdl_enter();
     b_update<DIM, STAGE>(P, Sx, Sy, Win, Wout, Acc, ctrl, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -1380,7 +1408,7 @@ __global__ void k_update(Params P, Sweep Sx, Sweep Sy, const double* __restrict_
 // One launch per kernel class covers the blocks of every solver of a batch: block b belongs
 // to solver s with boff[s] <= b < boff[s+1] and runs that solver's kernel body on its local
 // block index.  No block mixes solvers, so every result is bit-identical to stepping alone.
-__device__ __forceinline__ int find_solve(const int* __restrict__ boff, int n, int b)
+__device__ __forceinline__ int find_solve(const int* boff, int n, int b)
 {
     int lo = 0, hi = n;
     while (hi - lo > 1) {
@@ -1408,89 +1436,102 @@ __device__ __forceinline__ int find_solve(const int* __restrict__ boff, int n, i
     const long long id = lblk_ * blockDim.x + threadIdx.x;                               \
     (void)nblk_; (void)id;
 
-__global__ void kb_dt(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, const double* __restrict__ tend)
+__global__ void kb_dt(const SolveDesc* D, const int* boff, int n, const double* tend)
 {
+    pdl_enter();
     HGKS_BATCH_BLOCK();
     if (!(d.P.fixed_dt > 0.0)) b_dt(d.P, d.W, d.ctrl, d.h, id, nblk_ * blockDim.x);
     dt_finish(d.P, d.ctrl, tend[s_], (unsigned)nblk_);
 }
 
-__global__ void kb_ghost(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+__global__ void kb_ghost(const SolveDesc* D, const int* boff, int n, int stage)
 {
+    pdl_enter();
     HGKS_BATCH_BLOCK();
     if (d.ctrl->done) return;
     b_ghost(d.P, stage == 0 ? d.W : d.Ws, d.ctrl, stage, id);
 }
 
 template <int NV>
-__global__ void kb_raw_nflags(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+__global__ void kb_raw_nflags(const SolveDesc* D, const int* boff, int n, int stage)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     b_raw_nflags<NV>(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, id);
 }
 
 template <int NV>
-__global__ void kb_normal(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+__global__ void kb_normal(const SolveDesc* D, const int* boff, int n, int stage)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     b_normal<NV>(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, id);
 }
 
 template <int NV>
-__global__ void kb_normal_ao(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+__global__ void kb_normal_ao(const SolveDesc* D, const int* boff, int n, int stage)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     b_normal_ao<NV>(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, id, nblk_ * blockDim.x);
 }
 
 template <int NV>
-__global__ void kb_normal_small(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+__global__ void kb_normal_small(const SolveDesc* D, const int* boff, int n, int stage)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     b_normal_small<NV>(d.P, d.sw[dir], stage == 0 ? d.W : d.Ws, d.ctrl, stage, id);
 }
 
-__global__ void __launch_bounds__(kSmallTangBlock) kb_tang_small(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage, int rows)
+__global__ void __launch_bounds__(kSmallTangBlock) kb_tang_small(const SolveDesc* D, const int* boff, int n, int stage, int rows)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     tang_small_nl(d, dir, stage, (unsigned)lblk_, rows);
 }
 
-__global__ void kb_raw_tflags(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
+__global__ void kb_raw_tflags(const SolveDesc* D, const int* boff, int n)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     b_raw_tflags(d.P, d.sw[dir], d.ctrl, id);
 }
 
-__global__ void kb_tang(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+__global__ void kb_tang(const SolveDesc* D, const int* boff, int n, int stage)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     b_tang(d.P, d.sw[dir], d.ctrl, stage, id);
 }
 
-__global__ void kb_tang_ao(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n, int stage)
+__global__ void kb_tang_ao(const SolveDesc* D, const int* boff, int n, int stage)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     tang_ao_nl(d, dir, stage, id, nblk_ * blockDim.x);
 }
 
 template <int DIM, int STAGE, bool PRFIX>
-__global__ void __launch_bounds__(64, 4) kb_flux(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
+__global__ void __launch_bounds__(64, 4) kb_flux(const SolveDesc* D, const int* boff, int n)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     flux_nl<DIM, STAGE, PRFIX>(d, dir, id);
 }
 
 template <int DIM, int STAGE, bool PRFIX>
-__global__ void __launch_bounds__(kFluxSmallBlock) kb_flux_small(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
+__global__ void __launch_bounds__(kFluxSmallBlock) kb_flux_small(const SolveDesc* D, const int* boff, int n)
 {
+    pdl_enter();
     HGKS_BATCH_SWEEP_BLOCK();
     flux_small_nl<DIM, STAGE, PRFIX>(d, dir, id);
 }
 
 template <int DIM, int STAGE>
-__global__ void kb_update(const SolveDesc* __restrict__ D, const int* __restrict__ boff, int n)
+__global__ void kb_update(const SolveDesc* D, const int* boff, int n)
 {
+    pdl_enter();
     HGKS_BATCH_BLOCK();
     if (STAGE == 0) b_update<DIM, 0>(d.P, d.sw[0], d.sw[1], d.W, d.Ws, d.Acc, d.ctrl, id);
     else b_update<DIM, 1>(d.P, d.sw[0], d.sw[1], d.Ws, d.W, d.Acc, d.ctrl, id);
@@ -1619,6 +1660,22 @@ static void timed(hgks_solver* s, int cls, int nkernels, F&& launch)
     s->timers.push_back(TimerRec{cls, a, b});
 }
 
+template <class... K, class... A>
+static void launch_chained(void (*kernel)(K...), unsigned int grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, (K)args...);
+}
+
 // The sweep kernels of one stage, each class one launch over both sweeps (2D): nb[0] blocks for
 // the x sweep, then nb[1] for the y sweep.
 template <int DIM>
@@ -1643,23 +1700,23 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
     };
     unsigned int g;
     if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for((long long)S.nlines * (S.nn + 4), TPB); })))
-        timed(s, KC_RAWN, 1, [&] { k_raw_nflags<NV><<<g, TPB, 0, st>>>(D, (int)nb[0], stage); });
+        timed(s, KC_RAWN, 1, [&] { launch_chained(k_raw_nflags<NV>, g, TPB, 0, st, D, (int)nb[0], stage); });
     if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for((long long)S.nlines * S.nm, TPB); })))
-        timed(s, KC_NORMAL, 1, [&] { k_normal<NV><<<g, TPB, 0, st>>>(D, (int)nb[0], stage); });
+        timed(s, KC_NORMAL, 1, [&] { launch_chained(k_normal<NV>, g, TPB, 0, st, D, (int)nb[0], stage); });
     if ((g = pair(LARGE, [&](const Sweep& S) { return ao_blocks((long long)S.nlines * S.nm * 2 * 4); })))
-        timed(s, KC_NORMAL_AO, 1, [&] { k_normal_ao<NV><<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
+        timed(s, KC_NORMAL_AO, 1, [&] { launch_chained(k_normal_ao<NV>, g, 128, 0, st, D, (int)nb[0], stage); });
     if ((g = pair(SMALL, [](const Sweep& S) { return blocks_for(normal_small_threads(S), 128); })))
-        timed(s, KC_NORMAL, 1, [&] { k_normal_small<NV><<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
+        timed(s, KC_NORMAL, 1, [&] { launch_chained(k_normal_small<NV>, g, 128, 0, st, D, (int)nb[0], stage); });
     if constexpr (DIM == 2) {
         if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for(raw_t_threads(S), TPB); })))
-            timed(s, KC_RAWT, 1, [&] { k_raw_tflags<<<g, TPB, 0, st>>>(D, (int)nb[0]); });
+            timed(s, KC_RAWT, 1, [&] { launch_chained(k_raw_tflags, g, TPB, 0, st, D, (int)nb[0]); });
         if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for((long long)S.nt * S.nm, TPB); })))
-            timed(s, KC_TANG, 1, [&] { k_tang<<<g, TPB, 0, st>>>(D, (int)nb[0], stage); });
+            timed(s, KC_TANG, 1, [&] { launch_chained(k_tang, g, TPB, 0, st, D, (int)nb[0], stage); });
         if ((g = pair(LARGE, [&](const Sweep& S) { return ao_blocks((long long)S.nt * S.nm * 4 * 4); })))
-            timed(s, KC_TANG_AO, 1, [&] { k_tang_ao<<<g, 128, 0, st>>>(D, (int)nb[0], stage); });
+            timed(s, KC_TANG_AO, 1, [&] { launch_chained(k_tang_ao, g, 128, 0, st, D, (int)nb[0], stage); });
         const int rows = tang_small_rows(pair(SMALL, [](const Sweep& S) { return (unsigned)tang_small_blocks(S, 1); }));
         if ((g = pair(SMALL, [&](const Sweep& S) { return (unsigned)tang_small_blocks(S, rows); })))
-            timed(s, KC_TANG, 1, [&] { k_tang_small<<<g, kSmallTangBlock, 0, st>>>(D, (int)nb[0], stage, rows); });
+            timed(s, KC_TANG, 1, [&] { launch_chained(k_tang_small, g, kSmallTangBlock, 0, st, D, (int)nb[0], stage, rows); });
     }
     if (s->capture) {
         for (int d = 0; d < DIM; d++) {
@@ -1673,14 +1730,14 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
         constexpr bool PR = decltype(prfix)::value;
         if ((g = pair(LARGE, [](const Sweep& S) { return blocks_for(flux_threads(DIM, (long long)S.nt * S.nm), 64); })))
             timed(s, KC_FLUX, 1, [&] {
-                if (stage == 0) k_flux<DIM, 0, PR><<<g, 64, flux_smem(DIM, 64), st>>>(D, (int)nb[0]);
-                else k_flux<DIM, 1, PR><<<g, 64, flux_smem(DIM, 64), st>>>(D, (int)nb[0]);
+                if (stage == 0) launch_chained(k_flux<DIM, 0, PR>, g, 64, flux_smem(DIM, 64), st, D, (int)nb[0]);
+                else launch_chained(k_flux<DIM, 1, PR>, g, 64, flux_smem(DIM, 64), st, D, (int)nb[0]);
             });
         constexpr int T = kFluxSmallBlock;
         if ((g = pair(SMALL, [](const Sweep& S) { return blocks_for(flux_small_threads(DIM, (long long)S.nt * S.nm), T); })))
             timed(s, KC_FLUX, 1, [&] {
-                if (stage == 0) k_flux_small<DIM, 0, PR><<<g, T, flux_small_smem(DIM, PR, T), st>>>(D, (int)nb[0]);
-                else k_flux_small<DIM, 1, PR><<<g, T, flux_small_smem(DIM, PR, T), st>>>(D, (int)nb[0]);
+                if (stage == 0) launch_chained(k_flux_small<DIM, 0, PR>, g, T, flux_small_smem(DIM, PR, T), st, D, (int)nb[0]);
+                else launch_chained(k_flux_small<DIM, 1, PR>, g, T, flux_small_smem(DIM, PR, T), st, D, (int)nb[0]);
             });
     };
     if (P.fc.prfix != 0.0) flux(std::true_type{});
@@ -1694,12 +1751,12 @@ static void enqueue_stage(hgks_solver* s, int stage)
     const Params& P = s->P;
     cudaStream_t st = s->stream;
     if (stage == 1)
-        timed(s, KC_GHOST, 1, [&] { k_ghost<<<blocks_for(ghost_threads(P.g), TPB), TPB, 0, st>>>(P, s->Ws, s->ctrl); });
+        timed(s, KC_GHOST, 1, [&] { launch_chained(k_ghost, blocks_for(ghost_threads(P.g), TPB), TPB, 0, st, P, s->Ws, s->ctrl); });
     enqueue_sweeps<DIM>(s, stage);
     timed(s, KC_UPDATE, 1, [&] {
         long long n = (long long)(DIM == 2 ? P.g.ny : 1) * P.g.nx;
-        if (stage == 0) k_update<DIM, 0><<<blocks_for(n, TPB), TPB, 0, st>>>(P, s->sw[0], s->sw[1], s->W, s->Ws, s->Acc, s->ctrl);
-        else k_update<DIM, 1><<<blocks_for(n, TPB), TPB, 0, st>>>(P, s->sw[0], s->sw[1], s->Ws, s->W, s->Acc, s->ctrl);
+        if (stage == 0) launch_chained(k_update<DIM, 0>, blocks_for(n, TPB), TPB, 0, st, P, s->sw[0], s->sw[1], s->W, s->Ws, s->Acc, s->ctrl);
+        else launch_chained(k_update<DIM, 1>, blocks_for(n, TPB), TPB, 0, st, P, s->sw[0], s->sw[1], s->Ws, s->W, s->Acc, s->ctrl);
     });
 }
 
@@ -1716,7 +1773,7 @@ cudaError_t launch_step(hgks_solver* s, double t_end)
             const unsigned int cap = (unsigned)device_sm_count() * 4;
             if (nb > cap) nb = cap;
         }
-        k_dt_ghost<<<nb + blocks_for(ghost_threads(P.g), TPB), TPB, 0, st>>>(P, s->W, s->ctrl, h, t_end, (int)nb);
+        launch_chained(k_dt_ghost, nb + blocks_for(ghost_threads(P.g), TPB), TPB, 0, st, P, s->W, s->ctrl, h, t_end, (int)nb);
     });
     if (P.g.dim == 2) { enqueue_stage<2>(s, 0); enqueue_stage<2>(s, 1); }
     else { enqueue_stage<1>(s, 0); enqueue_stage<1>(s, 1); }
@@ -1820,11 +1877,11 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
     auto grid = [&](int c) { return (unsigned int)plan.nblk[c]; };
     auto tp = [&](int c) { return plan.tpb[c]; };
     mark(BK_DT, 0);
-    kb_dt<<<grid(BK_DT), tp(BK_DT), 0, st>>>(dd, bo(BK_DT), n, dtend);
+    launch_chained(kb_dt, grid(BK_DT), tp(BK_DT), 0, st, dd, bo(BK_DT), n, dtend);
     mark(BK_DT, 1);
     for (int stage = 0; stage < 2; stage++) {
         mark(BK_GHOST, 0);
-        kb_ghost<<<grid(BK_GHOST), tp(BK_GHOST), 0, st>>>(dd, bo(BK_GHOST), n, stage);
+        launch_chained(kb_ghost, grid(BK_GHOST), tp(BK_GHOST), 0, st, dd, bo(BK_GHOST), n, stage);
         mark(BK_GHOST, 1);
         // every sweep class: one launch over both sweeps of every solver it applies to
         auto sweep = [&](int c, auto launch) {
@@ -1834,28 +1891,28 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
             mark(c, 1);
         };
 #define HGKS_BY_DIM(kernel, c) sweep(c, [&] {                                                          \
-            if (dim == 2) kernel<4><<<grid(c), tp(c), 0, st>>>(dd, bo(c), n, stage);                      \
-            else kernel<3><<<grid(c), tp(c), 0, st>>>(dd, bo(c), n, stage); })
+            if (dim == 2) launch_chained(kernel<4>, grid(c), tp(c), 0, st, dd, bo(c), n, stage);                      \
+            else launch_chained(kernel<3>, grid(c), tp(c), 0, st, dd, bo(c), n, stage); })
         HGKS_BY_DIM(kb_raw_nflags, BK_RAWN);
         HGKS_BY_DIM(kb_normal, BK_NORMAL);
         HGKS_BY_DIM(kb_normal_ao, BK_NAO);
         HGKS_BY_DIM(kb_normal_small, BK_NSMALL);
 #undef HGKS_BY_DIM
-        sweep(BK_RAWT, [&] { kb_raw_tflags<<<grid(BK_RAWT), tp(BK_RAWT), 0, st>>>(dd, bo(BK_RAWT), n); });
-        sweep(BK_TANG, [&] { kb_tang<<<grid(BK_TANG), tp(BK_TANG), 0, st>>>(dd, bo(BK_TANG), n, stage); });
-        sweep(BK_TAO, [&] { kb_tang_ao<<<grid(BK_TAO), tp(BK_TAO), 0, st>>>(dd, bo(BK_TAO), n, stage); });
-        sweep(BK_TSMALL, [&] { kb_tang_small<<<grid(BK_TSMALL), kSmallTangBlock, 0, st>>>(dd, bo(BK_TSMALL), n, stage, plan.tang_rows); });
+        sweep(BK_RAWT, [&] { launch_chained(kb_raw_tflags, grid(BK_RAWT), tp(BK_RAWT), 0, st, dd, bo(BK_RAWT), n); });
+        sweep(BK_TANG, [&] { launch_chained(kb_tang, grid(BK_TANG), tp(BK_TANG), 0, st, dd, bo(BK_TANG), n, stage); });
+        sweep(BK_TAO, [&] { launch_chained(kb_tang_ao, grid(BK_TAO), tp(BK_TAO), 0, st, dd, bo(BK_TAO), n, stage); });
+        sweep(BK_TSMALL, [&] { launch_chained(kb_tang_small, grid(BK_TSMALL), kSmallTangBlock, 0, st, dd, bo(BK_TSMALL), n, stage, plan.tang_rows); });
         auto flux = [&](auto dimc, auto prfix) {
             constexpr int DIM = decltype(dimc)::value;
             constexpr bool PR = decltype(prfix)::value;
             const int cl = PR ? BK_FLUX_PR : BK_FLUX, cs = PR ? BK_FSMALL_PR : BK_FSMALL;
             sweep(cl, [&] {
-                if (stage == 0) kb_flux<DIM, 0, PR><<<grid(cl), tp(cl), flux_smem(DIM, tp(cl)), st>>>(dd, bo(cl), n);
-                else kb_flux<DIM, 1, PR><<<grid(cl), tp(cl), flux_smem(DIM, tp(cl)), st>>>(dd, bo(cl), n);
+                if (stage == 0) launch_chained(kb_flux<DIM, 0, PR>, grid(cl), tp(cl), flux_smem(DIM, tp(cl)), st, dd, bo(cl), n);
+                else launch_chained(kb_flux<DIM, 1, PR>, grid(cl), tp(cl), flux_smem(DIM, tp(cl)), st, dd, bo(cl), n);
             });
             sweep(cs, [&] {
-                if (stage == 0) kb_flux_small<DIM, 0, PR><<<grid(cs), tp(cs), flux_small_smem(DIM, PR, tp(cs)), st>>>(dd, bo(cs), n);
-                else kb_flux_small<DIM, 1, PR><<<grid(cs), tp(cs), flux_small_smem(DIM, PR, tp(cs)), st>>>(dd, bo(cs), n);
+                if (stage == 0) launch_chained(kb_flux_small<DIM, 0, PR>, grid(cs), tp(cs), flux_small_smem(DIM, PR, tp(cs)), st, dd, bo(cs), n);
+                else launch_chained(kb_flux_small<DIM, 1, PR>, grid(cs), tp(cs), flux_small_smem(DIM, PR, tp(cs)), st, dd, bo(cs), n);
             });
         };
         auto flux_dim = [&](auto dimc) { flux(dimc, std::false_type{}); flux(dimc, std::true_type{}); };
@@ -1864,11 +1921,11 @@ cudaError_t batch_enqueue_step(const BatchPlan& plan, const SolveDesc* dd, const
         mark(BK_UPD, 0);
         const int tu = tp(BK_UPD);
         if (dim == 2) {
-            if (stage == 0) kb_update<2, 0><<<grid(BK_UPD), tu, 0, st>>>(dd, bo(BK_UPD), n);
-            else kb_update<2, 1><<<grid(BK_UPD), tu, 0, st>>>(dd, bo(BK_UPD), n);
+            if (stage == 0) launch_chained(kb_update<2, 0>, grid(BK_UPD), tu, 0, st, dd, bo(BK_UPD), n);
+            else launch_chained(kb_update<2, 1>, grid(BK_UPD), tu, 0, st, dd, bo(BK_UPD), n);
         } else {
-            if (stage == 0) kb_update<1, 0><<<grid(BK_UPD), tu, 0, st>>>(dd, bo(BK_UPD), n);
-            else kb_update<1, 1><<<grid(BK_UPD), tu, 0, st>>>(dd, bo(BK_UPD), n);
+            if (stage == 0) launch_chained(kb_update<1, 0>, grid(BK_UPD), tu, 0, st, dd, bo(BK_UPD), n);
+            else launch_chained(kb_update<1, 1>, grid(BK_UPD), tu, 0, st, dd, bo(BK_UPD), n);
         }
         mark(BK_UPD, 1);
     }
@@ -1883,19 +1940,19 @@ static unsigned int copy_blocks(const GridGeom& g)
 
 cudaError_t launch_state_in(hgks_solver* s, const double* W, double t0)
 {
-    k_state_in<<<copy_blocks(s->P.g), TPB, 0, s->stream>>>(s->P.g, W, s->W, s->ctrl, t0);
+    launch_chained(k_state_in, copy_blocks(s->P.g), TPB, 0, s->stream, s->P.g, W, s->W, s->ctrl, t0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_noalloc_in(hgks_solver* s, const SolveDesc& self, const double* W)
 {
-    k_noalloc_in<<<copy_blocks(s->P.g), TPB, 0, s->stream>>>(self, s->d_self, W);
+    launch_chained(k_noalloc_in, copy_blocks(s->P.g), TPB, 0, s->stream, self, s->d_self, W);
     return cudaGetLastError();
 }
 
 cudaError_t launch_state_out(hgks_solver* s, double* W)
 {
-    k_state_out<<<copy_blocks(s->P.g), TPB, 0, s->stream>>>(s->P.g, s->W, W);
+    launch_chained(k_state_out, copy_blocks(s->P.g), TPB, 0, s->stream, s->P.g, s->W, W);
     return cudaGetLastError();
 }
 
