@@ -7,7 +7,7 @@ namespace hgks {
 // tangential velocity (2D: xi and the peculiar tangential velocity; 1D: xi alone).
 struct FluxConst {
     double gm1;            // gamma - 1
-    double hKt, ktp2;      // Kt/2, Kt + 2
+    double Kt, ktp2;       // Kt, Kt + 2
     double gq;             // (Kt + 3)/2: H = U^2/2 + gq h
     double k3, k6, hk6;    // Kt + 3, Kt + 6, (Kt + 6)/2
     double mu, c1, c2;
@@ -19,7 +19,7 @@ inline FluxConst flux_const(double gm1, double Kt, double mu, double c1, double 
 {
     FluxConst f;
     f.gm1 = gm1;
-    f.hKt = 0.5 * Kt; f.ktp2 = Kt + 2.0;
+    f.Kt = Kt; f.ktp2 = Kt + 2.0;
     f.gq = 0.5 * (Kt + 3.0);
     f.k3 = Kt + 3.0; f.k6 = Kt + 6.0; f.hk6 = 0.5 * (Kt + 6.0);
     f.mu = mu; f.c1 = c1; f.c2 = c2; f.prfix = prfix;

@@ -713,8 +713,8 @@ struct MState {
     double u2, H;                          // U^2 + h; H = (E + p)/rho, E without the tangential kinetic energy
 };
 
-// Slope constants of one side: ri/h and ri/(2 h^2) carry the 1/rho of <a> = dW/rho (Eq. (8)); 2 U.
-struct SlopeC { double rih, qh, U2; };
+// Slope constants of one side: ri/h and ri/(2 h^2) carry the 1/rho of <a> = dW/rho (Eq. (8)).
+struct SlopeC { double rih, qh; };
 
 // W_k-direction d in the frame of s, with what the closed forms share: R = d1 - U d0 (rho dU),
 // S = d1 + R, dp (pressure), d2, d3 in the frame.
@@ -801,50 +801,56 @@ HGKS_HD __forceinline__ void minus_w_t(const MState<DIM>& s, const FluxConst& fc
 }
 
 // Micro-slope a with <a> = d/rho (Eq. (8)), a.psi = a0 + a1 u + a2 c + a3 (u^2 + c^2 + xi^2)/2 in
-// the frame of s.  Kept as what the moments need: c0 = a0 + a3 Kt h/2, a1, ha3 = a3/2 (from
-// a3 = dh/h^2) and a2h = a2 h.
-struct Slope { double c0, a1, ha3, a2h; };
+// the frame of s.  Kept as what the moments need: with u_(n+2) = U u_(n+1) + (n+1) h u_n the polynomial
+// c0 + a1 u + (a3/2) u^2, c0 = a0 + a3 Kt h/2, gives T(n) = c0 u_n + b u_(n+1) + ha3 (n+1) h u_n with
+// b = a1 + U ha3, ha3 = a3/2 (from a3 = dh/h^2); y = 2 h ha3 and a2h = a2 h.
+struct Slope { double c0, b, ha3, y, a2h; };
 
 template <int DIM>
 HGKS_HD __forceinline__ void slope_solve(const Dir& d, const MState<DIM>& s, const SlopeC& k, Slope& a)
 {
     a.ha3 = k.qh * fma(-s.h, d.d0, d.dp);
-    a.a1 = fma(-k.U2, a.ha3, k.rih * d.R);
-    a.c0 = fma(-s.u2, a.ha3, fma(-s.U, a.a1, d.d0 * s.ri));
+    const double yh = s.h * a.ha3;
+    a.b = fma(-s.U, a.ha3, k.rih * d.R);
+    a.c0 = fma(-s.U, a.b, fma(d.d0, s.ri, -yh));
+    a.y = scale2<1>(yh);
     a.a2h = DIM == 2 ? s.ri * d.d2 : 0.0;
 }
 
-// Half-line moments: u[n] = rho <u^n> on one half line (n <= 6), and the constants of the energy
-// weight: kk = Kt h/2 = <c^2 + xi^2>/2, kh2 = Kt h^2.
-struct Mom { double u[7]; double kk, kh2; };
+// Half-line moments: u[n] = rho <u^n> on one half line (n <= 6), hu[n] = (n+1) h u[n] (n <= 4), and
+// Kh = Kt h = <c^2 + xi^2>.
+struct Mom { double u[7], hu[5]; double Kh; };
 
 // T(n) = <u^n (a.psi)>
 HGKS_HD __forceinline__ double mom_t(const Slope& a, const Mom& m, int n)
 {
-    return fma(a.c0, m.u[n], fma(a.a1, m.u[n + 1], a.ha3 * m.u[n + 2]));
+    return fma(a.c0, m.u[n], fma(a.b, m.u[n + 1], a.ha3 * m.hu[n]));
 }
 
-// <u^n psi (a.psi)> in the frame, given T(n), T(n+1), T(n+2) and z = kh2 ha3:
-// (c^2 + xi^2)/2 weighs T(n) with kk and the variance of the internal energy adds z u_n.
+// <u^n psi (a.psi)> in the frame, given T(n), T(n+1), T(n+2): c^2 + xi^2 weighs T(n) with Kh, and the variance
+// of the internal energy adds Kh y u_n.  The energy component is doubled here and in every sum over the
+// sides; flux_finish halves the sums (an exponent decrement).
 template <int DIM>
-HGKS_HD __forceinline__ void mom_g(const Slope& a, const Mom& m, double z, int n, double t0, double t1, double t2, double* out)
+HGKS_HD __forceinline__ void mom_g(const Slope& a, const Mom& m, int n, double t0, double t1, double t2, double* out)
 {
     out[0] = t0;
     out[1] = t1;
     if constexpr (DIM == 2) out[2] = a.a2h * m.u[n];
-    out[DIM + 1] = fma(0.5, t2, fma(m.kk, t0, z * m.u[n]));
+    out[DIM + 1] = fma(m.Kh, fma(a.y, m.u[n], t0), t2);
 }
 
-// acc (+)= the moment vector c of the frame of s as seen from the lab
-template <int DIM, bool FIRST>
+// acc (+)= the moment vector c of the frame of s as seen from the lab; TWICE: with doubled energy
+// component, which then gains V (2 c2 + V c0) where the energy gains V (c2 + V c0/2).
+template <int DIM, bool FIRST, bool TWICE>
 HGKS_HD __forceinline__ void add_lab(const MState<DIM>& s, const double* c, double* acc)
 {
     double l[DIM + 2];
     l[0] = c[0];
     l[1] = c[1];
     if constexpr (DIM == 2) {
+        const double in = TWICE ? fma(s.V, c[0], scale2<1>(c[2])) : fma(s.hV, c[0], c[2]);
         l[2] = FIRST ? fma(s.V, c[0], c[2]) : fma(s.V, c[0], acc[2] + c[2]);
-        l[3] = FIRST ? fma(s.V, fma(s.hV, c[0], c[2]), c[3]) : fma(s.V, fma(s.hV, c[0], c[2]), acc[3] + c[3]);
+        l[3] = FIRST ? fma(s.V, in, c[3]) : fma(s.V, in, acc[3] + c[3]);
     } else {
         l[2] = FIRST ? c[2] : acc[2] + c[2];
     }
@@ -854,15 +860,15 @@ HGKS_HD __forceinline__ void add_lab(const MState<DIM>& s, const double* c, doub
     for (int k = 2; k < DIM + 2; k++) acc[k] = l[k];
 }
 
-// The same for <u^n psi g> = (u_n, u_n+1, 0, (u_n+2 + Kt h u_n)/2).
+// The same for <u^n psi g> = (u_n, u_n+1, 0, (u_n+2 + Kt h u_n)/2), energy doubled.
 template <int DIM, bool FIRST>
 HGKS_HD __forceinline__ void add_psi_lab(const MState<DIM>& s, const Mom& m, int n, double* acc)
 {
-    const double en = fma(0.5, m.u[n + 2], m.kk * m.u[n]);
+    const double en = fma(m.Kh, m.u[n], m.u[n + 2]);
     if constexpr (DIM == 2) {
         const double v = s.V * m.u[n];
         acc[2] = FIRST ? v : acc[2] + v;
-        acc[3] = FIRST ? fma(s.hV, v, en) : fma(s.hV, v, acc[3] + en);
+        acc[3] = FIRST ? fma(s.V, v, en) : fma(s.V, v, acc[3] + en);
     } else {
         acc[2] = FIRST ? en : acc[2] + en;
     }
@@ -913,15 +919,18 @@ HGKS_HD __forceinline__ void half_moments(const MState<DIM>& s, double sl, int s
     m.u[1] = fma(s.U, m.u[0], sign > 0 ? e : -e);
     const double h2 = scale2<1>(s.h), hn[5] = {s.h, h2, s.h + h2, scale2<1>(h2), 5.0 * s.h};
 #pragma unroll
-    for (int n = 0; n < 5; n++) m.u[n + 2] = fma(s.U, m.u[n + 1], hn[n] * m.u[n]);
-    m.kk = fc.hKt * s.h;
-    m.kh2 = scale2<1>(m.kk) * s.h;
+    for (int n = 0; n < 5; n++) {
+        m.hu[n] = hn[n] * m.u[n];
+        m.u[n + 2] = fma(s.U, m.u[n + 1], m.hu[n]);
+    }
+    m.Kh = fc.Kt * s.h;
 }
 
-// Sums over the two sides (left over u > 0, right over u < 0), lab frame: the equilibrium state
-// and its slopes (Eqs. (46)-(47)) and the moments int u psi of the three non-equilibrium terms of
-// Eq. (10): S4 (g^k), S5 ((a1 u + a2 v) g^k), S6n (-A^k g^k).  D5, D6n: the density moments int psi of the
-// last two (Prandtl fix only).
+// Sums over the two sides (left over u > 0, right over u < 0), lab frame, energy components doubled
+// (one multiplication less per vector; with that and (n+1) h u_n kept beside the moments the flux
+// launch went from 4.02 to 3.79 ms at 1024^2): the equilibrium state and its slopes (Eqs. (46)-(47))
+// and the moments int u psi of the three non-equilibrium terms of Eq. (10): S4 (g^k), S5 ((a1 u +
+// a2 v) g^k), S6n (-A^k g^k).  D5, D6n: the density moments int psi of the last two (Prandtl fix only).
 template <int DIM>
 struct FluxSums { double Wc[DIM + 2], Wx[DIM + 2], Wy[DIM + 2], S4[DIM + 2], S5[DIM + 2], S6n[DIM + 2], D5[DIM + 2], D6n[DIM + 2]; };
 
@@ -942,7 +951,6 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
         const double lam = sl * sl;
         k.rih = scale2<1>(lam) * s.ri;
         k.qh = lam * k.rih;
-        k.U2 = scale2<1>(s.U);
     }
     Mom m;
     half_moments<DIM>(s, sl, left ? +1 : -1, fc, m);
@@ -953,48 +961,46 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
     in_frame<DIM>(s, fc, Wx, dx);
     slope_solve<DIM>(dx, s, k, a);
     const double ta0 = mom_t(a, m, 0), ta1 = mom_t(a, m, 1), ta2 = mom_t(a, m, 2);
-    const double za = m.kh2 * a.ha3;
-    mom_g<DIM>(a, m, za, 0, ta0, ta1, ta2, g);
-    add_lab<DIM, FIRST>(s, g, q.Wx);
+    mom_g<DIM>(a, m, 0, ta0, ta1, ta2, g);
+    add_lab<DIM, FIRST, true>(s, g, q.Wx);
     // int u psi (a1 u + a2 v) g of this side (L5) and, for the Prandtl fix, int psi (a1 u + a2 v) g
     double L5[NV], L[NV];
     const bool noneq = !fc.tau_zero;
     if (noneq) {
         const double ta3 = mom_t(a, m, 3), ta4 = mom_t(a, m, 4);
-        mom_g<DIM>(a, m, za, 2, ta2, ta3, ta4, L5);
-        if constexpr (PRFIX) mom_g<DIM>(a, m, za, 1, ta1, ta2, ta3, L);
+        mom_g<DIM>(a, m, 2, ta2, ta3, ta4, L5);
+        if constexpr (PRFIX) mom_g<DIM>(a, m, 1, ta1, ta2, ta3, L);
     }
     if constexpr (DIM == 2) {
         Slope b;
         in_frame<DIM>(s, fc, Wy, dy);
         slope_solve<DIM>(dy, s, k, b);
         const double tb0 = mom_t(b, m, 0), tb1 = mom_t(b, m, 1), tb2 = mom_t(b, m, 2);
-        const double zb = m.kh2 * b.ha3;
-        mom_g<DIM>(b, m, zb, 0, tb0, tb1, tb2, g);
-        add_lab<DIM, FIRST>(s, g, q.Wy);
+        mom_g<DIM>(b, m, 0, tb0, tb1, tb2, g);
+        add_lab<DIM, FIRST, true>(s, g, q.Wy);
         if (noneq) {
             // v = V + c: the c part has <u c psi (b.psi)> = b2 h u_1, b2 h u_2, h (T_b(1) + h b3 u_1)
-            // and b2 h (u_3 + (Kt + 2) h u_1)/2
-            const double y = scale2<1>(s.h) * b.ha3, kc = fc.ktp2 * s.h, hb = scale2<-1>(b.a2h);
+            // and b2 h (u_3 + (Kt + 2) h u_1)/2 (doubled)
+            const double kc = fc.ktp2 * s.h;
             if constexpr (PRFIX) {
                 L[0] = fma(s.V, g[0], fma(b.a2h, m.u[0], L[0]));
                 L[1] = fma(s.V, g[1], fma(b.a2h, m.u[1], L[1]));
-                L[2] = fma(s.V, g[2], fma(s.h, fma(y, m.u[0], tb0), L[2]));
-                L[3] = fma(s.V, g[3], fma(hb, fma(kc, m.u[0], m.u[2]), L[3]));
-                add_lab<DIM, FIRST>(s, L, q.D5);
+                L[2] = fma(s.V, g[2], fma(s.h, fma(b.y, m.u[0], tb0), L[2]));
+                L[3] = fma(s.V, g[3], fma(b.a2h, fma(kc, m.u[0], m.u[2]), L[3]));
+                add_lab<DIM, FIRST, true>(s, L, q.D5);
             }
             const double tb3 = mom_t(b, m, 3);
-            mom_g<DIM>(b, m, zb, 1, tb1, tb2, tb3, g);
+            mom_g<DIM>(b, m, 1, tb1, tb2, tb3, g);
             L5[0] = fma(s.V, g[0], L5[0] + g[2]);
             L5[1] = fma(s.V, g[1], fma(b.a2h, m.u[2], L5[1]));
-            L5[2] = fma(s.V, g[2], fma(s.h, fma(y, m.u[1], tb1), L5[2]));
-            L5[3] = fma(s.V, g[3], fma(hb, fma(kc, m.u[1], m.u[3]), L5[3]));
+            L5[2] = fma(s.V, g[2], fma(s.h, fma(b.y, m.u[1], tb1), L5[2]));
+            L5[3] = fma(s.V, g[3], fma(b.a2h, fma(kc, m.u[1], m.u[3]), L5[3]));
         }
     } else if constexpr (PRFIX) {
-        if (noneq) add_lab<DIM, FIRST>(s, L, q.D5);
+        if (noneq) add_lab<DIM, FIRST, true>(s, L, q.D5);
     }
     if (!noneq) return true;
-    add_lab<DIM, FIRST>(s, L5, q.S5);
+    add_lab<DIM, FIRST, true>(s, L5, q.S5);
     add_psi_lab<DIM, FIRST>(s, m, 1, q.S4);
     // time slope A from <a1 u + a2 v + A> = 0 (Eq. (9)), with the opposite sign
     Dir dt;
@@ -1002,12 +1008,11 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
     minus_w_t<DIM>(s, fc, dx, dy, dt);
     slope_solve<DIM>(dt, s, k, c);
     const double tc1 = mom_t(c, m, 1), tc2 = mom_t(c, m, 2), tc3 = mom_t(c, m, 3);
-    const double zc = m.kh2 * c.ha3;
-    mom_g<DIM>(c, m, zc, 1, tc1, tc2, tc3, g);
-    add_lab<DIM, FIRST>(s, g, q.S6n);
+    mom_g<DIM>(c, m, 1, tc1, tc2, tc3, g);
+    add_lab<DIM, FIRST, true>(s, g, q.S6n);
     if constexpr (PRFIX) {
-        mom_g<DIM>(c, m, zc, 0, mom_t(c, m, 0), tc1, tc2, g);
-        add_lab<DIM, FIRST>(s, g, q.D6n);
+        mom_g<DIM>(c, m, 0, mom_t(c, m, 0), tc1, tc2, g);
+        add_lab<DIM, FIRST, true>(s, g, q.D6n);
     }
     return true;
 }
@@ -1074,10 +1079,23 @@ HGKS_HD __forceinline__ void time_coefs(double dt, double tau, double* A0, doubl
 
 // Gas-kinetic flux at one Gauss point from the sums over the two sides and their pressures.
 template <int DIM, int STAGE, bool PRFIX>
-HGKS_HD __forceinline__ bool flux_finish(const FluxConst& fc, const FluxSums<DIM>& q, double pl, double pr, double dt,
+HGKS_HD __forceinline__ bool flux_finish(const FluxConst& fc, FluxSums<DIM>& q, double pl, double pr, double dt,
                                          double* o0, double* o1)
 {
     constexpr int NV = DIM + 2;
+    // the sums' energies are doubled
+    q.Wc[NV - 1] = scale2<-1>(q.Wc[NV - 1]);
+    q.Wx[NV - 1] = scale2<-1>(q.Wx[NV - 1]);
+    if constexpr (DIM == 2) q.Wy[NV - 1] = scale2<-1>(q.Wy[NV - 1]);
+    if (!fc.tau_zero) {
+        q.S4[NV - 1] = scale2<-1>(q.S4[NV - 1]);
+        q.S5[NV - 1] = scale2<-1>(q.S5[NV - 1]);
+        q.S6n[NV - 1] = scale2<-1>(q.S6n[NV - 1]);
+        if constexpr (PRFIX) {
+            q.D5[NV - 1] = scale2<-1>(q.D5[NV - 1]);
+            q.D6n[NV - 1] = scale2<-1>(q.D6n[NV - 1]);
+        }
+    }
     MState<DIM> sc;
     if (!make_state<DIM>(q.Wc, fc, sc)) return false;
 
@@ -1127,8 +1145,8 @@ HGKS_HD __forceinline__ bool flux_finish(const FluxConst& fc, const FluxSums<DIM
             if constexpr (STAGE == 0) c1[k] = fma(A1[1], M2[k], c1[k]);
         }
     }
-    add_lab<DIM, true>(sc, c0, o0);
-    if constexpr (STAGE == 0) add_lab<DIM, true>(sc, c1, o1);
+    add_lab<DIM, true, false>(sc, c0, o0);
+    if constexpr (STAGE == 0) add_lab<DIM, true, false>(sc, c1, o1);
     if (eq_only) return true;
 #pragma unroll
     for (int k = 0; k < NV; k++) {
