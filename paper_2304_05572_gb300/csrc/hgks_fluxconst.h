@@ -6,7 +6,7 @@ namespace hgks {
 // Kt = K + D - 1 counts the internal degrees of freedom as seen in the frame moving with the
 // tangential velocity (2D: xi and the peculiar tangential velocity; 1D: xi alone).
 struct FluxConst {
-    double gm1;            // gamma - 1
+    double gm1, rgm1;      // gamma - 1, 1/(gamma - 1)
     double Kt, ktp2;       // Kt, Kt + 2
     double gq;             // (Kt + 3)/2: H = U^2/2 + gq h
     double k3, k6, hk6;    // Kt + 3, Kt + 6, (Kt + 6)/2
@@ -18,7 +18,7 @@ struct FluxConst {
 inline FluxConst flux_const(double gm1, double Kt, double mu, double c1, double c2, double prfix, int viscous, int tau_zero)
 {
     FluxConst f;
-    f.gm1 = gm1;
+    f.gm1 = gm1; f.rgm1 = 1.0 / gm1;
     f.Kt = Kt; f.ktp2 = Kt + 2.0;
     f.gq = 0.5 * (Kt + 3.0);
     f.k3 = Kt + 3.0; f.k6 = Kt + 6.0; f.hk6 = 0.5 * (Kt + 6.0);

@@ -698,13 +698,15 @@ __device__ __forceinline__ void tang_ao_x4(const TangEig& e, const double (*x)[4
 // Every Maxwellian is handled in the frame that moves with its own tangential velocity V (2D):
 // there the peculiar tangential velocity c = v - V is one more internal degree of freedom beside
 // xi, odd moments of c vanish, and <psi (a.psi) u^n> takes the 1D form with Kt = K + 1 internal
-// degrees (1D: Kt = K) plus one product for the tangential momentum.  Derivatives are moved into
-// that frame (the energy loses V m + V^2 rho/2), the moments' sums back out of it, three
-// operations per vector each way.  On this part the flux is bound by the FP64 issue rate (one
-// warp instruction per 64 cycles and scheduler), so what counts is the number of FP64
-// instructions: with lab-frame moments in both directions the closed form took 1433 / 1389
-// operations per Gauss point (first / second stage), in the moving frames and with the simplified
-// time coefficients 897 / 824; the flux launch at 1024^2 went from 8.26 to 6.22 ms.
+// degrees (1D: Kt = K) plus one product for the tangential momentum; the moments' sums are moved
+// back out of the frame.  On this part the flux is bound by the FP64 issue rate (one warp
+// instruction per 64 cycles and scheduler), so what counts is the number of FP64 instructions.
+// Operations per Gauss point (first / second stage) and flux launch at 1024^2:
+//   lab-frame moments in both directions, solves for the micro-slopes      1433 / 1389   8.26 ms
+//   moving frames, simplified time coefficients                             897 /  824   6.22 ms
+//   divisions, roots, exp, erfc and the Gauss-point quartics in integers,
+//   doubled energy sums                                                     893 /  820   3.79 ms
+//   micro-slopes as derivatives of the primitives (struct Slope)            829 /  756   3.49 ms
 
 // Primitive description of one Maxwellian (Eq. (3)) in its own tangential frame: h = p/rho.
 template <int DIM>
@@ -712,9 +714,6 @@ struct MState {
     double rho, ri, U, hU, V, hV, p, h;   // hU, hV: halves
     double u2, H;                          // U^2 + h; H = (E + p)/rho, E without the tangential kinetic energy
 };
-
-// Slope constants of one side: ri/h and ri/(2 h^2) carry the 1/rho of <a> = dW/rho (Eq. (8)).
-struct SlopeC { double rih, qh; };
 
 // W_k-direction d in the frame of s, with what the closed forms share: R = d1 - U d0 (rho dU),
 // S = d1 + R, dp (pressure), d2, d3 in the frame.
@@ -800,43 +799,74 @@ HGKS_HD __forceinline__ void minus_w_t(const MState<DIM>& s, const FluxConst& fc
     n.dp = fc.gm1 * fma(-s.hU, n.S, n.d3);
 }
 
-// Micro-slope a with <a> = d/rho (Eq. (8)), a.psi = a0 + a1 u + a2 c + a3 (u^2 + c^2 + xi^2)/2 in
-// the frame of s.  Kept as what the moments need: with u_(n+2) = U u_(n+1) + (n+1) h u_n the polynomial
-// c0 + a1 u + (a3/2) u^2, c0 = a0 + a3 Kt h/2, gives T(n) = c0 u_n + b u_(n+1) + ha3 (n+1) h u_n with
-// b = a1 + U ha3, ha3 = a3/2 (from a3 = dh/h^2); y = 2 h ha3 and a2h = a2 h.
-struct Slope { double c0, b, ha3, y, a2h; };
+// Micro-slope of one side (Eq. (8)).  <a> = dW/rho makes (a.psi) g the derivative of g along d,
+// so it is kept as the derivatives of the primitives, al = d ln rho, be = dU, ga = dV, de = dh,
+// ka = Kt dh, and every moment is the derivative of a half-line moment: no solve for a, moments up to
+// u^4 rather than u^6, and the time slope from the primitive Euler equations (14 operations against
+// 24 through the conserved ones).
+struct Slope { double al, be, ga, de, ka; };
+
+// What the conversion from conserved derivatives needs: lU = U/(2h); e = (gamma-1)/rho;
+// z = |(U, V)|^2/2 - h/(gamma-1).
+struct SlopeC { double lU, e, z; };
 
 template <int DIM>
-HGKS_HD __forceinline__ void slope_solve(const Dir& d, const MState<DIM>& s, const SlopeC& k, Slope& a)
+HGKS_HD __forceinline__ void slope_of(const MState<DIM>& s, const FluxConst& fc, const SlopeC& k, const double* d, Slope& a)
 {
-    a.ha3 = k.qh * fma(-s.h, d.d0, d.dp);
-    const double yh = s.h * a.ha3;
-    a.b = fma(-s.U, a.ha3, k.rih * d.R);
-    a.c0 = fma(-s.U, a.b, fma(d.d0, s.ri, -yh));
-    a.y = scale2<1>(yh);
-    a.a2h = DIM == 2 ? s.ri * d.d2 : 0.0;
+    a.al = s.ri * d[0];
+    a.be = s.ri * fma(-s.U, d[0], d[1]);
+    double x = fma(-s.U, d[1], fma(k.z, d[0], d[DIM + 1]));
+    if constexpr (DIM == 2) {
+        a.ga = s.ri * fma(-s.V, d[0], d[2]);
+        x = fma(-s.V, d[2], x);
+    } else {
+        a.ga = 0.0;
+    }
+    a.de = k.e * x;
+    a.ka = fc.Kt * a.de;
 }
 
-// Half-line moments: u[n] = rho <u^n> on one half line (n <= 6), hu[n] = (n+1) h u[n] (n <= 4), and
-// Kh = Kt h = <c^2 + xi^2>.
-struct Mom { double u[7], hu[5]; double Kh; };
-
-// T(n) = <u^n (a.psi)>
-HGKS_HD __forceinline__ double mom_t(const Slope& a, const Mom& m, int n)
+// -W_t of the slopes a (x) and b (y) from the Euler compatibility (Eq. (9)), as a slope: the Euler
+// equations in the primitives.
+template <int DIM>
+HGKS_HD __forceinline__ void slope_minus_t(const MState<DIM>& s, const FluxConst& fc, const Slope& a, const Slope& b, Slope& c)
 {
-    return fma(a.c0, m.u[n], fma(a.b, m.u[n + 1], a.ha3 * m.hu[n]));
+    const double px = fma(s.h, a.al, a.de), gh = fc.gm1 * s.h;        // p_x/rho
+    if constexpr (DIM == 2) {
+        const double div = a.be + b.ga;
+        c.al = fma(s.U, a.al, fma(s.V, b.al, div));
+        c.be = fma(s.U, a.be, fma(s.V, b.be, px));
+        c.ga = fma(s.U, a.ga, fma(s.V, b.ga, fma(s.h, b.al, b.de)));
+        c.de = fma(s.U, a.de, fma(s.V, b.de, gh * div));
+    } else {
+        c.al = fma(s.U, a.al, a.be);
+        c.be = fma(s.U, a.be, px);
+        c.ga = 0.0;
+        c.de = fma(s.U, a.de, gh * a.be);
+    }
+    c.ka = fc.Kt * c.de;
 }
 
-// <u^n psi (a.psi)> in the frame, given T(n), T(n+1), T(n+2): c^2 + xi^2 weighs T(n) with Kh, and the variance
-// of the internal energy adds Kh y u_n.  The energy component is doubled here and in every sum over the
-// sides; flux_finish halves the sums (an exponent decrement).
+// Half-line moments: u[n] = rho <u^n> on one half line (n <= 4) with the multiples that the
+// derivatives need, G = d u[0]/dU (the density at u = 0, signed), hG its half, and Kh = Kt h = <c^2 + xi^2>.
+struct Mom { double u[5], G, hG, u1x2, u1x3, u2x3, u2x6, u3x4, Kh; };
+
+// T(n) = <u^n (a.psi)>, the derivative of u[n]: d/dh = (d/dU)^2/2, d u[0]/dU = G, d u[1]/dU = u[0].
+HGKS_HD __forceinline__ double mom_t0(const Slope& a, const Mom& m, const SlopeC& k) { return fma(a.al, m.u[0], fma(-k.lU, a.de, a.be) * m.G); }
+HGKS_HD __forceinline__ double mom_t1(const Slope& a, const Mom& m) { return fma(a.al, m.u[1], fma(a.be, m.u[0], a.de * m.hG)); }
+HGKS_HD __forceinline__ double mom_t2(const Slope& a, const Mom& m) { return fma(a.al, m.u[2], fma(a.be, m.u1x2, a.de * m.u[0])); }
+HGKS_HD __forceinline__ double mom_t3(const Slope& a, const Mom& m) { return fma(a.al, m.u[3], fma(a.be, m.u2x3, a.de * m.u1x3)); }
+HGKS_HD __forceinline__ double mom_t4(const Slope& a, const Mom& m) { return fma(a.al, m.u[4], fma(a.be, m.u3x4, a.de * m.u2x6)); }
+
+// <u^n psi (a.psi)> in the frame, given T(n), T(n+1), T(n+2).  The energy component (of u^2 + Kt h) is doubled
+// here and in every sum over the sides; flux_finish halves the sums (an exponent decrement).
 template <int DIM>
 HGKS_HD __forceinline__ void mom_g(const Slope& a, const Mom& m, int n, double t0, double t1, double t2, double* out)
 {
     out[0] = t0;
     out[1] = t1;
-    if constexpr (DIM == 2) out[2] = a.a2h * m.u[n];
-    out[DIM + 1] = fma(m.Kh, fma(a.y, m.u[n], t0), t2);
+    if constexpr (DIM == 2) out[2] = a.ga * m.u[n];
+    out[DIM + 1] = fma(m.Kh, t0, fma(a.ka, m.u[n], t2));
 }
 
 // acc (+)= the moment vector c of the frame of s as seen from the lab; TWICE: with doubled energy
@@ -907,7 +937,10 @@ HGKS_HD __forceinline__ void half_moments(const MState<DIM>& s, double sl, int s
     const double x = sl * s.U;
     double ex2, E;
     exp_erfc(x, ex2, E);
-    const double e = ex2 * (0.56418958354775628695 * s.p * sl);   // rho h sqrt(lam)/sqrt(pi), rho h = p
+    const double g0 = ex2 * (0.56418958354775628695 * sl);          // sqrt(lam/pi) exp(-lam U^2)
+    const double e = s.p * g0, G = s.rho * g0;                      // rho h = p
+    m.G = sign > 0 ? G : -G;
+    m.hG = scale2<-1>(m.G);
 #ifdef __CUDA_ARCH__
     const bool neg = __double2hiint(x) < 0;         // (at x = 0 both forms below give half the mass)
 #else
@@ -917,18 +950,20 @@ HGKS_HD __forceinline__ void half_moments(const MState<DIM>& s, double sl, int s
     const double hr = scale2<-1>(s.rho);
     m.u[0] = into ? fma(-hr, E, s.rho) : hr * E;
     m.u[1] = fma(s.U, m.u[0], sign > 0 ? e : -e);
-    const double h2 = scale2<1>(s.h), hn[5] = {s.h, h2, s.h + h2, scale2<1>(h2), 5.0 * s.h};
-#pragma unroll
-    for (int n = 0; n < 5; n++) {
-        m.hu[n] = hn[n] * m.u[n];
-        m.u[n + 2] = fma(s.U, m.u[n + 1], m.hu[n]);
-    }
+    m.u[2] = fma(s.U, m.u[1], s.h * m.u[0]);
+    m.u1x2 = scale2<1>(m.u[1]);
+    m.u1x3 = 3.0 * m.u[1];
+    m.u[3] = fma(s.U, m.u[2], s.h * m.u1x2);
+    m.u2x3 = 3.0 * m.u[2];
+    m.u2x6 = scale2<1>(m.u2x3);
+    m.u[4] = fma(s.U, m.u[3], s.h * m.u2x3);
+    m.u3x4 = scale2<2>(m.u[3]);
     m.Kh = fc.Kt * s.h;
 }
 
 // Sums over the two sides (left over u > 0, right over u < 0), lab frame, energy components doubled
-// (one multiplication less per vector; with that and (n+1) h u_n kept beside the moments the flux
-// launch went from 4.02 to 3.79 ms at 1024^2): the equilibrium state and its slopes (Eqs. (46)-(47))
+// (one multiplication less per vector; the flux launch went from
+// 4.02 to 3.79 ms at 1024^2): the equilibrium state and its slopes (Eqs. (46)-(47))
 // and the moments int u psi of the three non-equilibrium terms of Eq. (10): S4 (g^k), S5 ((a1 u +
 // a2 v) g^k), S6n (-A^k g^k).  D5, D6n: the density moments int psi of the last two (Prandtl fix only).
 template <int DIM>
@@ -946,55 +981,50 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
     if (!make_state<DIM>(W, fc, s)) return false;
     p = s.p;
     const double sl = rsqrt_nr(scale2<1>(s.h));      // sqrt(lambda)
-    SlopeC k;
-    {
-        const double lam = sl * sl;
-        k.rih = scale2<1>(lam) * s.ri;
-        k.qh = lam * k.rih;
-    }
     Mom m;
     half_moments<DIM>(s, sl, left ? +1 : -1, fc, m);
     add_psi_lab<DIM, FIRST>(s, m, 0, q.Wc);
-    Dir dx, dy;
-    Slope a;
+    SlopeC k;
+    k.lU = sl * (sl * s.U);
+    k.e = fc.gm1 * s.ri;
+    k.z = fma(s.hU, s.U, -(fc.rgm1 * s.h));
+    if constexpr (DIM == 2) k.z = fma(s.hV, s.V, k.z);
+    Slope a, b;
     double g[NV];
-    in_frame<DIM>(s, fc, Wx, dx);
-    slope_solve<DIM>(dx, s, k, a);
-    const double ta0 = mom_t(a, m, 0), ta1 = mom_t(a, m, 1), ta2 = mom_t(a, m, 2);
+    slope_of<DIM>(s, fc, k, Wx, a);
+    const double ta0 = mom_t0(a, m, k), ta1 = mom_t1(a, m), ta2 = mom_t2(a, m);
     mom_g<DIM>(a, m, 0, ta0, ta1, ta2, g);
     add_lab<DIM, FIRST, true>(s, g, q.Wx);
     // int u psi (a1 u + a2 v) g of this side (L5) and, for the Prandtl fix, int psi (a1 u + a2 v) g
     double L5[NV], L[NV];
     const bool noneq = !fc.tau_zero;
     if (noneq) {
-        const double ta3 = mom_t(a, m, 3), ta4 = mom_t(a, m, 4);
+        const double ta3 = mom_t3(a, m), ta4 = mom_t4(a, m);
         mom_g<DIM>(a, m, 2, ta2, ta3, ta4, L5);
         if constexpr (PRFIX) mom_g<DIM>(a, m, 1, ta1, ta2, ta3, L);
     }
     if constexpr (DIM == 2) {
-        Slope b;
-        in_frame<DIM>(s, fc, Wy, dy);
-        slope_solve<DIM>(dy, s, k, b);
-        const double tb0 = mom_t(b, m, 0), tb1 = mom_t(b, m, 1), tb2 = mom_t(b, m, 2);
+        slope_of<DIM>(s, fc, k, Wy, b);
+        const double tb0 = mom_t0(b, m, k), tb1 = mom_t1(b, m), tb2 = mom_t2(b, m);
         mom_g<DIM>(b, m, 0, tb0, tb1, tb2, g);
         add_lab<DIM, FIRST, true>(s, g, q.Wy);
         if (noneq) {
-            // v = V + c: the c part has <u c psi (b.psi)> = b2 h u_1, b2 h u_2, h (T_b(1) + h b3 u_1)
-            // and b2 h (u_3 + (Kt + 2) h u_1)/2 (doubled)
+            // v = V + c: the c part has <u^n c psi (b.psi)> = dV u_n, dV u_(n+1), h T_b(n) + dh u_n
+            // and dV (u_(n+2) + (Kt + 2) h u_n) (doubled)
             const double kc = fc.ktp2 * s.h;
             if constexpr (PRFIX) {
-                L[0] = fma(s.V, g[0], fma(b.a2h, m.u[0], L[0]));
-                L[1] = fma(s.V, g[1], fma(b.a2h, m.u[1], L[1]));
-                L[2] = fma(s.V, g[2], fma(s.h, fma(b.y, m.u[0], tb0), L[2]));
-                L[3] = fma(s.V, g[3], fma(b.a2h, fma(kc, m.u[0], m.u[2]), L[3]));
+                L[0] = fma(s.V, g[0], fma(b.ga, m.u[0], L[0]));
+                L[1] = fma(s.V, g[1], fma(b.ga, m.u[1], L[1]));
+                L[2] = fma(s.V, g[2], fma(s.h, tb0, fma(b.de, m.u[0], L[2])));
+                L[3] = fma(s.V, g[3], fma(b.ga, fma(kc, m.u[0], m.u[2]), L[3]));
                 add_lab<DIM, FIRST, true>(s, L, q.D5);
             }
-            const double tb3 = mom_t(b, m, 3);
+            const double tb3 = mom_t3(b, m);
             mom_g<DIM>(b, m, 1, tb1, tb2, tb3, g);
             L5[0] = fma(s.V, g[0], L5[0] + g[2]);
-            L5[1] = fma(s.V, g[1], fma(b.a2h, m.u[2], L5[1]));
-            L5[2] = fma(s.V, g[2], fma(s.h, fma(b.y, m.u[1], tb1), L5[2]));
-            L5[3] = fma(s.V, g[3], fma(b.a2h, fma(kc, m.u[1], m.u[3]), L5[3]));
+            L5[1] = fma(s.V, g[1], fma(b.ga, m.u[2], L5[1]));
+            L5[2] = fma(s.V, g[2], fma(s.h, tb1, fma(b.de, m.u[1], L5[2])));
+            L5[3] = fma(s.V, g[3], fma(b.ga, fma(kc, m.u[1], m.u[3]), L5[3]));
         }
     } else if constexpr (PRFIX) {
         if (noneq) add_lab<DIM, FIRST, true>(s, L, q.D5);
@@ -1003,15 +1033,13 @@ HGKS_HD __forceinline__ bool flux_side(const FluxConst& fc, const double* W, con
     add_lab<DIM, FIRST, true>(s, L5, q.S5);
     add_psi_lab<DIM, FIRST>(s, m, 1, q.S4);
     // time slope A from <a1 u + a2 v + A> = 0 (Eq. (9)), with the opposite sign
-    Dir dt;
     Slope c;
-    minus_w_t<DIM>(s, fc, dx, dy, dt);
-    slope_solve<DIM>(dt, s, k, c);
-    const double tc1 = mom_t(c, m, 1), tc2 = mom_t(c, m, 2), tc3 = mom_t(c, m, 3);
+    slope_minus_t<DIM>(s, fc, a, b, c);
+    const double tc1 = mom_t1(c, m), tc2 = mom_t2(c, m), tc3 = mom_t3(c, m);
     mom_g<DIM>(c, m, 1, tc1, tc2, tc3, g);
     add_lab<DIM, FIRST, true>(s, g, q.S6n);
     if constexpr (PRFIX) {
-        mom_g<DIM>(c, m, 0, mom_t(c, m, 0), tc1, tc2, g);
+        mom_g<DIM>(c, m, 0, mom_t0(c, m, k), tc1, tc2, g);
         add_lab<DIM, FIRST, true>(s, g, q.D6n);
     }
     return true;
