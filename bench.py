@@ -56,10 +56,13 @@ N_SIDE = 1024
 WORKLOAD = "four-quadrant 2D Riemann problem, 1024^2 cells, hybrid WENO-AO HGKS, S2O4"
 
 # Algorithmic FP64 work of the step (add / sub, mul, div, sqrt, exp and erfc count one each, fma
-# two), kept fixed here so that the yardstick does not move when a kernel changes:
+# two), of the algorithm as the kernels now run it (a change of the algebra moves it):
 # * the flux per Gauss point: the closed form of the flux kernel (2D Euler, tau > 0), counted on
-#   the host by paper_2304_05572_gb300/flopcount.py: 1433 operations in the first stage (F(dt/2)
-#   and the F^n + dt/6 dF^n combination), 1389 in the second; on sweeps of 49 152 segments or
+#   the host by paper_2304_05572_gb300/flopcount.py: 829 operations in the first stage (F(dt/2)
+#   and the F^n + dt/6 dF^n combination), 756 in the second (1433 and 1389 with lab-frame moments
+#   and solved micro-slopes); part of them (the quotients, roots, exp, erfc and the Gauss-point
+#   quartics) runs in integer units, so the fraction of the FP64 peak may pass the FP64 pipe's
+#   own utilisation; on sweeps of 49 152 segments or
 #   more the kernel also reconstructs its Gauss point's smooth tangential passes
 #   (FLUX_KERNEL_TANG_FLOP_PER_GP); one launch covers both sweeps of a stage;
 # * the rest of the step per cell-stage (indicator, reconstruction, update, time step), counted on
@@ -67,10 +70,10 @@ WORKLOAD = "four-quadrant 2D Riemann problem, 1024^2 cells, hybrid WENO-AO HGKS,
 #   these formulas as the paper prints them): every cell smooth 2721.3, every cell troubled
 #   19486.7, the hybrid step 3525.5 at its troubled fraction 0.41 %; a run at another troubled
 #   fraction f moves the hybrid figure along the troubled-minus-smooth slope.  (The oracle's own
-#   flux integrates every moment literally, ORACLE_FLUX_FLOP_PER_GP operations, five times the
+#   flux integrates every moment literally, ORACLE_FLUX_FLOP_PER_GP operations, nine times the
 #   closed form: a roofline on that count would exceed the peak, so the flux enters with its
 #   closed-form count.)
-FLUX_ALG_FLOP_PER_GP = (1433.0 + 1389.0) / 2
+FLUX_ALG_FLOP_PER_GP = (829.0 + 756.0) / 2
 ORACLE_FLUX_FLOP_PER_GP = 7025.0
 # On large sweeps the flux kernel also reconstructs its Gauss point's smooth tangential passes
 # (the quartic of Sec. 2.3.3 at the Gauss point): 16 values and 8 tangential derivatives of 5
