@@ -176,8 +176,9 @@ typedef struct hgks_batch hgks_batch;
 #define HGKS_BATCH_AUTOTUNE 2   /* choose the block size of each kernel class on the first steps (see hgks_batch_step) */
 
 /* Group n >= 1 solvers of the same dimension on the current device.  One
- * batched step issues one launch per kernel class (24 per step in 2D, the sweep
- * classes covering both sweeps) whose blocks cover every solver's interfaces;
+ * batched step issues one launch per kernel class that any solver needs (at most 24 per
+ * step in 2D, the sweep classes covering both sweeps; small and large sweeps have classes
+ * of their own) whose blocks cover every solver's interfaces;
  * each block works for exactly one solver (and one sweep) with that solver's own
  * arithmetic, so every result is bit-identical
  * to stepping the solver alone.  The solvers keep their own state, dt, time and
@@ -210,7 +211,7 @@ int hgks_batch_update(hgks_batch* b, hgks_solver* const* solvers, int n);
  * With HGKS_BATCH_AUTOTUNE on a batch not tuned yet, the first (up to) 4 of the
  * nsteps steps are taken one at a time with a wait after each: one with the
  * default block sizes, then one with each of three candidate sizes per kernel
- * class, timed per class with CUDA events; the fastest size of each class is
+ * class (the flux and the small sweeps' tangential kernel have fixed sizes), timed per class with CUDA events; the fastest size of each class is
  * kept for the rest of the batch's life.  These are real steps (results do not
  * depend on the block size).  Otherwise the call returns after enqueueing (no
  * wait); use hgks_batch_sync to wait.  A graph captured earlier is rebuilt
@@ -266,8 +267,8 @@ int hgks_probe_fp64(void* stream, double* tflops, double* ms, int* sms);
 
 /* Check of the flux's reciprocal and reciprocal square root (a measurement
  * helper like the probe above; the paper has no counterpart).  The flux forms 1/x
- * and 1/sqrt(x) as the hardware's approximations refined by two Newton-Raphson
- * steps instead of a division or square root; this evaluates both on n >= 1
+ * and 1/sqrt(x) in 64-bit fixed point from the hardware's single-precision
+ * approximations instead of a division or square root; this evaluates both on n >= 1
  * arguments spread log-uniformly over 1e-8..1e8 (both signs for 1/x) on the
  * current device (default stream; the call waits) and stores in max_ulp[0] the
  * largest distance of 1/x, in units in the last place, from the correctly

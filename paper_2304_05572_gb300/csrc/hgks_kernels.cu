@@ -4,9 +4,10 @@
 // Per stage: ghost fill -> for each sweep (x, then y in 2D):
 //   raw normal flags -> normal reconstruction (linear inline, troubled sides appended to a
 //   work list with warp-aggregated atomics) -> dense WENO-AO pass over that list ->
-//   [2D: raw tangential flags -> Gauss-point reconstruction (linear inline, troubled passes
-//   compacted the same way) -> dense WENO-AO pass] -> gas-kinetic flux per Gauss point
-// -> stage update.  dt is reduced, clipped to t_end and applied on the device.
+//   [2D: raw tangential flags -> spread flags and work list of the troubled passes -> dense
+//   WENO-AO pass] -> gas-kinetic flux per Gauss point (which reconstructs the smooth passes itself)
+// -> stage update.  Sweeps below 49152 segments take one launch per reconstruction direction instead
+// (k_normal_small, k_tang_small) and the flux with one side of a Gauss point per warp (k_flux_small).  dt is reduced, clipped to t_end and applied on the device.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -336,6 +337,27 @@ __device__ __forceinline__ void warp_push(unsigned int* cnt, uint32_t* list, boo
     if (pred) stc(list + base + __popc(mask & ((1u << lane) - 1u)), item, rg);
 }
 
+// The same for up to four items a lane, item | X for every set bit X of `bits`, with one atomic: the
+// appends of all warps of a sweep meet on one counter.
+template <class R>
+__device__ __forceinline__ void warp_push4(unsigned int* cnt, uint32_t* list, unsigned int bits, uint32_t item, const R& rg)
+{
+    unsigned int mask[4];
+    int total = 0;
+#pragma unroll
+    for (int X = 0; X < 4; X++) { mask[X] = __ballot_sync(0xffffffffu, (bits >> X) & 1u); total += __popc(mask[X]); }
+    if (!total) return;
+    const int lane = threadIdx.x & 31;
+    unsigned int base = 0;
+    if (lane == 0) base = atomicAdd(cnt, (unsigned int)total);
+    base = __shfl_sync(0xffffffffu, base, 0);
+#pragma unroll
+    for (int X = 0; X < 4; X++) {
+        if ((bits >> X) & 1u) stc(list + base + __popc(mask[X] & ((1u << lane) - 1u)), item | (uint32_t)X, rg);
+        base += __popc(mask[X]);
+    }
+}
+
 // ---------------------------------------------------------------- normal pass
 // local state access: component k of cell n on line t
 __device__ __forceinline__ const double* cellp(const Params& P, const Sweep& S, const double* W, int t, int n)
@@ -434,7 +456,7 @@ __device__ __forceinline__ void b_normal(const Params& P, const Sweep& S, const 
     }
     bool counted = active && t >= 0 && t < S.nt && m < S.nn;
     warp_count(&ctrl->troubled[stage][S.dir][0], counted && fl[1] ? 1u : 0u);
-    warp_count(&ctrl->examined[stage][S.dir][0], counted ? 1u : 0u);
+    if (id == 0) atomicAdd(&ctrl->examined[stage][S.dir][0], (unsigned long long)S.nt * S.nn);
 #pragma unroll
     for (int side = 0; side < 2; side++) {
         bool push = active && fl[side];
@@ -578,7 +600,9 @@ __global__ void k_normal_ao(const SolveDesc* D, int nb0, int stage)
 // Such a sweep's time is made of launches (3 us each) and of each thread's chain of FP64 instructions (31 ns
 // each): with one launch per direction in place of three (flags, linear pass, compacted WENO-AO) and the
 // step's five control and ghost launches in two, a step of 200 cells in 1D went from 133 to 90 us, of
-// 48 x 48 from 210 to 136.  Compaction and shared flags pay from about 49152 segments on
+// 48 x 48 from 210 to 136.  Compaction and shared flags pay from about 49152 segments on:
+// 200^2 (40200 segments) 714 us a step in this form, 749 in the other; 250^2 (62750) 990 and 941 (both before
+// launches overlapped the drain of the one before and the flux's last changes, which are common to both).
 constexpr int kSmallCells = 6;
 
 template <int NV>
@@ -671,44 +695,55 @@ __device__ __forceinline__ double lineval(const Sweep& S, int X, int k, int t, i
     return ldc(S.line + (long long)(X * 4 + k) * plane + (long long)(t - S.tlo) * S.nm + m, S);
 }
 
-// Large sweeps: each thread takes kTRows consecutive lines of one interface, so that a line value is
-// loaded and truncated once for up to 5 windows (8 rows instead of 20 for 4 segments).
+// Large sweeps: each thread takes kTRows consecutive lines of one interface and one of the four passes, so
+// that a line value is loaded and truncated once for up to 5 windows (8 rows instead of 20 for 4 segments);
+// the four warps of a group take the four passes of the same 32 items and combine their bits through
+// shared memory.  The launch lasts as long as its slowest warps, those on a shock, whose windows go
+// through the exact chains one after the other: with all four passes in one thread (64 windows instead of 16)
+// the four-quadrant step's launches took 64 us at 512^2 and 124 at 1024^2, so 36 and 106.
 constexpr int kTRows = 4;
+static_assert(kTRows == 4, "a warp of a group stores one row");
 
 __device__ __forceinline__ void b_raw_tflags(const Params& P, const Sweep& S, const Ctrl* ctrl, long long id)
 {
-    if (ctrl->done) return;
-    const int m = (int)(id % S.nm);
-    const int r0 = (int)(id / S.nm) * kTRows;              // row of rawT: line r0 - 1
+    if (ctrl->done) return;                                // the same for the block
+    __shared__ unsigned int words[512];                    // the block's threads (at most 512, a multiple of 128)
+    const int X = (int)(id >> 5) & 3, tid = threadIdx.x;
+    const unsigned item = (unsigned)(id >> 7) * 32u + (unsigned)(tid & 31);
+    const unsigned rg = item / (unsigned)S.nm;
+    const int m = (int)(item - rg * (unsigned)S.nm);
+    const int r0 = (int)rg * kTRows;                       // row of rawT: line r0 - 1
     const int rows = S.nt + 2 - r0 < kTRows ? S.nt + 2 - r0 : kTRows;
-    if (rows <= 0) return;
-    unsigned bits[kTRows] = {};
-    if (P.recon_mode == HGKS_RECON_HYBRID) {
+    unsigned word = 0;                                     // row r's bits in byte r
+    if (rows > 0 && P.recon_mode == HGKS_RECON_HYBRID) {
 #pragma unroll 1
-        for (int X = 0; X < 4; X++) {
-#pragma unroll 1
-            for (int k = 0; k < 4; k++) {
-                double q[kTRows + 4];
-                float f[kTRows + 4];
+        for (int k = 0; k < 4; k++) {
+            double q[kTRows + 4];
+            float f[kTRows + 4];
 #pragma unroll
-                for (int s = 0; s < kTRows + 4; s++) {
-                    // (lines past the last window repeat the last one: loaded, not used)
-                    q[s] = lineval(S, X, k, r0 - 3 + (s < rows + 4 ? s : rows + 3), m);
-                    f[s] = fixed::to_float(q[s]);
-                }
-#pragma unroll
-                for (int r = 0; r < kTRows; r++)
-                    if (r < rows) bits[r] |= (unsigned)indicator_raw<false>(q + r, f + r, S.Z1t) << X;
+            for (int s = 0; s < kTRows + 4; s++) {
+                // (lines past the last window repeat the last one: loaded, not used)
+                q[s] = lineval(S, X, k, r0 - 3 + (s < rows + 4 ? s : rows + 3), m);
+                f[s] = fixed::to_float(q[s]);
             }
+#pragma unroll
+            for (int r = 0; r < kTRows; r++)
+                if (r < rows) word |= (unsigned)indicator_raw<false>(q + r, f + r, S.Z1t) << (8 * r + X);
         }
     }
-#pragma unroll
-    for (int r = 0; r < kTRows; r++)
-        if (r < rows) stc(S.rawT + (long long)(r0 + r) * S.nm + m, bits[r], S);
+    words[tid] = word;
+    __syncthreads();
+    if (X < rows) {                                        // (pass X's warp stores row X)
+        const unsigned* w = words + (tid & ~127) + (tid & 31);
+        stc(S.rawT + (long long)(r0 + X) * S.nm + m, ((w[0] | w[32] | w[64] | w[96]) >> (8 * X)) & 0xFFu, S);
+    }
 }
 
 // Threads of the raw tangential flag kernel on sweep S.
-inline long long raw_t_threads(const Sweep& S) { return (long long)((S.nt + 2 + kTRows - 1) / kTRows) * S.nm; }
+inline long long raw_t_threads(const Sweep& S)
+{
+    return ((long long)((S.nt + 2 + kTRows - 1) / kTRows) * S.nm + 31) / 32 * 128;
+}
 
 __global__ void k_raw_tflags(const SolveDesc* D, int nb0)
 {
@@ -751,12 +786,10 @@ __device__ __forceinline__ void b_tang(const Params& P, const Sweep& S, Ctrl* ct
         stc(S.flagT + id, bits, S);
     }
     warp_count(&ctrl->troubled[stage][S.dir][1], active ? (unsigned)__popc(bits) : 0u);
-    warp_count(&ctrl->examined[stage][S.dir][1], active ? 4u : 0u);
-#pragma unroll
-    for (int X = 0; X < 4; X++) {
-        bool f = active && ((bits >> X) & 1);
-        warp_push(&ctrl->cnt[S.dir][1], S.itemsT, f, (uint32_t)((((long long)t * S.nm + m) << 2) | X), S);
-    }
+    // (a count known beforehand; with an atomic per warp for it and one per pass for the list the launch waited
+    // on those few addresses: 54 us at 1024^2, now 16)
+    if (id == 0) atomicAdd(&ctrl->examined[stage][S.dir][1], 4ull * (unsigned long long)total);
+    warp_push4(&ctrl->cnt[S.dir][1], S.itemsT, bits, (uint32_t)(((long long)t * S.nm + m) << 2), S);
 }
 
 __global__ void k_tang(const SolveDesc* D, int nb0, int stage)
@@ -1573,7 +1606,7 @@ cudaError_t launch_dfma_probe(cudaStream_t st, int blocks, int iters)
 }
 
 // ---------------------------------------------------------------- reciprocal check
-// The flux's Newton-refined reciprocal (rcp_nr) against IEEE division, and its reciprocal square
+// The flux's fixed-point reciprocal (rcp_nr) against IEEE division, and its reciprocal square
 // root (rsqrt_nr) against IEEE division by the IEEE square root, on n arguments spread
 // log-uniformly over 1e-8..1e8 (both signs for the reciprocal; splitmix64 hashes of the index);
 // the largest differences in units in the last place go to g_rcp_max_ulp[0], [1].

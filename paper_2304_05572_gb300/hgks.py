@@ -364,7 +364,7 @@ def hgks_debug_bounds():
 
 
 def hgks_check_reciprocal(n: int = 1 << 24):
-    """(1/x, 1/sqrt(x)): largest distances in ulps of the flux's Newton-refined reciprocal and
+    """(1/x, 1/sqrt(x)): largest distances in ulps of the flux's fixed-point reciprocal and
     reciprocal square root from their IEEE counterparts over n arguments (see include/hgks.h)."""
     u = (ctypes.c_ulonglong * 2)()
     rc = lib().hgks_check_reciprocal(int(n), u)
