@@ -176,9 +176,9 @@ typedef struct hgks_batch hgks_batch;
 #define HGKS_BATCH_AUTOTUNE 2   /* choose the block size of each kernel class on the first steps (see hgks_batch_step) */
 
 /* Group n >= 1 solvers of the same dimension on the current device.  One
- * batched step issues one launch per kernel class that any solver needs (at most 24 per
- * step in 2D, the sweep classes covering both sweeps; small and large sweeps have classes
- * of their own) whose blocks cover every solver's interfaces;
+ * batched step issues one launch per kernel class that any solver needs (at most 13 per
+ * stage beside the time step's and the ghost cells', the sweep classes covering both
+ * sweeps; small and large sweeps have classes of their own) whose blocks cover every solver's interfaces;
  * each block works for exactly one solver (and one sweep) with that solver's own
  * arithmetic, so every result is bit-identical
  * to stepping the solver alone.  The solvers keep their own state, dt, time and
