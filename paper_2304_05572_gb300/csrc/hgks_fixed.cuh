@@ -2,8 +2,8 @@
 // fixed point.
 //
 // The FP64 pipe of this part takes one warp instruction per 64 cycles and scheduler (measured
-// 65-76, comparisons and conversions from and to doubles included), while the integer pipe issues a 32 x 32 + 64 bit multiply-add in 2 and everything else in
-// 1 (a 64 x 64 -> 64 bit high product: 10-22).  A function whose arguments and results have a known
+// 65-76, comparisons and conversions from and to doubles included), while the integer pipe issues a
+// 32 x 32 + 64 bit multiply-add in 2 and everything else in 1 (a 64 x 64 -> 64 bit high product: 10-22).  A function whose arguments and results have a known
 // range is therefore cheaper in integers, at more bits than a double carries: each routine below
 // works with 61-63 fraction bits, rounds once, and is within one unit in the last place of the exact
 // result (tests/test_fixed_point.py, which compiles this header for the host).

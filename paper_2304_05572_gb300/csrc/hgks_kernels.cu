@@ -1237,7 +1237,7 @@ __device__ __forceinline__ void b_flux(const Params& P, const Sweep& S, Ctrl* ct
     store_flux<DIM, STAGE>(S, o, o0, o1);
 }
 
-// Small sweeps: the two sides of a Gauss point on two warps, so that a thread's chain is one side (about 190
+// Small sweeps: the two sides of a Gauss point on two warps, so that a thread's chain is one side (about 160
 // FP64 instructions) and, on the left side's warp, the sums' completion (about 150) instead of two sides and
 // the completion.  2D: 4 warps on the same 32 segments (side = warp & 1, Gauss point = warp >> 1 of the 4);
 // 1D: 2 warps.  The right side's sums and the second point's fluxes go through shared memory, one column
@@ -1338,7 +1338,8 @@ __device__ __noinline__ void flux_nl(const SolveDesc& d, int dir, long long id)
 
 // 64-thread blocks, at least 4 per SM: the register budget this leaves (up to 256 per thread at
 // 8 warps per SM) lets the flux keep its working set in registers (measured 3.5 % faster than
-// under a 128-thread bound at the same occupancy)
+// under a 128-thread bound at the same occupancy, when the flux took all 255; it takes 138 now, 174 with
+// the Prandtl fix)
 template <int DIM, int STAGE, bool PRFIX>
 __global__ void __launch_bounds__(64, 4) k_flux(const SolveDesc* D, int nb0)
 {

@@ -57,3 +57,27 @@ def test_flags_at_thresholds(scale, zeta1):
     assert np.array_equal(fg, want), int((fg != want).sum())
     if scale == 0:
         assert 0.05 < want.mean() < 0.999
+
+
+@pytest.mark.parametrize("nx,ny", [(7101, 7), (12300, 4), (9900, 5), (231, 230)])
+def test_large_sweep_tangential_flags_ragged(nx, ny):
+    """Sweeps from 49152 segments on: the flag kernel takes 4 lines and one pass per thread, 32 interfaces
+    per warp; sides that leave 1, 2, 3 and 0 lines in the last group and interfaces across the group edge.
+    First-stage flags are decided on identical inputs, so they and the counters are exact."""
+    from paper_2304_05572_gb300 import _build, hgks
+    _build.build()
+    oracle.build()
+    cfg, W, _ = P.riemann4_2d(nx, ny=ny)
+    fo = oracle.step_flags(cfg, W)[2]
+    g = hgks.Solver(cfg)
+    g.hgks_set_flag_capture(True)
+    g.hgks_set_state(W)
+    g.hgks_step(1e9, 1, wait=False)
+    st = g.hgks_get_stats()
+    for d in range(2):
+        fg = g.hgks_get_flags(0, d, 1)
+        assert np.array_equal(fg, fo[(0, d, "tang")]), d
+        assert fg.any()
+        assert st["troubled"][0, d, 1] == sum(bin(v).count("1") * int((fg == v).sum()) for v in range(16))
+        assert st["examined"][0, d, 1] == 4 * fg.size
+    g.hgks_destroy_solver()
