@@ -44,8 +44,10 @@ HGKS_FX u64 bits_of(double x) { u64 b; memcpy(&b, &x, 8); return b; }
 HGKS_FX double of_bits(u64 b) { double x; memcpy(&x, &b, 8); return x; }
 HGKS_FX u32 float_bits(float x) { u32 b; memcpy(&b, &x, 4); return b; }
 HGKS_FX float float_of(u32 b) { float x; memcpy(&x, &b, 4); return x; }
+#ifndef HGKS_FX_OWN_SEEDS               // (a check may bring seeds as far off as the hardware's may be)
 HGKS_FX float approx_rcp(float x) { return 1.0f / x; }
 HGKS_FX float approx_rsqrt(float x) { return 1.0f / std::sqrt(x); }
+#endif
 HGKS_FX int clz32(u32 x) { return __builtin_clz(x); }
 #endif
 
@@ -124,13 +126,20 @@ HGKS_FX double scale2(double x)
     return of_bits(((u64)h << 32) | (u32)b);
 }
 
+// A starting value for the two below: the approximation, which may lie a rounding outside [1/2, 1) at the
+// mantissa's ends, brought inside and as a fraction in 2^-32.
+HGKS_FX u32 seed(float y0)
+{
+    y0 = y0 < 0.99999994f ? y0 : 0.99999994f;
+    y0 = y0 > 0.5f ? y0 : 0.5f;
+    return (float_bits(y0) << 8) | 0x80000000u;
+}
+
 // 1/m for m in [1, 2) given in units of 2^-63, as r 2^-63, r in (2^62, 2^63], within 2 units: the 23-bit
 // reciprocal of the leading bits and one third-order Newton step, 1/m = y (1 + e + e^2), e = 1 - m y.
 HGKS_FX u64 rcp_mantissa(u64 m)
 {
-    float y0 = approx_rcp(float_of(0x3F800000u | (u32)(m << 1 >> 41)));
-    y0 = y0 < 0.99999994f ? y0 : 0.99999994f;                              // (1/2, 1)
-    const u32 y = (float_bits(y0) << 8) | 0x80000000u;                     // 2^-32
+    const u32 y = seed(approx_rcp(float_of(0x3F800000u | (u32)(m << 1 >> 41))));
     const u64 p = (u64)(u32)(m >> 32) * y + (((u64)(u32)m * y) >> 32);     // m y, 2^-63
     const i64 e = (i64)(0x8000000000000000ull - p);                        // |e| < 2^42
     const i64 eh = (int)(e >> 12);
@@ -142,9 +151,7 @@ HGKS_FX u64 rcp_mantissa(u64 m)
 // the same with 1/sqrt(m) = y (1 + e/2 + 3 e^2/8), e = 1 - m y^2.
 HGKS_FX u64 rsqrt_mantissa(u64 m, u32 frac, u32 odd)
 {
-    float y0 = approx_rsqrt(float_of((odd ? 0x3F800000u : 0x40000000u) | frac));
-    y0 = y0 < 0.99999994f ? y0 : 0.99999994f;
-    const u32 y = (float_bits(y0) << 8) | 0x80000000u;                     // 2^-32, [1/2, 1)
+    const u32 y = seed(approx_rsqrt(float_of((odd ? 0x3F800000u : 0x40000000u) | frac)));
     const u64 p = umulhi(m, (u64)y * y);                                   // m y^2, 2^-62
     const i64 e = (i64)(0x4000000000000000ull - p);                        // e in 2^-62 = e/2 in 2^-63
     const i64 eh = (int)(e >> 11);                                         // 2^-51
