@@ -178,7 +178,9 @@ __device__ __noinline__ int indicator_exact_nl(ex q0, ex q1, ex q2, ex q3, ex q4
 // FP32 with a margin above its rounding errors; only a test that falls inside its margin is decided by
 // the exact chain.
 //   Step 1: |D| against Z1 from the truncated window: truncation (2^-23) and four roundings (2^-24) of terms
-//     |c| m with coefficients summing to 20, m = max |q|: error below 20 m (2^-23 + 4 2^-24) = 7.2e-6 m.
+//     |c| m with coefficients summing to 20, m = max |q|: error below 20 m (2^-23 + 4 2^-24) = 7.2e-6 m.  A
+//     value below 2^-126 counts as 0, which adds up to 20 2^-126 = 2.4e-37: within the 1e-6 Z1 kept back
+//     for Z1 above 1e-30, below which the test is not taken.
 //   Steps 2, 3 on D, N, d = q3 - q1, s = (q1 + q3) - 2 q2, rounded as the exact chain rounds them (10 FP64
 //     operations): xbar = 1.7 N/D and xhat = -d/(2 s) (s = 2 ah2, the halves are exact), their FP32 ratios
 //     within 2^-20 relative; margins 1e-5.  Quantities outside 1e-30..1e30 go to the exact chain, and
@@ -194,7 +196,8 @@ __device__ __forceinline__ int indicator_raw(const double* q, const float* f, do
     const float m = fmaxf(fmaxf(fmaxf(fabsf(f[0]), fabsf(f[1])), fmaxf(fabsf(f[3]), fabsf(f[4]))), fabsf(f[2]));
     const float Df = fmaf(-10.0f, f[2], fmaf(4.0f, f[0], f[1]) + fmaf(4.0f, f[4], f[3]));
     // (an infinity among the f makes the sum infinite or a NaN: the comparison fails)
-    if (fmaf(8.0e-6f, m, fabsf(Df)) < 0.999999f * fixed::to_float(Z1)) return 0;
+    const float Zf = fixed::to_float(Z1);
+    if (Zf > 1e-30f && fmaf(8.0e-6f, m, fabsf(Df)) < 0.999999f * Zf) return 0;
     const ex q0(q[0]), q1(q[1]), q2(q[2]), q3(q[3]), q4(q[4]);
     const ex D = xfma(ex(-10.0), q2, xfma(ex(4.0), q0, q1) + xfma(ex(4.0), q4, q3));
     if (fixed::abs_le(D.v, Z1)) return 0;
