@@ -129,6 +129,22 @@ void fill_params(const hgks_config* c, Params& P)
     P.eps = c->eps;
 }
 
+// Small sweeps spread an item over lanes (shorter FP64 chains per thread) and take one launch per
+// reconstruction direction; the line is placed by measurement (see k_normal_small).  In 1D, where a sweep is the
+// normal pass and the flux alone, it lies lower when that pass may hold troubled sides, whose lane groups repeat
+// the eigenvectors: where a full pass gives every side a lane of its own in the compacted form.  us per step,
+// this form against the compacted one:
+//   WENO-AO everywhere, 16 400 / 20 000 / 49 000 cells: 205, 205 / 249, 212 / 563, 398; 64 solves of 16 400
+//     batched: 11 295, 6546;
+//   hybrid, nearly every side troubled, 64 solves of 20 000 / 30 000 cells batched: 13 770, 7639 / 20 620, 11 663;
+//   hybrid, Sod tube (few troubled sides) of 16 400 / 30 000 / 37 000 cells: 79, 92 / 105, 109 / 112, 110; 64
+//     solves of 16 400 batched: 2105, 1531.
+bool small_sweep(const hgks_config* c, const Sweep& S)
+{
+    if (c->dim == 1 && c->recon_mode != HGKS_RECON_LINEAR && 2 * (long long)S.nm >= kAoOneLaneMin) return false;
+    return (long long)S.nt * S.nm < 49152;
+}
+
 void fill_sweeps(const hgks_config* c, const Params& P, Sweep* sw)
 {
     const GridGeom& g = P.g;
@@ -141,9 +157,7 @@ void fill_sweeps(const hgks_config* c, const Params& P, Sweep* sw)
         S.nt = c->dim == 2 ? (d == 0 ? g.ny : g.nx) : 1;
         S.nm = S.nn + 1;
         S.nlines = c->dim == 2 ? S.nt + 6 : 1;
-        // small sweeps spread an item over lanes (shorter FP64 chains per thread) and take one launch per
-        // reconstruction direction; the line is placed by measurement (see k_normal_small)
-        S.small = (long long)S.nt * S.nm < 49152 ? 1 : 0;
+        S.small = small_sweep(c, S) ? 1 : 0;
         S.tlo = c->dim == 2 ? -3 : 0;
         S.sN = d == 0 ? 1 : g.pitch;
         S.sT = d == 0 ? g.pitch : 1;

@@ -15,6 +15,15 @@ namespace hgks {
 constexpr int NG = 4;            // ghost layers: the widest stencil (a Step-4 spread of 5-cell tests) reaches 4 cells
 constexpr int MAXNV = 4;
 
+// Troubled items of one compacted WENO-AO pass at or above which every item gets one lane, below
+// which an aligned group of 4 lanes (one characteristic field per lane).  The lane-group form
+// repeats the eigenvector work in each of its lanes (about 1.9 times the FP64 instructions per
+// item) and pays only while the items leave the schedulers short of warps; measured on this part
+// (512^2 and 1024^2 four-quadrant steps, 200x100 tube, thresholds 8192 / 32768 / 131072) the
+// crossover lies near 32768 items.  A constant, not a function of the launch, so that a solve
+// takes the same form in its own kernels and in batched ones.
+constexpr unsigned int kAoOneLaneMin = 32768;
+
 // Device control block of one solver: time, dt, status and counters.  All
 // step logic that would otherwise need a host round trip lives here.
 struct Ctrl {
@@ -48,7 +57,7 @@ struct Sweep {
     int nn, nt;                // cells normal / tangential
     int nm;                    // interfaces per line (nn + 1)
     int nlines;                // lines with normal reconstruction (nt + 6 in 2D, 1 in 1D)
-    int small;                 // below 49152 interface segments: one launch per reconstruction direction (lane groups)
+    int small;                 // one launch per reconstruction direction (lane groups): see small_sweep in hgks_api.cu
     int tlo;                   // first line index (-3 in 2D, 0 in 1D)
     long long sN, sT;          // state strides for +1 in n / t
     int perm[4];               // local component -> global component
