@@ -1,6 +1,7 @@
 // hgks_api.cu -- the C ABI of the solver (declared in include/hgks.h): configuration
 // checks, the device memory pool of a solver, state transfer, the step loop, parity
 // hooks (flags), per-kernel timing and batched stepping.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -336,15 +337,38 @@ extern "C" const char* hgks_last_error(const hgks_solver* s)
     return s ? s->err : g_create_err;
 }
 
-// Plain device memory of the solver's device: a kernel may read and write it directly (memory of another
-// device, managed or mapped memory goes through the runtime's copies).
+// The start and size of the allocation that a device address lies in (the driver's cuMemGetAddressRange, looked
+// up once); false if it knows none.
+static bool allocation_of(const void* p, uintptr_t& base, size_t& size)
+{
+    typedef CUresult (*Query)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Query query = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (Query)f : nullptr;
+    }();
+    CUdeviceptr b = 0;
+    if (!query || query(&b, &size, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return false;
+    base = (uintptr_t)b;
+    return true;
+}
+
+// A state in plain device memory of the solver's device that lies whole in one allocation: a kernel may read and
+// write it directly.  Memory of another device, managed or mapped memory, and a buffer that reaches past its
+// allocation go through the runtime's copies, which refuse what they always refused.
 static bool own_device_memory(const hgks_solver* s, const void* p)
 {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { (void)cudaGetLastError(); return false; }
     int dev = -1;
+    uintptr_t base = 0;
+    size_t size = 0;
+    const GridGeom& g = s->P.g;
     return a.type == cudaMemoryTypeDevice && a.device == s->device && cudaGetDevice(&dev) == cudaSuccess && dev == s->device
-           && (uintptr_t)p % sizeof(double) == 0;
+           && (uintptr_t)p % sizeof(double) == 0 && allocation_of(p, base, size)
+           && inside_allocation(base, size, (uintptr_t)p, (size_t)g.nv * g.ny * g.nx * sizeof(double));
 }
 
 extern "C" int hgks_set_state(hgks_solver* s, const double* W, int on_device, double t0)

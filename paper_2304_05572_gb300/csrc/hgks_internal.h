@@ -24,6 +24,12 @@ constexpr int MAXNV = 4;
 // takes the same form in its own kernels and in batched ones.
 constexpr unsigned int kAoOneLaneMin = 32768;
 
+// Whether [p, p + bytes) lies in the allocation [base, base + size).
+inline bool inside_allocation(uintptr_t base, size_t size, uintptr_t p, size_t bytes)
+{
+    return p >= base && bytes <= size && p - base <= size - bytes;
+}
+
 // Device control block of one solver: time, dt, status and counters.  All
 // step logic that would otherwise need a host round trip lives here.
 struct Ctrl {
