@@ -25,10 +25,10 @@ The default line also carries
 Other workloads (--workload batched | served | recon_cost | ns_tube | vortex) print
 their own line.
 
-The roofline is FP64-ALU bound: the numerator counts the algorithmic FP64 work (fixed
-counts, see FLUX_ALG_FLOP_PER_GP); the peak is the device's SM count x 4 FP64 flop per
-clock x the SM clock sampled during the timed region, with the DFMA-chain probe
-(hgks_probe_fp64) reported beside it.
+The roofline is bound by the FP64 pipe: the numerator counts the instructions that run on
+it (FLUX_FP64_INSTR_PER_GP, STEP_FP64_INSTR_PER_CELL_STAGE), the peak is the device's SM
+count x 2 such instructions per clock x the SM clock sampled during the timed region, with
+the DFMA-chain probe (hgks_probe_fp64) and the algorithmic operation rate beside it.
 
 --impl reference times the CPU oracle (the plain FP64 restatement of the
 paper's method) on the host cores, on the same 1024^2 problem.
@@ -55,14 +55,25 @@ UNIT = "Mcell-stage/s"
 N_SIDE = 1024
 WORKLOAD = "four-quadrant 2D Riemann problem, 1024^2 cells, hybrid WENO-AO HGKS, S2O4"
 
-# Algorithmic FP64 work of the step (add / sub, mul, div, sqrt, exp and erfc count one each, fma
-# two), of the algorithm as the kernels now run it (a change of the algebra moves it):
+# Roofline.  The FP64 pipe takes one warp instruction per 64 cycles and scheduler, whatever it is (an FMA as
+# an addition, a comparison or a conversion), so the numerators are the instructions that run on it and the
+# denominator is that issue rate.  Counts by ncu (smsp__inst_executed_pipe_fp64, lane instructions = 32 per warp
+# instruction) on one 1024^2 four-quadrant step, 0.58 % of its passes troubled
+# (profiles/step_kernels_riemann512_ncu.md): 494 and 446 per Gauss point of the two stages' flux launches on
+# sweeps of 49 152 segments or more (the launch covers both sweeps and reconstructs the smooth tangential passes
+# in integers); 2162 per cell-stage of the whole step.
+FLUX_FP64_INSTR_PER_GP = (494.0 + 446.0) / 2
+STEP_FP64_INSTR_PER_CELL_STAGE = 2162.0
+FP64_INSTR_PER_CLOCK_AND_SM = 2.0          # 4 schedulers x 32 lanes / 64 cycles
+
+# Algorithmic FP64 work of the step (add / sub, mul, div, sqrt, exp and erfc count one each, fma two), of the
+# algorithm as the kernels now run it (a change of the algebra moves it).  Quotients, roots, exp, erfc, the
+# Gauss-point quartics and most of the indicator run in integer and FP32 units, so this rate is no share of the
+# FP64 peak and is printed without one:
 # * the flux per Gauss point: the closed form of the flux kernel (2D Euler, tau > 0), counted on
 #   the host by paper_2304_05572_gb300/flopcount.py: 829 operations in the first stage (F(dt/2)
 #   and the F^n + dt/6 dF^n combination), 756 in the second (1433 and 1389 with lab-frame moments
-#   and solved micro-slopes); part of them (the quotients, roots, exp, erfc and the Gauss-point
-#   quartics) runs in integer units, so the fraction of the FP64 peak may pass the FP64 pipe's
-#   own utilisation; on sweeps of 49 152 segments or
+#   and solved micro-slopes); on sweeps of 49 152 segments or
 #   more the kernel also reconstructs its Gauss point's smooth tangential passes
 #   (FLUX_KERNEL_TANG_FLOP_PER_GP); one launch covers both sweeps of a stage;
 # * the rest of the step per cell-stage (indicator, reconstruction, update, time step), counted on
@@ -71,8 +82,7 @@ WORKLOAD = "four-quadrant 2D Riemann problem, 1024^2 cells, hybrid WENO-AO HGKS,
 #   19486.7, the hybrid step 3525.5 at its troubled fraction 0.41 %; a run at another troubled
 #   fraction f moves the hybrid figure along the troubled-minus-smooth slope.  (The oracle's own
 #   flux integrates every moment literally, ORACLE_FLUX_FLOP_PER_GP operations, nine times the
-#   closed form: a roofline on that count would exceed the peak, so the flux enters with its
-#   closed-form count.)
+#   closed form, and does not enter.)
 FLUX_ALG_FLOP_PER_GP = (829.0 + 756.0) / 2
 ORACLE_FLUX_FLOP_PER_GP = 7025.0
 # On large sweeps the flux kernel also reconstructs its Gauss point's smooth tangential passes
@@ -82,11 +92,32 @@ ORACLE_FLUX_FLOP_PER_GP = 7025.0
 FLUX_KERNEL_TANG_FLOP_PER_GP = 16 * 9 + 8 * 9 + 2 * 6 + 8
 NONFLUX_FLOP_PER_CELL_STAGE = {"linear": 2721.3, "wenoao": 19486.7, "hybrid": 3525.5,
                                "hybrid_troubled_fraction": 0.004106}
-# DRAM bytes (read + write) per flux launch (both sweeps), one ncu pass over a whole 1024^2 step
-# with the caches carried from kernel to kernel (--cache-control none), as the step runs: first
-# stage 275.5 MB read + 118.6 MB written, second stage 275.6 + 61.5 MB; per Gauss point of the
-# launch (4 * 1024 * 1025 of them).
-FLUX_DRAM_BYTES_PER_GP = (275.49e6 + 118.56e6 + 275.58e6 + 61.50e6) / 2 / (4 * 1024 * 1025)
+# DRAM bytes (read + write) per flux launch (both sweeps) of a 1024^2 step with the caches carried from
+# kernel to kernel (ncu --cache-control none), as the step runs: first stage 276.5 MB read + 122.3 MB written,
+# second stage 276.1 + 64.2 MB; per Gauss point of the launch (4 * 1024 * 1025 of them).
+FLUX_DRAM_BYTES_PER_GP = (276.53e6 + 122.28e6 + 276.09e6 + 64.22e6) / 2 / (4 * 1024 * 1025)
+
+
+def fp64_issue_peak(n_sm, mhz):
+    """FP64 instructions (lanes) per second that n_sm SMs can issue at mhz."""
+    return n_sm * FP64_INSTR_PER_CLOCK_AND_SM * mhz * 1e6
+
+
+def flux_roofline(n, avg_launch_ms, n_sm, mhz):
+    """(achieved, peak, fraction) of the n^2 step's flux launches, in FP64 instructions a second; None on
+    sweeps below 49 152 segments, whose flux kernel is another."""
+    if n * (n + 1) < 49152:
+        return None
+    achieved = FLUX_FP64_INSTR_PER_GP * 4 * n * (n + 1) / (avg_launch_ms * 1e-3)
+    peak = fp64_issue_peak(n_sm, mhz)
+    return achieved, peak, achieved / peak
+
+
+def step_roofline(mcell_stages_per_s, n_sm, mhz):
+    """The same of the whole step, from one GPU's rate in Mcell-stage/s."""
+    achieved = STEP_FP64_INSTR_PER_CELL_STAGE * mcell_stages_per_s * 1e6
+    peak = fp64_issue_peak(n_sm, mhz)
+    return achieved, peak, achieved / peak
 
 
 def algorithmic_flop_per_cell_stage(n, troubled_fraction):
@@ -629,49 +660,51 @@ def main():
     e2e_value = replica_throughput(world, cells, e2e_steps, e2e_s)
     state_bytes = int(W0.nbytes)
 
-    # ---- FP64 peak of this GPU: the SM count of the device x 4 FP64 flop per clock and SM (two
-    # FP64 instruction issues, the unit count behind the nominal 1.25 TFLOP/s) x the median SM clock
-    # of the timed region.  The DFMA-chain probe (its clock sampled while it runs) is reported
-    # beside it: chains of one FP64 operation reach 84 % of that issue rate, while the flux kernel's
-    # instruction mix reaches 90 % (ncu), so the probe is not a ceiling and the unit count is.
+    # ---- FP64 issue rate of this GPU at the median SM clock of the timed region.  The DFMA-chain probe (its
+    # clock sampled while it runs) is reported beside it: chains of one FP64 operation reach 84 % of that issue
+    # rate, while the flux kernel's instruction mix reaches 88 % (ncu), so the probe is not a ceiling.
     clocks = clk.summary()
     with ClockSampler(local_rank if "CUDA_VISIBLE_DEVICES" not in os.environ else 0) as clkp:
         probe_tflops, probe_ms, n_sm = hgks.hgks_probe_fp64(stream)
     probe_mhz = clkp.summary()["sm_mhz"] or clocks["sm_mhz"]
     run_mhz = clocks["sm_mhz"] or probe_mhz or 2070.0
-    peak_tflops = n_sm * 4 * run_mhz / 1e6
 
-    # ---- dominant kernel roofline (FP64 ALU) on the algorithmic count
+    # ---- dominant kernel roofline (FP64 pipe)
     flux_ms, flux_calls = timing.get("gks_flux", (0.0, 0))
     launches = int(stats.get("launches", 0)) - launches0     # kernels of the timed steps only
     roofline = None
-    if flux_calls:
+    fr = flux_roofline(n, flux_ms / flux_calls, n_sm, run_mhz) if flux_calls else None
+    if fr:
         avg_ms = flux_ms / flux_calls
         gp_per_launch = 2 * 2 * (n + 1) * n      # Gauss points of both sweeps (one launch per stage)
-        # the kernel's work per Gauss point: the flux, and on sweeps of 49 152 segments or more the
-        # fused reconstruction of the smooth tangential passes
-        per_gp = FLUX_ALG_FLOP_PER_GP + (FLUX_KERNEL_TANG_FLOP_PER_GP if n * (n + 1) >= 49152 else 0.0)
-        achieved = per_gp * gp_per_launch / (avg_ms * 1e-3) / 1e12
-        roofline = {"bound": "alu", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
-                    "frac": achieved / peak_tflops,
+        # the kernel's algorithmic work per Gauss point: the flux and the fused reconstruction of the
+        # smooth tangential passes
+        per_gp = FLUX_ALG_FLOP_PER_GP + FLUX_KERNEL_TANG_FLOP_PER_GP
+        roofline = {"bound": "alu", "achieved": fr[0] / 1e12, "peak": fr[1] / 1e12, "unit": "T FP64 instructions/s",
+                    "frac": fr[2],
                     "traffic": FLUX_DRAM_BYTES_PER_GP * gp_per_launch if n == N_SIDE else None,
                     "kernel": "gks_flux", "avg_launch_ms": avg_ms,
-                    "flop_per_launch": per_gp * gp_per_launch,
-                    "unit_of_work": "Gauss point: %.0f algorithmic FP64 operations = flux %.0f (closed form; the "
-                                    "oracle's literal moment integration takes %.0f) + reconstruction of the smooth "
-                                    "tangential passes %.0f" % (per_gp, FLUX_ALG_FLOP_PER_GP, ORACLE_FLUX_FLOP_PER_GP,
-                                                                 per_gp - FLUX_ALG_FLOP_PER_GP),
-                    "peak_note": "derived: %d SMs (device attribute) x 4 FP64 flop/clk/SM x %s MHz (median SM "
+                    "fp64_instr_per_launch": FLUX_FP64_INSTR_PER_GP * gp_per_launch,
+                    "algorithmic": {"tflops": per_gp * gp_per_launch / (avg_ms * 1e-3) / 1e12,
+                                    "flop_per_launch": per_gp * gp_per_launch,
+                                    "note": "per Gauss point %.0f algorithmic operations = flux %.0f (closed form; the "
+                                            "oracle's literal moment integration takes %.0f) + reconstruction of the "
+                                            "smooth tangential passes %.0f; part of them runs in integer units"
+                                            % (per_gp, FLUX_ALG_FLOP_PER_GP, ORACLE_FLUX_FLOP_PER_GP,
+                                               FLUX_KERNEL_TANG_FLOP_PER_GP)},
+                    "unit_of_work": "Gauss point: %.0f instructions on the FP64 pipe (ncu)" % FLUX_FP64_INSTR_PER_GP,
+                    "peak_note": "derived: %d SMs (device attribute) x 2 FP64 instructions/clk/SM x %s MHz (median SM "
                                  "clock of the timed region); the DFMA-chain probe hgks_probe_fp64 gives %.3f "
                                  "TFLOP/s at %s MHz (%.2f flop/clk/SM)"
                                  % (n_sm, run_mhz, probe_tflops, probe_mhz,
                                     probe_tflops * 1e6 / (n_sm * probe_mhz) if probe_mhz else float("nan"))}
     shares = {k: round(v[0] / max(1e-9, sum(x[0] for x in timing.values())), 4) for k, v in timing.items() if v[1]}
-    if roofline is not None and NONFLUX_FLOP_PER_CELL_STAGE["hybrid"] is not None:
+    if roofline is not None:
         fpcs = algorithmic_flop_per_cell_stage(n, float(troubled))
-        step_tflops = fpcs * value / world * 1e6 / 1e12
-        roofline["whole_step"] = {"flop_per_cell_stage": fpcs, "achieved": step_tflops,
-                                  "frac": step_tflops / peak_tflops, "unit": "TFLOP/s",
+        sr = step_roofline(value / world, n_sm, run_mhz)
+        roofline["whole_step"] = {"fp64_instr_per_cell_stage": STEP_FP64_INSTR_PER_CELL_STAGE, "achieved": sr[0] / 1e12,
+                                  "frac": sr[2], "unit": "T FP64 instructions/s",
+                                  "algorithmic": {"flop_per_cell_stage": fpcs, "tflops": fpcs * value / world / 1e6},
                                   "troubled_fraction": float(troubled)}
 
     line = {
@@ -690,8 +723,7 @@ def main():
         "kernel_time_share": shares,
         # the same throughput with the dt reduction and the ghost fills taken out (the value above
         # is the whole step, those included)
-        "value_without_dt_and_ghost": value / max(1e-9, 1.0 - shares.get("dt", 0.0) - shares.get("ghost", 0.0)
-                                                  - shares.get("misc", 0.0)),
+        "value_without_dt_and_ghost": value / max(1e-9, 1.0 - shares.get("dt", 0.0) - shares.get("ghost", 0.0)),
         "clocks": clocks,
         "wall_s_timed": t_wall,
     }
