@@ -1001,14 +1001,14 @@ __device__ __forceinline__ void b_tang_small(const Params& P, const Sweep& S, co
 }
 
 // Blocks of the small tangential launch on sweep S with `rows` lines a block; rows from the number of blocks
-// that leaves: up to 8 while a launch still has 16 blocks for each of 152 SMs.
+// that leaves: up to 8 while a launch still has 16 blocks for each SM.
 inline long long tang_small_blocks(const Sweep& S, int rows)
 {
     return (long long)((S.nm + kSmallCols - 1) / kSmallCols) * ((S.nt + rows - 1) / rows);
 }
-inline int tang_small_rows(long long blocks1)     // blocks1: blocks of the whole launch with one line a block
+inline int tang_small_rows(long long blocks1, int sms)     // blocks1: blocks of the whole launch with one line a block
 {
-    const long long r = blocks1 / (16 * 152);
+    const long long r = blocks1 / (16 * sms);
     return r < 1 ? 1 : r > kSmallRowsMax ? kSmallRowsMax : (int)r;
 }
 
@@ -1739,7 +1739,7 @@ static void enqueue_sweeps(hgks_solver* s, int stage)
             timed(s, KC_TANG, 1, [&] { launch_chained(k_tang, g, TPB, 0, st, D, (int)nb[0], stage); });
         if ((g = pair(LARGE, [&](const Sweep& S) { return ao_blocks((long long)S.nt * S.nm * 4 * 4); })))
             timed(s, KC_TANG_AO, 1, [&] { launch_chained(k_tang_ao, g, 128, 0, st, D, (int)nb[0], stage); });
-        const int rows = tang_small_rows(pair(SMALL, [](const Sweep& S) { return (unsigned)tang_small_blocks(S, 1); }));
+        const int rows = tang_small_rows(pair(SMALL, [](const Sweep& S) { return (unsigned)tang_small_blocks(S, 1); }), sms);
         if ((g = pair(SMALL, [&](const Sweep& S) { return (unsigned)tang_small_blocks(S, rows); })))
             timed(s, KC_TANG, 1, [&] { launch_chained(k_tang_small, g, kSmallTangBlock, 0, st, D, (int)nb[0], stage, rows); });
     }
@@ -1874,7 +1874,7 @@ void batch_plan(const std::vector<const SolveDesc*>& descs, int dim, const int* 
     for (int c = 0; c < BK_COUNT; c++) plan.tpb[c] = tpb[c];
     long long blocks1 = 0;
     for (int u = 0; u < 2 * n; u++) blocks1 += batch_unit_blocks(*descs[u >> 1], dim, BK_TSMALL, u & 1, tpb[BK_TSMALL], 1);
-    plan.tang_rows = tang_small_rows(blocks1);
+    plan.tang_rows = tang_small_rows(blocks1, device_sm_count());
     plan.boff.assign((size_t)BK_COUNT * stride, 0);
     for (int c = 0; c < BK_COUNT; c++) {
         int* bo = plan.boff.data() + (size_t)c * stride;
