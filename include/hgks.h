@@ -317,8 +317,8 @@ int hgks_check_reciprocal(long long n, unsigned long long* max_ulp);
  * looks up the array's device address (cudaGetSymbolAddress, with that device
  * current); make that first call before any stream capture.  All calls share
  * the one array: calls whose work overlaps on the GPU race and corrupt each
- * other, so issue them one after another (for example on one stream).  Each
- * call clears the array before use.
+ * other, so issue them one after another (for example on one stream).  No
+ * call's result depends on what an earlier one left in the array.
  * Errors: HGKS_EINVAL (bad config, NULL buffer, grid too large), HGKS_ECUDA;
  * the message is in hgks_last_error(NULL), kept per calling thread. */
 int hgks_step_noalloc(const hgks_config* cfg, const double* W_in, double* W_out, int* status, void* stream);

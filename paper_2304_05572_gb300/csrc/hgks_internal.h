@@ -71,7 +71,7 @@ struct Sweep {
     uint8_t* rawN;             // [nlines][nn + 4]   raw normal flags, cells -2..nn+1
     uint8_t* flagN;            // [nlines][nn + 2]   final normal flags, cells -1..nn
     double* line;              // [4][nv][nlines][nm] Q^l, Q^r, Q^l_n, Q^r_n
-    uint8_t* rawT;             // [nt + 4][nm]       raw tangential flag bits, lines -2..nt+1
+    uint8_t* rawT;             // [nt + 2][nm]       raw tangential flag bits, lines -1..nt
     uint8_t* flagT;            // [nt][nm]           final tangential flag bits
     double* gp;                // [2][6][nv][nt][nm] Gauss-point states
     double* flux;              // [2][nv][nt][nm] segment fluxes (Gauss points combined; global component order)

@@ -6,8 +6,10 @@
 //   work list with warp-aggregated atomics) -> dense WENO-AO pass over that list ->
 //   [2D: raw tangential flags -> spread flags and work list of the troubled passes -> dense
 //   WENO-AO pass] -> gas-kinetic flux per Gauss point (which reconstructs the smooth passes itself)
-// -> stage update.  Sweeps below 49152 segments take one launch per reconstruction direction instead
-// (k_normal_small, k_tang_small) and the flux with one side of a Gauss point per warp (k_flux_small).  dt is reduced, clipped to t_end and applied on the device.
+// -> stage update.  Small sweeps (small_sweep in hgks_api.cu: below 49152 segments, in 1D below 16384 interfaces
+// unless linear) take one launch per reconstruction direction instead (k_normal_small, k_tang_small) and the flux
+// with one side of a Gauss point per warp (k_flux_small).  dt is reduced, clipped to t_end and applied on the
+// device.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -591,9 +593,13 @@ __global__ void k_normal_ao(const SolveDesc* D, int nb0, int stage)
 // Such a sweep's time is made of launches (3 us each) and of each thread's chain of FP64 instructions (31 ns
 // each): with one launch per direction in place of three (flags, linear pass, compacted WENO-AO) and the
 // step's five control and ghost launches in two, a step of 200 cells in 1D went from 133 to 90 us, of
-// 48 x 48 from 210 to 136.  Compaction and shared flags pay from about 49152 segments on:
-// 200^2 (40200 segments) 714 us a step in this form, 749 in the other; 250^2 (62750) 990 and 941 (both before
-// launches overlapped the drain of the one before and the flux's last changes, which are common to both).
+// 48 x 48 from 210 to 136.  Compaction and shared flags pay on larger sweeps.  The line of 49152 segments was placed
+// when 200^2 (40200 segments) took 714 us a step in this form against 749 in the other, 250^2 990 against 941.
+// With the present kernels (us per step, this form against the other; both forms' flux included) the two
+// meet lower, and the line has not been moved since:
+//   four-quadrant 64^2 173, 224; 100^2 257, 287; 141^2 377, 389; 180^2 523, 461; 200^2 626, 547; 221^2 744, 612;
+//   viscous tube with the Prandtl fix 200 x 100 364, 418; 280 x 140 604, 616; 312 x 156 726, 718;
+//   WENO-AO everywhere 64^2 280, 275; 100^2 563, 526; 200^2 2041, 1591.
 constexpr int kSmallCells = 6;
 
 template <int NV>

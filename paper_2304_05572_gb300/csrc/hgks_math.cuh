@@ -187,9 +187,9 @@ __device__ __noinline__ int indicator_exact_nl(ex q0, ex q1, ex q2, ex q3, ex q4
 //     s = 0 does unless d = 0, where xhat = 0.
 // The exact chain takes 5 FP64 slots of the pipe on smooth data and, behind Step 1, four IEEE
 // divisions more, where one troubled lane holds up its warp.  Raw flags per step at 1024^2: normal
-// 253 -> 160 us, tangential 702 -> 251 us (with the shared row loads of b_raw_tflags_x1).
-// CALL: the exact chain behind a call, where three windows a thread would otherwise unroll it three times
-// (a call costs the large sweeps' tangential flags 20 %, 254 -> 300 us at 1024^2).
+// 253 -> 163 us, tangential 702 -> 220 us (with the shared row loads of b_raw_tflags).
+// CALL: the exact chain behind a call, for b_tang_small, whose three uses would each hold a copy of it (the
+// large sweeps' tangential flags unroll four and are 31 % slower behind a call: 220 -> 288 us at 1024^2).
 template <bool CALL>
 __device__ __forceinline__ int indicator_raw(const double* q, const float* f, double Z1)
 {
